@@ -247,7 +247,8 @@ nd_status nd_autotune(nd_incidence* inc, int32_t passes, void* stream, int32_t* 
 /* Counters of the last nd_snd / nd_and / nd_iterate_k call on this handle,
  * pass by pass: changed[i] = r-cliques whose tau changed in pass i,
  * evaluated[i] = h-index evaluations in pass i (active r-cliques for AND),
- * incidences[i] = incidences (s-cliques) streamed by those evaluations.
+ * incidences[i] = incidences (s-cliques) of the evaluated r-cliques; an
+ * evaluation that is settled before the end of its row reads only a part.
  * Any array may be NULL.  Fills at most cap entries and returns the number
  * of passes in *passes. */
 nd_status nd_last_passes(const nd_incidence* inc, int64_t* changed, int64_t* evaluated, int64_t* incidences,

@@ -16,11 +16,16 @@
 //   3. otherwise H lies in [count, tau(R)) and is found by binary search on
 //      h over the register-resident rho values, testing
 //      #{rho >= h} >= h (Def. 3).  No histogram, no sort.
-// A warp or a CTA (longer rows) streams its row instead: one pass counts
-// rho >= tau(R); if that fails, each further pass bins rho into at most 256
-// shared-memory counters over the interval [lo, hi) that holds H, and the
-// suffix sums at the bin edges cut the interval 256-fold, so H is exact after
-// 1-2 more streaming passes whatever the row length.
+// A warp or a CTA (longer rows) streams its row instead (warp_hindex): it
+// counts rho >= tau(R) and stops at tau(R) of them; a row that fails, or is
+// expected to, goes through a shared-memory histogram of rho over the values
+// that can be H, whose suffix sums give H.
+// What bounds a pass: the L1 wavefronts of the gathers, and in the early
+// passes the instructions of the search.  R-MAT scale-20 k-truss (1.17G
+// incidences), SND to convergence in 57 passes: 113.1 ms, against 184.3 ms
+// with 64-bit row offsets, a runtime division per binned value, whole rows
+// read in every pass and 16-bit values cached in shared memory between a
+// count and its search; AND 53.0 against 72.9 ms, AND-nn 63.6 against 105.8.
 // The paper's linear-time hashmap h-index (Section 4.4) is replaced by this
 // tau-bounded count; both compute Def. 3 exactly.
 //
@@ -36,24 +41,15 @@
 // slot, and the frontier has one bit per slot.  k_pass_otf is the same update
 // with no stored incidence: it finds each edge's triangles again by
 // intersecting adjacency lists on every pass.
-#include <cooperative_groups.h>
-#include <cooperative_groups/reduce.h>
-
 #include "nd_internal.cuh"
-
-namespace cg = cooperative_groups;
 
 namespace {
 
 constexpr int kThreads = 256;
-#ifndef ND_WARP_UNROLL
-#define ND_WARP_UNROLL 4  // streamed incidences in flight per lane (warp / CTA rows)
-#endif
-constexpr int kWarpUnroll = ND_WARP_UNROLL;
 #ifndef ND_WARP_CHUNK
 #define ND_WARP_CHUNK 16  // consecutive warp tasks per counter grab
 #endif
-constexpr int kWarpChunk = ND_WARP_CHUNK;
+constexpr int kWarpChunk = ND_WARP_CHUNK;  // at most: pass_chunk
 #ifndef ND_NOTIFY_UNROLL
 #define ND_NOTIFY_UNROLL 4  // notification entries in flight per lane ((2,3))
 #endif
@@ -75,20 +71,21 @@ __device__ __forceinline__ uint32_t ld_front(const uint32_t* p) {
     return __ldcg(p);
 #endif
 }
-#ifndef ND_CORE_AND_CTA_FIRST
-#define ND_CORE_AND_CTA_FIRST 1  // (1,2) AND: the CTA rows (hub vertices) before the warp tasks
-#endif
-#ifndef ND_RHO_CACHE
-#define ND_RHO_CACHE 1024  // rho values a warp keeps in shared memory for the search passes (0 = none)
-#endif
-constexpr int kRhoCache = ND_RHO_CACHE;
+// histogram words per warp: 512 bins in the passes where most rows search, 256
+// in the late ones.  Every KB of them is taken from L1 and its gathers.
+// Measured (R-MAT scale-20 k-truss / scale-24 k-core / Chung-Lu 100K (3,4)):
+// the first 16 SND passes 43.2 / 24.0 / 18.6 ms with 256 words, 44.0 / 25.7 /
+// 20.3 with 512; passes 17-32 28.3 / 20.7 / 17.8 ms with 128 words, 29.0 /
+// 20.5 / 17.5 with 256.
+constexpr int kHistWords = 256;
+constexpr int kLateHistWords = 128;
+static_assert(kHistWords % 128 == 0 && kLateHistWords % 128 == 0, "cleared and selected in blocks of 128 words");
 
 // Work of one pass: rows longer than the CTA threshold are taken one per
 // block from a per-pass counter; all other rows form warp tasks that warps
 // take in chunks from a second counter.
 
 struct SweepParams {
-    const int64_t* __restrict__ inc_ptr;
     const uint32_t* __restrict__ inc;
     const int32_t* tin;   // SND: tau of the previous pass; AND: same array as tout
     int32_t* tout;
@@ -108,6 +105,8 @@ struct SweepParams {
     const int32_t* __restrict__ ev;
     const nd_item* __restrict__ items;
     int64_t lo[ND_NB], hi[ND_NB];  // bucket ranges in items
+    int chunk;                     // warp tasks per counter grab (pass_chunk)
+    bool direct;                   // AND: rows are expected to fail the count (see warp_hindex)
     const uint32_t* cur;  // AND + notification: frontier read in this pass
     uint32_t* next;       // and the frontier written for the next pass
     const uint32_t* members;  // PartialAnd: only members are notified (null = everyone)
@@ -150,38 +149,38 @@ __device__ __forceinline__ uint32_t ld_id(const uint32_t* p) {
     return RO ? __ldcs(p) : __ldg(p);
 }
 
-template <int Q, bool RO, typename T>
-__device__ __forceinline__ int32_t rho_at(const uint32_t* __restrict__ inc, const T* tau, int64_t j) {
-    if (Q == 1) {
-        return ld_tau<RO>(tau + ld_id<RO>(inc + j));
-    } else if (Q == 2) {
-        const uint2* p = reinterpret_cast<const uint2*>(inc) + j;
-        uint2 id = RO ? __ldcs(p) : __ldg(p);
-        return min(ld_tau<RO>(tau + id.x), ld_tau<RO>(tau + id.y));
-    } else {
-        const uint32_t* p = inc + 3 * j;
-        uint32_t a = ld_id<RO>(p), b = ld_id<RO>(p + 1), c = ld_id<RO>(p + 2);
-        return min(min(ld_tau<RO>(tau + a), ld_tau<RO>(tau + b)), ld_tau<RO>(tau + c));
-    }
-}
-
-// rho of incidence j, as a functor for the h-index routines below
+// rho of entry j of a row, as a functor for the h-index routines below: the
+// row's base address once, 32-bit offsets from it (the passes are bound by
+// instructions as much as by the gathers; 64-bit offsets per entry cost both
+// registers and issue slots)
 template <int Q, bool RO, typename T>
 struct Rho {
-    const uint32_t* __restrict__ inc;
+    const uint32_t* __restrict__ row;
     const T* tau;
-    __device__ __forceinline__ int32_t operator()(int64_t j) const { return rho_at<Q, RO>(inc, tau, j); }
+    __device__ __forceinline__ int32_t operator()(int j) const {
+        if constexpr (Q == 1) {
+            return ld_tau<RO>(tau + ld_id<RO>(row + j));
+        } else if constexpr (Q == 2) {
+            const uint2* p = reinterpret_cast<const uint2*>(row) + j;
+            const uint2 id = RO ? __ldcs(p) : __ldg(p);
+            return min(ld_tau<RO>(tau + id.x), ld_tau<RO>(tau + id.y));
+        } else {
+            const uint32_t* p = row + 3 * (int64_t)j;
+            const uint32_t a = ld_id<RO>(p), b = ld_id<RO>(p + 1), c = ld_id<RO>(p + 2);
+            return min(min(ld_tau<RO>(tau + a), ld_tau<RO>(tau + b)), ld_tau<RO>(tau + c));
+        }
+    }
 };
 
 // (2,3) rows with tau(R) > 65535 (so d_s > 65535, CTA rows): exact values,
 // CSR position -> edge id -> tau
 template <bool RO>
 struct RhoExact2 {
-    const uint32_t* __restrict__ inc;
+    const uint32_t* __restrict__ row;
     const uint32_t* __restrict__ eid;
     const int32_t* tau;
-    __device__ __forceinline__ int32_t operator()(int64_t j) const {
-        const uint2 id = __ldg(reinterpret_cast<const uint2*>(inc) + j);
+    __device__ __forceinline__ int32_t operator()(int j) const {
+        const uint2 id = __ldg(reinterpret_cast<const uint2*>(row) + j);
         return min(ld_tau<RO>(tau + __ldg(eid + id.x)), ld_tau<RO>(tau + __ldg(eid + id.y)));
     }
 };
@@ -193,202 +192,277 @@ constexpr int32_t kTau16Max = 65535;
 // the 16-bit copy measured 3% slower there (Chung-Lu 100K (3,4) with planted
 // cliques) against 6% faster for a scale-24 k-core.
 template <int Q, bool RO>
-__device__ __forceinline__ auto make_rho(const SweepParams& P) {
-    if constexpr (Q == 3) return Rho<3, RO, int32_t>{P.inc, P.tin};
-    else return Rho<Q, RO, uint16_t>{P.inc, P.gin};
+__device__ __forceinline__ auto make_rho(const SweepParams& P, int64_t jb) {
+    if constexpr (Q == 3) return Rho<3, RO, int32_t>{P.inc + 3 * jb, P.tin};
+    else return Rho<Q, RO, uint16_t>{P.inc + Q * jb, P.gin};
 }
 
-// H({rho_j}) clipped to t, for one r-clique, by a group of G lanes; the row
-// (at most G*C <= 1024 incidences, so t <= 1024) is held in registers as
-// min(rho, t), two 16-bit values per register.
+// f(rho(j)) for the entries j in [i, end), STEP lanes wide: four loads per
+// lane in flight, without tests while whole blocks are left; the rest is one
+// block with a test per entry (rho = -1 past the end, which no step counts).
+template <int STEP, typename F, typename G>
+__device__ __forceinline__ void stream_row(const F& rho, int i, int end, G&& f) {
+    const int lane = STEP == 32 ? (threadIdx.x & 31) : threadIdx.x;
+    for (; end - i >= 4 * STEP; i += 4 * STEP) {
+        int32_t r[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) r[u] = rho(i + u * STEP + lane);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) f(i + u * STEP + lane, r[u]);
+    }
+    if (end - i > 2 * STEP) {
+        int32_t r[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int j = i + u * STEP + lane;
+            r[u] = j < end ? rho(j) : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) f(i + u * STEP + lane, r[u]);
+    } else if (end > i) {
+        int32_t r[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int j = i + u * STEP + lane;
+            r[u] = j < end ? rho(j) : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) f(i + u * STEP + lane, r[u]);
+    }
+}
+
+// H({rho_j}) clipped to t, for one r-clique per group of G lanes (t = 0 for
+// a group without a row); the row (at most G*C <= 64 entries, so t <= 64) is
+// held in registers as min(rho, t), four 8-bit values per register.  dmax:
+// the longest row of the warp's groups.  Every lane of the warp takes part
+// in every step.
 template <int G, int C, typename F>
-__device__ __forceinline__ int32_t group_hindex(const cg::thread_block_tile<G>& g, const F& rho,
-                                                int64_t jb, int64_t je, int32_t t) {
-    static_assert(C % 2 == 0, "values are packed in pairs");
-    const int lane = g.thread_rank();
-    if (t <= 0) return 0;
-    uint32_t pk[C / 2];
+__device__ __forceinline__ int32_t group_hindex(const F& rho, int d, int dmax, int32_t t) {
+    static_assert(G * C <= 64, "values fit 7 bits, with one spare for the comparison");
+    const int lane = threadIdx.x & (G - 1);
+    constexpr int W = (C + 3) / 4;
+    constexpr unsigned kHigh = 0x80808080u;
+    unsigned pk[W];
     int cnt = 0;
 #pragma unroll
-    for (int c = 0; c < C; c += 2) {
-        const int64_t j0 = jb + lane + (int64_t)c * G, j1 = j0 + G;
-        const int32_t r0 = (j0 < je) ? rho(j0) : 0;
-        const int32_t r1 = (j1 < je) ? rho(j1) : 0;
-        cnt += (r0 >= t) + (r1 >= t);
-        pk[c / 2] = (uint32_t)min(r0, t) | ((uint32_t)min(r1, t) << 16);
+    for (int w = 0; w < W; ++w) {
+        pk[w] = kHigh;
+        if (w == 0 || dmax > 4 * w * G) {  // the same for the whole warp
+            int32_t r[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                if (4 * w + c < C) {
+                    const int j = lane + (4 * w + c) * G;
+                    r[c] = j < d ? rho(j) : 0;
+                }
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                if (4 * w + c < C) {
+                    cnt += (r[c] >= t);
+                    pk[w] |= (unsigned)max(min(r[c], t), 0) << (8 * c);
+                }
+        }
     }
-    cnt = cg::reduce(g, cnt, cg::plus<int>());
-    if (cnt >= t) return t;
-    int lo = cnt, hi = t;  // #{rho >= lo} >= lo holds; at hi it fails
-    while (hi - lo > 1) {
-        const int mid = lo + ((hi - lo) >> 1);
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+    if (cnt >= t) cnt = t;
+    int lo = cnt, hi = max(t, cnt + 1);  // #{rho >= lo} >= lo holds; at hi it fails (or H = t is settled)
+    while (__any_sync(0xffffffffu, hi - lo > 1)) {
+        const int mid = (lo + hi) >> 1;  // >= 1 where it is used
+        const unsigned m4 = (unsigned)mid * 0x01010101u;
         int c2 = 0;
 #pragma unroll
-        for (int c = 0; c < C / 2; ++c)
-            c2 += ((int)(pk[c] & 0xffffu) >= mid) + ((int)(pk[c] >> 16) >= mid);
-        c2 = cg::reduce(g, c2, cg::plus<int>());
-        if (c2 >= mid) lo = mid; else hi = mid;
+        for (int w = 0; w < W; ++w) c2 += __popc((pk[w] - m4) & kHigh);  // bytes >= mid; no borrow crosses a byte
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1) c2 += __shfl_xor_sync(0xffffffffu, c2, o);
+        if (hi - lo > 1) {
+            if (c2 >= mid) lo = mid; else hi = mid;
+        }
     }
-    return lo;
+    return max(min(lo, t), 0);
 }
 
-// Bin selection of one k-ary search step, by one full warp.  bins[0..255]
-// count rho in [lo + b*width, lo + (b+1)*width), bins[256] counts rho >= hi.
-// #{rho >= lo + b*width} is the suffix sum from b; the answer H lies in
-// [k, next edge) for the largest bin edge k whose suffix is >= k (bin 0
-// always qualifies, because #{rho >= lo} >= lo).  Each lane owns 8 bins.
-// P16: the counters are 16 bits, two to a word (bin b in word b/2), for
-// rows of fewer than 65,536 entries; 129 words instead of 257.
-template <bool P16>
-__device__ __forceinline__ unsigned bin_count(const unsigned* bins, int b) {
-    if constexpr (P16) return (bins[b >> 1] >> ((b & 1) << 4)) & 0xffffu;
-    return bins[b];
+// the smallest shift that maps [0, span) onto fewer than `bins` values
+__device__ __forceinline__ int bin_shift(unsigned span, int bins) {
+    const int s = (32 - __clz(span - 1)) - (31 - __clz(bins));
+    return span > 1 && s > 0 ? s : 0;
 }
 
-template <bool P16>
-__device__ __forceinline__ void select_bin(const unsigned* bins, int lo, int hi, int width, int nb,
-                                           int* nlo, int* nhi) {
+// The bin of a histogram that holds H, by one full warp.  Bin b counts rho in
+// [lo + (b << shift), lo + ((b + 1) << shift)); `above` counts rho past the
+// last bin.  #{rho >= lo + (b << shift)} is above plus the suffix sum from b,
+// and H lies in the last bin whose sum reaches its lower edge (bin 0 always
+// qualifies: #{rho >= lo} >= lo).  Blocks of 128 bins from the top, four to a
+// lane; returns the bin, and in `above` the count past it.
+// PK: 16-bit counters, bin b in half b / HW of word b % HW.
+template <bool PK, int HW>
+__device__ __forceinline__ int select_bin(const unsigned* bins, int lo, int shift, int nb, int& above) {
     const int lane = threadIdx.x & 31;
-    unsigned own = 0;
+    for (int c = (nb - 1) >> 7;; --c) {
+        const int b0 = 128 * c;
+        uint4 w = *reinterpret_cast<const uint4*>(bins + (PK ? (b0 & (HW - 1)) : b0) + 4 * lane);
+        if (PK) {
+            if (b0 >= HW) w = make_uint4(w.x >> 16, w.y >> 16, w.z >> 16, w.w >> 16);
+            else w = make_uint4(w.x & 0xffffu, w.y & 0xffffu, w.z & 0xffffu, w.w & 0xffffu);
+        }
+        const int s3 = (int)w.w, s2 = s3 + (int)w.z, s1 = s2 + (int)w.y, s0 = s1 + (int)w.x;
+        int incl = s0;  // suffix over the lanes
 #pragma unroll
-    for (int k = 0; k < 8; ++k) own += bin_count<P16>(bins, 8 * lane + k);
-    unsigned incl = own;  // inclusive prefix over lanes
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        unsigned v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_down_sync(0xffffffffu, incl, o);
+            if (lane + o < 32) incl += v;
+        }
+        const int after = above + incl - s0;  // rho past this lane's bins
+        // lower edges; unsigned, because those of the padding past nb may leave 31 bits
+        const unsigned e0 = (unsigned)lo + ((unsigned)(b0 + 4 * lane) << shift), w1 = 1u << shift;
+        int best = -1, past = 0;
+        if ((unsigned)(after + s0) >= e0) { best = 0; past = after + s1; }
+        if ((unsigned)(after + s1) >= e0 + w1) { best = 1; past = after + s2; }
+        if ((unsigned)(after + s2) >= e0 + 2 * w1) { best = 2; past = after + s3; }
+        if ((unsigned)(after + s3) >= e0 + 3 * w1) { best = 3; past = after; }
+        const unsigned hit = __ballot_sync(0xffffffffu, best >= 0);
+        if (hit || c == 0) {
+            const int src = hit ? 31 - __clz(hit) : 0;
+            above = __shfl_sync(0xffffffffu, past, src);
+            return b0 + 4 * src + max(__shfl_sync(0xffffffffu, best, src), 0);
+        }
+        above += __shfl_sync(0xffffffffu, incl, 0);
     }
-    const unsigned total = __shfl_sync(0xffffffffu, incl, 31);
-    int64_t run = (int64_t)bin_count<P16>(bins, 256) + (total - incl);  // rho at or above this lane's bins
-    int best = -1;
-#pragma unroll
-    for (int k = 7; k >= 0; --k) {
-        const int b = 8 * lane + k;
-        run += bin_count<P16>(bins, b);
-        if (best < 0 && run >= (int64_t)lo + (int64_t)b * width) best = b;
-    }
-    const unsigned hit = __ballot_sync(0xffffffffu, best >= 0);
-    const int b = __shfl_sync(0xffffffffu, best, 31 - __clz(hit));
-    *nlo = lo + b * width;
-    const int e = (b + 1 < nb) ? lo + (b + 1) * width : hi;
-    *nhi = e < hi ? e : hi;
 }
 
-template <bool P16>
-__device__ __forceinline__ void kary_bin(unsigned* bins, int32_t r, int lo, int hi, int width) {
-    if (r < lo) return;
-    const int b = r >= hi ? 256 : (r - lo) / width;
-    if constexpr (P16) atomicAdd(&bins[b >> 1], 1u << ((b & 1) << 4));
-    else atomicAdd(&bins[b], 1u);
-}
-
-// words of one set of bins: 257 counters, packed or not
-template <bool P16>
-__device__ __forceinline__ int bin_words() { return P16 ? 129 : 257; }
-
-// H({rho_j}) clipped to t by one warp, streaming the row: one pass counts
-// rho >= t; if that fails, k-ary search with 256 shared-memory bins per
-// streaming pass (at most 2 passes for t <= 65536).  The counting pass keeps
-// min(rho, t) of the row's first ncache entries in `cache` (16 bits: a warp
-// row has t <= d_s < 65536), so the search passes read them from shared
-// memory instead of gathering them again; only entries past ncache are
-// streamed again.
-// P16: packed 16-bit bins, for rows of fewer than 65,536 entries
-template <bool P16 = false, typename F>
-__device__ __forceinline__ int32_t warp_hindex(const F& rho, int64_t jb, int64_t je, int32_t t, unsigned* bins,
-                                               uint16_t* cache = nullptr, int ncache = 0) {
+// H({rho_j}) clipped to t by one warp, streaming the row.
+// count first (direct = false): count rho >= t, reading no further than the
+// count still needs: t entries at or above t settle H = t.  Rows are in
+// order of the third vertex's degree class where the build renumbers, so the
+// entries that reach t come early: at convergence a row is read to about
+// 0.58 of its length (R-MAT scale 18 k-truss; the floor, t entries, is 0.47).
+// A row that fails is streamed again into a histogram over [count, t).
+// direct: straight into the histogram over [0, t) (rows that are expected to
+// fail: the early passes, and rows that changed in the pass before).
+// The histogram has up to 2 * HW bins (PK: 16-bit counters, two to a word, for
+// rows of fewer than 65,536 entries; else HW bins of 32 bits), one per value
+// while t allows, so H is exact after one sweep there, and after two for
+// longer rows.
+template <bool PK, int HW, typename F>
+__device__ __forceinline__ int32_t warp_hindex(const F& rho, int d, int32_t t, bool direct, unsigned* bins) {
     const int lane = threadIdx.x & 31;
     if (t <= 0) return 0;
-    int cnt = 0;
-    if (!cache || t > 65535) ncache = 0;
-    const int64_t jc = jb + ncache;  // entries [jb, jc) go to the cache
-#pragma unroll kWarpUnroll
-    for (int64_t j = jb + lane; j < je; j += 32) {
-        const int32_t r = rho(j);
-        cnt += (r >= t);
-        if (j < jc) cache[j - jb] = (uint16_t)min(r, t);
+    int lo = 0, hi = t, above = 0;
+    if (!direct) {
+        int cnt = 0, have = 0;
+        for (int i = 0; i < d;) {
+            const int end = min(d, i + max((t - have + 31) & ~31, 64));
+            stream_row<32>(rho, i, end, [&](int, int32_t r) { cnt += (r >= t); });
+            i = end;
+            have = (int)__reduce_add_sync(0xffffffffu, (unsigned)cnt);
+            if (have >= t) return t;
+        }
+        lo = above = have;  // #{rho >= lo} >= lo holds; at hi it fails
+        if (hi - lo <= 1) return lo;
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-    if (cnt >= t) return t;
-    __syncwarp();  // the cache is complete
-    int lo = cnt, hi = t;
-    while (hi - lo > 1) {
-        const int span = hi - lo;
-        const int nb = span < 256 ? span : 256;
-        const int width = (span + nb - 1) / nb;
-        for (int i = lane; i < bin_words<P16>(); i += 32) bins[i] = 0;
+    for (;;) {
+        const unsigned span = (unsigned)(hi - lo);
+        const int shift = bin_shift(span, PK ? 2 * HW : HW);
+        const int nb = (int)((span - 1) >> shift) + 1;
+        for (int i = 0; i < min(nb, HW); i += 128)  // whole blocks of 128, as select_bin reads them
+            *reinterpret_cast<uint4*>(bins + i + 4 * lane) = make_uint4(0u, 0u, 0u, 0u);
         __syncwarp();
-        for (int64_t j = jb + lane; j < jc && j < je; j += 32)
-            kary_bin<P16>(bins, (int32_t)cache[j - jb], lo, hi, width);
-        for (int64_t j = jc + lane; j < je; j += 32) kary_bin<P16>(bins, rho(j), lo, hi, width);
+        int ge = 0;
+        stream_row<32>(rho, 0, d, [&](int, int32_t r) {
+            const unsigned x = (unsigned)(r - lo);
+            if (x < span) {
+                const unsigned b = x >> shift;
+                if (PK) atomicAdd(bins + (b & (HW - 1)), b < (unsigned)HW ? 1u : 0x10000u);
+                else atomicAdd(bins + b, 1u);
+            } else {
+                ge += (r >= hi);
+            }
+        });
         __syncwarp();
-        int nlo, nhi;
-        select_bin<P16>(bins, lo, hi, width, nb, &nlo, &nhi);
-        lo = nlo;
-        hi = nhi;
+        if (direct) {
+            above = (int)__reduce_add_sync(0xffffffffu, (unsigned)ge);
+            if (above >= t) return t;
+            direct = false;
+        }
+        const int b = select_bin<PK, HW>(bins, lo, shift, nb, above);
+        lo += b << shift;
+        hi = min(hi, lo + (1 << shift));
+        if (hi - lo <= 1) return lo;
         __syncwarp();
     }
-    return lo;
 }
 
-// The same by the whole CTA (the longest rows); warp 0 selects the bin.
-// The first ncache entries are kept in `cache` as for a warp.
-template <typename F>
-__device__ __forceinline__ int32_t cta_hindex(const F& rho, int64_t jb, int64_t je, int32_t t,
-                                              unsigned* bins /* 257 */, int* bounds /* 2 */,
-                                              uint16_t* cache = nullptr, int ncache = 0) {
+// entries of a CTA row between two tests of its count, at least
+constexpr int kCtaSegment = 2048;
+
+// The same by the whole CTA (the longest rows): 32-bit counters, as many bins
+// as the block's histogram has words; warp 0 selects the bin.
+template <int WORDS, typename F>
+__device__ __forceinline__ int32_t cta_hindex(const F& rho, int d, int32_t t, bool direct, unsigned* bins,
+                                              int* bounds /* 8 */) {
     if (t <= 0) return 0;
-    int cnt = 0;
-    if (!cache || t > 65535) ncache = 0;
-    const int64_t jc = jb + ncache;
-#pragma unroll kWarpUnroll
-    for (int64_t j = jb + threadIdx.x; j < je; j += kThreads) {
-        const int32_t r = rho(j);
-        cnt += (r >= t);
-        if (j < jc) cache[j - jb] = (uint16_t)min(r, t);
-    }
+    auto total = [&](int v) {
+        const unsigned w = __reduce_add_sync(0xffffffffu, (unsigned)v);
+        if ((threadIdx.x & 31) == 0) bounds[threadIdx.x >> 5] = (int)w;
+        __syncthreads();
+        int tot = 0;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-    if ((threadIdx.x & 31) == 0) bins[threadIdx.x >> 5] = (unsigned)cnt;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned tot = 0;
-        for (int w = 0; w < kThreads / 32; ++w) tot += bins[w];
-        bounds[0] = (int)tot;
+        for (int i = 0; i < kThreads / 32; ++i) tot += bounds[i];
+        __syncthreads();
+        return tot;
+    };
+    int lo = 0, hi = t, above = 0;
+    if (!direct) {
+        int cnt = 0, have = 0;
+        for (int i = 0; i < d;) {
+            const int need = max((t - have + 4 * kThreads - 1) & ~(4 * kThreads - 1), kCtaSegment);
+            const int end = d - i > need ? i + need : d;
+            stream_row<kThreads>(rho, i, end, [&](int, int32_t r) { cnt += (r >= t); });
+            i = end;
+            have = total(cnt);
+            if (have >= t) return t;
+        }
+        lo = above = have;
+        if (hi - lo <= 1) return lo;
     }
-    __syncthreads();
-    cnt = bounds[0];
-    __syncthreads();
-    if (cnt >= t) return t;
-    int lo = cnt, hi = t;  // #{rho >= lo} >= lo holds; at hi it fails
-    while (hi - lo > 1) {
-        const int span = hi - lo;
-        const int nb = span < 256 ? span : 256;
-        const int width = (span + nb - 1) / nb;
-        for (int i = threadIdx.x; i <= 256; i += kThreads) bins[i] = 0;
+    for (;;) {
+        const unsigned span = (unsigned)(hi - lo);
+        const int shift = bin_shift(span, WORDS);
+        const int nb = (int)((span - 1) >> shift) + 1;
+        for (int i = threadIdx.x; i < ((nb + 127) & ~127); i += kThreads) bins[i] = 0;
         __syncthreads();
-        for (int64_t j = jb + threadIdx.x; j < jc && j < je; j += kThreads)
-            kary_bin<false>(bins, (int32_t)cache[j - jb], lo, hi, width);
-        for (int64_t j = jc + threadIdx.x; j < je; j += kThreads)
-            kary_bin<false>(bins, rho(j), lo, hi, width);
-        __syncthreads();
+        int ge = 0;
+        stream_row<kThreads>(rho, 0, d, [&](int, int32_t r) {
+            const unsigned x = (unsigned)(r - lo);
+            if (x < span) atomicAdd(bins + (x >> shift), 1u);
+            else ge += (r >= hi);
+        });
+        if (direct) {
+            above = total(ge);  // with its barriers, the bins are complete too
+            if (above >= t) return t;
+            direct = false;
+        } else {
+            __syncthreads();
+        }
         if (threadIdx.x < 32) {
-            int nlo, nhi;
-            select_bin<false>(bins, lo, hi, width, nb, &nlo, &nhi);
-            if (threadIdx.x == 0) { bounds[0] = nlo; bounds[1] = nhi; }
+            const int b = select_bin<false, WORDS>(bins, lo, shift, nb, above);
+            if (threadIdx.x == 0) { bounds[0] = b; bounds[1] = above; }
         }
         __syncthreads();
-        lo = bounds[0];
-        hi = bounds[1];
+        lo += bounds[0] << shift;
+        above = bounds[1];
         __syncthreads();
+        hi = min(hi, lo + (1 << shift));
+        if (hi - lo <= 1) return lo;
     }
-    return lo;
 }
 
-// the new tau of R; (2,3) also writes it to both CSR entries of the edge
+// the new tau of R; (2,3) also writes it to both CSR entries of the edge.
+// SND writes the buffer of two passes ago: where that holds h already (old),
+// all its copies do, and nothing is written.
 template <int Q>
-__device__ __forceinline__ void store_tau(const SweepParams& P, uint32_t R, int32_t h) {
+__device__ __forceinline__ void store_tau(const SweepParams& P, uint32_t R, int32_t h, int32_t old) {
+    if (h == old) return;
     P.tout[R] = h;
     const uint16_t v = (uint16_t)min(h, kTau16Max);
     if (Q == 2) {
@@ -554,103 +628,101 @@ __device__ __forceinline__ nd_item load_item(const nd_item* __restrict__ items, 
     return it;
 }
 
-// work items [first, first + 32/G): one r-clique per group of G lanes of the
-// calling warp
-template <int Q, int G, int C, bool AND, bool NOTIFY, bool GB = false>
-__device__ __forceinline__ void run_groups(const SweepParams& P, int64_t first, int64_t last,
-                                           unsigned long long& changed, unsigned long long& evals,
-                                           unsigned long long& incs) {
-    auto g = cg::tiled_partition<G>(cg::this_thread_block());
-    const int lane = g.thread_rank();
-    // the group's index inside its warp, from the lane id (G divides 32)
+// counters of one thread over a pass.  FULL (AND with notification, batches):
+// evaluated rows and their incidences too; the other passes evaluate every
+// row, so the host knows both.
+template <bool FULL>
+struct Tally {
+    unsigned changed = 0, evals = 0;
+    unsigned long long incs = 0;
+    __device__ __forceinline__ void row(uint32_t d, bool ch) {
+        if (FULL) {
+            evals++;
+            incs += d;
+        }
+        changed += ch;
+    }
+};
+
+// tau(R) (t0), its value clipped at d_s for the search (t: a no-op for every
+// valid tau, which is <= d_s; changes are detected against the stored value),
+// and what the output buffer holds (old; for AND the same array)
+template <bool AND>
+__device__ __forceinline__ void load_tau(const SweepParams& P, const nd_item& it, int32_t& t0, int32_t& t,
+                                         int32_t& old) {
+    t0 = ld_tau<!AND>(P.tin + it.R);
+    old = AND ? t0 : P.tout[it.R];
+    t = min(t0, (int32_t)min(it.d, (uint32_t)INT32_MAX));
+}
+
+// work items [first, last): one r-clique per group of G lanes of the calling
+// warp, at most 32/G of them
+template <int Q, int G, int C, bool AND, bool GB, bool FULL>
+__device__ __forceinline__ void run_groups(const SweepParams& P, int64_t first, int64_t last, Tally<FULL>& n) {
     const int64_t i = first + (int64_t)((threadIdx.x & 31) / G);
-    if (i >= last) return;
+    const bool ok = i < last;
+    const nd_item it = load_item(P.items, ok ? i : first);
+    const bool run = ok && !graph_done<GB>(P, it.R);
+    int32_t t0, t, old;
+    load_tau<AND>(P, it, t0, t, old);
+    const int d = run ? (int)it.d : 0;
+    if (!run) t = 0;
+    const int dmax = (int)__reduce_max_sync(0xffffffffu, (unsigned)d);
+    const int32_t h = group_hindex<G, C>(make_rho<Q, !AND>(P, it.jb), d, dmax, t);
+    if (run && (threadIdx.x & (G - 1)) == 0) {
+        n.row(it.d, h != t0);
+        if (h != t0) graph_changed<GB>(P, it.R);
+        store_tau<Q>(P, it.R, h, old);
+    }
+}
+
+// one r-clique per warp (rows of the warp bucket), streamed
+template <int Q, bool AND, bool NOTIFY, bool GB, int HW, bool FULL>
+__device__ __forceinline__ void run_warp_row(const SweepParams& P, const nd_item& it, unsigned* bins,
+                                             Tally<FULL>& n) {
+    const uint32_t R = it.R;
+    if (graph_done<GB>(P, R)) return;
+    int32_t t0, t, old;
+    load_tau<AND>(P, it, t0, t, old);
+    const int32_t h = warp_hindex<true, HW>(make_rho<Q, !AND>(P, it.jb), (int)it.d, t,
+                                             P.direct || (!AND && old != t0), bins);
+    const int lane = threadIdx.x & 31;
+    if (lane == 0) {
+        n.row(it.d, h != t0);
+        if (h != t0) graph_changed<GB>(P, R);
+        store_tau<Q>(P, R, h, old);
+    }
+    if (AND && NOTIFY && h != t0) notify_row<Q>(P, it.jb, it.jb + it.d, h, lane, 32);
+    __syncwarp();  // the bins are free again
+}
+
+// one r-clique per CTA (rows past the warp threshold)
+template <int Q, bool AND, bool NOTIFY, bool GB, int WORDS, bool FULL>
+__device__ __forceinline__ void run_cta(const SweepParams& P, int64_t i, unsigned* bins, int* bounds,
+                                        Tally<FULL>& n) {
     const nd_item it = load_item(P.items, i);
     const uint32_t R = it.R;
-    const int64_t jb = it.jb, je = it.jb + it.d;
     if (AND && NOTIFY && !in_frontier<Q>(P, R)) return;
-    if (graph_done<GB>(P, R)) return;
-    const int32_t t0 = ld_tau<!AND>(P.tin + R);
-    // H <= d_s, so tau is clipped at d_s for the search (a no-op for every
-    // valid tau, which is <= d_s); changes are detected against the stored value
-    const int32_t t = min(t0, (int32_t)it.d);
-    const int32_t h = group_hindex<G, C>(g, make_rho<Q, !AND>(P), jb, je, t);
-    if (lane == 0) {
-        evals++;
-        incs += it.d;
-        if (h != t0) {
-            changed++;
-            graph_changed<GB>(P, R);
-        }
-        if (!AND || h != t0) store_tau<Q>(P, R, h);
+    if (graph_done<GB>(P, R)) return;  // the same R for the whole block
+    int32_t t0, t, old;
+    load_tau<AND>(P, it, t0, t, old);
+    __syncthreads();  // AND: every thread has read tau(R) before it is written
+    const int d = (int)it.d;
+    const bool direct = P.direct || (!AND && old != t0);
+    int32_t h;
+    if (Q == 2 && t > kTau16Max)  // only then can a saturated value matter
+        h = cta_hindex<WORDS>(RhoExact2<!AND>{P.inc + 2 * it.jb, P.eid, P.tin}, d, t, direct, bins, bounds);
+    else if (Q == 1 && t > kTau16Max)
+        h = cta_hindex<WORDS>(Rho<Q, !AND, int32_t>{P.inc + it.jb, P.tin}, d, t, direct, bins, bounds);
+    else
+        h = cta_hindex<WORDS>(make_rho<Q, !AND>(P, it.jb), d, t, direct, bins, bounds);
+    if (threadIdx.x == 0) {
+        n.row(it.d, h != t0);
+        if (h != t0) graph_changed<GB>(P, R);
+        store_tau<Q>(P, R, h, old);
     }
-    if (AND && NOTIFY && h != t0) notify_row<Q>(P, jb, je, h, lane, G);
-}
-
-// one r-clique per warp (rows of the warp bucket), streamed.  CHECK: test
-// the frontier here (false when the caller has already selected active rows)
-template <int Q, bool AND, bool NOTIFY, bool CHECK = true, bool GB = false, bool PK = true>
-__device__ __forceinline__ void run_warp_row(const SweepParams& P, const nd_item& it, unsigned* bins,
-                                             uint16_t* cache, unsigned long long& changed, unsigned long long& evals,
-                                             unsigned long long& incs) {
-    const int lane = threadIdx.x & 31;
-    const uint32_t R = it.R;
-    if (CHECK && AND && NOTIFY && !in_frontier<Q>(P, R)) return;
-    if (graph_done<GB>(P, R)) return;
-    const int32_t t0 = ld_tau<!AND>(P.tin + R);
-    // H <= d_s, so tau is clipped at d_s for the search (a no-op for every
-    // valid tau, which is <= d_s); changes are detected against the stored value
-    const int32_t t = min(t0, (int32_t)it.d);
-    const int64_t jb = it.jb, je = it.jb + it.d;
-    // a warp row has d_s <= the warp threshold (at most 8,192), so 16-bit bins hold its counts
-    const int32_t h = warp_hindex<PK>(make_rho<Q, !AND>(P), jb, je, t, bins, cache, kRhoCache);
-    if (lane == 0) {
-        evals++;
-        incs += it.d;
-        if (h != t0) {
-            changed++;
-            graph_changed<GB>(P, R);
-        }
-        if (!AND || h != t0) store_tau<Q>(P, R, h);
-    }
-    if (AND && NOTIFY && h != t0) notify_row<Q>(P, jb, je, h, lane, 32);
-}
-
-// one r-clique per CTA (rows longer than 2048 incidences)
-template <int Q, bool AND, bool NOTIFY, bool GB = false>
-__device__ __forceinline__ void run_cta(const SweepParams& P, int64_t first, int64_t last,
-                                        unsigned* bins, int* bounds, uint16_t* cache, int ncache,
-                                        unsigned long long& changed,
-                                        unsigned long long& evals, unsigned long long& incs) {
-    for (int64_t i = first; i < last; ++i) {
-        const nd_item it = load_item(P.items, i);
-        const uint32_t R = it.R;
-        if (AND && NOTIFY && !in_frontier<Q>(P, R)) continue;
-        if (graph_done<GB>(P, R)) continue;  // the same R for the whole block
-        const int32_t t0 = ld_tau<!AND>(P.tin + R);
-        // H <= d_s, so tau is clipped at d_s for the search (a no-op for every
-        // valid tau, which is <= d_s); changes are detected against the stored value
-        const int32_t t = min(t0, (int32_t)it.d);
-        const int64_t jb = it.jb, je = it.jb + it.d;
-        int32_t h;
-        if (Q == 2 && t > kTau16Max)  // only then can a saturated value matter
-            h = cta_hindex(RhoExact2<!AND>{P.inc, P.eid, P.tin}, jb, je, t, bins, bounds);
-        else if (Q == 1 && t > kTau16Max)
-            h = cta_hindex(Rho<Q, !AND, int32_t>{P.inc, P.tin}, jb, je, t, bins, bounds);
-        else
-            h = cta_hindex(make_rho<Q, !AND>(P), jb, je, t, bins, bounds, cache, ncache);
-        if (threadIdx.x == 0) {
-            evals++;
-            incs += it.d;
-            if (h != t0) {
-                changed++;
-                graph_changed<GB>(P, R);
-            }
-            if (!AND || h != t0) store_tau<Q>(P, R, h);
-        }
-        if (AND && NOTIFY && h != t0) notify_row<Q>(P, jb, je, h, threadIdx.x, kThreads);
-        __syncthreads();
-    }
+    if (AND && NOTIFY && h != t0) notify_row<Q>(P, it.jb, it.jb + d, h, threadIdx.x, kThreads);
+    __syncthreads();
 }
 
 // AND with notification: the frontier bits of the rows [a, b) of a warp
@@ -714,35 +786,27 @@ __device__ __forceinline__ int nth_set_bit(unsigned m, int k) {
 // notification), instead of by each row's own G lanes while the groups whose
 // rows did not change wait.
 template <int Q, int G, int C>
-__device__ __forceinline__ void run_groups_active(const SweepParams& P, int64_t a, unsigned mask,
-                                                  unsigned long long& changed, unsigned long long& evals,
-                                                  unsigned long long& incs) {
+__device__ __forceinline__ void run_groups_active(const SweepParams& P, int64_t a, unsigned mask, Tally<true>& n) {
     constexpr int NG = 32 / G;
-    auto g = cg::tiled_partition<G>(cg::this_thread_block());
     const int lane = threadIdx.x & 31;
     const int grp = lane / G;
     const int cnt = __popc(mask);
     for (int base = 0; base < cnt; base += NG) {
         const int k = base + grp;  // this group's k-th active row
-        int64_t jb = 0;
-        int32_t h = 0, dn = 0;
-        if (k < cnt) {  // uniform inside the group
-            const int64_t i = a + nth_set_bit(mask, k);
-            const nd_item it = load_item(P.items, i);
-            const int32_t t0 = ld_tau<false>(P.tin + it.R);
-            const int32_t t = min(t0, (int32_t)it.d);
-            jb = it.jb;
-            h = group_hindex<G, C>(g, make_rho<Q, false>(P), jb, jb + it.d, t);
-            if (g.thread_rank() == 0) {
-                evals++;
-                incs += it.d;
-                if (h != t0) {
-                    changed++;
-                    store_tau<Q>(P, it.R, h);
-                }
-            }
-            dn = (h != t0) ? (int32_t)it.d : 0;
+        const bool run = k < cnt;
+        const nd_item it = load_item(P.items, a + nth_set_bit(mask, run ? k : 0));
+        int32_t t0, t, old;
+        load_tau<true>(P, it, t0, t, old);
+        const int64_t jb = it.jb;
+        const int d = run ? (int)it.d : 0;
+        if (!run) t = 0;
+        const int dmax = (int)__reduce_max_sync(0xffffffffu, (unsigned)d);
+        const int32_t h = group_hindex<G, C>(make_rho<Q, false>(P, jb), d, dmax, t);
+        if (run && (lane & (G - 1)) == 0) {
+            n.row(it.d, h != t0);
+            store_tau<Q>(P, it.R, h, old);
         }
+        const int32_t dn = h != t0 ? d : 0;
         // merged notification over the changed rows of this round
         int tot = 0;
 #pragma unroll
@@ -765,59 +829,50 @@ __device__ __forceinline__ void run_groups_active(const SweepParams& P, int64_t 
     }
 }
 
-#ifndef ND_PASS_MIN_BLOCKS
-#define ND_PASS_MIN_BLOCKS 6  // resident blocks per SM the register budget targets (6 measured best)
-#endif
-#ifndef ND_PACKED_BINS_Q2
-#define ND_PACKED_BINS_Q2 0  // (2,3) passes with the packed bins too (measured slower on the R-MAT k-truss)
-#endif
-#ifndef ND_CARVEOUT_FN0
-#define ND_CARVEOUT_FN0 1  // request the carve-out for the first batch's kernel too
-#endif
-#ifndef ND_NC_CARVEOUT
-#define ND_NC_CARVEOUT 1  // the late-pass kernel asks for the carve-out it needs (0: the driver's choice)
-#endif
-#ifndef ND_NC_MIN_BLOCKS
-#define ND_NC_MIN_BLOCKS 6  // the late-pass kernel without the rho cache
-#endif
-#ifndef ND_AND_MIN_BLOCKS
-#define ND_AND_MIN_BLOCKS 6   // the same for the AND pass with notification
-#endif
+// the block's counters, added to the pass's
+template <bool FULL>
+__device__ __forceinline__ void flush_tally(const SweepParams& P, const Tally<FULL>& n) {
+    __shared__ unsigned s_ch[kThreads / 32], s_ev[kThreads / 32];
+    __shared__ unsigned long long s_in[kThreads / 32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const unsigned ch = __reduce_add_sync(0xffffffffu, n.changed);
+    unsigned ev = 0;
+    unsigned long long in = 0;
+    if (FULL) {
+        ev = __reduce_add_sync(0xffffffffu, n.evals);
+        in = n.incs;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) in += __shfl_xor_sync(0xffffffffu, in, o);
+    }
+    if (lane == 0) { s_ch[wid] = ch; s_ev[wid] = ev; s_in[wid] = in; }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned long long a = 0, e = 0, c = 0;
+        for (int w = 0; w < kThreads / 32; ++w) { a += s_ch[w]; e += s_ev[w]; c += s_in[w]; }
+        if (a) atomicAdd(P.ctr, a);
+        if (e) atomicAdd(P.ctr + 1, e);
+        if (c) atomicAdd(P.ctr + 3, c);
+    }
+}
+
+constexpr int kPassBlocks = 6;  // resident blocks per SM the register budget of every pass kernel targets
+
 // GB: a batch handle's SND / AND-nn pass, which skips the rows of graphs
 // that have converged
-// NC: no rho cache, for the late passes of a run, where few rows search:
-// without its 16 KB per block the SM keeps more of its memory as L1 for the
-// gathers
-template <int Q, bool AND, bool NOTIFY, bool GB = false, bool NC = false>
-__global__ void __launch_bounds__(kThreads, NC ? ND_NC_MIN_BLOCKS
-                                               : ((AND && NOTIFY) ? ND_AND_MIN_BLOCKS : ND_PASS_MIN_BLOCKS))
-    k_pass(SweepParams P) {
+// LATE: the passes after the first of a run, where few rows search: a
+// quarter of the histogram, and the shared memory it frees serves as L1 for
+// the gathers
+template <int Q, bool AND, bool NOTIFY, bool GB, bool LATE>
+__global__ void __launch_bounds__(kThreads, kPassBlocks) k_pass(SweepParams P) {
     if (P.prev != nullptr && *(volatile const unsigned long long*)P.prev == 0ull) return;  // converged
-    constexpr int kRC = NC ? 0 : kRhoCache;
-    // k-ary search bins.  (1,2) and (3,4): one packed set per warp (16-bit
-    // counters), and a 32-bit set for the CTA rows in the last 1,040 bytes of
-    // the block's rho cache, which a CTA row then does not use for values;
-    // that keeps six blocks within a 132 KB shared-memory carve-out, and the
-    // rest of the SM's memory serves as L1 (R-MAT scale-26 k-core: 794 against
-    // 825 ms per step; Chung-Lu 100K (3,4): 121.9 against 126.8 ms).  (2,3): one
-    // 32-bit set per warp, the CTA rows using warp 0's (the packed layout
-    // measured 262.8 against 258.9 ms per step on the R-MAT scale-20 k-truss).
-    // PK: packed warp bins and the CTA bins in the cache (ND_PACKED_BINS_Q2
-    // selects it for (2,3))
-    constexpr bool PK = Q != 2 || ND_PACKED_BINS_Q2;
-    constexpr int kCtaBinWords = 260;
-    constexpr int kCtaCache = kRC > 0 ? (kThreads / 32) * kRC - (PK ? 2 * kCtaBinWords : 0) : 0;
-    static_assert(kRC == 0 || kCtaCache > 0, "the rho cache holds the CTA bins");
-    __shared__ unsigned bins[kThreads / 32][PK ? 132 : 260];
-    __shared__ __align__(16) uint16_t rho_cache[kThreads / 32][kRC > 0 ? kRC : 1];  // per warp; a CTA row uses all
-    __shared__ unsigned cta_bins_own[(kRC > 0 && PK) ? 1 : kCtaBinWords];
-    uint16_t* const wcache = kRC > 0 ? rho_cache[threadIdx.x >> 5] : nullptr;
-    uint16_t* const bcache = kRC > 0 ? &rho_cache[0][0] : nullptr;
-    unsigned* const cta_bins =
-        (kRC > 0 && PK) ? reinterpret_cast<unsigned*>(&rho_cache[0][0] + kCtaCache) : (PK ? cta_bins_own : bins[0]);
-    __shared__ int bounds[2];
+    constexpr bool FULL = NOTIFY || GB;
+    constexpr int HW = LATE ? kLateHistWords : kHistWords;
+    constexpr int kWords = (kThreads / 32) * HW;  // a CTA row uses every warp's histogram
+    __shared__ __align__(16) unsigned hist[kThreads / 32][HW];
+    __shared__ int bounds[kThreads / 32];
     __shared__ unsigned long long s_chunk;
-    unsigned long long changed = 0, evals = 0, incs = 0;
+    unsigned* const bins = hist[threadIdx.x >> 5];
+    Tally<FULL> n;
     // phase 1: rows longer than the CTA threshold, one per block at a time,
     // taken from a per-pass counter (longest rows first)
     const int64_t n3 = P.hi[3] - P.lo[3];
@@ -829,8 +884,7 @@ __global__ void __launch_bounds__(kThreads, NC ? ND_NC_MIN_BLOCKS
             const int64_t c = (int64_t)s_chunk;
             __syncthreads();
             if (c >= n3) break;
-            run_cta<Q, AND, NOTIFY, GB>(P, P.lo[3] + c, P.lo[3] + c + 1, cta_bins, bounds, bcache, kCtaCache,
-                                        changed, evals, incs);
+            run_cta<Q, AND, NOTIFY, GB, kWords>(P, P.lo[3] + c, &hist[0][0], bounds, n);
         }
     };
     // AND updates in place, so a row evaluated later in a pass already sees
@@ -843,29 +897,29 @@ __global__ void __launch_bounds__(kThreads, NC ? ND_NC_MIN_BLOCKS
     // rest of the pass had finished (18% of the AND time of an R-MAT scale
     // 26 k-core in ncu), so (1,2) AND takes them first.
     constexpr bool kShortFirst = AND;
-    constexpr bool kCtaFirst = !AND || (Q == 1 && ND_CORE_AND_CTA_FIRST);
+    constexpr bool kCtaFirst = !AND || Q == 1;
     if (kCtaFirst) cta_phase();
     // phase 2: warp tasks (one warp row, four 8-lane rows or eight 4-lane
     // rows), longest first (SND) or shortest first (AND).  Each warp takes
-    // chunks of kWarpChunk
-    // consecutive tasks from a per-pass counter (one atomic per chunk, no
-    // barrier): consecutive r-cliques share a vertex and gather from the
-    // same part of tau, and dynamic chunks keep the warps balanced even when
-    // only a scattered subset of r-cliques is active (AND).
+    // chunks of P.chunk consecutive tasks from a per-pass counter (one atomic
+    // per chunk, no barrier): consecutive r-cliques share a vertex and gather
+    // from the same part of tau, and dynamic chunks keep the warps balanced
+    // even when only a scattered subset of r-cliques is active (AND).
     const int64_t n2 = P.hi[2] - P.lo[2];
     const int64_t t1 = (P.hi[1] - P.lo[1] + 3) / 4;
     const int64_t t0 = (P.hi[0] - P.lo[0] + 7) / 8;
     const int64_t tasks = n2 + t1 + t0;
     const int lane32 = threadIdx.x & 31;
+    const int chunk = P.chunk;
+    const int64_t nchunks = (tasks + chunk - 1) / chunk;
     for (;;) {
         unsigned long long c = 0;
         if (lane32 == 0) c = atomicAdd(P.ctr + 4, 1ull);
         c = __shfl_sync(0xffffffffu, c, 0);
-        const int64_t nchunks = (tasks + kWarpChunk - 1) / kWarpChunk;
         if ((int64_t)c >= nchunks) break;
         const int64_t cc = kShortFirst ? nchunks - 1 - (int64_t)c : (int64_t)c;
-        int64_t t = cc * kWarpChunk;
-        const int64_t te = min(t + (int64_t)kWarpChunk, tasks);
+        int64_t t = cc * chunk;
+        const int64_t te = min(t + (int64_t)chunk, tasks);
         if constexpr (AND && NOTIFY) {
             // the chunk's rows per bucket, their frontier bits tested up front;
             // only active rows are evaluated
@@ -879,8 +933,7 @@ __global__ void __launch_bounds__(kThreads, NC ? ND_NC_MIN_BLOCKS
                     const int b = __ffs(mm) - 1;
                     mm &= mm - 1;
                     const nd_item it = load_item(P.items, P.lo[2] + t + b);
-                    run_warp_row<Q, AND, NOTIFY, false, false, PK>(P, it, bins[threadIdx.x >> 5], wcache, changed,
-                                                                   evals, incs);
+                    run_warp_row<Q, AND, NOTIFY, false, HW>(P, it, bins, n);
                 }
             }
             const int64_t t1_lo = max(t, n2), t1_hi = min(te, n2 + t1);
@@ -891,7 +944,7 @@ __global__ void __launch_bounds__(kThreads, NC ? ND_NC_MIN_BLOCKS
                 active_masks<Q, W1>(P, a, b, mk);
 #pragma unroll
                 for (int w = 0; w < W1; ++w)
-                    if (mk[w]) run_groups_active<Q, 8, 8>(P, a + 32 * w, mk[w], changed, evals, incs);
+                    if (mk[w]) run_groups_active<Q, 8, 8>(P, a + 32 * w, mk[w], n);
             }
             const int64_t t0_lo = max(t, n2 + t1);
             if (t0_lo < te) {
@@ -901,60 +954,46 @@ __global__ void __launch_bounds__(kThreads, NC ? ND_NC_MIN_BLOCKS
                 active_masks<Q, W0>(P, a, b, mk);
 #pragma unroll
                 for (int w = 0; w < W0; ++w)
-                    if (mk[w]) run_groups_active<Q, 4, 2>(P, a + 32 * w, mk[w], changed, evals, incs);
+                    if (mk[w]) run_groups_active<Q, 4, 2>(P, a + 32 * w, mk[w], n);
             }
-            continue;
-        }
-        const int64_t e2 = min(te, n2);
-        if (t < e2) {
-            // warp rows: the next row's work item is loaded before this one runs
-            nd_item it = load_item(P.items, P.lo[2] + t);
-            while (t < e2) {
-                nd_item nx;
-                if (t + 1 < e2) nx = load_item(P.items, P.lo[2] + t + 1);
-                run_warp_row<Q, AND, NOTIFY, true, GB, PK>(P, it, bins[threadIdx.x >> 5], wcache, changed, evals,
-                                                           incs);
-                it = nx;
-                ++t;
+        } else {
+            const int64_t e2 = min(te, n2);
+            if (t < e2) {
+                // warp rows: the next row's work item is loaded before this one runs
+                nd_item it = load_item(P.items, P.lo[2] + t);
+                while (t < e2) {
+                    nd_item nx;
+                    if (t + 1 < e2) nx = load_item(P.items, P.lo[2] + t + 1);
+                    run_warp_row<Q, AND, NOTIFY, GB, HW>(P, it, bins, n);
+                    it = nx;
+                    ++t;
+                }
             }
-        }
-        for (; t < te; ++t) {
-            if (t < n2 + t1) {
-                const int64_t first = P.lo[1] + 4 * (t - n2);
-                run_groups<Q, 8, 8, AND, NOTIFY, GB>(P, first, min(first + 4, P.hi[1]), changed, evals, incs);
-            } else {
-                const int64_t first = P.lo[0] + 8 * (t - n2 - t1);
-                run_groups<Q, 4, 2, AND, NOTIFY, GB>(P, first, min(first + 8, P.hi[0]), changed, evals, incs);
+            for (; t < te; ++t) {
+                if (t < n2 + t1) {
+                    const int64_t first = P.lo[1] + 4 * (t - n2);
+                    run_groups<Q, 8, 8, AND, GB>(P, first, min(first + 4, P.hi[1]), n);
+                } else {
+                    const int64_t first = P.lo[0] + 8 * (t - n2 - t1);
+                    run_groups<Q, 4, 2, AND, GB>(P, first, min(first + 8, P.hi[0]), n);
+                }
             }
         }
     }
     if (!kCtaFirst) cta_phase();
-    __shared__ unsigned long long s_ch[kThreads / 32], s_ev[kThreads / 32], s_in[kThreads / 32];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        changed += __shfl_xor_sync(0xffffffffu, changed, o);
-        evals += __shfl_xor_sync(0xffffffffu, evals, o);
-        incs += __shfl_xor_sync(0xffffffffu, incs, o);
-    }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) { s_ch[wid] = changed; s_ev[wid] = evals; s_in[wid] = incs; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long a = 0, e = 0, c = 0;
-        for (int w = 0; w < kThreads / 32; ++w) { a += s_ch[w]; e += s_ev[w]; c += s_in[w]; }
-        if (a) atomicAdd(P.ctr, a);
-        if (e) atomicAdd(P.ctr + 1, e);
-        if (c) atomicAdd(P.ctr + 3, c);
-    }
+    flush_tally(P, n);
 }
 
+// tau_0 = d_s in a; b (SND's other buffer): -1, which no pass has stored, for
+// every row that a pass evaluates, so that the first pass writes them all and
+// takes them for rows that have just changed (see warp_hindex)
 __global__ void k_init_tau(int64_t N, const int64_t* __restrict__ inc_ptr, int32_t* __restrict__ a,
                            int32_t* __restrict__ b) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N;
          i += (int64_t)gridDim.x * blockDim.x) {
         int32_t d = (int32_t)(inc_ptr[i + 1] - inc_ptr[i]);
         a[i] = d;
-        if (b) b[i] = d;
+        if (b) b[i] = d ? -1 : 0;
     }
 }
 
@@ -1050,7 +1089,7 @@ struct RhoOtf {
     const uint16_t* tau16;
     const uint32_t* __restrict__ eid;
     const int32_t* tau32;
-    __device__ __forceinline__ int32_t operator()(int64_t j) const {
+    __device__ __forceinline__ int32_t operator()(int j) const {
         const int32_t w = __ldg(col + sb + j);
         const int k = nd_lower_bound_n(col + lb, ln, w);
         if (k >= ln || __ldg(col + lb + k) != w) return -1;
@@ -1063,12 +1102,12 @@ struct RhoOtf {
 constexpr int kOtfChunk = 4;  // rows per counter grab
 
 template <bool AND, bool NOTIFY>
-__global__ void __launch_bounds__(kThreads, ND_PASS_MIN_BLOCKS) k_pass_otf(SweepParams P) {
+__global__ void __launch_bounds__(kThreads, kPassBlocks) k_pass_otf(SweepParams P) {
     if (P.prev != nullptr && *(volatile const unsigned long long*)P.prev == 0ull) return;  // converged
-    __shared__ unsigned bins[kThreads / 32][260];
-    unsigned long long changed = 0, evals = 0, incs = 0;
+    __shared__ __align__(16) unsigned hist[kThreads / 32][kHistWords];
+    Tally<true> n;
     const int lane = threadIdx.x & 31;
-    unsigned* wb = bins[threadIdx.x >> 5];
+    unsigned* const bins = hist[threadIdx.x >> 5];
     const int64_t first = P.lo[0], rows = P.hi[ND_NB - 1] - P.lo[0];
     for (;;) {
         unsigned long long c = 0;
@@ -1081,8 +1120,9 @@ __global__ void __launch_bounds__(kThreads, ND_PASS_MIN_BLOCKS) k_pass_otf(Sweep
             const nd_item it = load_item(P.items, first + rows - 1 - t);  // longest first
             const uint32_t R = it.R;
             if (AND && NOTIFY && !in_frontier<2>(P, R)) continue;
-            const int32_t tr = ld_tau<!AND>(P.tin + R);
-            const int32_t tc = min(tr, (int32_t)it.d);
+            int32_t tr, tc, old;
+            load_tau<AND>(P, it, tr, tc, old);
+            const bool direct = P.direct || (!AND && old != tr);
             const int32_t x = __ldg(P.eu + R), y = __ldg(P.ev + R);
             const int64_t xb = __ldg(P.rp + x), xe = __ldg(P.rp + x + 1);
             const int64_t yb = __ldg(P.rp + y), ye = __ldg(P.rp + y + 1);
@@ -1090,17 +1130,16 @@ __global__ void __launch_bounds__(kThreads, ND_PASS_MIN_BLOCKS) k_pass_otf(Sweep
             const int64_t sb = xs ? xb : yb, se = xs ? xe : ye;
             const int64_t lb = xs ? yb : xb, le = xs ? ye : xe;
             int32_t h;
+            const int ln = (int)(le - lb), sn = (int)(se - sb);
             if (tc > kTau16Max)
-                h = warp_hindex(RhoOtf<!AND, true>{P.col, sb, lb, (int)(le - lb), P.gin, P.eid, P.tin}, 0, se - sb,
-                                tc, wb);
+                h = warp_hindex<false, kHistWords>(RhoOtf<!AND, true>{P.col, sb, lb, ln, P.gin, P.eid, P.tin}, sn, tc, direct,
+                                            bins);
             else
-                h = warp_hindex(RhoOtf<!AND, false>{P.col, sb, lb, (int)(le - lb), P.gin, P.eid, P.tin}, 0, se - sb,
-                                tc, wb);
+                h = warp_hindex<false, kHistWords>(RhoOtf<!AND, false>{P.col, sb, lb, ln, P.gin, P.eid, P.tin}, sn, tc, direct,
+                                            bins);
             if (lane == 0) {
-                evals++;
-                incs += it.d;
-                if (h != tr) changed++;
-                if (!AND || h != tr) store_tau<2>(P, R, h);
+                n.row(it.d, h != tr);
+                store_tau<2>(P, R, h, old);
             }
             if (AND && NOTIFY && h != tr) {
                 // notify the other two edges of every triangle, found again
@@ -1115,70 +1154,28 @@ __global__ void __launch_bounds__(kThreads, ND_PASS_MIN_BLOCKS) k_pass_otf(Sweep
             }
         }
     }
-    __shared__ unsigned long long s_ch[kThreads / 32], s_ev[kThreads / 32], s_in[kThreads / 32];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        changed += __shfl_xor_sync(0xffffffffu, changed, o);
-        evals += __shfl_xor_sync(0xffffffffu, evals, o);
-        incs += __shfl_xor_sync(0xffffffffu, incs, o);
-    }
-    const int wid = threadIdx.x >> 5;
-    if (lane == 0) { s_ch[wid] = changed; s_ev[wid] = evals; s_in[wid] = incs; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long a = 0, e = 0, c2 = 0;
-        for (int w = 0; w < kThreads / 32; ++w) { a += s_ch[w]; e += s_ev[w]; c2 += s_in[w]; }
-        if (a) atomicAdd(P.ctr, a);
-        if (e) atomicAdd(P.ctr + 1, e);
-        if (c2) atomicAdd(P.ctr + 3, c2);
-    }
+    flush_tally(P, n);
 }
 
 typedef void (*pass_fn)(SweepParams);
 
-#ifndef ND_LATE_FROM
-#define ND_LATE_FROM 16  // the first pass (0-based) of a run that takes the late-pass kernel
-#endif
-#ifndef ND_AND_LATE_FROM
-#define ND_AND_LATE_FROM 16  // the same for AND with notification
-#endif
-static_assert(ND_LATE_FROM >= 0 && ND_LATE_FROM <= ND_BATCH, "the late kernel starts within the first batch");
-static_assert(ND_AND_LATE_FROM >= 0 && ND_AND_LATE_FROM <= ND_BATCH, "the late kernel starts within the first batch");
-#ifndef ND_LATE_NOCACHE
-#define ND_LATE_NOCACHE 2  // passes after the first batch without the rho cache: 0 none, 1 SND, 2 SND and AND
-#endif
-pass_fn pick(const nd_incidence* h, int mode, bool late = false) {
+// the pass kernel of a run; late: for the passes from kLateFrom on
+constexpr int kLateFrom = ND_BATCH;
+template <int Q>
+pass_fn pick_q(int mode, bool batch, bool late) {
+    if (mode == ND_AND) return late ? k_pass<Q, true, true, false, true> : k_pass<Q, true, true, false, false>;
+    if (mode == ND_SND) {
+        if (batch) return late ? k_pass<Q, false, false, true, true> : k_pass<Q, false, false, true, false>;
+        return late ? k_pass<Q, false, false, false, true> : k_pass<Q, false, false, false, false>;
+    }
+    if (batch) return late ? k_pass<Q, true, false, true, true> : k_pass<Q, true, false, true, false>;
+    return late ? k_pass<Q, true, false, false, true> : k_pass<Q, true, false, false, false>;
+}
+pass_fn pick(const nd_incidence* h, int mode, bool late) {
     // mode: ND_SND, ND_AND (notify), ND_AND_NN
-    const int q = h->q;
-    if (late && !h->otf) {
-        const bool gb = h->gid && mode != ND_AND;  // a batch's SND / AND-nn pass
-        if (mode == ND_SND && ND_LATE_NOCACHE >= 1) {
-            if (gb)
-                return q == 1 ? k_pass<1, false, false, true, true>
-                              : (q == 2 ? k_pass<2, false, false, true, true> : k_pass<3, false, false, true, true>);
-            return q == 1 ? k_pass<1, false, false, false, true>
-                          : (q == 2 ? k_pass<2, false, false, false, true> : k_pass<3, false, false, false, true>);
-        }
-        if (mode == ND_AND && ND_LATE_NOCACHE >= 2)
-            return q == 1 ? k_pass<1, true, true, false, true>
-                          : (q == 2 ? k_pass<2, true, true, false, true> : k_pass<3, true, true, false, true>);
-        if (mode == ND_AND_NN && ND_LATE_NOCACHE >= 2) {
-            if (gb)
-                return q == 1 ? k_pass<1, true, false, true, true>
-                              : (q == 2 ? k_pass<2, true, false, true, true> : k_pass<3, true, false, true, true>);
-            return q == 1 ? k_pass<1, true, false, false, true>
-                          : (q == 2 ? k_pass<2, true, false, false, true> : k_pass<3, true, false, false, true>);
-        }
-    }
     if (h->otf) return mode == ND_SND ? k_pass_otf<false, false> : (mode == ND_AND ? k_pass_otf<true, true> : k_pass_otf<true, false>);
-    if (h->gid && mode != ND_AND) {  // a batch: converged graphs are skipped
-        if (q == 1) return mode == ND_SND ? k_pass<1, false, false, true> : k_pass<1, true, false, true>;
-        if (q == 2) return mode == ND_SND ? k_pass<2, false, false, true> : k_pass<2, true, false, true>;
-        return mode == ND_SND ? k_pass<3, false, false, true> : k_pass<3, true, false, true>;
-    }
-    if (q == 1) return mode == ND_SND ? k_pass<1, false, false> : (mode == ND_AND ? k_pass<1, true, true> : k_pass<1, true, false>);
-    if (q == 2) return mode == ND_SND ? k_pass<2, false, false> : (mode == ND_AND ? k_pass<2, true, true> : k_pass<2, true, false>);
-    return mode == ND_SND ? k_pass<3, false, false> : (mode == ND_AND ? k_pass<3, true, true> : k_pass<3, true, false>);
+    const bool batch = h->gid && mode != ND_AND;  // converged graphs are skipped
+    return h->q == 1 ? pick_q<1>(mode, batch, late) : (h->q == 2 ? pick_q<2>(mode, batch, late) : pick_q<3>(mode, batch, late));
 }
 
 // bucket ranges of a pass
@@ -1208,6 +1205,18 @@ int pass_grid(const nd_incidence* h, const void* fn, int64_t units) {
     return (int)(g < 1 ? 1 : g);
 }
 
+// warp tasks per counter grab: kWarpChunk where there are many, fewer where
+// that would leave the resident warps with less than kChunksPerWarp grabs
+// each.  A graph of 2,000 vertices has 250 tasks: in chunks of 16 they kept 16
+// warps busy, one after the other (26 us per pass).  R-MAT of 100,003 vertices:
+// the first 16 SND passes 3.2 ms with 8 grabs, 3.9 with 4, 3.2 with 16 (whose
+// late passes are 12% slower).
+constexpr int kChunksPerWarp = 8;
+int pass_chunk(int64_t tasks, int grid) {
+    const int64_t c = tasks / ((int64_t)(grid > 0 ? grid : 1) * (kThreads / 32) * kChunksPerWarp);
+    return (int)(c < 1 ? 1 : (c > kWarpChunk ? kWarpChunk : c));
+}
+
 nd_status ensure_state(nd_incidence* h, bool and_mode, cudaStream_t st) {
     const int64_t N = h->num_r > 0 ? h->num_r : 1;
     if (!h->tau[0]) ND_TRY(nd_alloc((void**)&h->tau[0], sizeof(int32_t) * N, st, h));
@@ -1234,29 +1243,34 @@ nd_status ensure_state(nd_incidence* h, bool and_mode, cudaStream_t st) {
 
 
 // the smallest shared-memory carve-out (percent of the SM's maximum) that
-// holds the resident blocks of a pass kernel (all are built for 6 per SM)
+// holds the resident blocks of a pass kernel (all are built for kPassBlocks)
 nd_status request_carveout(const void* fn) {
-    static_assert(ND_PASS_MIN_BLOCKS == 6 && ND_AND_MIN_BLOCKS == 6 && ND_NC_MIN_BLOCKS == 6,
-                  "the carve-out is sized for six blocks per SM");
     cudaFuncAttributes fa;
     int dev = 0, max_sm = 0;
     ND_CUDA(cudaFuncGetAttributes(&fa, fn));
     ND_CUDA(cudaGetDevice(&dev));
     ND_CUDA(cudaDeviceGetAttribute(&max_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
     if (max_sm <= 0) return ND_OK;
-    const int64_t need = 6 * ((int64_t)fa.sharedSizeBytes + 1024);
+    const int64_t need = kPassBlocks * ((int64_t)fa.sharedSizeBytes + 1024);
     int pct = (int)((100 * need + max_sm - 1) / max_sm);  // rounded up to a supported carve-out
     if (pct > 100) pct = 100;
     ND_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, pct));
     return ND_OK;
 }
 
+// AND passes whose rows go straight to the histogram.  AND over a run with 0 /
+// 2 / 4 / 6 / 8 of them: 55.7 / 53.9 / 52.6 / 53.0 / 53.9 ms on the R-MAT
+// scale-20 k-truss, 71.9 / 68.0 / 66.1 / 62.9 / 62.7 on the scale-24 k-core
+constexpr int kAndDirect = 6;
+
 // parameters of one pass: its counter slot, the slot of the pass before it
 // (-1: none), and the parity of its index in the run (SND reads tau[parity]
 // and writes the other buffer; AND reads the frontier front[parity])
+// and whether an AND pass takes its rows for changing ones (its first passes)
 SweepParams pass_params(const nd_incidence* h, int mode, const SweepParams& P0, int slot, int prev_slot,
-                        int parity) {
+                        int parity, bool direct) {
     SweepParams P = P0;
+    P.direct = direct;
     P.ctr = h->counters + ND_SLOT * slot;
     P.prev = prev_slot < 0 ? nullptr : h->counters + ND_SLOT * prev_slot;
     if (P.gid) {
@@ -1287,7 +1301,7 @@ SweepParams pass_params(const nd_incidence* h, int mode, const SweepParams& P0, 
 // capture) so that it also serves the legacy default stream.  On any
 // failure the handle falls back to ordinary launches for this kind.
 void make_batch_graph(nd_incidence* h, int mode, int kind, const SweepParams& P0, int grid0, pass_fn fn0,
-                      int grid1, pass_fn fn1, int late_from, int64_t words) {
+                      int grid1, pass_fn fn1, int64_t words) {
     const int base = (kind == 2) ? ND_BATCH : 0;
     cudaGraph_t g = nullptr;
     cudaGraphExec_t ex = nullptr;
@@ -1306,7 +1320,7 @@ void make_batch_graph(nd_incidence* h, int mode, int kind, const SweepParams& P0
         // a batch starts at an even pass; its first pass reads the last slot
         // of the other half (the caller puts the previous pass's counters there)
         const int prev_slot = k > 0 ? base + k - 1 : (kind == 0 ? -1 : (base ^ ND_BATCH) + ND_BATCH - 1);
-        SweepParams P = pass_params(h, mode, P0, base + k, prev_slot, k & 1);
+        SweepParams P = pass_params(h, mode, P0, base + k, prev_slot, k & 1, mode != ND_SND && kind == 0 && k < kAndDirect);
         if (mode == ND_AND) {
             cudaMemsetParams ms = {};
             ms.dst = P.next;
@@ -1332,8 +1346,7 @@ void make_batch_graph(nd_incidence* h, int mode, int kind, const SweepParams& P0
         if (!ok) break;
         cudaKernelNodeParams kp = {};
         void* args[] = {&P};
-        // passes from late_from on (in the run) take the late-pass kernel
-        const bool late = (kind == 0 ? k : ND_BATCH + k) >= late_from;
+        const bool late = (kind == 0 ? k : ND_BATCH + k) >= kLateFrom;
         kp.func = (void*)(late ? fn1 : fn0);
         kp.gridDim = dim3(late ? grid1 : grid0);
         kp.blockDim = dim3(kThreads);
@@ -1461,7 +1474,6 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
         ND_CUDA(cudaGetLastError());
     }
     SweepParams P;
-    P.inc_ptr = h->inc_ptr;
     P.inc = h->inc;
     P.epos = h->e_pos;
     P.eid = h->eid;
@@ -1483,21 +1495,22 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
         P.gid = h->gid;
     }
     plan_buckets(h, P);
-    // the first batch of passes, where rows still search, keeps the rho
-    // cache; later batches may run a kernel without it
-    pass_fn fn0 = pick(h, mode), fn1 = pick(h, mode, true);
-    const int late_from = mode == ND_SND ? ND_LATE_FROM : ND_AND_LATE_FROM;
-    // ask for a shared-memory carve-out that just holds each kernel's six
+    pass_fn fn0 = pick(h, mode, false), fn1 = pick(h, mode, true);
+    // ask for a shared-memory carve-out that just holds each kernel's
     // resident blocks (plus the 1 KB each block reserves), leaving the rest
     // of the SM's memory as L1 for the gathers.  Left to itself the driver
     // chose 132 KB for the late-pass kernel, where 64 KB suffice.
-    if (ND_NC_CARVEOUT && !h->otf) {
-        if (ND_CARVEOUT_FN0) ND_TRY(request_carveout((const void*)fn0));
-        if (fn1 != fn0) ND_TRY(request_carveout((const void*)fn1));
+    if (!h->otf) {
+        ND_TRY(request_carveout((const void*)fn0));
+        ND_TRY(request_carveout((const void*)fn1));
     }
     const int64_t units = pass_units(h, P);
     const int grid0 = units > 0 ? pass_grid(h, (const void*)fn0, units) : 0;
     const int grid1 = units > 0 ? pass_grid(h, (const void*)fn1, units) : 0;
+    P.chunk = pass_chunk(units - (P.hi[3] - P.lo[3]), grid0 < grid1 ? grid0 : grid1);
+    // passes that evaluate every row do not count rows and incidences (Tally)
+    const bool counted = h->otf || mode == ND_AND || P.gid;
+    const int64_t all_rows = P.hi[ND_NB - 1] - P.lo[0], all_incs = h->num_inc;
     const int kBatch = ND_BATCH;
     // Thm. 3 / Lemma 2: SND settles within the number of degree levels, at
     // most N_R, and AND never needs more passes than SND.  A run longer than
@@ -1527,7 +1540,7 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
         // graphs hold the plain parameters; runs with members or a stopping rule launch directly
         if (nb == kBatch && grid0 > 0 && !members && (start & 1) == 0 && !h->pass_graph_failed[mode][kind]) {
             if (!h->pass_graph[mode][kind])
-                make_batch_graph(h, mode, kind, P, grid0, fn0, grid1, fn1, late_from, words);
+                make_batch_graph(h, mode, kind, P, grid0, fn0, grid1, fn1, words);
             if (h->pass_graph[mode][kind]) {
                 // the graph's first pass reads the last slot of the other half
                 const int want = (base ^ ND_BATCH) + ND_BATCH - 1;
@@ -1543,12 +1556,13 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
         if (!launched) {
             ND_CUDA(cudaMemsetAsync(h->counters + ND_SLOT * base, 0, sizeof(unsigned long long) * ND_SLOT * nb, st));
             for (int k = 0; k < nb; ++k, ++pass) {
-                SweepParams Pk = pass_params(h, mode, P, base + k, k > 0 ? base + k - 1 : last_slot, pass & 1);
+                SweepParams Pk = pass_params(h, mode, P, base + k, k > 0 ? base + k - 1 : last_slot, pass & 1,
+                                             mode != ND_SND && pass < kAndDirect);
                 if (mode == ND_AND)
                     ND_CUDA(cudaMemsetAsync(Pk.next, 0, sizeof(uint32_t) * words, st));
                 if (Pk.gid) ND_CUDA(cudaMemsetAsync(Pk.gact_out, 0, (size_t)h->ngraphs, st));
                 if (grid0 > 0) {
-                    const bool late = pass >= late_from;
+                    const bool late = pass >= kLateFrom;
                     nd_prof_scope ps(pname, st);
                     (late ? fn1 : fn0)<<<late ? grid1 : grid0, kThreads, 0, st>>>(Pk);
                     ND_CUDA(cudaGetLastError());
@@ -1562,7 +1576,7 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
         for (int k = 0; k < nb; ++k) {
             const int32_t p = start + k;
             unsigned long long ch = h->h_counters[ND_SLOT * (base + k)];
-            unsigned long long ev = h->h_counters[ND_SLOT * (base + k) + 1];
+            unsigned long long ev = counted ? h->h_counters[ND_SLOT * (base + k) + 1] : (unsigned long long)all_rows;
             // r-cliques with d_s = 0 are never launched: tau = H(empty) = 0 = d_s.
             // They count as evaluated in every SND / AND-nn pass and in the first
             // AND pass, as in the paper's sequential loops (in a batch, whose
@@ -1570,7 +1584,7 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
             if ((mode != ND_AND && !h->gid) || p == 0) ev += (unsigned long long)h->num_zero;
             h->last_changed.push_back((int64_t)ch);
             h->last_evals.push_back((int64_t)ev);
-            h->last_incs.push_back((int64_t)h->h_counters[ND_SLOT * (base + k) + 3]);
+            h->last_incs.push_back(counted ? (int64_t)h->h_counters[ND_SLOT * (base + k) + 3] : all_incs);
             *evals += (int64_t)ev;
             if (!and_mode) last_written = (p & 1) ^ 1;
             if (ch == 0) { done = true; break; }

@@ -1,0 +1,69 @@
+"""GPU rows at the edges of the h-index kernels, against the CPU oracle.
+
+A power-law background gives tau many values; hub vertices (for (1,2)) and
+pairs of adjacent hubs (for (2,3)) get rows of exactly the lengths where the
+evaluation changes: the lane-group, warp and CTA buckets, blocks of 64 and
+128 streamed entries, and histograms that hold one value per bin, several
+values per bin, or need a second sweep.  Integers: every comparison is exact.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1704_00386_gb300 import graphs as G
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+LENGTHS = (7, 8, 9, 63, 64, 65, 127, 128, 129, 255, 256, 257, 511, 512, 513, 1024, 2047, 2048, 2049, 4095, 4097, 5900)
+
+
+@pytest.fixture(scope="module")
+def nd():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1704_00386_gb300 import nd as _nd
+    _nd.load()
+    return _nd
+
+
+def _rows_graph(pairs: bool):
+    n0 = 6000
+    rng = np.random.default_rng(31)
+    src, dst = [x.tolist() for x in G.chung_lu(n0, 2.1, 60.0 if not pairs else 24.0, seed=33)]
+    n = n0
+    for k in LENGTHS:
+        nb = rng.choice(n0, size=k, replace=False).tolist()
+        for h in ((n, n + 1) if pairs else (n,)):
+            src += [h] * k
+            dst += nb
+        if pairs:
+            src.append(n)
+            dst.append(n + 1)
+        n += 2 if pairs else 1
+    return G.to_csr(n, src, dst)
+
+
+@pytest.mark.parametrize("r", [1, 2])
+def test_rows_at_the_edges(nd, r):
+    rp, col = _rows_graph(pairs=r == 2)
+    g = oracle.Graph(rp, col, r, r + 1)
+    inc = nd.build_incidence(torch.from_numpy(rp).cuda(), torch.from_numpy(col).cuda(), r, r + 1)
+    ds = inc.s_degree().cpu().numpy()
+    np.testing.assert_array_equal(ds, g.s_degree())
+    assert set(LENGTHS) <= set(ds.tolist())
+    kap = g.peel()
+    tau, iters = inc.snd()
+    assert iters == g.snd()[2]
+    np.testing.assert_array_equal(tau.cpu().numpy(), kap)
+    for k in (1, 2, 3, 4):
+        tk, _ = inc.iterate_k("snd", k)
+        np.testing.assert_array_equal(tk.cpu().numpy(), g.snd(max_sweeps=k)[0])
+    # from a given tau the first pass counts before it searches
+    t1, _ = inc.iterate_k("snd", 1)
+    t3, _ = inc.iterate_k("snd", 2, tau=t1)
+    np.testing.assert_array_equal(t3.cpu().numpy(), g.snd(max_sweeps=3)[0])
+    for notify in (True, False):
+        np.testing.assert_array_equal(inc.and_(notify=notify)[0].cpu().numpy(), kap)
+    ta, _ = inc.iterate_k("and", 1 << 20, tau=t1)
+    np.testing.assert_array_equal(ta.cpu().numpy(), kap)

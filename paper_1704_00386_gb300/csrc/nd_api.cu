@@ -128,8 +128,55 @@ static void keep_pool(int dev) {
     });
 }
 
-// bounded wait: poll the stream instead of blocking forever
+// Pinned blocks for the handles' counters and read-backs.  Pinning a page
+// takes longer than a small decomposition, so up to kPinnedKept blocks of
+// freed handles wait for the next ones; the rest are given back.  Any thread
+// may take and put blocks; a block is put only after its handle's stream has
+// drained.
+namespace {
+constexpr size_t kPinnedBytes = sizeof(unsigned long long) * ND_SLOT * ND_RING + sizeof(int64_t) * ND_READ;
+constexpr size_t kPinnedKept = 64;
+std::mutex g_pinned_mu;
+std::vector<void*> g_pinned;
+}  // namespace
+
+void* nd_pinned_get() {
+    {
+        std::lock_guard<std::mutex> lk(g_pinned_mu);
+        if (!g_pinned.empty()) {
+            void* p = g_pinned.back();
+            g_pinned.pop_back();
+            return p;
+        }
+    }
+    void* p = nullptr;
+    if (cudaHostAlloc(&p, kPinnedBytes, cudaHostAllocPortable) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return p;
+}
+
+void nd_pinned_put(void* p) {
+    if (!p) return;
+    {
+        std::lock_guard<std::mutex> lk(g_pinned_mu);
+        if (g_pinned.size() < kPinnedKept) {
+            try {
+                g_pinned.push_back(p);
+                return;
+            } catch (...) {
+            }
+        }
+    }
+    cudaFreeHost(p);
+}
+
+// bounded wait: poll the stream instead of blocking forever.  A sleep of 20 us
+// takes three times that to return, so the first kSpinSeconds only poll: most
+// waits of a small decomposition end there.
 static std::atomic<double> g_wait_limit{600.0};
+constexpr double kSpinSeconds = 1e-3;
 
 nd_status nd_wait(cudaStream_t st) {
     const double seconds = g_wait_limit.load();
@@ -138,13 +185,15 @@ nd_status nd_wait(cudaStream_t st) {
         cudaError_t e = cudaStreamQuery(st);
         if (e == cudaSuccess) return ND_OK;
         if (e != cudaErrorNotReady) return nd_cuda_fail(e, "cudaStreamQuery", __FILE__, __LINE__);
-        if (std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count() > seconds) {
+        const double waited = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
+        if (waited > seconds) {
             char buf[96];
             snprintf(buf, sizeof(buf), "stream did not finish within %g s", seconds);
             nd_set_error(buf);
             return ND_E_TIMEOUT;
         }
-        std::this_thread::sleep_for(std::chrono::microseconds(20));
+        if (waited < kSpinSeconds) std::this_thread::yield();
+        else std::this_thread::sleep_for(std::chrono::microseconds(20));
     }
 }
 
@@ -204,8 +253,8 @@ void nd_free(nd_incidence* h) {
     }
     nd_release(h->rp, st);
     nd_release(h->col, st);
-    if (h->h_counters) cudaFreeHost(h->h_counters);
     cudaStreamSynchronize(st);
+    nd_pinned_put(h->h_counters);
     delete h;
 }
 
@@ -278,6 +327,13 @@ static nd_status build_common(const nd_csr* g, int r, int s, cudaStream_t st, nd
     if (cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         h->sm_count = 152;
     h->last_stream = st;
+    h->h_counters = (unsigned long long*)nd_pinned_get();
+    if (!h->h_counters) {
+        delete h;
+        nd_set_error("pinned host allocation failed");
+        return ND_E_NOMEM;
+    }
+    h->h_read = (int64_t*)(h->h_counters + ND_SLOT * ND_RING);
     nd_status rc = nd_build_graph(h, g, st, r == 2 && !h->otf && relabel);
     if (rc == ND_OK && r == 2 && !h->otf && relabel) rc = nd_relabel_truss_graph(h, st);
     if (rc == ND_OK && r >= 2) rc = nd_build_edges(h, st);

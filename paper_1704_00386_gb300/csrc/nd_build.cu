@@ -201,7 +201,12 @@ __global__ void k_validate_split(int64_t n, int64_t nnz, const int64_t* __restri
             continue;
         }
         if (is_long_row(b, e)) {  // counted by k_validate_long
-            if (lane == 0) { nlow[u] = 0; upcnt[u] = 0; }
+            if (lane == 0) {
+                nlow[u] = 0;
+                upcnt[u] = 0;
+                // a graph of at most kLongRow vertices: too long to be simple
+                if (n <= kLongRow) atomicOr(err, 2);
+            }
             continue;
         }
         int low = 0, found = 0;
@@ -1050,32 +1055,78 @@ __device__ __forceinline__ int bucket_of(int64_t d, int3 t) {
     return d == 0 ? -1 : (d <= t.x ? 0 : (d <= t.y ? 1 : (d <= t.z ? 2 : 3)));
 }
 
-__global__ void k_bucket_flags(int64_t N, const int64_t* __restrict__ inc_ptr, int b, int3 thr,
-                               int64_t* __restrict__ flags, unsigned long long* __restrict__ inc_sum) {
-    unsigned long long local = 0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        int64_t d = inc_ptr[i + 1] - inc_ptr[i];
-        bool in = bucket_of(d, thr) == b;
-        flags[i] = in;
-        if (in) local += (unsigned long long)d;
+// rows per block: kThreads at a time, in order
+constexpr int kBucketTile = 2048;
+
+// cnt[b * nblocks + block] = rows of the block's tile in bucket b
+__global__ void __launch_bounds__(kThreads) k_bucket_count(int64_t N, const int64_t* __restrict__ inc_ptr, int3 thr,
+                                                           int64_t nblocks, int64_t* __restrict__ cnt) {
+    __shared__ unsigned c[ND_NB];
+    if (threadIdx.x < ND_NB) c[threadIdx.x] = 0;
+    __syncthreads();
+    const int64_t t0 = (int64_t)blockIdx.x * kBucketTile;
+    unsigned own[ND_NB] = {0, 0, 0, 0};
+#pragma unroll
+    for (int k = 0; k < kBucketTile / kThreads; ++k) {
+        const int64_t i = t0 + k * kThreads + threadIdx.x;
+        const int b = i < N ? bucket_of(inc_ptr[i + 1] - inc_ptr[i], thr) : -1;
+#pragma unroll
+        for (int q = 0; q < ND_NB; ++q) own[q] += (b == q);
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) local += __shfl_xor_sync(kFull, local, o);
-    if ((threadIdx.x & 31) == 0 && local) atomicAdd(inc_sum, local);
+    for (int q = 0; q < ND_NB; ++q) {
+        const unsigned w = __reduce_add_sync(kFull, own[q]);
+        if ((threadIdx.x & 31) == 0 && w) atomicAdd(&c[q], w);
+    }
+    __syncthreads();
+    if (threadIdx.x < ND_NB) cnt[threadIdx.x * nblocks + blockIdx.x] = c[threadIdx.x];
 }
 
-__global__ void k_bucket_scatter(int64_t N, const int64_t* __restrict__ inc_ptr, int b, int3 thr,
-                                 const int64_t* __restrict__ pos, nd_item* __restrict__ items) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        int64_t d = inc_ptr[i + 1] - inc_ptr[i];
-        if (bucket_of(d, thr) == b) {
-            nd_item it;
-            it.jb = inc_ptr[i];
-            it.R = (uint32_t)i;
-            it.d = (uint32_t)d;
-            items[pos[i]] = it;
+// the work items of the tile's rows, in order inside their bucket: start of
+// (bucket, block) in off, plus the earlier rows of the bucket in the tile
+__global__ void __launch_bounds__(kThreads) k_bucket_scatter(int64_t N, const int64_t* __restrict__ inc_ptr, int3 thr,
+                                                             int64_t nblocks, const int64_t* __restrict__ off,
+                                                             nd_item* __restrict__ items) {
+    constexpr int kWarps = kThreads / 32;
+    __shared__ unsigned wcnt[2][kWarps][ND_NB];  // two rounds' buffers: one barrier per round
+    int64_t run[ND_NB];
+#pragma unroll
+    for (int q = 0; q < ND_NB; ++q) run[q] = off[q * nblocks + blockIdx.x];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t t0 = (int64_t)blockIdx.x * kBucketTile;
+    for (int k = 0; k < kBucketTile / kThreads && t0 + k * kThreads < N; ++k) {
+        const int64_t i = t0 + k * kThreads + threadIdx.x;
+        int64_t jb = 0, d = 0;
+        if (i < N) {
+            jb = inc_ptr[i];
+            d = inc_ptr[i + 1] - jb;
+        }
+        const int b = i < N ? bucket_of(d, thr) : -1;
+        unsigned before = 0;
+#pragma unroll
+        for (int q = 0; q < ND_NB; ++q) {
+            const unsigned m = __ballot_sync(kFull, b == q);
+            if (b == q) before = __popc(m & lanemask_lt());
+            if (lane == 0) wcnt[k & 1][w][q] = __popc(m);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < ND_NB; ++q) {
+            unsigned mine = 0, all = 0;
+#pragma unroll
+            for (int v = 0; v < kWarps; ++v) {
+                const unsigned c = wcnt[k & 1][v][q];
+                all += c;
+                if (v < w) mine += c;
+            }
+            if (b == q) {
+                nd_item it;
+                it.jb = jb;
+                it.R = (uint32_t)i;
+                it.d = (uint32_t)d;
+                items[run[q] + mine + before] = it;
+            }
+            run[q] += all;
         }
     }
 }
@@ -1142,15 +1193,24 @@ __global__ void k_gather_i64(const int64_t* __restrict__ src, const int64_t* __r
 
 int grid_cap(const nd_incidence* h) { return (h->sm_count > 0 ? h->sm_count : 152) * 8; }
 
-nd_status read_flag(int* dflag, int* hval, cudaStream_t st) {
-    ND_CUDA(cudaMemcpyAsync(hval, dflag, sizeof(int), cudaMemcpyDeviceToHost, st));
-    ND_TRY(nd_wait(st));
+// device words to the handle's pinned words [at, at + count): valid after the
+// next nd_wait, so one wait serves several of them
+nd_status fetch(nd_incidence* h, int at, const void* d, int count, cudaStream_t st) {
+    ND_CUDA(cudaMemcpyAsync(h->h_read + at, d, sizeof(int64_t) * count, cudaMemcpyDeviceToHost, st));
     return ND_OK;
 }
 
-nd_status read_i64(const int64_t* d, int64_t* hv, cudaStream_t st) {
-    ND_CUDA(cudaMemcpyAsync(hv, d, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+nd_status read_flag(nd_incidence* h, const int* dflag, int* hval, cudaStream_t st) {
+    ND_CUDA(cudaMemcpyAsync(h->h_read, dflag, sizeof(int), cudaMemcpyDeviceToHost, st));
     ND_TRY(nd_wait(st));
+    *hval = *(const int*)h->h_read;
+    return ND_OK;
+}
+
+nd_status read_i64(nd_incidence* h, const int64_t* d, int64_t* hv, cudaStream_t st) {
+    ND_TRY(fetch(h, 0, d, 1, st));
+    ND_TRY(nd_wait(st));
+    *hv = h->h_read[0];
     return ND_OK;
 }
 
@@ -1162,7 +1222,9 @@ nd_status read_i64(const int64_t* d, int64_t* hv, cudaStream_t st) {
 // (a host scan over the few such rows); kept on the handle for the edge ids
 static nd_status find_long_rows(nd_incidence* h, cudaStream_t st) {
     h->long_count = h->long_segs = 0;
-    if (h->n == 0 || h->nnz <= kLongRow) return ND_OK;
+    // a simple graph of n vertices has no row past n - 1 entries; the
+    // validation refuses one that is longer
+    if (h->n <= kLongRow || h->nnz <= kLongRow) return ND_OK;
     const int64_t cap = h->nnz / kLongRow + 1;
     ND_TRY(nd_alloc((void**)&h->long_rows, sizeof(int32_t) * cap, st, h));
     nd_tmp<int64_t> len(st);
@@ -1173,9 +1235,9 @@ static nd_status find_long_rows(nd_incidence* h, cudaStream_t st) {
     k_long_rows<<<nd_blocks_for(h->n, kThreads, grid_cap(h) * 4), kThreads, 0, st>>>(
         h->n, h->nnz, h->rp, h->long_rows, len, (unsigned long long)cap, cnt);
     ND_CUDA(cudaGetLastError());
-    unsigned long long c = 0;
-    ND_CUDA(cudaMemcpyAsync(&c, cnt.p, sizeof(c), cudaMemcpyDeviceToHost, st));
-    ND_TRY(nd_wait(st));
+    int64_t cc = 0;
+    ND_TRY(read_i64(h, (const int64_t*)cnt.p, &cc, st));
+    const unsigned long long c = (unsigned long long)cc;
     if (c > (unsigned long long)cap) {  // overlapping rows: not an offset array
         nd_set_error("row_ptr is not a valid offset array");
         return ND_E_INVAL;
@@ -1213,14 +1275,12 @@ static nd_status validate_split(nd_incidence* h, cudaStream_t st, bool by_length
     // reverse entries for the edge ids and the (2,3) adjacency layout (build only)
     if (mirror && h->r >= 2 && g->nnz > 0 && g->nnz < (int64_t)UINT32_MAX)
         ND_TRY(nd_alloc((void**)&h->mirror, sizeof(uint32_t) * g->nnz, st, h));
-    nd_tmp<int> derr(st);
-    ND_TRY(derr.alloc(1));
-    ND_CUDA(cudaMemsetAsync(derr, 0, sizeof(int), st));
     // k-core builds (no reverse entries needed) decide symmetry by fingerprint
     const bool fp = h->r == 1;
     nd_tmp<unsigned long long> dsearched(st);
-    ND_TRY(dsearched.alloc(3));  // [0] searching entries found, [1..2] fingerprint sums
-    ND_CUDA(cudaMemsetAsync(dsearched, 0, 3 * sizeof(unsigned long long), st));
+    ND_TRY(dsearched.alloc(4));  // [0] searching entries found, [1..2] fingerprint sums, [3] error bits
+    ND_CUDA(cudaMemsetAsync(dsearched, 0, 4 * sizeof(unsigned long long), st));
+    int* const derr = (int*)(dsearched.p + 3);
     ND_CUDA(cudaMemsetAsync(h->up_start, 0, sizeof(int64_t) * (g->n + 1), st));
     ND_TRY(find_long_rows(h, st));
     if (g->n > 0) {
@@ -1238,20 +1298,19 @@ static nd_status validate_split(nd_incidence* h, cudaStream_t st, bool by_length
             ND_CUDA(cudaGetLastError());
         }
     }
-    int herr = 0;
-    ND_TRY(read_flag(derr, &herr, st));
+    ND_TRY(nd_scan_i64(h->up_start, g->n, st));
+    // everything the host decides on, with one wait
+    ND_TRY(fetch(h, 0, dsearched.p, 4, st));
+    ND_TRY(fetch(h, 4, h->up_start + g->n, 1, st));
+    ND_TRY(nd_wait(st));
+    const int herr = *(const int*)(h->h_read + 3);
     if (herr) {
         nd_set_error(herr & 1 ? "row_ptr is not a valid offset array"
                               : "col is not simple, sorted and symmetric");
         return ND_E_INVAL;
     }
-    ND_TRY(nd_scan_i64(h->up_start, g->n, st));
-    int64_t m = 0, found = 0;
-    unsigned long long hs[3] = {0, 0, 0};
-    ND_TRY(read_i64(h->up_start + g->n, &m, st));
-    ND_CUDA(cudaMemcpyAsync(hs, dsearched.p, sizeof(hs), cudaMemcpyDeviceToHost, st));
-    ND_TRY(nd_wait(st));
-    found = (int64_t)hs[0];
+    const int64_t m = h->h_read[4], found = h->h_read[0];
+    const unsigned long long hs[3] = {0, (unsigned long long)h->h_read[1], (unsigned long long)h->h_read[2]};
     if (fp ? (hs[1] != 0 || hs[2] != 0 || 2 * m != g->nnz) : (2 * found != g->nnz || 2 * m != g->nnz)) {
         // every searching entry has its reverse; a surplus of the others is
         // an entry without one
@@ -1386,7 +1445,7 @@ nd_status nd_relabel_truss_edges(nd_incidence* h, cudaStream_t st) {
         ND_CUDA(cudaGetLastError());
     }
     int herr = 0;
-    ND_TRY(read_flag(derr, &herr, st));
+    ND_TRY(read_flag(h, derr, &herr, st));
     if (herr) { nd_set_error("an edge of the relabelled graph is missing from the caller's (internal fault)"); return ND_E_CUDA; }
     nd_release(h->c_rp, st);
     nd_release(h->c_col, st);
@@ -1534,10 +1593,12 @@ static nd_status sort_tri_rows(nd_incidence* h, cudaStream_t st) {
     }
     nd_tmp<uint32_t> over(st);
     nd_tmp<unsigned long long> over_ctr(st);
-    nd_status rc = over.alloc(N);
+    // no adjacency list of n <= 32 * kRankWords vertices needs more words
+    const bool can_overflow = h->n > 32 * (int64_t)kRankWords;
+    nd_status rc = over.alloc(can_overflow ? N : 1);
     if (rc == ND_OK) rc = over_ctr.alloc(2);
     if (rc != ND_OK) { cudaFreeAsync(dst, st); return rc; }
-    ND_CUDA(cudaMemsetAsync(over_ctr, 0, sizeof(unsigned long long) * 2, st));
+    if (can_overflow) ND_CUDA(cudaMemsetAsync(over_ctr, 0, sizeof(unsigned long long) * 2, st));
     const size_t smem = sizeof(uint32_t) * 2 * kRankWords * kRankWarps;
     ND_CUDA(cudaFuncSetAttribute(k_row_rank<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     {
@@ -1549,8 +1610,12 @@ static nd_status sort_tri_rows(nd_incidence* h, cudaStream_t st) {
         ND_CUDA(cudaGetLastError());
     }
     unsigned long long hc[2] = {0, 0};
-    ND_CUDA(cudaMemcpyAsync(hc, over_ctr.p, sizeof(hc), cudaMemcpyDeviceToHost, st));
-    ND_TRY(nd_wait(st));
+    if (can_overflow) {
+        ND_TRY(fetch(h, 0, over_ctr.p, 2, st));
+        ND_TRY(nd_wait(st));
+        hc[0] = (unsigned long long)h->h_read[0];
+        hc[1] = (unsigned long long)h->h_read[1];
+    }
     if (hc[0] > 0) {
         // rows whose shorter adjacency list needs more than kRankWords words
         const int warps = 64;
@@ -1568,6 +1633,10 @@ static nd_status sort_tri_rows(nd_incidence* h, cudaStream_t st) {
     return ND_OK;
 }
 
+// smaller (2,3) builds search twice: their searches are a few microseconds,
+// less than the launches, the scan and the wait that size the records
+constexpr int64_t kRecordMinEdges = 1 << 16;
+
 nd_status nd_build_tri_incidence(nd_incidence* h, cudaStream_t st) {
     const int64_t m = h->m;
     h->num_r = m;
@@ -1584,14 +1653,14 @@ nd_status nd_build_tri_incidence(nd_incidence* h, cudaStream_t st) {
     nd_tmp<int64_t> rec_ptr(st);
     nd_tmp<uint32_t> rec(st), rec_cnt(st);
     bool use_rec = false;
-    if (h->adj && !h->otf && rec_ptr.alloc(m + 1) == ND_OK) {
+    if (h->adj && !h->otf && m >= kRecordMinEdges && rec_ptr.alloc(m + 1) == ND_OK) {
         k_rec_bound<<<nd_blocks_for(m, kThreads, grid_cap(h) * 4), kThreads, 0, st>>>(m, o.out_ptr, o.out_src,
                                                                                      o.out_col, rec_ptr);
         ND_CUDA(cudaGetLastError());
         ND_CUDA(cudaMemsetAsync(rec_ptr.p + m, 0, sizeof(int64_t), st));
         ND_TRY(nd_scan_i64(rec_ptr, m, st));
         int64_t slots = 0;
-        ND_TRY(read_i64(rec_ptr.p + m, &slots, st));
+        ND_TRY(read_i64(h, rec_ptr.p + m, &slots, st));
         use_rec = rec.alloc(slots) == ND_OK && rec_cnt.alloc(m) == ND_OK;
         if (!use_rec) nd_set_error("");
     }
@@ -1614,7 +1683,7 @@ nd_status nd_build_tri_incidence(nd_incidence* h, cudaStream_t st) {
         ND_CUDA(cudaGetLastError());
     }
     ND_TRY(nd_scan_i64(h->inc_ptr, m, st));
-    ND_TRY(read_i64(h->inc_ptr + m, &h->num_inc, st));
+    ND_TRY(read_i64(h, h->inc_ptr + m, &h->num_inc, st));
     if (h->otf) {
         // no stored incidence: the counts (d_s, tau_0 and the buckets) are all
         // that is kept; every pass finds the triangles again
@@ -1680,7 +1749,7 @@ nd_status nd_build_triangles(nd_incidence* h, cudaStream_t st) {
         ND_CUDA(cudaGetLastError());
     }
     ND_TRY(nd_scan_i64(h->tri_ptr, h->m, st));
-    ND_TRY(read_i64(h->tri_ptr + h->m, &h->num_tri, st));
+    ND_TRY(read_i64(h, h->tri_ptr + h->m, &h->num_tri, st));
     if (h->num_tri >= (int64_t)UINT32_MAX) { nd_set_error("more than 2^32-1 triangles"); return ND_E_TOO_LARGE; }
     ND_TRY(nd_alloc((void**)&h->tri_w, sizeof(int32_t) * (h->num_tri > 0 ? h->num_tri : 1), st, h));
     ND_TRY(nd_alloc((void**)&h->tri_e, sizeof(uint32_t) * (h->num_tri > 0 ? h->num_tri : 1), st, h));
@@ -1733,7 +1802,7 @@ nd_status nd_build_k4_incidence(nd_incidence* h, cudaStream_t st) {
     }
     ND_TRY(nd_scan_i64(kptr, T, st));
     int64_t K = 0;
-    ND_TRY(read_i64(kptr.p + T, &K, st));
+    ND_TRY(read_i64(h, kptr.p + T, &K, st));
     nd_tmp<uint4> k4(st);
     ND_TRY(k4.alloc(K));
     if (K > 0) {
@@ -1743,7 +1812,14 @@ nd_status nd_build_k4_incidence(nd_incidence* h, cudaStream_t st) {
         ND_CUDA(cudaGetLastError());
     }
     ND_TRY(nd_scan_i64(h->inc_ptr, T, st));
-    ND_TRY(read_i64(h->inc_ptr + T, &h->num_inc, st));
+    ND_TRY(fetch(h, 0, h->inc_ptr + T, 1, st));
+    ND_CUDA(cudaMemcpyAsync(h->h_read + 1, derr, sizeof(int), cudaMemcpyDeviceToHost, st));
+    ND_TRY(nd_wait(st));
+    h->num_inc = h->h_read[0];
+    if (*(const int*)(h->h_read + 1)) {
+        nd_set_error("internal: a triangle of a 4-clique was not found");
+        return ND_E_INVAL;
+    }
     ND_TRY(nd_alloc((void**)&h->inc, sizeof(uint32_t) * 3 * (h->num_inc > 0 ? h->num_inc : 1), st, h));
     if (K > 0) {
         nd_prof_scope ps("k4_fill", st);
@@ -1762,9 +1838,6 @@ nd_status nd_build_k4_incidence(nd_incidence* h, cudaStream_t st) {
         }
         ND_CUDA(cudaGetLastError());
     }
-    int herr = 0;
-    ND_TRY(read_flag(derr, &herr, st));
-    if (herr) { nd_set_error("internal: a triangle of a 4-clique was not found"); return ND_E_INVAL; }
     return ND_OK;
 }
 
@@ -1774,40 +1847,36 @@ nd_status nd_build_buckets(nd_incidence* h, cudaStream_t st) {
     for (auto& row : h->pass_graph)
         for (auto& ex : row)
             if (ex) { cudaGraphExecDestroy(ex); ex = nullptr; }
-    const int3 thr = make_int3(h->thr[0], h->thr[1], h->thr[2]);
-    nd_tmp<int64_t> flags(st);
-    nd_tmp<unsigned long long> sums(st);
-    ND_TRY(flags.alloc(N + 1));
-    ND_TRY(sums.alloc(ND_NB));
-    ND_CUDA(cudaMemsetAsync(sums, 0, sizeof(unsigned long long) * ND_NB, st));
+    for (int b = 0; b <= ND_NB; ++b) h->bucket_lo[b] = 0;
+    h->num_zero = N;
     if (!h->items) ND_TRY(nd_alloc((void**)&h->items, sizeof(nd_item) * (N > 0 ? N : 1), st, h));
-    int blocks = nd_blocks_for(N, kThreads, grid_cap(h) * 2);
-    int64_t lo = 0;
-    for (int b = 0; b < ND_NB; ++b) {
-        h->bucket_lo[b] = lo;
-        if (N == 0) continue;
-        ND_CUDA(cudaMemsetAsync(flags.p + N, 0, sizeof(int64_t), st));
-        {
-            nd_prof_scope ps("buckets", st);
-            k_bucket_flags<<<blocks, kThreads, 0, st>>>(N, h->inc_ptr, b, thr, flags, sums.p + b);
-            ND_CUDA(cudaGetLastError());
-        }
-        ND_TRY(nd_scan_i64(flags, N, st));
-        {
-            nd_prof_scope ps("buckets", st);
-            k_bucket_scatter<<<blocks, kThreads, 0, st>>>(N, h->inc_ptr, b, thr, flags, h->items + lo);
-            ND_CUDA(cudaGetLastError());
-        }
-        int64_t cnt = 0;
-        ND_TRY(read_i64(flags.p + N, &cnt, st));
-        lo += cnt;
+    if (N == 0) return ND_OK;
+    // a stable counting sort of the rows by bucket: the counts per (bucket,
+    // tile), one scan, one scatter, and the five bounds read back at once.
+    // One flag array, scan and read-back per bucket before: 0.16 of the 1.1 ms
+    // of a 10,000-edge k-truss, and 16 B more per row of scratch.
+    const int3 thr = make_int3(h->thr[0], h->thr[1], h->thr[2]);
+    const int64_t nblocks = (N + kBucketTile - 1) / kBucketTile;
+    nd_tmp<int64_t> cnt(st);
+    ND_TRY(cnt.alloc(ND_NB * nblocks + 1));
+    {
+        nd_prof_scope ps("buckets", st);
+        k_bucket_count<<<(unsigned)nblocks, kThreads, 0, st>>>(N, h->inc_ptr, thr, nblocks, cnt);
+        ND_CUDA(cudaGetLastError());
     }
-    h->bucket_lo[ND_NB] = lo;
-    unsigned long long hs[ND_NB] = {0, 0, 0, 0};
-    ND_CUDA(cudaMemcpyAsync(hs, sums, sizeof(hs), cudaMemcpyDeviceToHost, st));
+    ND_CUDA(cudaMemsetAsync(cnt.p + ND_NB * nblocks, 0, sizeof(int64_t), st));
+    ND_TRY(nd_scan_i64(cnt, ND_NB * nblocks, st));
+    {
+        nd_prof_scope ps("buckets", st);
+        k_bucket_scatter<<<(unsigned)nblocks, kThreads, 0, st>>>(N, h->inc_ptr, thr, nblocks, cnt, h->items);
+        ND_CUDA(cudaGetLastError());
+    }
+    // the first entry of every bucket's counts, and the total
+    ND_CUDA(cudaMemcpy2DAsync(h->h_read, sizeof(int64_t), cnt.p, sizeof(int64_t) * nblocks, sizeof(int64_t),
+                              ND_NB + 1, cudaMemcpyDeviceToHost, st));
     ND_TRY(nd_wait(st));
-    for (int b = 0; b < ND_NB; ++b) h->bucket_inc[b] = (int64_t)hs[b];
-    h->num_zero = N - lo;
+    for (int b = 0; b <= ND_NB; ++b) h->bucket_lo[b] = h->h_read[b];
+    h->num_zero = N - h->bucket_lo[ND_NB];
     return ND_OK;
 }
 
@@ -1839,7 +1908,8 @@ nd_status nd_union_device(const nd_union_part* parts_host, int count, int64_t n,
     }
     ND_CUDA(cudaMemcpyAsync(urp + n, &nnz, sizeof(int64_t), cudaMemcpyHostToDevice, st));
     int herr = 0;
-    ND_TRY(read_flag(derr, &herr, st));
+    ND_CUDA(cudaMemcpyAsync(&herr, derr.p, sizeof(int), cudaMemcpyDeviceToHost, st));
+    ND_TRY(nd_wait(st));
     if (herr) {
         nd_set_error(herr & 1 ? "a graph of the batch has an invalid row_ptr"
                               : "a graph of the batch has a neighbour id outside its own vertex range");

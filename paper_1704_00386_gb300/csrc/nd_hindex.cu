@@ -1234,10 +1234,7 @@ nd_status ensure_state(nd_incidence* h, bool and_mode, cudaStream_t st) {
         ND_TRY(nd_alloc((void**)&h->front[0], sizeof(uint32_t) * words, st, h));
         ND_TRY(nd_alloc((void**)&h->front[1], sizeof(uint32_t) * words, st, h));
     }
-    if (!h->counters) {
-        ND_TRY(nd_alloc((void**)&h->counters, sizeof(unsigned long long) * ND_SLOT * ND_RING, st, h));
-        ND_CUDA(cudaMallocHost((void**)&h->h_counters, sizeof(unsigned long long) * ND_SLOT * ND_RING));
-    }
+    if (!h->counters) ND_TRY(nd_alloc((void**)&h->counters, sizeof(unsigned long long) * ND_SLOT * ND_RING, st, h));
     return ND_OK;
 }
 
@@ -1537,8 +1534,13 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
         if (stop_active > 0.0) nb = 1;  // the stopping rule looks at every pass
         const int kind = batch == 0 ? 0 : ((batch & 1) ? 2 : 1);
         bool launched = false;
-        // graphs hold the plain parameters; runs with members or a stopping rule launch directly
-        if (nb == kBatch && grid0 > 0 && !members && (start & 1) == 0 && !h->pass_graph_failed[mode][kind]) {
+        // graphs hold the plain parameters; runs with members or a stopping
+        // rule launch directly, and so does the first batch of its kind on a
+        // handle: building a graph costs more than its launches, and many
+        // handles run each mode once
+        const bool seen = h->batch_seen[mode][kind];
+        if (nb == kBatch) h->batch_seen[mode][kind] = true;
+        if (nb == kBatch && seen && grid0 > 0 && !members && (start & 1) == 0 && !h->pass_graph_failed[mode][kind]) {
             if (!h->pass_graph[mode][kind])
                 make_batch_graph(h, mode, kind, P, grid0, fn0, grid1, fn1, words);
             if (h->pass_graph[mode][kind]) {

@@ -120,14 +120,14 @@ struct nd_incidence {
     // degree-bucketed processing order
     nd_item* items = nullptr;      // [num_r - num_zero], bucket by bucket
     int64_t bucket_lo[ND_NB + 1] = {0, 0, 0, 0, 0};
-    int64_t bucket_inc[ND_NB] = {0, 0, 0, 0};
     int64_t num_zero = 0;          // r-cliques with d_s = 0 (kappa = 0, never updated)
     int32_t thr[3] = {8, 64, 2048};  // bucket thresholds t0, t1, t2
     // iteration state
     int32_t* tau[2] = {nullptr, nullptr};
     uint32_t* front[2] = {nullptr, nullptr};
     unsigned long long* counters = nullptr;  // ring of per-pass counters
-    unsigned long long* h_counters = nullptr;  // pinned host mirror
+    unsigned long long* h_counters = nullptr;  // pinned host mirror, at the head of the handle's pinned block
+    int64_t* h_read = nullptr;                 // ND_READ pinned words after it, for counts read back in the build
     std::vector<int64_t> last_changed, last_evals, last_incs;
     int64_t bytes = 0;
     cudaStream_t last_stream = 0;  // stream of the latest call on this handle
@@ -136,6 +136,7 @@ struct nd_incidence {
     cudaGraphExec_t pass_graph[3][3] = {{nullptr, nullptr, nullptr}, {nullptr, nullptr, nullptr},
                                         {nullptr, nullptr, nullptr}};
     bool pass_graph_failed[3][3] = {{false, false, false}, {false, false, false}, {false, false, false}};
+    bool batch_seen[3][3] = {{false, false, false}, {false, false, false}, {false, false, false}};
     // set while a call uses the iteration state (nd_claim); a second call
     // meanwhile gets ND_E_BUSY
     std::atomic<int> busy{0};
@@ -167,6 +168,12 @@ struct nd_claim {
 // passes are enqueued in batches of ND_BATCH; the per-pass counters (ND_SLOT
 // u64 each) live in two halves of ND_BATCH slots used by alternate batches
 enum { ND_BATCH = 16, ND_RING = 2 * ND_BATCH, ND_SLOT = 6 };
+enum { ND_READ = 16 };
+
+// a pinned block for a handle's counters and read-backs, from a bounded pool
+// (nd_api.cu); null if there is no memory
+void* nd_pinned_get();
+void nd_pinned_put(void* p);
 
 // wait for a stream with a time limit (ND_E_TIMEOUT past it)
 nd_status nd_wait(cudaStream_t st);

@@ -1,8 +1,13 @@
 // Exclusive prefix sums over int64 (offsets of every CSR this library builds).
 //
-// Three-phase scan: each 256-thread block reduces a tile of 2048 elements,
-// the tile sums are scanned (recursively), then each tile is scanned and
-// offset.  HBM-bound: two reads and one write of the array.
+// Two launches whatever the length: every block of a grid of at most
+// kMaxBlocks sums its contiguous share of the array, then every block adds up
+// the sums before its own (at most kMaxBlocks values, from L2) and scans its
+// share tile by tile.  Arrays of a few tiles take the second launch alone.
+// No recursion over tile sums, and no block waits for another.
+// HBM-bound for long arrays: two reads and one write.  A recursive tile scan
+// before: three launches, an allocation and a memset per level; a build of
+// 10,000 edges spent 0.14 of its 1.1 ms in eight of them.
 #include "nd_internal.cuh"
 
 namespace {
@@ -10,6 +15,8 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kItems = 8;
 constexpr int kTile = kThreads * kItems;
+constexpr int kMaxBlocks = 608;   // 4 per SM of a 152-SM GPU; the second launch reads as many sums per block
+constexpr int64_t kOneBlock = 4;  // tiles that one block scans alone
 
 __device__ __forceinline__ int64_t warp_incl_scan(int64_t v) {
     const int lane = threadIdx.x & 31;
@@ -21,83 +28,113 @@ __device__ __forceinline__ int64_t warp_incl_scan(int64_t v) {
     return v;
 }
 
-// exclusive scan of one value per thread across the block; returns the
-// block total through *total
-__device__ __forceinline__ int64_t block_excl_scan(int64_t v, int64_t* total) {
+// exclusive scan of one value per thread across the block, and the block's total
+__device__ __forceinline__ int64_t block_excl_scan(int64_t v, int64_t& total) {
     __shared__ int64_t warp_sums[kThreads / 32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int64_t incl = warp_incl_scan(v);
+    const int64_t incl = warp_incl_scan(v);
     if (lane == 31) warp_sums[wid] = incl;
     __syncthreads();
-    if (wid == 0) {
-        int64_t w = (lane < kThreads / 32) ? warp_sums[lane] : 0;
-        int64_t wi = warp_incl_scan(w);
-        if (lane < kThreads / 32) warp_sums[lane] = wi - w;  // exclusive prefix of warp sums
-        if (lane == kThreads / 32 - 1) *total = wi;
+    int64_t before = 0, all = 0;
+#pragma unroll
+    for (int w = 0; w < kThreads / 32; ++w) {
+        const int64_t s = warp_sums[w];
+        if (w < wid) before += s;
+        all += s;
     }
     __syncthreads();
-    int64_t r = warp_sums[wid] + incl - v;
-    __syncthreads();
-    return r;
+    total = all;
+    return before + incl - v;
 }
 
-__global__ void k_tile_sums(const int64_t* __restrict__ a, int64_t n, int64_t* __restrict__ sums) {
-    __shared__ int64_t tot;
-    int64_t base = (int64_t)blockIdx.x * kTile + (int64_t)threadIdx.x * kItems;
-    int64_t s = 0;
+// the kItems values of a thread from a[base]; base is a multiple of kItems
+// and a comes from the allocator, so whole groups load as 16-byte pairs
+__device__ __forceinline__ void load_items(const int64_t* __restrict__ a, int64_t base, int64_t n, int64_t (&v)[kItems]) {
+    if (base + kItems <= n) {
+        const longlong2* p = reinterpret_cast<const longlong2*>(a + base);
 #pragma unroll
-    for (int i = 0; i < kItems; ++i)
-        if (base + i < n) s += a[base + i];
-    block_excl_scan(s, &tot);
-    if (threadIdx.x == 0) sums[blockIdx.x] = tot;
-}
-
-__global__ void k_tile_scan(int64_t* __restrict__ a, int64_t n, const int64_t* __restrict__ offs) {
-    __shared__ int64_t tot;
-    int64_t base = (int64_t)blockIdx.x * kTile + (int64_t)threadIdx.x * kItems;
-    int64_t v[kItems];
-    int64_t s = 0;
-#pragma unroll
-    for (int i = 0; i < kItems; ++i) {
-        v[i] = (base + i < n) ? a[base + i] : 0;
-        s += v[i];
-    }
-    int64_t run = block_excl_scan(s, &tot) + (offs ? offs[blockIdx.x] : 0);
-#pragma unroll
-    for (int i = 0; i < kItems; ++i)
-        if (base + i < n) {
-            int64_t x = v[i];
-            a[base + i] = run;
-            run += x;
+        for (int i = 0; i < kItems / 2; ++i) {
+            const longlong2 x = p[i];
+            v[2 * i] = x.x;
+            v[2 * i + 1] = x.y;
         }
+    } else {
+#pragma unroll
+        for (int i = 0; i < kItems; ++i) v[i] = base + i < n ? a[base + i] : 0;
+    }
 }
 
-nd_status scan_rec(int64_t* data, int64_t count, cudaStream_t st) {
-    const int64_t n = count + 1;  // the trailing slot receives the total
-    const int64_t tiles = (n + kTile - 1) / kTile;
-    if (tiles == 1) {
-        k_tile_scan<<<1, kThreads, 0, st>>>(data, n, nullptr);
-        ND_CUDA(cudaGetLastError());
-        return ND_OK;
+// sums[b] = sum of block b's share, tiles [b * share, (b + 1) * share)
+__global__ void __launch_bounds__(kThreads) k_share_sums(const int64_t* __restrict__ a, int64_t n, int64_t share,
+                                                         int64_t* __restrict__ sums) {
+    int64_t s = 0;
+    for (int64_t t = 0; t < share; ++t) {
+        const int64_t base = ((int64_t)blockIdx.x * share + t) * kTile + (int64_t)threadIdx.x * kItems;
+        int64_t v[kItems];
+        load_items(a, base, n, v);
+#pragma unroll
+        for (int i = 0; i < kItems; ++i) s += v[i];
     }
-    int64_t* sums = nullptr;
-    ND_CUDA(cudaMallocAsync((void**)&sums, sizeof(int64_t) * (tiles + 1), st));
-    ND_CUDA(cudaMemsetAsync(sums + tiles, 0, sizeof(int64_t), st));
-    k_tile_sums<<<(unsigned)tiles, kThreads, 0, st>>>(data, n, sums);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) { cudaFreeAsync(sums, st); return nd_cuda_fail(e, "k_tile_sums", __FILE__, __LINE__); }
-    nd_status s = scan_rec(sums, tiles, st);  // sums[tiles] = grand total (unused)
-    if (s != ND_OK) { cudaFreeAsync(sums, st); return s; }
-    k_tile_scan<<<(unsigned)tiles, kThreads, 0, st>>>(data, n, sums);
-    e = cudaGetLastError();
-    cudaFreeAsync(sums, st);
-    if (e != cudaSuccess) return nd_cuda_fail(e, "k_tile_scan", __FILE__, __LINE__);
-    return ND_OK;
+    int64_t total;
+    block_excl_scan(s, total);
+    if (threadIdx.x == 0) sums[blockIdx.x] = total;
+}
+
+__global__ void __launch_bounds__(kThreads) k_share_scan(int64_t* __restrict__ a, int64_t n, int64_t share,
+                                                         const int64_t* __restrict__ sums) {
+    int64_t run = 0;
+    if (sums) {
+        int64_t s = 0, total;
+        for (int i = threadIdx.x; i < (int)blockIdx.x; i += kThreads) s += sums[i];
+        block_excl_scan(s, total);
+        run = total;
+    }
+    for (int64_t t = 0; t < share; ++t) {
+        const int64_t tile = ((int64_t)blockIdx.x * share + t) * kTile;
+        if (tile >= n) break;  // the same for the whole block
+        const int64_t base = tile + (int64_t)threadIdx.x * kItems;
+        int64_t v[kItems], s = 0, total;
+        load_items(a, base, n, v);
+#pragma unroll
+        for (int i = 0; i < kItems; ++i) s += v[i];
+        int64_t at = run + block_excl_scan(s, total);
+        if (base + kItems <= n) {
+            longlong2* p = reinterpret_cast<longlong2*>(a + base);
+#pragma unroll
+            for (int i = 0; i < kItems / 2; ++i) {
+                p[i] = make_longlong2(at, at + v[2 * i]);
+                at += v[2 * i] + v[2 * i + 1];
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < kItems; ++i)
+                if (base + i < n) {
+                    a[base + i] = at;
+                    at += v[i];
+                }
+        }
+        run += total;
+    }
 }
 
 }  // namespace
 
 nd_status nd_scan_i64(int64_t* data, int64_t count, cudaStream_t st) {
     nd_prof_scope ps("scan", st);
-    return scan_rec(data, count, st);
+    const int64_t n = count + 1;  // the trailing slot receives the total
+    const int64_t tiles = (n + kTile - 1) / kTile;
+    if (tiles <= kOneBlock) {
+        k_share_scan<<<1, kThreads, 0, st>>>(data, n, tiles, nullptr);
+        ND_CUDA(cudaGetLastError());
+        return ND_OK;
+    }
+    const int64_t share = (tiles + kMaxBlocks - 1) / kMaxBlocks;
+    const unsigned blocks = (unsigned)((tiles + share - 1) / share);
+    nd_tmp<int64_t> sums(st);
+    ND_TRY(sums.alloc(blocks));
+    k_share_sums<<<blocks, kThreads, 0, st>>>(data, n, share, sums);
+    ND_CUDA(cudaGetLastError());
+    k_share_scan<<<blocks, kThreads, 0, st>>>(data, n, share, sums);
+    ND_CUDA(cudaGetLastError());
+    return ND_OK;
 }

@@ -109,6 +109,9 @@ struct SweepParams {
     bool direct;                   // AND: rows are expected to fail the count (see warp_hindex)
     const uint32_t* cur;  // AND + notification: frontier read in this pass
     uint32_t* next;       // and the frontier written for the next pass
+    // relabelled (1,2) runs from d_s: the largest degree, so the largest tau, of
+    // the ids from 2^o on; rows are ordered by floor(log2 id).  Null: no bound
+    const int32_t* __restrict__ oct_max;
     const uint32_t* members;  // PartialAnd: only members are notified (null = everyone)
     // batches, SND and AND-nn: graph of every r-clique, the graphs that changed
     // in the previous pass (gact_in) and those changing in this one (gact_out);
@@ -196,6 +199,30 @@ __device__ __forceinline__ auto make_rho(const SweepParams& P, int64_t jb) {
     if constexpr (Q == 3) return Rho<3, RO, int32_t>{P.inc + 3 * jb, P.tin};
     else return Rho<Q, RO, uint16_t>{P.inc + Q * jb, P.gin};
 }
+
+// What a row's order says about the entries that are still to come.  Rows of a
+// relabelled (1,2) graph are ordered by floor(log2 id), and ids by degree
+// class, so past an entry of octave o no tau exceeds oct_max[o].
+struct NoBound {
+    static constexpr bool kOn = false;
+    __device__ __forceinline__ bool past(int) const { return false; }
+    __device__ __forceinline__ int max_from(int) const { return INT32_MAX; }
+};
+// the first id from which on no vertex has degree >= h (whole warp)
+__device__ __forceinline__ uint32_t id_limit(const int32_t* __restrict__ oct_max, int32_t h) {
+    const unsigned m = __ballot_sync(0xffffffffu, __ldg(oct_max + (threadIdx.x & 31)) < h);
+    return m ? 1u << (__ffs(m) - 1) : 0xffffffffu;
+}
+struct IdBound {
+    static constexpr bool kOn = true;
+    const uint32_t* __restrict__ row;
+    const int32_t* __restrict__ oct_max;
+    uint32_t limit;  // of the row's tau
+    // can no entry from j on reach the row's tau?  (j - 1 has just been read)
+    __device__ __forceinline__ bool past(int j) const { return __ldg(row + j - 1) >= limit; }
+    // the largest tau from entry j on
+    __device__ __forceinline__ int max_from(int j) const { return __ldg(oct_max + 31 - __clz(__ldg(row + j) | 1u)); }
+};
 
 // f(rho(j)) for the entries j in [i, end), STEP lanes wide: four loads per
 // lane in flight, without tests while whole blocks are left; the rest is one
@@ -343,8 +370,10 @@ __device__ __forceinline__ int select_bin(const unsigned* bins, int lo, int shif
 // rows of fewer than 65,536 entries; else HW bins of 32 bits), one per value
 // while t allows, so H is exact after one sweep there, and after two for
 // longer rows.
-template <bool PK, int HW, typename F>
-__device__ __forceinline__ int32_t warp_hindex(const F& rho, int d, int32_t t, bool direct, unsigned* bins) {
+// bound: a count also stops where the rest of the row cannot reach t.
+template <bool PK, int HW, typename F, typename B>
+__device__ __forceinline__ int32_t warp_hindex(const F& rho, const B& bound, int d, int32_t t, bool direct,
+                                               unsigned* bins) {
     const int lane = threadIdx.x & 31;
     if (t <= 0) return 0;
     int lo = 0, hi = t, above = 0;
@@ -356,6 +385,7 @@ __device__ __forceinline__ int32_t warp_hindex(const F& rho, int d, int32_t t, b
             i = end;
             have = (int)__reduce_add_sync(0xffffffffu, (unsigned)cnt);
             if (have >= t) return t;
+            if (bound.past(end)) break;
         }
         lo = above = have;  // #{rho >= lo} >= lo holds; at hi it fails
         if (hi - lo <= 1) return lo;
@@ -396,10 +426,15 @@ __device__ __forceinline__ int32_t warp_hindex(const F& rho, int d, int32_t t, b
 constexpr int kCtaSegment = 2048;
 
 // The same by the whole CTA (the longest rows): 32-bit counters, as many bins
-// as the block's histogram has words; warp 0 selects the bin.
-template <int WORDS, typename F>
-__device__ __forceinline__ int32_t cta_hindex(const F& rho, int d, int32_t t, bool direct, unsigned* bins,
-                                              int* bounds /* 8 */) {
+// as the block's histogram has words; warp 0 selects the bin.  A sweep also
+// stops where u, the most the rest of the row can reach, is settled: once
+// #{rho >= u} >= u, H is at least u, and the rest counts for no larger value.
+// That is what keeps the hub rows of a k-core short: on R-MAT scale 20 the
+// rows past 2,048 entries hold 22% of all entries, and a search needs a third
+// of those, a converged count an eighth.
+template <int WORDS, typename F, typename B>
+__device__ __forceinline__ int32_t cta_hindex(const F& rho, const B& bound, int d, int32_t t, bool direct,
+                                              unsigned* bins, int* bounds /* 8 */) {
     if (t <= 0) return 0;
     auto total = [&](int v) {
         const unsigned w = __reduce_add_sync(0xffffffffu, (unsigned)v);
@@ -421,6 +456,7 @@ __device__ __forceinline__ int32_t cta_hindex(const F& rho, int d, int32_t t, bo
             i = end;
             have = total(cnt);
             if (have >= t) return t;
+            if (bound.past(end)) break;
         }
         lo = above = have;
         if (hi - lo <= 1) return lo;
@@ -431,12 +467,26 @@ __device__ __forceinline__ int32_t cta_hindex(const F& rho, int d, int32_t t, bo
         const int nb = (int)((span - 1) >> shift) + 1;
         for (int i = threadIdx.x; i < ((nb + 127) & ~127); i += kThreads) bins[i] = 0;
         __syncthreads();
-        int ge = 0;
-        stream_row<kThreads>(rho, 0, d, [&](int, int32_t r) {
-            const unsigned x = (unsigned)(r - lo);
-            if (x < span) atomicAdd(bins + (x >> shift), 1u);
-            else ge += (r >= hi);
-        });
+        int ge = 0, u = hi;  // u: the last bound tested
+        for (int i = 0; i < d;) {
+            const int end = B::kOn && d - i > kCtaSegment ? i + kCtaSegment : d;
+            stream_row<kThreads>(rho, i, end, [&](int, int32_t r) {
+                const unsigned x = (unsigned)(r - lo);
+                if (x < span) atomicAdd(bins + (x >> shift), 1u);
+                else ge += (r >= hi);
+            });
+            i = end;
+            if (!B::kOn || i >= d) continue;
+            const int m = max(bound.max_from(i), lo);
+            if (m >= u) continue;  // the same for every thread
+            u = m;
+            __syncthreads();  // the bins so far are complete
+            // #{rho >= u} from the bins at or past u
+            int c = direct ? ge : (threadIdx.x == 0 ? above : 0);
+            for (int b = (int)(((unsigned)(u - lo) + (1u << shift) - 1) >> shift) + threadIdx.x; b < nb; b += kThreads)
+                c += (int)bins[b];
+            if (total(c) >= u) break;
+        }
         if (direct) {
             above = total(ge);  // with its barriers, the bins are complete too
             if (above >= t) return t;
@@ -548,6 +598,8 @@ __device__ __forceinline__ void notify_row(const SweepParams& P, int64_t jb, int
         // (1,2), (3,4): ids of r-cliques; the same overlap, kNotifyUnroll
         // entries (Q ids each) and their bit words loaded before any test
         constexpr int U = Q == 1 ? kNotifyUnroll : 2;
+        // a relabelled (1,2) row: from this id on every tau is below h
+        const uint32_t limit = Q == 1 && P.oct_max ? id_limit(P.oct_max, h) : 0xffffffffu;
         for (int64_t j0 = jb + first; j0 < je; j0 += (int64_t)U * step) {
             uint32_t id[U][Q], wd[U][Q];
 #pragma unroll
@@ -556,9 +608,10 @@ __device__ __forceinline__ void notify_row(const SweepParams& P, int64_t jb, int
 #pragma unroll
                 for (int k = 0; k < Q; ++k) id[u][k] = j < je ? __ldg(P.inc + Q * j + k) : 0u;
             }
+            if (Q == 1 && id[0][0] >= limit) break;  // so are this lane's later entries
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                const bool ok = j0 + (int64_t)u * step < je;
+                const bool ok = j0 + (int64_t)u * step < je && (Q != 1 || id[u][0] < limit);
 #pragma unroll
                 for (int k = 0; k < Q; ++k) wd[u][k] = ok ? ld_front(P.next + (id[u][k] >> 5)) : 0xffffffffu;
             }
@@ -684,8 +737,14 @@ __device__ __forceinline__ void run_warp_row(const SweepParams& P, const nd_item
     if (graph_done<GB>(P, R)) return;
     int32_t t0, t, old;
     load_tau<AND>(P, it, t0, t, old);
-    const int32_t h = warp_hindex<true, HW>(make_rho<Q, !AND>(P, it.jb), (int)it.d, t,
-                                             P.direct || (!AND && old != t0), bins);
+    const bool direct = P.direct || (!AND && old != t0);
+    int32_t h;
+    if (Q == 1 && P.oct_max)
+        h = warp_hindex<true, HW>(make_rho<Q, !AND>(P, it.jb),
+                                  IdBound{P.inc + it.jb, P.oct_max, direct ? 0u : id_limit(P.oct_max, t)}, (int)it.d, t,
+                                  direct, bins);
+    else
+        h = warp_hindex<true, HW>(make_rho<Q, !AND>(P, it.jb), NoBound{}, (int)it.d, t, direct, bins);
     const int lane = threadIdx.x & 31;
     if (lane == 0) {
         n.row(it.d, h != t0);
@@ -710,12 +769,16 @@ __device__ __forceinline__ void run_cta(const SweepParams& P, int64_t i, unsigne
     const int d = (int)it.d;
     const bool direct = P.direct || (!AND && old != t0);
     int32_t h;
-    if (Q == 2 && t > kTau16Max)  // only then can a saturated value matter
-        h = cta_hindex<WORDS>(RhoExact2<!AND>{P.inc + 2 * it.jb, P.eid, P.tin}, d, t, direct, bins, bounds);
-    else if (Q == 1 && t > kTau16Max)
-        h = cta_hindex<WORDS>(Rho<Q, !AND, int32_t>{P.inc + it.jb, P.tin}, d, t, direct, bins, bounds);
-    else
-        h = cta_hindex<WORDS>(make_rho<Q, !AND>(P, it.jb), d, t, direct, bins, bounds);
+    if (Q == 2 && t > kTau16Max) {  // only then can a saturated value matter
+        h = cta_hindex<WORDS>(RhoExact2<!AND>{P.inc + 2 * it.jb, P.eid, P.tin}, NoBound{}, d, t, direct, bins, bounds);
+    } else if (Q == 1 && t > kTau16Max) {
+        h = cta_hindex<WORDS>(Rho<Q, !AND, int32_t>{P.inc + it.jb, P.tin}, NoBound{}, d, t, direct, bins, bounds);
+    } else if (Q == 1 && P.oct_max) {
+        const IdBound bound{P.inc + it.jb, P.oct_max, id_limit(P.oct_max, t)};
+        h = cta_hindex<WORDS>(make_rho<Q, !AND>(P, it.jb), bound, d, t, direct, bins, bounds);
+    } else {
+        h = cta_hindex<WORDS>(make_rho<Q, !AND>(P, it.jb), NoBound{}, d, t, direct, bins, bounds);
+    }
     if (threadIdx.x == 0) {
         n.row(it.d, h != t0);
         if (h != t0) graph_changed<GB>(P, R);
@@ -1132,10 +1195,10 @@ __global__ void __launch_bounds__(kThreads, kPassBlocks) k_pass_otf(SweepParams 
             int32_t h;
             const int ln = (int)(le - lb), sn = (int)(se - sb);
             if (tc > kTau16Max)
-                h = warp_hindex<false, kHistWords>(RhoOtf<!AND, true>{P.col, sb, lb, ln, P.gin, P.eid, P.tin}, sn, tc, direct,
+                h = warp_hindex<false, kHistWords>(RhoOtf<!AND, true>{P.col, sb, lb, ln, P.gin, P.eid, P.tin}, NoBound{}, sn, tc, direct,
                                             bins);
             else
-                h = warp_hindex<false, kHistWords>(RhoOtf<!AND, false>{P.col, sb, lb, ln, P.gin, P.eid, P.tin}, sn, tc, direct,
+                h = warp_hindex<false, kHistWords>(RhoOtf<!AND, false>{P.col, sb, lb, ln, P.gin, P.eid, P.tin}, NoBound{}, sn, tc, direct,
                                             bins);
             if (lane == 0) {
                 n.row(it.d, h != tr);
@@ -1480,6 +1543,7 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
     P.ev = h->e_v;
     P.items = h->items;
     P.members = members;
+    P.oct_max = tau_in_dev ? nullptr : h->oct_max;  // tau <= d_s holds for the library's own start
     // batches, SND and AND-nn: every graph starts active (AND with
     // notification needs nothing more: a converged graph notifies no one)
     P.gid = nullptr;
@@ -1534,13 +1598,13 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
         if (stop_active > 0.0) nb = 1;  // the stopping rule looks at every pass
         const int kind = batch == 0 ? 0 : ((batch & 1) ? 2 : 1);
         bool launched = false;
-        // graphs hold the plain parameters; runs with members or a stopping
-        // rule launch directly, and so does the first batch of its kind on a
+        // graphs hold the plain parameters; runs with members, a stopping rule
+        // or a tau of the caller's launch directly, and so does the first batch of its kind on a
         // handle: building a graph costs more than its launches, and many
         // handles run each mode once
         const bool seen = h->batch_seen[mode][kind];
         if (nb == kBatch) h->batch_seen[mode][kind] = true;
-        if (nb == kBatch && seen && grid0 > 0 && !members && (start & 1) == 0 && !h->pass_graph_failed[mode][kind]) {
+        if (nb == kBatch && seen && grid0 > 0 && !members && !tau_in_dev && (start & 1) == 0 && !h->pass_graph_failed[mode][kind]) {
             if (!h->pass_graph[mode][kind])
                 make_batch_graph(h, mode, kind, P, grid0, fn0, grid1, fn1, words);
             if (h->pass_graph[mode][kind]) {

@@ -98,6 +98,9 @@ struct nd_incidence {
     int32_t* to_new = nullptr;  // [num_r] caller's r-clique id -> internal id
     int32_t* to_old = nullptr;  // [num_r] internal r-clique id -> caller's id
     int32_t* vto_old = nullptr;
+    // (1,2), relabelled: [32] the largest degree of the ids from 2^o on; rows
+    // are ordered by floor(log2 id)
+    int32_t* oct_max = nullptr;
     int64_t *c_rp = nullptr, *c_up = nullptr;
     int32_t *c_col = nullptr, *c_nlow = nullptr;
     bool adj = false;
@@ -168,7 +171,7 @@ struct nd_claim {
 // passes are enqueued in batches of ND_BATCH; the per-pass counters (ND_SLOT
 // u64 each) live in two halves of ND_BATCH slots used by alternate batches
 enum { ND_BATCH = 16, ND_RING = 2 * ND_BATCH, ND_SLOT = 6 };
-enum { ND_READ = 16 };
+enum { ND_READ = 64 };
 
 // a pinned block for a handle's counters and read-backs, from a bounded pool
 // (nd_api.cu); null if there is no memory

@@ -326,13 +326,39 @@ __device__ __forceinline__ int octave_of(uint32_t id) { return 31 - __clz(id | 1
 
 constexpr int kSortRow = 512;  // entries of a row that one warp orders in shared memory
 
+// How a row is ordered: the key of the entry at CSR position p, its bucket
+// (0..31, the order of the row), where row u's output begins, and the write.
+struct NewIdOrder {  // k-core relabelling: new ids, by octave
+    const int32_t* __restrict__ col;
+    const int32_t* __restrict__ to_new;
+    const int64_t* __restrict__ nrp;
+    int32_t* __restrict__ ncol;
+    __device__ __forceinline__ uint32_t key(int64_t p) const { return (uint32_t)to_new[col[p]]; }
+    static __device__ __forceinline__ int bucket(uint32_t key) { return octave_of(key); }
+    __device__ __forceinline__ int64_t begin(int64_t u, int64_t) const { return nrp[to_new[u]]; }
+    __device__ __forceinline__ void write(int64_t at, int64_t, uint32_t key) const { ncol[at] = (int32_t)key; }
+};
+struct DegreeOrder {  // no-storage passes: the caller's ids with their slots, by degree class, high first
+    const int64_t* __restrict__ rp;
+    const int32_t* __restrict__ col;
+    int32_t* __restrict__ vertex;
+    uint32_t* __restrict__ slot;
+    __device__ __forceinline__ uint32_t key(int64_t p) const {
+        const int32_t v = col[p];
+        return (uint32_t)degree_class(rp[v + 1] - rp[v]);  // a neighbour has a neighbour: below 32
+    }
+    static __device__ __forceinline__ int bucket(uint32_t key) { return (int)key; }
+    __device__ __forceinline__ int64_t begin(int64_t, int64_t b) const { return b; }
+    __device__ __forceinline__ void write(int64_t at, int64_t p, uint32_t) const {
+        vertex[at] = col[p];
+        slot[at] = (uint32_t)p;
+    }
+};
+
 // one warp per row of up to kSortRow entries; up to 32 are ranked across the
 // warp, longer rows go through 32 shared counters
-__global__ void __launch_bounds__(kThreads) k_relabel_rows(int64_t n, const int64_t* __restrict__ rp,
-                                                           const int32_t* __restrict__ col,
-                                                           const int32_t* __restrict__ to_new,
-                                                           const int64_t* __restrict__ nrp,
-                                                           int32_t* __restrict__ ncol) {
+template <typename K>
+__global__ void __launch_bounds__(kThreads) k_order_rows(int64_t n, const int64_t* __restrict__ rp, K k) {
     __shared__ uint32_t stage[kThreads / 32][kSortRow];
     __shared__ uint32_t cur[kThreads / 32][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -341,20 +367,23 @@ __global__ void __launch_bounds__(kThreads) k_relabel_rows(int64_t n, const int6
         const int64_t len = rp[u + 1] - b;
         if (len == 0 || len > kSortRow) continue;  // k_sort_count, k_sort_scatter
         const int d = (int)len;
-        int32_t* const out = ncol + nrp[to_new[u]];
+        const int64_t out = k.begin(u, b);
         if (d <= 32) {
-            const uint32_t id = lane < d ? (uint32_t)to_new[col[b + lane]] : 0xffffffffu;
+            const uint32_t key = lane < d ? k.key(b + lane) : 0xffffffffu;
             int rank = 0;
-            for (int o = 0; o < d; ++o) rank += (__shfl_sync(kFull, id, o) < id);
-            if (lane < d) out[rank] = (int32_t)id;
+            for (int o = 0; o < d; ++o) {
+                const uint32_t x = __shfl_sync(kFull, key, o);
+                rank += x < key || (x == key && o < lane);
+            }
+            if (lane < d) k.write(out + rank, b + lane, key);
             continue;
         }
         cur[w][lane] = 0;
         __syncwarp();
         for (int j = lane; j < d; j += 32) {
-            const uint32_t id = (uint32_t)to_new[col[b + j]];
-            stage[w][j] = id;
-            atomicAdd(&cur[w][octave_of(id)], 1u);
+            const uint32_t key = k.key(b + j);
+            stage[w][j] = key;
+            atomicAdd(&cur[w][K::bucket(key)], 1u);
         }
         __syncwarp();
         const uint32_t c = cur[w][lane];
@@ -367,8 +396,8 @@ __global__ void __launch_bounds__(kThreads) k_relabel_rows(int64_t n, const int6
         cur[w][lane] = incl - c;
         __syncwarp();
         for (int j = lane; j < d; j += 32) {
-            const uint32_t id = stage[w][j];
-            out[atomicAdd(&cur[w][octave_of(id)], 1u)] = (int32_t)id;
+            const uint32_t key = stage[w][j];
+            k.write(out + atomicAdd(&cur[w][K::bucket(key)], 1u), b + j, key);
         }
         __syncwarp();
     }
@@ -411,8 +440,8 @@ struct sort_segment {
     }
 };
 
-__global__ void __launch_bounds__(kThreads) k_sort_count(const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
-                                                         const int32_t* __restrict__ to_new,
+template <typename K>
+__global__ void __launch_bounds__(kThreads) k_sort_count(const int64_t* __restrict__ rp, K k,
                                                          const int32_t* __restrict__ rows,
                                                          const int64_t* __restrict__ seg_off, int64_t count,
                                                          int64_t segs, int64_t* __restrict__ cells) {
@@ -422,17 +451,15 @@ __global__ void __launch_bounds__(kThreads) k_sort_count(const int64_t* __restri
         const sort_segment x(sg, rows, seg_off, count, rp);
         cnt[w][lane] = 0;
         __syncwarp();
-        for (int64_t p = x.pb + lane; p < x.pe; p += 32) atomicAdd(&cnt[w][octave_of((uint32_t)to_new[col[p]])], 1u);
+        for (int64_t p = x.pb + lane; p < x.pe; p += 32) atomicAdd(&cnt[w][K::bucket(k.key(p))], 1u);
         __syncwarp();
         cells[x.cell + lane * x.stride] = cnt[w][lane];
         __syncwarp();
     }
 }
 
-__global__ void __launch_bounds__(kThreads) k_sort_scatter(const int64_t* __restrict__ rp,
-                                                           const int32_t* __restrict__ col,
-                                                           const int32_t* __restrict__ to_new,
-                                                           const int64_t* __restrict__ nrp, int32_t* __restrict__ ncol,
+template <typename K>
+__global__ void __launch_bounds__(kThreads) k_sort_scatter(const int64_t* __restrict__ rp, K k,
                                                            const int32_t* __restrict__ rows,
                                                            const int64_t* __restrict__ seg_off, int64_t count,
                                                            int64_t segs, const int64_t* __restrict__ cells) {
@@ -442,10 +469,10 @@ __global__ void __launch_bounds__(kThreads) k_sort_scatter(const int64_t* __rest
         const sort_segment x(sg, rows, seg_off, count, rp);
         cur[w][lane] = (uint32_t)(cells[x.cell + lane * x.stride] - cells[x.row_cell]);
         __syncwarp();
-        int32_t* const out = ncol + nrp[to_new[x.u]];
+        const int64_t out = k.begin(x.u, x.b);
         for (int64_t p = x.pb + lane; p < x.pe; p += 32) {
-            const uint32_t id = (uint32_t)to_new[col[p]];
-            out[atomicAdd(&cur[w][octave_of(id)], 1u)] = (int32_t)id;
+            const uint32_t key = k.key(p);
+            k.write(out + atomicAdd(&cur[w][K::bucket(key)], 1u), p, key);
         }
         __syncwarp();
     }
@@ -1572,6 +1599,57 @@ nd_status nd_relabel_truss_edges(nd_incidence* h, cudaStream_t st) {
     return ND_OK;
 }
 
+// the rows of h->rp too long for one warp, as segments
+struct nd_row_segments {
+    nd_tmp<int32_t> rows;
+    nd_tmp<int64_t> off;
+    int64_t listed = 0, segs = 0;
+    explicit nd_row_segments(cudaStream_t st) : rows(st), off(st) {}
+    // waits once, for what has been fetched before too
+    nd_status list(nd_incidence* h, cudaStream_t st) {
+        const int64_t cap = h->nnz / kSortRow + 1;
+        nd_tmp<unsigned long long> count(st);
+        ND_TRY(rows.alloc(cap));
+        ND_TRY(off.alloc(cap + 1));
+        ND_TRY(count.alloc(1));
+        ND_CUDA(cudaMemsetAsync(off, 0, sizeof(int64_t) * (cap + 1), st));
+        ND_CUDA(cudaMemsetAsync(count, 0, sizeof(unsigned long long), st));
+        k_sort_list<<<nd_blocks_for(h->n, kThreads, grid_cap(h) * 4), kThreads, 0, st>>>(h->n, h->rp, rows, off, count);
+        ND_CUDA(cudaGetLastError());
+        ND_TRY(nd_scan_i64(off, cap, st));
+        ND_TRY(fetch(h, 0, count.p, 1, st));
+        ND_TRY(fetch(h, 1, off.p + cap, 1, st));
+        ND_TRY(nd_wait(st));
+        listed = h->h_read[0];
+        segs = h->h_read[1];
+        return ND_OK;
+    }
+};
+
+// every row of h->rp in the order of k's buckets
+template <typename K>
+static nd_status order_rows(nd_incidence* h, const K& k, const nd_row_segments& sg, cudaStream_t st) {
+    k_order_rows<K><<<nd_blocks_for(h->n * 32, kThreads, grid_cap(h) * 4), kThreads, 0, st>>>(h->n, h->rp, k);
+    ND_CUDA(cudaGetLastError());
+    if (sg.segs == 0) return ND_OK;
+    const int blocks = nd_blocks_for(sg.segs * 32, kThreads, grid_cap(h) * 4);
+    nd_tmp<int64_t> cells(st);
+    ND_TRY(cells.alloc(32 * sg.segs + 1));
+    ND_CUDA(cudaMemsetAsync(cells.p + 32 * sg.segs, 0, sizeof(int64_t), st));
+    k_sort_count<K><<<blocks, kThreads, 0, st>>>(h->rp, k, sg.rows, sg.off, sg.listed, sg.segs, cells);
+    ND_CUDA(cudaGetLastError());
+    ND_TRY(nd_scan_i64(cells, 32 * sg.segs, st));
+    k_sort_scatter<K><<<blocks, kThreads, 0, st>>>(h->rp, k, sg.rows, sg.off, sg.listed, sg.segs, cells);
+    ND_CUDA(cudaGetLastError());
+    return ND_OK;
+}
+
+nd_status nd_rows_by_degree(nd_incidence* h, int32_t* vertex, uint32_t* slot, cudaStream_t st) {
+    nd_row_segments segments(st);
+    ND_TRY(segments.list(h, st));
+    return order_rows(h, DegreeOrder{h->rp, h->col, vertex, slot}, segments, st);
+}
+
 nd_status nd_relabel_by_degree(nd_incidence* h, cudaStream_t st) {
     const int64_t n = h->n, nnz = h->nnz;
     if (n >= kRelabelMinVertices) {
@@ -1579,23 +1657,8 @@ nd_status nd_relabel_by_degree(nd_incidence* h, cudaStream_t st) {
         ND_TRY(nd_alloc((void**)&h->to_new, sizeof(int32_t) * n, st, h));
         ND_TRY(nd_alloc((void**)&h->to_old, sizeof(int32_t) * n, st, h));
         ND_TRY(class_ids(h, h->to_new, h->to_old, st, kReadClasses));
-        // the rows too long for one warp, as segments
-        const int64_t cap = nnz / kSortRow + 1;
-        nd_tmp<int32_t> rows(st);
-        nd_tmp<int64_t> seg_off(st), cells(st);
-        nd_tmp<unsigned long long> count(st);
-        ND_TRY(rows.alloc(cap));
-        ND_TRY(seg_off.alloc(cap + 1));
-        ND_TRY(count.alloc(1));
-        ND_CUDA(cudaMemsetAsync(seg_off, 0, sizeof(int64_t) * (cap + 1), st));
-        ND_CUDA(cudaMemsetAsync(count, 0, sizeof(unsigned long long), st));
-        k_sort_list<<<nd_blocks_for(n, kThreads, grid_cap(h) * 4), kThreads, 0, st>>>(n, h->rp, rows, seg_off, count);
-        ND_CUDA(cudaGetLastError());
-        ND_TRY(nd_scan_i64(seg_off, cap, st));
-        ND_TRY(fetch(h, 0, count.p, 1, st));
-        ND_TRY(fetch(h, 1, seg_off.p + cap, 1, st));
-        ND_TRY(nd_wait(st));
-        const int64_t listed = h->h_read[0], segs = h->h_read[1];
+        nd_row_segments segments(st);
+        ND_TRY(segments.list(h, st));
         // the largest degree in octave o and past it: that of the class of its first id
         int32_t* const oct_max = (int32_t*)(h->h_read + kReadOctaves);
         for (int o = 0; o < 32; ++o) {
@@ -1614,22 +1677,7 @@ nd_status nd_relabel_by_degree(nd_incidence* h, cudaStream_t st) {
         ND_CUDA(cudaGetLastError());
         ND_TRY(nd_scan_i64(nrp, n, st));
         ND_TRY(nd_alloc((void**)&ncol, sizeof(int32_t) * (nnz > 0 ? nnz : 1), st, h));
-        if (nnz > 0) {
-            k_relabel_rows<<<nd_blocks_for(n * 32, kThreads, grid_cap(h) * 4), kThreads, 0, st>>>(
-                n, h->rp, h->col, h->to_new, nrp, ncol);
-            ND_CUDA(cudaGetLastError());
-            if (segs > 0) {
-                const int blocks = nd_blocks_for(segs * 32, kThreads, grid_cap(h) * 4);
-                ND_TRY(cells.alloc(32 * segs + 1));
-                ND_CUDA(cudaMemsetAsync(cells.p + 32 * segs, 0, sizeof(int64_t), st));
-                k_sort_count<<<blocks, kThreads, 0, st>>>(h->rp, h->col, h->to_new, rows, seg_off, listed, segs, cells);
-                ND_CUDA(cudaGetLastError());
-                ND_TRY(nd_scan_i64(cells, 32 * segs, st));
-                k_sort_scatter<<<blocks, kThreads, 0, st>>>(h->rp, h->col, h->to_new, nrp, ncol, rows, seg_off, listed,
-                                                            segs, cells);
-                ND_CUDA(cudaGetLastError());
-            }
-        }
+        if (nnz > 0) ND_TRY(order_rows(h, NewIdOrder{h->col, h->to_new, nrp, ncol}, segments, st));
         nd_release(h->rp, st);
         nd_release(h->col, st);
         h->rp = nrp;

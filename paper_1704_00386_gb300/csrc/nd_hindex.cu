@@ -103,6 +103,12 @@ struct SweepParams {
     const int32_t* __restrict__ col;
     const int32_t* __restrict__ eu;
     const int32_t* __restrict__ ev;
+    const int32_t* __restrict__ hub_of;  // hub index of a vertex, -1 for the others; null: no hub tables
+    const uint2* __restrict__ hub_bits;  // per hub hub_words x (neighbour bits of 32 ids, neighbours below them)
+    int64_t hub_words;
+    const int32_t* __restrict__ by_degree;  // with hub tables: the adjacency lists by degree class, and
+    const uint32_t* __restrict__ slot_of;   // the CSR slot of every entry
+    bool bounded;                           // tau <= d_s throughout: a run from d_s
     const nd_item* __restrict__ items;
     int64_t lo[ND_NB], hi[ND_NB];  // bucket ranges in items
     int chunk;                     // warp tasks per counter grab (pass_chunk)
@@ -1144,80 +1150,307 @@ __global__ void k_add_const(const int32_t* __restrict__ in, int64_t n, int32_t c
 // (the same slots the stored layout lists); a missing one returns -1, which
 // no h-index step counts (every bound is >= 0).  One warp per row, longest
 // rows first, in chunks from a counter.
+//
+// Finding the w: 32 entries of the shorter list at a time, in order.
+//  - Where the longer list is a hub's, its table (k_hub_tables) holds one bit
+//    per vertex and a count per 32 of them: one 8-byte load tells whether w is
+//    a neighbour and at which entry.  No order is needed for that, so the
+//    shorter list is walked by degree class, high first: the w of high degree
+//    close most triangles and hold the largest tau, and past a class no tau
+//    exceeds its degrees (DegreeBound).
+//  - Otherwise, where the lists are of like length (kMergeRatio), blocks of 128
+//    entries of the longer one pass through shared memory, each loaded once
+//    per sweep, and a lane searches its w there;
+//  - otherwise every lane searches the rest of the longer list.
+// A search of the whole list per entry (the only way before) takes some 250 L1
+// wavefronts per 32 entries of a list of 4,000, because its lanes part after
+// the first steps.  The blocks alone were little faster: about 150 instructions
+// per 32 entries; a table takes 25.  SND of an R-MAT k-truss of 50,021 vertices
+// (33.4M incidences, 101 passes): 109 ms with searches, 95 with blocks, 45 with
+// tables, 34 with the lists by degree class (late passes 0.31 ms; 0.43 in CSR
+// order).
+constexpr int kMergeRatio = 16;
+constexpr int kOtfBlock = 128;
+
 template <bool RO, bool EXACT>
-struct RhoOtf {
-    const int32_t* __restrict__ col;
-    int64_t sb, lb;  // first slots of N(s) and N(l)
-    int ln;          // |N(l)|
+struct OtfRow {
+    const int32_t* __restrict__ scol;   // N(s), sn entries: in CSR order from slot sb, or
+    const uint32_t* __restrict__ slot;  // with a table, by degree class, and their slots
+    const int32_t* __restrict__ lcol;  // N(l), ln entries from CSR slot lb
+    int64_t sb, lb;
+    int sn, ln;
+    const uint2* __restrict__ table;  // of the longer list's vertex, or null
+    int32_t* buf;  // kOtfBlock words of the warp
     const uint16_t* tau16;
     const uint32_t* __restrict__ eid;
     const int32_t* tau32;
-    __device__ __forceinline__ int32_t operator()(int j) const {
-        const int32_t w = __ldg(col + sb + j);
-        const int k = nd_lower_bound_n(col + lb, ln, w);
-        if (k >= ln || __ldg(col + lb + k) != w) return -1;
-        const int64_t ps = sb + j, pl = lb + k;
+    mutable int at;   // merging: the block in buf starts here; searching: no earlier entry can match
+    mutable int last;  // merging: the largest vertex in buf
+
+    __device__ __forceinline__ void load_block() const {
+        const int lane = threadIdx.x & 31;
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < kOtfBlock / 32; ++u) {
+            const int k = at + 32 * u + lane;
+            buf[32 * u + lane] = k < ln ? __ldg(lcol + k) : INT32_MAX;
+        }
+        __syncwarp();
+        last = buf[kOtfBlock - 1];
+    }
+
+    // the entry of w in the longer list, -1 if it is none
+    static __device__ __forceinline__ int at_table(uint2 x, int32_t w) {
+        const unsigned below = (1u << (w & 31)) - 1u;
+        return (x.x >> (w & 31)) & 1u ? (int)(x.y + __popc(x.x & below)) : -1;
+    }
+
+    // f(k) for the entries [i, end) of N(s), 32 at a time: entry i + lane is in
+    // N(l) at k, or k = -1.  Sweeps start at 0 and go on where they stopped.
+    template <typename G>
+    __device__ __forceinline__ void match(int i, int end, G&& f) const {
+        const int lane = threadIdx.x & 31;
+        if (table) {
+            for (; end - i >= 64; i += 64) {  // two blocks in flight
+                int32_t w[2];
+                uint2 x[2];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) w[u] = __ldg(scol + i + 32 * u + lane);
+#pragma unroll
+                for (int u = 0; u < 2; ++u) x[u] = __ldg(table + (w[u] >> 5));
+#pragma unroll
+                for (int u = 0; u < 2; ++u) f(i + 32 * u + lane, at_table(x[u], w[u]));
+            }
+            for (; i < end; i += 32) {
+                const int j = i + lane;
+                int k = -1;
+                if (j < end) {
+                    const int32_t w = __ldg(scol + j);
+                    k = at_table(__ldg(table + (w >> 5)), w);
+                }
+                f(j, k);
+            }
+            return;
+        }
+        const bool merge = ln <= kMergeRatio * (int64_t)sn;
+        if (i == 0) {
+            at = 0;
+            if (merge) load_block();
+        }
+        for (; i < end; i += 32) {
+            const int j = i + lane;
+            const int32_t w = j < end ? __ldg(scol + j) : INT32_MAX;
+            int k = -1;
+            if (merge) {
+                const int32_t top = __reduce_max_sync(0xffffffffu, j < end ? w : 0);
+                bool open = j < end;
+                for (;;) {
+                    if (open && w <= last) {
+                        int lo = 0;  // entries of the block below w
+#pragma unroll
+                        for (int h = kOtfBlock / 2; h > 0; h >>= 1) lo += buf[lo + h - 1] < w ? h : 0;
+                        if (buf[lo] == w) k = at + lo;
+                        open = false;
+                    }
+                    if (top <= last || at + kOtfBlock >= ln) break;
+                    at += kOtfBlock;
+                    load_block();
+                }
+            } else {
+                int p = ln;
+                if (j < end) {
+                    p = at + nd_lower_bound_n(lcol + at, ln - at, w);
+                    if (p < ln && __ldg(lcol + p) == w) k = p;
+                }
+                at = __shfl_sync(0xffffffffu, p, min(end - i, 32) - 1);
+            }
+            f(j, k);
+        }
+    }
+    __device__ __forceinline__ int32_t rho(int j, int k) const {
+        if (k < 0) return -1;
+        const int64_t ps = slot ? (int64_t)__ldg(slot + j) : sb + j, pl = lb + k;
         if (EXACT) return min(ld_tau<RO>(tau32 + __ldg(eid + ps)), ld_tau<RO>(tau32 + __ldg(eid + pl)));
         return min(ld_tau<RO>(tau16 + ps), ld_tau<RO>(tau16 + pl));
     }
 };
 
-constexpr int kOtfChunk = 4;  // rows per counter grab
+// a list by degree class: past an entry of degree d, no edge to a later entry
+// has a tau above the largest degree of d's class, less one
+struct DegreeBound {
+    static constexpr bool kOn = true;
+    const int32_t* __restrict__ scol;  // null: the list is in another order
+    const int64_t* __restrict__ rp;
+    int32_t t;
+    __device__ __forceinline__ bool past(int j) const {
+        if (!scol) return false;
+        const int32_t w = __ldg(scol + j - 1);
+        const unsigned d = (unsigned)(__ldg(rp + w + 1) - __ldg(rp + w));
+        return (0xffffffffu >> __clz(d)) - 1 < (unsigned)t;
+    }
+};
+
+template <int STEP, bool RO, bool EXACT, typename G>
+__device__ __forceinline__ void stream_row(const OtfRow<RO, EXACT>& row, int i, int end, G&& f) {
+    row.match(i, end, [&](int j, int k) { f(j, row.rho(j, k)); });
+}
+
+// rows per counter grab.  What a row needs before its first list entry is a
+// chain of five loads (work item, endpoints, list bounds, hub number); the
+// lanes of a warp walk the chains of a whole grab at once.
+// Rows of the warp bucket come four at a time and CTA rows alone: in grabs of
+// eight, a few warps held the longest rows and a first pass took 1.26 instead
+// of 0.66 ms.
+constexpr int kOtfChunk = 8, kOtfChunk2 = 4;
 
 template <bool AND, bool NOTIFY>
 __global__ void __launch_bounds__(kThreads, kPassBlocks) k_pass_otf(SweepParams P) {
     if (P.prev != nullptr && *(volatile const unsigned long long*)P.prev == 0ull) return;  // converged
     __shared__ __align__(16) unsigned hist[kThreads / 32][kHistWords];
+    __shared__ int32_t blocks[kThreads / 32][kOtfBlock];
     Tally<true> n;
     const int lane = threadIdx.x & 31;
     unsigned* const bins = hist[threadIdx.x >> 5];
+    int32_t* const buf = blocks[threadIdx.x >> 5];
     const int64_t first = P.lo[0], rows = P.hi[ND_NB - 1] - P.lo[0];
+    const int64_t n3 = P.hi[3] - P.lo[3], n2 = P.hi[2] - P.lo[2], g2 = (n2 + kOtfChunk2 - 1) / kOtfChunk2;
     for (;;) {
         unsigned long long c = 0;
         if (lane == 0) c = atomicAdd(P.ctr + 4, 1ull);
         c = __shfl_sync(0xffffffffu, c, 0);
-        const int64_t t0 = (int64_t)c * kOtfChunk;
-        if (t0 >= rows) break;
-        const int64_t t1 = min(t0 + (int64_t)kOtfChunk, rows);
-        for (int64_t t = t0; t < t1; ++t) {
-            const nd_item it = load_item(P.items, first + rows - 1 - t);  // longest first
-            const uint32_t R = it.R;
-            if (AND && NOTIFY && !in_frontier<2>(P, R)) continue;
-            int32_t tr, tc, old;
-            load_tau<AND>(P, it, tr, tc, old);
-            const bool direct = P.direct || (!AND && old != tr);
+        // the grab's rows [r0, r0 + take): one at a time of the CTA bucket,
+        // kOtfChunk2 of the warp bucket, then kOtfChunk
+        int64_t g = (int64_t)c, r0 = 0;
+        int take = 1;
+        if (g < n3) {
+            r0 = g;
+        } else if ((g -= n3) < g2) {
+            r0 = n3 + g * kOtfChunk2;
+            take = (int)min((int64_t)kOtfChunk2, n3 + n2 - r0);
+        } else {
+            r0 = n3 + n2 + (g - g2) * kOtfChunk;
+            if (r0 >= rows) break;
+            take = (int)min((int64_t)kOtfChunk, rows - r0);
+        }
+        // lane l: row r0 + l of the pass, longest rows first
+        bool run = lane < take;
+        uint32_t R = 0, d = 0, my_sb = 0, my_lb = 0;  // CSR slots fit 32 bits for (2,3)
+        int32_t my_t0 = 0, my_old = 0;
+        int my_sn = 0, my_ln = 0, my_hub = -1;
+        if (run) {
+            const nd_item it = load_item(P.items, first + rows - 1 - r0 - lane);
+            R = it.R;
+            d = it.d;
+            if (AND && NOTIFY) run = in_frontier<2>(P, R);
+        }
+        if (run) {
+            my_t0 = ld_tau<!AND>(P.tin + R);
+            my_old = AND ? my_t0 : P.tout[R];
             const int32_t x = __ldg(P.eu + R), y = __ldg(P.ev + R);
             const int64_t xb = __ldg(P.rp + x), xe = __ldg(P.rp + x + 1);
             const int64_t yb = __ldg(P.rp + y), ye = __ldg(P.rp + y + 1);
             const bool xs = (xe - xb) <= (ye - yb);
-            const int64_t sb = xs ? xb : yb, se = xs ? xe : ye;
-            const int64_t lb = xs ? yb : xb, le = xs ? ye : xe;
+            my_sb = (uint32_t)(xs ? xb : yb);
+            my_lb = (uint32_t)(xs ? yb : xb);
+            my_sn = (int)(xs ? xe - xb : ye - yb);
+            my_ln = (int)(xs ? ye - yb : xe - xb);
+            if (P.hub_of) my_hub = __ldg(P.hub_of + (xs ? y : x));
+        }
+        for (unsigned todo = __ballot_sync(0xffffffffu, run); todo; todo &= todo - 1) {
+            const int l = __ffs(todo) - 1;
+            const int64_t sb = __shfl_sync(0xffffffffu, my_sb, l), lb = __shfl_sync(0xffffffffu, my_lb, l);
+            const int sn = __shfl_sync(0xffffffffu, my_sn, l), ln = __shfl_sync(0xffffffffu, my_ln, l);
+            const int hub = __shfl_sync(0xffffffffu, my_hub, l);
+            const int32_t t0 = __shfl_sync(0xffffffffu, my_t0, l), old = __shfl_sync(0xffffffffu, my_old, l);
+            const int32_t t = min(t0, (int32_t)__shfl_sync(0xffffffffu, d, l));
+            const bool direct = P.direct || (!AND && old != t0);
+            const uint2* const table = hub >= 0 ? P.hub_bits + hub * P.hub_words : nullptr;
+            const int32_t* const scol = (table && P.by_degree ? P.by_degree : P.col) + sb;
+            const uint32_t* const slot = table && P.by_degree ? P.slot_of + sb : nullptr;
+            const OtfRow<!AND, false> row{scol, slot, P.col + lb, sb, lb, sn, ln, table, buf, P.gin, P.eid, P.tin, 0, 0};
             int32_t h;
-            const int ln = (int)(le - lb), sn = (int)(se - sb);
-            if (tc > kTau16Max)
-                h = warp_hindex<false, kHistWords>(RhoOtf<!AND, true>{P.col, sb, lb, ln, P.gin, P.eid, P.tin}, NoBound{}, sn, tc, direct,
-                                            bins);
-            else
-                h = warp_hindex<false, kHistWords>(RhoOtf<!AND, false>{P.col, sb, lb, ln, P.gin, P.eid, P.tin}, NoBound{}, sn, tc, direct,
-                                            bins);
-            if (lane == 0) {
-                n.row(it.d, h != tr);
+            if (t > kTau16Max) {
+                const OtfRow<!AND, true> exact{scol, slot, P.col + lb, sb, lb, sn, ln, table, buf,
+                                               P.gin, P.eid, P.tin, 0, 0};
+                h = warp_hindex<false, kHistWords>(exact, NoBound{}, sn, t, direct, bins);
+            } else {
+                h = warp_hindex<false, kHistWords>(row, DegreeBound{slot && P.bounded ? scol : nullptr, P.rp, t}, sn, t,
+                                                   direct, bins);
+            }
+            if (lane == l) {
+                n.row(d, h != t0);
                 store_tau<2>(P, R, h, old);
             }
-            if (AND && NOTIFY && h != tr) {
+            if (AND && NOTIFY && h != t0) {
                 // notify the other two edges of every triangle, found again
-                for (int64_t j = lane; j < se - sb; j += 32) {
-                    const int32_t w = __ldg(P.col + sb + j);
-                    const int k = nd_lower_bound_n(P.col + lb, (int)(le - lb), w);
-                    if (k >= (int)(le - lb) || __ldg(P.col + lb + k) != w) continue;
-                    const uint32_t ps = (uint32_t)(sb + j), pl = (uint32_t)(lb + k);
-                    notify_pos(P, ps, h);
-                    notify_pos(P, pl, h);
+                const DegreeBound bound{slot && P.bounded ? scol : nullptr, P.rp, h};
+                for (int i = 0; i < sn;) {
+                    const int end = min(sn, i + 256);
+                    row.match(i, end, [&](int j, int k) {
+                        if (k < 0) return;
+                        notify_pos(P, slot ? __ldg(slot + j) : (uint32_t)(sb + j), h);
+                        notify_pos(P, (uint32_t)(lb + k), h);
+                    });
+                    i = end;
+                    if (bound.past(i)) break;  // no later edge has a tau of h or more
                 }
             }
+            __syncwarp();  // the bins and the block are free again
         }
     }
     flush_tally(P, n);
+}
+
+// vertices by floor(log2 degree)
+__global__ void k_degree_classes(int64_t n, const int64_t* __restrict__ rp, unsigned long long* __restrict__ cnt) {
+    __shared__ unsigned c[32];
+    if (threadIdx.x < 32) c[threadIdx.x] = 0;
+    __syncthreads();
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t d = rp[v + 1] - rp[v];
+        if (d > 0) atomicAdd(&c[31 - __clz((unsigned)min(d, (int64_t)INT32_MAX))], 1u);
+    }
+    __syncthreads();
+    if (threadIdx.x < 32 && c[threadIdx.x]) atomicAdd(cnt + threadIdx.x, (unsigned long long)c[threadIdx.x]);
+}
+
+// hub numbers of the vertices of at least min_degree neighbours
+__global__ void k_number_hubs(int64_t n, const int64_t* __restrict__ rp, int64_t min_degree,
+                              int32_t* __restrict__ hub_of, int32_t* __restrict__ hubs, int* __restrict__ count) {
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
+        int h = -1;
+        if (rp[v + 1] - rp[v] >= min_degree) {
+            h = atomicAdd(count, 1);
+            hubs[h] = (int32_t)v;
+        }
+        hub_of[v] = h;
+    }
+}
+
+// the table of every hub, one block each: word w covers the vertices
+// [32 w, 32 w + 32), x = which of them are neighbours, y = neighbours below.
+// The list is sorted, so a word's entries are one run: its first entry (found
+// by a search, as the word's count below) writes the word alone.
+__global__ void __launch_bounds__(kThreads) k_hub_tables(const int32_t* __restrict__ hubs,
+                                                         const int64_t* __restrict__ rp,
+                                                         const int32_t* __restrict__ col, int64_t words,
+                                                         uint2* __restrict__ tables) {
+    const int32_t v = hubs[blockIdx.x];
+    const int64_t b = rp[v];
+    const int d = (int)(rp[v + 1] - b);
+    uint2* const t = tables + (int64_t)blockIdx.x * words;
+    for (int64_t w = threadIdx.x; w < words; w += kThreads) {
+        const int64_t lo = 32 * w;  // below n, so a vertex id
+        int j = nd_lower_bound_n(col + b, d, (int32_t)lo);
+        const unsigned below = (unsigned)j;
+        unsigned bits = 0;
+        for (; j < d; ++j) {
+            const int64_t x = (int64_t)__ldg(col + b + j) - lo;
+            if (x >= 32) break;
+            bits |= 1u << x;
+        }
+        t[w] = make_uint2(bits, below);
+    }
 }
 
 typedef void (*pass_fn)(SweepParams);
@@ -1471,6 +1704,68 @@ nd_status nd_classic_truss(const int32_t* in, int64_t n, int32_t* out, cudaStrea
     return ND_OK;
 }
 
+namespace {
+
+// the hub tables of a run without a stored incidence, in the run's own
+// workspace.  The largest degree class whose tables, with those of the
+// classes above, fit kHubBytes (an L2's worth: past that the probes would go
+// to DRAM) bounds the hubs.  Small graphs, and a device without the memory,
+// do without.
+constexpr int64_t kHubBytes = int64_t(128) << 20;
+constexpr int64_t kHubMinEntries = 1 << 18;  // below, the tables cost more than the passes
+constexpr int kHubMinClass = 5;              // lists of 32 entries are searched as fast
+
+struct hub_tables {
+    nd_tmp<int32_t> of, list, by_degree;
+    nd_tmp<uint32_t> slot_of;
+    nd_tmp<uint2> bits;
+    explicit hub_tables(cudaStream_t st) : of(st), list(st), by_degree(st), slot_of(st), bits(st) {}
+};
+
+nd_status make_hub_tables(nd_incidence* h, hub_tables* t, SweepParams& P, cudaStream_t st) {
+    const int64_t words = (h->n + 31) / 32;
+    if (h->nnz < kHubMinEntries) return ND_OK;
+    nd_tmp<unsigned long long> cnt(st);
+    nd_tmp<int> count(st);
+    ND_TRY(cnt.alloc(32));
+    ND_TRY(count.alloc(1));
+    ND_CUDA(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long) * 32, st));
+    ND_CUDA(cudaMemsetAsync(count, 0, sizeof(int), st));
+    const int blocks = nd_blocks_for(h->n, kThreads, h->sm_count * 8);
+    nd_prof_scope ps("hub_tables", st, 3);
+    k_degree_classes<<<blocks, kThreads, 0, st>>>(h->n, h->rp, cnt);
+    ND_CUDA(cudaGetLastError());
+    ND_CUDA(cudaMemcpyAsync(h->h_read, cnt, sizeof(unsigned long long) * 32, cudaMemcpyDeviceToHost, st));
+    ND_TRY(nd_wait(st));
+    int64_t hubs = 0;
+    int k = 32;
+    while (k > kHubMinClass && (hubs + h->h_read[k - 1]) * words * (int64_t)sizeof(uint2) <= kHubBytes) hubs += h->h_read[--k];
+    if (hubs == 0) return ND_OK;
+    if (t->of.alloc(h->n) != ND_OK || t->list.alloc(hubs) != ND_OK || t->bits.alloc(hubs * words) != ND_OK ||
+        t->by_degree.alloc(h->nnz) != ND_OK || t->slot_of.alloc(h->nnz) != ND_OK) {
+        nd_set_error("");
+        return ND_OK;
+    }
+    k_number_hubs<<<blocks, kThreads, 0, st>>>(h->n, h->rp, (int64_t)1 << k, t->of, t->list, count);
+    ND_CUDA(cudaGetLastError());
+    k_hub_tables<<<(unsigned)hubs, kThreads, 0, st>>>(t->list, h->rp, h->col, words, t->bits);
+    ND_CUDA(cudaGetLastError());
+    const nd_status rc = nd_rows_by_degree(h, t->by_degree, t->slot_of, st);
+    if (rc == ND_E_NOMEM) {
+        nd_set_error("");
+        return ND_OK;
+    }
+    ND_TRY(rc);
+    P.by_degree = t->by_degree;
+    P.slot_of = t->slot_of;
+    P.hub_of = t->of;
+    P.hub_bits = t->bits;
+    P.hub_words = words;
+    return ND_OK;
+}
+
+}  // namespace
+
 // Runs passes of `mode` until a pass changes nothing or max_passes passes ran.
 // Passes are enqueued in batches; each pass reads the previous pass's counter
 // on the device and returns at once if it was zero, so the host only reads
@@ -1543,7 +1838,8 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
     P.ev = h->e_v;
     P.items = h->items;
     P.members = members;
-    P.oct_max = tau_in_dev ? nullptr : h->oct_max;  // tau <= d_s holds for the library's own start
+    P.bounded = !tau_in_dev;  // tau <= d_s holds for the library's own start
+    P.oct_max = P.bounded ? h->oct_max : nullptr;
     // batches, SND and AND-nn: every graph starts active (AND with
     // notification needs nothing more: a converged graph notifies no one)
     P.gid = nullptr;
@@ -1556,6 +1852,13 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
         P.gid = h->gid;
     }
     plan_buckets(h, P);
+    hub_tables hubs(st);
+    P.hub_of = nullptr;
+    P.hub_bits = nullptr;
+    P.hub_words = 0;
+    P.by_degree = nullptr;
+    P.slot_of = nullptr;
+    if (h->otf) ND_TRY(make_hub_tables(h, &hubs, P, st));
     pass_fn fn0 = pick(h, mode, false), fn1 = pick(h, mode, true);
     // ask for a shared-memory carve-out that just holds each kernel's
     // resident blocks (plus the 1 KB each block reserves), leaving the rest
@@ -1598,13 +1901,13 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
         if (stop_active > 0.0) nb = 1;  // the stopping rule looks at every pass
         const int kind = batch == 0 ? 0 : ((batch & 1) ? 2 : 1);
         bool launched = false;
-        // graphs hold the plain parameters; runs with members, a stopping rule
-        // or a tau of the caller's launch directly, and so does the first batch of its kind on a
+        // graphs hold the plain parameters; runs with members, a stopping rule,
+        // a tau of the caller's or tables of their own launch directly, and so does the first batch of its kind on a
         // handle: building a graph costs more than its launches, and many
         // handles run each mode once
         const bool seen = h->batch_seen[mode][kind];
         if (nb == kBatch) h->batch_seen[mode][kind] = true;
-        if (nb == kBatch && seen && grid0 > 0 && !members && !tau_in_dev && (start & 1) == 0 && !h->pass_graph_failed[mode][kind]) {
+        if (nb == kBatch && seen && grid0 > 0 && !members && !tau_in_dev && !h->otf && (start & 1) == 0 && !h->pass_graph_failed[mode][kind]) {
             if (!h->pass_graph[mode][kind])
                 make_batch_graph(h, mode, kind, P, grid0, fn0, grid1, fn1, words);
             if (h->pass_graph[mode][kind]) {

@@ -231,6 +231,9 @@ nd_status nd_build_triangles(nd_incidence* h, cudaStream_t st);
 nd_status nd_build_k4_incidence(nd_incidence* h, cudaStream_t st);
 nd_status nd_build_buckets(nd_incidence* h, cudaStream_t st);
 nd_status nd_relabel_by_degree(nd_incidence* h, cudaStream_t st);
+// every adjacency list of h->rp / h->col in order of the neighbours' degree
+// class, high first: the neighbours and their CSR slots (nnz each)
+nd_status nd_rows_by_degree(nd_incidence* h, int32_t* vertex, uint32_t* slot, cudaStream_t st);
 nd_status nd_relabel_truss_graph(nd_incidence* h, cudaStream_t st);
 nd_status nd_relabel_truss_edges(nd_incidence* h, cudaStream_t st);
 // out[idx[i]] = in[i] (scatter) or out[i] = in[idx[i]] (gather), n int32 values on st

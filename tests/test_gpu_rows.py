@@ -69,3 +69,29 @@ def test_rows_at_the_edges(nd, r, pad):
         np.testing.assert_array_equal(inc.and_(notify=notify)[0].cpu().numpy(), kap)
     ta, _ = inc.iterate_k("and", 1 << 20, tau=t1)
     np.testing.assert_array_equal(ta.cpu().numpy(), kap)
+
+
+def test_no_storage_rows_with_hub_tables(nd):
+    """The no-storage passes of a graph large enough for hub tables: lists by
+    degree class, their bound, and the lists below the tables' degree."""
+    n, s, d = G.rmat(14, 16, seed=61)
+    rp, col = G.to_csr(n, s, d)
+    assert rp[-1] >= 1 << 18
+    g = oracle.ParallelSND(rp, col, 2, threads=8)
+    inc = nd.build_incidence(torch.from_numpy(rp).cuda(), torch.from_numpy(col).cuda(), 2, 3, on_the_fly=True)
+    for k in (1, 2, 5):
+        tk, _ = inc.iterate_k("snd", k)
+        np.testing.assert_array_equal(tk.cpu().numpy(), g.snd(max_sweeps=k)[0])
+    t1, _ = inc.iterate_k("snd", 1)
+    t3, _ = inc.iterate_k("snd", 2, tau=t1)
+    np.testing.assert_array_equal(t3.cpu().numpy(), g.snd(max_sweeps=3)[0])
+    kap, passes = inc.snd()
+    kap = kap.cpu().numpy()
+    want = g.snd()
+    np.testing.assert_array_equal(kap, want[0])
+    for notify in (True, False):
+        np.testing.assert_array_equal(inc.and_(notify=notify)[0].cpu().numpy(), kap)
+    stored = nd.build_incidence(torch.from_numpy(rp).cuda(), torch.from_numpy(col).cuda(), 2, 3)
+    members = torch.arange(0, inc.num_r, 3, dtype=torch.int32, device="cuda")
+    np.testing.assert_array_equal(inc.and_partial(members)[0].cpu().numpy(),
+                                  stored.and_partial(members)[0].cpu().numpy())

@@ -88,6 +88,8 @@ nd_prof_scope::~nd_prof_scope() {
 // per-handle device memory limit (nd_set_handle_memory_limit; 0 = none)
 static std::atomic<int64_t> g_handle_limit{0};
 
+int64_t nd_handle_limit() { return g_handle_limit.load(); }
+
 nd_status nd_alloc(void** p, size_t bytes, cudaStream_t st, nd_incidence* owner) {
     if (bytes == 0) bytes = 16;
     const int64_t limit = g_handle_limit.load();
@@ -242,7 +244,7 @@ void nd_free(nd_incidence* h) {
     void* ptrs[] = {h->nlow, h->up_start, h->eid, h->e_u, h->e_v, h->tri_ptr, h->tri_w, h->tri_e,
                     h->items, h->tau[0], h->tau[1], h->front[0], h->front[1], h->counters,
                     h->mirror, h->e_pos, h->tg[0], h->tg[1], h->long_rows, h->long_seg, h->to_new, h->to_old,
-                    h->vto_old, h->oct_max, h->c_rp, h->c_up, h->c_col, h->c_nlow, h->gid, h->gact[0], h->gact[1]};
+                    h->vto_old, h->oct_max, h->t_pos, h->t_id, h->c_rp, h->c_up, h->c_col, h->c_nlow, h->gid, h->gact[0], h->gact[1]};
     for (void* p : ptrs) nd_release(p, st);
     for (auto& row : h->pass_graph)
         for (auto& ex : row)
@@ -349,8 +351,7 @@ static nd_status build_common(const nd_csr* g, int r, int s, cudaStream_t st, nd
         } else if (r == 2) {
             rc = nd_build_tri_incidence(h, st);
         } else {
-            rc = nd_build_triangles(h, st);
-            if (rc == ND_OK) rc = nd_build_k4_incidence(h, st);
+            rc = nd_build_k4_incidence(h, st);
         }
     }
     if (rc == ND_OK) apply_tuned(h, dev);

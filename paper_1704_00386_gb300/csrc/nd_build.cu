@@ -9,8 +9,8 @@
 //   (2,3)  triangle {u,v,w} -> one pair per edge: the CSR slots of its other
 //          two edges at the edge's endpoints (found once each, by degree
 //          orientation), each row then ordered by the third vertex;
-//   (3,4)  triangle (u,v,w): x in N(u) /\ N(v) /\ N(w) -> the ids of the
-//          triangles {u,v,x}, {u,w,x}, {v,w,x}.
+//   (3,4)  triangle (u,v,w): the z in the triangle lists of its three edges
+//          -> the slots of {u,v,z}, {u,w,z}, {v,w,z} in those lists.
 // Every step is a count pass, an exclusive scan and a fill pass over the same
 // enumeration.  Intersections: one warp per list pair; the lanes walk the
 // shorter list in order and binary-search each element in the other list(s)
@@ -983,203 +983,184 @@ k_row_rank(int64_t N, const int64_t* __restrict__ inc_ptr, const int32_t* __rest
     }
 }
 
-// ---- (3,4) step 1: canonical triangle list (one warp per edge) -------------
-// Edge (u,v), u<v, owns the triangles (u,v,w) with w > v: w in the parts of
-// N(u) and N(v) above v.  COUNT: ptr[e] = number owned.  FILL: tri_w, tri_e.
+// ---- (3,4): the triangles of every edge, and the 4-cliques of every triangle --
+// The list of edge (u,v) holds every triangle on it, by third vertex: the
+// common neighbours of u and v, one warp per edge.  Third vertices above v
+// make the canonical triangles (u < v < w, lexicographic, grouped by edge in
+// tri_ptr / tri_w / tri_e).  A triangle stands in the lists of its three edges.
+// The 4-cliques of triangle {u,v,w} are then the z in all three of them: one
+// warp per triangle intersects the lists, which are far shorter than the
+// neighbourhoods (a planted clique of k vertices: k - 2), and writes its row in
+// order of z, with no atomics, no cursors and no search for triangle ids.
+// Listing every 4-clique once by degree orientation, with three id searches
+// each and a scatter into four rows, took 18.5 ms for 55M 4-cliques (Chung-Lu
+// 100K with planted cliques) and left the rows unordered.
 template <bool FILL>
-__global__ void k_triangle_list(int64_t m, const int64_t* __restrict__ rp,
-                                const int32_t* __restrict__ col, const int32_t* __restrict__ nlow,
-                                const int64_t* __restrict__ up_start, const int32_t* __restrict__ e_u,
-                                const int32_t* __restrict__ e_v, int64_t* __restrict__ ptr,
-                                int32_t* __restrict__ tri_w, uint32_t* __restrict__ tri_e) {
+__global__ void __launch_bounds__(kThreads) k_edge_lists(int64_t m, const int64_t* __restrict__ rp,
+                                                         const int32_t* __restrict__ col,
+                                                         const uint32_t* __restrict__ eid,
+                                                         const int32_t* __restrict__ e_u,
+                                                         const int32_t* __restrict__ e_v, int64_t* __restrict__ lptr,
+                                                         int64_t* __restrict__ tri_ptr, int32_t* __restrict__ lw,
+                                                         uint32_t* __restrict__ lid, int32_t* __restrict__ tri_w,
+                                                         uint32_t* __restrict__ tri_e, uint32_t* __restrict__ te,
+                                                         uint32_t* __restrict__ t_pos) {
+    __shared__ int32_t bufs[kThreads / 32][nd_list_cursor::kBlock];
     const int lane = threadIdx.x & 31;
     for (int64_t e = warp_id_global(); e < m; e += warp_count_global()) {
         const int32_t u = e_u[e], v = e_v[e];
-        // position of v in row u follows from the edge id; entries after it are > v
-        int64_t ab = rp[u] + nlow[u] + (e - up_start[u]) + 1, ae = rp[u + 1];
-        int64_t bb = rp[v] + nlow[v], be = rp[v + 1];
-        if (ae - ab > be - bb) { int64_t t = ab; ab = bb; bb = t; t = ae; ae = be; be = t; }
-        int64_t out = FILL ? ptr[e] : 0;
-        int64_t cnt = 0;
-        int64_t lo = bb;
-        for (int64_t base = ab; base < ae; base += 32) {
-            int64_t p = base + lane;
-            bool found = false;
-            int64_t pb = 0;
-            int32_t x = 0;
-            if (p < ae) {
-                x = __ldg(col + p);
-                pb = lower_bound_i32(col, lo, be, x);
-                found = (pb < be) && (__ldg(col + pb) == x);
-            }
-            unsigned bal = __ballot_sync(kFull, found);
-            if (FILL && found) {
-                int64_t slot = out + cnt + __popc(bal & lanemask_lt());
-                tri_w[slot] = x;
-                tri_e[slot] = (uint32_t)e;
-            }
-            cnt += __popc(bal);
-            int64_t last_pb = __shfl_sync(kFull, pb, 31);
-            if (base + 32 <= ae) lo = last_pb;
-        }
-        if (!FILL && lane == 0) ptr[e] = cnt;
-    }
-}
-
-// ---- (3,4): 4-cliques by degree orientation ---------------------------------
-// Every 4-clique {a,b,w,x} with a before b before w before x (degree order) is
-// found exactly once, as x in out(a) /\ out(b) /\ out(w) for the oriented
-// triangle (a,b,w).  Its four triangles get their canonical ids (lexicographic
-// u<v<w, grouped by edge (u,v) in tri_ptr / tri_w) from one binary search
-// each, because the six edge ids are known from the out-lists.  The 4-cliques
-// are listed once (4 triangle ids each), then scattered into the incidence
-// rows through per-triangle cursors; row order is therefore unspecified.
-
-struct otri {  // oriented triangle a -> b -> w and its edge ids
-    int32_t a, b, w;
-    uint32_t e_ab, e_aw, e_bw;
-};
-
-// one warp per oriented edge a -> b: the oriented triangles (a, b, w)
-template <bool FILL>
-__global__ void k_otri(int64_t m, const int64_t* __restrict__ out_ptr, const int32_t* __restrict__ out_col,
-                       const uint32_t* __restrict__ out_eid, const int32_t* __restrict__ out_src,
-                       int64_t* __restrict__ ptr, otri* __restrict__ tris) {
-    const int lane = threadIdx.x & 31;
-    for (int64_t k = warp_id_global(); k < m; k += warp_count_global()) {
-        const int32_t a = out_src[k], b = out_col[k];
-        const uint32_t e_ab = out_eid[k];
-        int64_t ab = out_ptr[a], ae = out_ptr[a + 1], bb = out_ptr[b], be = out_ptr[b + 1];
-        bool a_is_a = true;
-        if (ae - ab > be - bb) {
-            int64_t t = ab; ab = bb; bb = t; t = ae; ae = be; be = t;
-            a_is_a = false;
-        }
-        const int64_t out = FILL ? ptr[k] : 0;
-        int64_t cnt = 0, lo = bb;
-        for (int64_t base = ab; base < ae; base += 32) {
-            const int64_t p = base + lane;
-            bool found = false;
-            int64_t pb = 0;
-            int32_t x = 0;
-            if (p < ae) {
-                x = __ldg(out_col + p);
-                pb = lower_bound_i32(out_col, lo, be, x);
-                found = (pb < be) && (__ldg(out_col + pb) == x);
-            }
-            const unsigned bal = __ballot_sync(kFull, found);
-            if (FILL && found) {
-                const uint32_t e1 = __ldg(out_eid + p), e2 = __ldg(out_eid + pb);
-                otri t;
-                t.a = a; t.b = b; t.w = x; t.e_ab = e_ab;
-                t.e_aw = a_is_a ? e1 : e2;
-                t.e_bw = a_is_a ? e2 : e1;
-                tris[out + cnt + __popc(bal & lanemask_lt())] = t;
-            }
-            cnt += __popc(bal);
-            const int64_t last_pb = __shfl_sync(kFull, pb, 31);
-            if (base + 32 <= ae) lo = last_pb;
-        }
-        if (!FILL && lane == 0) ptr[k] = cnt;
-    }
-}
-
-// canonical id of the triangle on vertices p, q, r with edge ids epq, epr, eqr
-__device__ __forceinline__ uint32_t canon_tri(int32_t p, int32_t q, int32_t r, uint32_t epq, uint32_t epr,
-                                              uint32_t eqr, const int64_t* __restrict__ tri_ptr,
-                                              const int32_t* __restrict__ tri_w, bool* ok) {
-    // the smallest two vertex ids own the triangle; the largest is its third vertex
-    uint32_t edge;
-    int32_t third;
-    if (p > q && p > r) { edge = eqr; third = p; }
-    else if (q > r) { edge = epr; third = q; }
-    else { edge = epq; third = r; }
-    const int64_t lo = __ldg(tri_ptr + edge), hi = __ldg(tri_ptr + edge + 1);
-    const int64_t pos = lower_bound_i32(tri_w, lo, hi, third);
-    if (pos >= hi || __ldg(tri_w + pos) != third) { *ok = false; return 0; }
-    return (uint32_t)pos;
-}
-
-// one warp per oriented triangle: x in out(a) /\ out(b) /\ out(w).
-// MODE 0 counts the 4-cliques of the triangle into ptr[t]; MODE 1 writes
-// their four canonical triangle ids at ptr[t] (scanned) and counts the
-// incidences of each triangle in rowcnt.
-template <int MODE>
-__global__ void k_k4(int64_t T, const otri* __restrict__ tris, const int64_t* __restrict__ out_ptr,
-                     const int32_t* __restrict__ out_col, const uint32_t* __restrict__ out_eid,
-                     const int64_t* __restrict__ tri_ptr, const int32_t* __restrict__ tri_w,
-                     int64_t* __restrict__ ptr, uint4* __restrict__ k4, unsigned long long* __restrict__ rowcnt,
-                     int* __restrict__ err) {
-    const int lane = threadIdx.x & 31;
-    for (int64_t t = warp_id_global(); t < T; t += warp_count_global()) {
-        const otri tr = tris[t];
-        const int32_t vtx[3] = {tr.a, tr.b, tr.w};
-        int64_t rb[3], re[3];
-#pragma unroll
-        for (int i = 0; i < 3; ++i) { rb[i] = out_ptr[vtx[i]]; re[i] = out_ptr[vtx[i] + 1]; }
-        int A = 0;
-        if (re[1] - rb[1] < re[A] - rb[A]) A = 1;
-        if (re[2] - rb[2] < re[A] - rb[A]) A = 2;
-        const int B1 = (A == 0) ? 1 : 0, B2 = (A == 2) ? 1 : 2;
-        const int64_t out = MODE ? ptr[t] : 0;
-        int64_t cnt = 0;
-        bool ok = true;
-        uint32_t id0 = 0;  // MODE 1: the triangle (a,b,w) itself, shared by all its 4-cliques
-        if (MODE == 1) {
-            if (ptr[t + 1] == out) continue;  // no 4-clique here
-            id0 = canon_tri(tr.a, tr.b, tr.w, tr.e_ab, tr.e_aw, tr.e_bw, tri_ptr, tri_w, &ok);
-        }
-        for (int64_t base = rb[A]; base < re[A]; base += 32) {
-            const int64_t p = base + lane;
-            bool found = false;
-            int64_t pos[3] = {0, 0, 0};
-            int32_t x = 0;
-            if (p < re[A]) {
-                x = __ldg(out_col + p);
-                pos[A] = p;
-                pos[B1] = lower_bound_i32(out_col, rb[B1], re[B1], x);
-                if (pos[B1] < re[B1] && __ldg(out_col + pos[B1]) == x) {
-                    pos[B2] = lower_bound_i32(out_col, rb[B2], re[B2], x);
-                    found = (pos[B2] < re[B2]) && (__ldg(out_col + pos[B2]) == x);
+        const int64_t ub = rp[u], ue = rp[u + 1], vb = rp[v], ve = rp[v + 1];
+        const bool us = ue - ub <= ve - vb;  // walk the shorter list
+        const int64_t sb = us ? ub : vb, lb = us ? vb : ub;
+        const int sn = (int)(us ? ue - ub : ve - vb), ln = (int)(us ? ve - vb : ue - ub);
+        const int64_t out = FILL ? lptr[e] : 0, tri = FILL ? tri_ptr[e] : 0;
+        int64_t cnt = 0, up = 0;
+        nd_list_cursor cur;
+        cur.start(col + lb, ln, sn, bufs[threadIdx.x >> 5]);
+        for (int j0 = 0; j0 < sn; j0 += 32) {
+            const int j = j0 + lane;
+            const int32_t w = j < sn ? __ldg(col + sb + j) : 0;
+            const int k = cur.find(w, j < sn, __reduce_max_sync(kFull, w));
+            const unsigned all = __ballot_sync(kFull, k >= 0), high = __ballot_sync(kFull, k >= 0 && w > v);
+            if (FILL && k >= 0) {
+                const int64_t slot = out + cnt + __popc(all & lanemask_lt());
+                lw[slot] = w;
+                if (w > v) {
+                    const int64_t id = tri + up + __popc(high & lanemask_lt());
+                    lid[slot] = (uint32_t)id;
+                    tri_w[id] = w;
+                    tri_e[id] = (uint32_t)e;
+                    te[3 * id] = (uint32_t)e;
+                    if (t_pos) t_pos[3 * id] = (uint32_t)slot;
+                } else {
+                    // the edge {u,w}, whose list of canonical triangles holds
+                    // this one (k_list_ids)
+                    lid[slot] = __ldg(eid + (us ? sb + j : lb + k));
                 }
             }
-            const unsigned bal = __ballot_sync(kFull, found);
-            if (MODE == 1 && found) {
-                const uint32_t e_ax = __ldg(out_eid + pos[0]), e_bx = __ldg(out_eid + pos[1]),
-                               e_wx = __ldg(out_eid + pos[2]);
-                uint4 ids;
-                ids.x = id0;
-                ids.y = canon_tri(tr.a, tr.b, x, tr.e_ab, e_ax, e_bx, tri_ptr, tri_w, &ok);
-                ids.z = canon_tri(tr.a, tr.w, x, tr.e_aw, e_ax, e_wx, tri_ptr, tri_w, &ok);
-                ids.w = canon_tri(tr.b, tr.w, x, tr.e_bw, e_bx, e_wx, tri_ptr, tri_w, &ok);
-                k4[out + cnt + __popc(bal & lanemask_lt())] = ids;
-                atomicAdd(rowcnt + ids.y, 1ull);
-                atomicAdd(rowcnt + ids.z, 1ull);
-                atomicAdd(rowcnt + ids.w, 1ull);
-            }
-            cnt += __popc(bal);
+            cnt += __popc(all);
+            up += __popc(high);
         }
-        if (MODE == 1 && cnt > 0 && lane == 0) atomicAdd(rowcnt + id0, (unsigned long long)cnt);
-        if (MODE == 1 && !__all_sync(kFull, ok) && lane == 0) atomicOr(err, 4);
-        if (MODE == 0 && lane == 0) ptr[t] = cnt;
+        if (!FILL && lane == 0) {
+            lptr[e] = cnt;
+            tri_ptr[e] = up;
+        }
+        __syncwarp();
     }
 }
 
-// one thread per 4-clique: add it to the rows of its four triangles
-template <typename C>
-__global__ void k_k4_scatter(int64_t K, const uint4* __restrict__ k4, C* __restrict__ cursor,
-                             uint32_t* __restrict__ inc) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < K; i += (int64_t)gridDim.x * blockDim.x) {
-        const uint4 q = k4[i];
-        const uint32_t id[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            uint32_t* d = inc + 3 * (int64_t)atomicAdd(cursor + id[k], (C)1);
-            int o = 0;
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-                if (j != k) d[o++] = id[j];
+// the ids of the list entries whose third vertex w is below v: v's place among
+// the canonical triangles of the edge {u,w} (left in lid)
+__global__ void k_list_ids(int64_t m, const int32_t* __restrict__ e_u, const int32_t* __restrict__ e_v,
+                           const int64_t* __restrict__ lptr, const int32_t* __restrict__ lw,
+                           uint32_t* __restrict__ lid, const int64_t* __restrict__ tri_ptr,
+                           const int32_t* __restrict__ tri_w, uint32_t* __restrict__ te,
+                           uint32_t* __restrict__ t_pos) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t e = warp_id_global(); e < m; e += warp_count_global()) {
+        const int64_t b = lptr[e], low = (lptr[e + 1] - b) - (tri_ptr[e + 1] - tri_ptr[e]);
+        if (low == 0) continue;
+        const int32_t u = e_u[e], v = e_v[e];
+        for (int64_t s = b + lane; s < b + low; s += 32) {
+            const int32_t w = lw[s];
+            const uint32_t o = lid[s];
+            const int64_t id = lower_bound_i32(tri_w, tri_ptr[o], tri_ptr[o + 1], v);
+            lid[s] = (uint32_t)id;
+            const int64_t at = 3 * id + (w < u ? 2 : 1);
+            te[at] = (uint32_t)e;
+            if (t_pos) t_pos[at] = (uint32_t)s;
         }
+    }
+}
+
+// The 4-cliques of every triangle.  FILL: its row, three runs of d words (the
+// slot of z in each of the three lists, or the triangle there: IDS), ordered
+// by z; else their number.  Eight triangles per warp at a time: their list
+// bounds, a chain of two loads, are fetched by eight lanes at once.
+template <bool FILL, bool IDS>
+__global__ void __launch_bounds__(kThreads) k_k4_rows(int64_t T, const uint32_t* __restrict__ te,
+                                                      const int64_t* __restrict__ lptr,
+                                                      const int32_t* __restrict__ lw,
+                                                      const uint32_t* __restrict__ lid,
+                                                      int64_t* __restrict__ inc_ptr, uint32_t* __restrict__ inc) {
+    __shared__ int32_t bufs[kThreads / 32][2][nd_list_cursor::kBlock];
+    const int lane = threadIdx.x & 31;
+    constexpr int kAtOnce = 8;
+    const int64_t groups = (T + kAtOnce - 1) / kAtOnce;
+    for (int64_t g = warp_id_global(); g < groups; g += warp_count_global()) {
+        const int64_t t0 = g * kAtOnce;
+        int64_t b[3] = {0, 0, 0}, jb = 0;  // shortest list first
+        int n[3] = {0, 0, 0}, d = 0;
+        bool run = lane < kAtOnce && t0 + lane < T;
+        if (run && FILL) {
+            jb = inc_ptr[t0 + lane];
+            d = (int)(inc_ptr[t0 + lane + 1] - jb);
+            run = d > 0;
+        }
+        if (run) {
+            uint32_t e[3];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) e[i] = __ldg(te + 3 * (t0 + lane) + i);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                b[i] = __ldg(lptr + e[i]);
+                n[i] = (int)(__ldg(lptr + e[i] + 1) - b[i]);
+            }
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {  // sort by length: (0,1), (1,2), (0,1)
+                const int x = i & 1, y = x + 1;
+                if (n[x] > n[y]) {
+                    const int tn = n[x];
+                    n[x] = n[y];
+                    n[y] = tn;
+                    const int64_t tb = b[x];
+                    b[x] = b[y];
+                    b[y] = tb;
+                }
+            }
+        }
+        int count = 0;  // lane l: 4-cliques of triangle t0 + l
+        // every list holds the triangle's own third vertex, so a 4-clique needs two
+        for (unsigned todo = __ballot_sync(kFull, run && n[0] > 1); todo; todo &= todo - 1) {
+            const int l = __ffs(todo) - 1;
+            int64_t lb[3];
+            int ln[3];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                lb[i] = __shfl_sync(kFull, b[i], l);
+                ln[i] = __shfl_sync(kFull, n[i], l);
+            }
+            uint32_t* row = nullptr;
+            int rd = 0;
+            if (FILL) {
+                row = inc + 3 * __shfl_sync(kFull, jb, l);
+                rd = __shfl_sync(kFull, d, l);
+            }
+            nd_list_cursor B, C;
+            B.start(lw + lb[1], ln[1], ln[0], bufs[threadIdx.x >> 5][0]);
+            C.start(lw + lb[2], ln[2], ln[0], bufs[threadIdx.x >> 5][1]);
+            int cnt = 0;
+            for (int j0 = 0; j0 < ln[0]; j0 += 32) {
+                const int j = j0 + lane;
+                const int32_t z = j < ln[0] ? __ldg(lw + lb[0] + j) : 0;
+                const int32_t top = __reduce_max_sync(kFull, z);
+                const int kb = B.find(z, j < ln[0], top);
+                if (!__any_sync(kFull, kb >= 0)) continue;
+                const int kc = C.find(z, kb >= 0, top);
+                const unsigned hit = __ballot_sync(kFull, kc >= 0);
+                if (FILL && kc >= 0) {
+                    const int at = cnt + __popc(hit & lanemask_lt());
+                    const int64_t s0 = lb[0] + j, s1 = lb[1] + kb, s2 = lb[2] + kc;
+                    row[at] = IDS ? lid[s0] : (uint32_t)s0;
+                    row[at + rd] = IDS ? lid[s1] : (uint32_t)s1;
+                    row[at + 2 * (int64_t)rd] = IDS ? lid[s2] : (uint32_t)s2;
+                }
+                cnt += __popc(hit);
+            }
+            if (lane == l) count = cnt;
+            __syncwarp();
+        }
+        if (!FILL && lane < kAtOnce && t0 + lane < T) inc_ptr[t0 + lane] = count;
     }
 }
 
@@ -1730,7 +1711,7 @@ nd_status nd_build_edges(nd_incidence* h, cudaStream_t st) {
     return ND_OK;
 }
 
-// oriented out-lists (degree order), used by the (2,3) and (3,4) builds
+// oriented out-lists (degree order) of the (2,3) build
 struct nd_oriented {
     nd_tmp<int64_t> out_ptr;
     nd_tmp<int32_t> out_col, out_src;
@@ -1925,106 +1906,77 @@ nd_status nd_build_tri_incidence(nd_incidence* h, cudaStream_t st) {
     return ND_OK;
 }
 
-nd_status nd_build_triangles(nd_incidence* h, cudaStream_t st) {
-    ND_TRY(nd_alloc((void**)&h->tri_ptr, sizeof(int64_t) * (h->m + 1), st, h));
-    ND_CUDA(cudaMemsetAsync(h->tri_ptr, 0, sizeof(int64_t) * (h->m + 1), st));
-    int blocks = nd_blocks_for(h->m * 32, kThreads, grid_cap(h) * 4);
-    if (h->m > 0) {
-        nd_prof_scope ps("tri_list_count", st);
-        k_triangle_list<false><<<blocks, kThreads, 0, st>>>(h->m, h->rp, h->col, h->nlow, h->up_start,
-                                                            h->e_u, h->e_v, h->tri_ptr, nullptr,
-                                                            nullptr);
-        ND_CUDA(cudaGetLastError());
-    }
-    ND_TRY(nd_scan_i64(h->tri_ptr, h->m, st));
-    ND_TRY(read_i64(h, h->tri_ptr + h->m, &h->num_tri, st));
-    if (h->num_tri >= (int64_t)UINT32_MAX) { nd_set_error("more than 2^32-1 triangles"); return ND_E_TOO_LARGE; }
-    ND_TRY(nd_alloc((void**)&h->tri_w, sizeof(int32_t) * (h->num_tri > 0 ? h->num_tri : 1), st, h));
-    ND_TRY(nd_alloc((void**)&h->tri_e, sizeof(uint32_t) * (h->num_tri > 0 ? h->num_tri : 1), st, h));
-    if (h->num_tri > 0) {
-        nd_prof_scope ps("tri_list_fill", st);
-        k_triangle_list<true><<<blocks, kThreads, 0, st>>>(h->m, h->rp, h->col, h->nlow, h->up_start,
-                                                           h->e_u, h->e_v, h->tri_ptr, h->tri_w,
-                                                           h->tri_e);
-        ND_CUDA(cudaGetLastError());
-    }
-    return ND_OK;
+// may a (3,4) handle of T triangles and M incidences take the list layout?
+// Its slots have 32 bits, and what it holds beyond the id layout must not make
+// a handle miss the memory limit that would do without.
+static bool list_layout_fits(const nd_incidence* h, int64_t T, int64_t M) {
+    if (3 * T >= (int64_t)UINT32_MAX) return false;
+    const int64_t limit = nd_handle_limit();
+    if (limit <= 0) return true;
+    const int64_t extra = 24 * T + 12 * T + T;          // t_pos, t_id; two 16-bit copies; frontier bits
+    const int64_t rest = 12 * M + 16 * T + 8 * T + 4 * T + (1 << 16);  // incidence, items, tau, a batch's graph ids
+    return h->bytes + extra + rest <= limit;
 }
 
 nd_status nd_build_k4_incidence(nd_incidence* h, cudaStream_t st) {
-    const int64_t T = h->num_tri, m = h->m;
-    h->num_r = T;
-    ND_TRY(nd_alloc((void**)&h->inc_ptr, sizeof(int64_t) * (T + 1), st, h));
-    ND_CUDA(cudaMemsetAsync(h->inc_ptr, 0, sizeof(int64_t) * (T + 1), st));
-    if (T == 0) { h->num_inc = 0; ND_TRY(nd_alloc((void**)&h->inc, 16, st, h)); return ND_OK; }
-    nd_oriented o(st);
-    ND_TRY(orient_graph(h, &o, st));
-    nd_tmp<int64_t> optr(st), kptr(st);  // oriented triangles per oriented edge; 4-cliques per triangle
-    nd_tmp<otri> tris(st);
-    nd_tmp<int> derr(st);
-    ND_TRY(optr.alloc(m + 1));
-    ND_TRY(kptr.alloc(T + 1));
-    ND_TRY(tris.alloc(T));
-    ND_TRY(derr.alloc(1));
-    ND_CUDA(cudaMemsetAsync(derr, 0, sizeof(int), st));
-    ND_CUDA(cudaMemsetAsync(optr.p + m, 0, sizeof(int64_t), st));
-    ND_CUDA(cudaMemsetAsync(kptr.p + T, 0, sizeof(int64_t), st));
+    const int64_t m = h->m;
+    ND_TRY(nd_alloc((void**)&h->tri_ptr, sizeof(int64_t) * (m + 1), st, h));
+    ND_CUDA(cudaMemsetAsync(h->tri_ptr, 0, sizeof(int64_t) * (m + 1), st));
+    nd_tmp<int64_t> lptr(st);
+    ND_TRY(lptr.alloc(m + 1));
+    ND_CUDA(cudaMemsetAsync(lptr, 0, sizeof(int64_t) * (m + 1), st));
     const int eblocks = nd_blocks_for(m * 32, kThreads, grid_cap(h) * 4);
-    const int tblocks = nd_blocks_for(T * 32, kThreads, grid_cap(h) * 4);
-    {
-        nd_prof_scope ps("otri", st);
-        k_otri<false><<<eblocks, kThreads, 0, st>>>(m, o.out_ptr, o.out_col, o.out_eid, o.out_src, optr, nullptr);
+    if (m > 0) {
+        nd_prof_scope ps("edge_lists", st);
+        k_edge_lists<false><<<eblocks, kThreads, 0, st>>>(m, h->rp, h->col, h->eid, h->e_u, h->e_v, lptr, h->tri_ptr,
+                                                          nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);
         ND_CUDA(cudaGetLastError());
     }
-    ND_TRY(nd_scan_i64(optr, m, st));
+    ND_TRY(nd_scan_i64(lptr, m, st));
+    ND_TRY(nd_scan_i64(h->tri_ptr, m, st));
+    ND_TRY(read_i64(h, h->tri_ptr + m, &h->num_tri, st));
+    const int64_t T = h->num_tri;
+    if (T >= (int64_t)UINT32_MAX) { nd_set_error("more than 2^32-1 triangles"); return ND_E_TOO_LARGE; }
+    h->num_r = T;
+    ND_TRY(nd_alloc((void**)&h->tri_w, sizeof(int32_t) * (T > 0 ? T : 1), st, h));
+    ND_TRY(nd_alloc((void**)&h->tri_e, sizeof(uint32_t) * (T > 0 ? T : 1), st, h));
+    ND_TRY(nd_alloc((void**)&h->inc_ptr, sizeof(int64_t) * (T + 1), st, h));
+    ND_CUDA(cudaMemsetAsync(h->inc_ptr + T, 0, sizeof(int64_t), st));
+    if (T == 0) { h->num_inc = 0; ND_TRY(nd_alloc((void**)&h->inc, 16, st, h)); return ND_OK; }
+    nd_tmp<int32_t> lw(st);
+    nd_tmp<uint32_t> lid(st), te(st), t_pos(st);
+    ND_TRY(lw.alloc(3 * T));
+    ND_TRY(lid.alloc(3 * T));
+    ND_TRY(te.alloc(3 * T));
+    if (3 * T < (int64_t)UINT32_MAX) ND_TRY(t_pos.alloc(3 * T));
     {
-        nd_prof_scope ps("otri", st);
-        k_otri<true><<<eblocks, kThreads, 0, st>>>(m, o.out_ptr, o.out_col, o.out_eid, o.out_src, optr, tris);
+        nd_prof_scope ps("edge_lists", st, 2);
+        k_edge_lists<true><<<eblocks, kThreads, 0, st>>>(m, h->rp, h->col, h->eid, h->e_u, h->e_v, lptr, h->tri_ptr, lw,
+                                                         lid, h->tri_w, h->tri_e, te, t_pos);
+        ND_CUDA(cudaGetLastError());
+        k_list_ids<<<eblocks, kThreads, 0, st>>>(m, h->e_u, h->e_v, lptr, lw, lid, h->tri_ptr, h->tri_w, te, t_pos);
         ND_CUDA(cudaGetLastError());
     }
+    const int tblocks = nd_blocks_for(T * 4, kThreads, grid_cap(h) * 4);
     {
         nd_prof_scope ps("k4_count", st);
-        k_k4<0><<<tblocks, kThreads, 0, st>>>(T, tris, o.out_ptr, o.out_col, o.out_eid, h->tri_ptr, h->tri_w,
-                                              kptr, nullptr, nullptr, derr);
-        ND_CUDA(cudaGetLastError());
-    }
-    ND_TRY(nd_scan_i64(kptr, T, st));
-    int64_t K = 0;
-    ND_TRY(read_i64(h, kptr.p + T, &K, st));
-    nd_tmp<uint4> k4(st);
-    ND_TRY(k4.alloc(K));
-    if (K > 0) {
-        nd_prof_scope ps("k4_list", st);
-        k_k4<1><<<tblocks, kThreads, 0, st>>>(T, tris, o.out_ptr, o.out_col, o.out_eid, h->tri_ptr, h->tri_w,
-                                              kptr, k4, (unsigned long long*)h->inc_ptr, derr);
+        k_k4_rows<false, false><<<tblocks, kThreads, 0, st>>>(T, te, lptr, lw, lid, h->inc_ptr, nullptr);
         ND_CUDA(cudaGetLastError());
     }
     ND_TRY(nd_scan_i64(h->inc_ptr, T, st));
-    ND_TRY(fetch(h, 0, h->inc_ptr + T, 1, st));
-    ND_CUDA(cudaMemcpyAsync(h->h_read + 1, derr, sizeof(int), cudaMemcpyDeviceToHost, st));
-    ND_TRY(nd_wait(st));
-    h->num_inc = h->h_read[0];
-    if (*(const int*)(h->h_read + 1)) {
-        nd_set_error("internal: a triangle of a 4-clique was not found");
-        return ND_E_INVAL;
-    }
+    ND_TRY(read_i64(h, h->inc_ptr + T, &h->num_inc, st));
+    const bool slots = list_layout_fits(h, T, h->num_inc);
     ND_TRY(nd_alloc((void**)&h->inc, sizeof(uint32_t) * 3 * (h->num_inc > 0 ? h->num_inc : 1), st, h));
-    if (K > 0) {
+    if (h->num_inc > 0) {
         nd_prof_scope ps("k4_fill", st);
-        const int kb = nd_blocks_for(K, kThreads, grid_cap(h) * 4);
-        if (h->num_inc < (int64_t)UINT32_MAX) {  // 32-bit slot atomics
-            nd_tmp<unsigned> cursor(st);
-            ND_TRY(cursor.alloc(T));
-            k_narrow_u32<<<nd_blocks_for(T, kThreads, grid_cap(h) * 4), kThreads, 0, st>>>(T, h->inc_ptr, cursor);
-            ND_CUDA(cudaGetLastError());
-            k_k4_scatter<unsigned><<<kb, kThreads, 0, st>>>(K, k4, cursor.p, h->inc);
-        } else {
-            nd_tmp<unsigned long long> cursor(st);
-            ND_TRY(cursor.alloc(T));
-            ND_CUDA(cudaMemcpyAsync(cursor, h->inc_ptr, sizeof(int64_t) * T, cudaMemcpyDeviceToDevice, st));
-            k_k4_scatter<unsigned long long><<<kb, kThreads, 0, st>>>(K, k4, cursor.p, h->inc);
-        }
+        auto fill = slots ? k_k4_rows<true, false> : k_k4_rows<true, true>;
+        fill<<<tblocks, kThreads, 0, st>>>(T, te, lptr, lw, lid, h->inc_ptr, h->inc);
         ND_CUDA(cudaGetLastError());
+    }
+    if (slots) {
+        h->t_pos = t_pos.take();
+        h->t_id = lid.take();
+        h->bytes += (int64_t)sizeof(uint32_t) * 6 * T;
     }
     return ND_OK;
 }

@@ -38,7 +38,8 @@
 //
 // (2,3) uses the adjacency layout: incidence entries are the CSR slots of
 // the other two edges, the gathers read a 16-bit copy of tau indexed by CSR
-// slot, and the frontier has one bit per slot.  k_pass_otf is the same update
+// slot, and the frontier has one bit per slot.  (3,4) does the same with the
+// slots of the edges' triangle lists, three per triangle.  k_pass_otf is the same update
 // with no stored incidence: it finds each edge's triangles again by
 // intersecting adjacency lists on every pass.
 #include "nd_internal.cuh"
@@ -81,6 +82,18 @@ constexpr int kHistWords = 256;
 constexpr int kLateHistWords = 128;
 static_assert(kHistWords % 128 == 0 && kLateHistWords % 128 == 0, "cleared and selected in blocks of 128 words");
 
+// The kinds of incidence rows a pass kernel is built for: Q = 1, 2, 3 for
+// (1,2), (2,3) and (3,4) in the layouts above; kIds for a (3,4) handle whose
+// entries are triangle ids.
+constexpr int kIds = 4;
+// ids per entry; (3,4) rows hold them as three runs of d words, so that a warp
+// loads 32 entries with three coalesced loads
+template <int Q>
+constexpr int kWords = Q == kIds ? 3 : Q;
+// are the ids slots?
+template <int Q>
+constexpr bool kSlots = Q == 2 || Q == 3;
+
 // Work of one pass: rows longer than the CTA threshold are taken one per
 // block from a per-pass counter; all other rows form warp tasks that warps
 // take in chunks from a second counter.
@@ -91,13 +104,14 @@ struct SweepParams {
     int32_t* tout;
     // gathers: a copy of tau in 16 bits saturated at 65535, exact for every
     // row with tau(R) <= 65535 (the row only looks at min(rho, tau(R))); a
-    // row above that (a CTA row) gathers tin.  Indexed by CSR position for
-    // (2,3), where an updated edge writes both of its entries (e_pos), and by
-    // vertex for (1,2); (3,4) gathers tin.
+    // row above that (a CTA row) gathers tin.  Indexed by slot for (2,3) and
+    // (3,4), where an updated r-clique writes all of its slots (epos, tpos), and
+    // by vertex for (1,2); kIds gathers tin.
     const uint16_t* gin;
     uint16_t* gout;
-    const uint2* __restrict__ epos;
-    const uint32_t* __restrict__ eid;  // CSR position -> edge id (notification)
+    const uint2* __restrict__ epos;     // (2,3): the two slots of an edge
+    const uint32_t* __restrict__ tpos;  // (3,4): the three slots of a triangle
+    const uint32_t* __restrict__ eid;   // slot -> r-clique
     // (2,3) without a stored incidence: the graph and the edge endpoints
     const int64_t* __restrict__ rp;
     const int32_t* __restrict__ col;
@@ -165,6 +179,7 @@ __device__ __forceinline__ uint32_t ld_id(const uint32_t* p) {
 template <int Q, bool RO, typename T>
 struct Rho {
     const uint32_t* __restrict__ row;
+    int d;  // (3,4): the length of the row's runs
     const T* tau;
     __device__ __forceinline__ int32_t operator()(int j) const {
         if constexpr (Q == 1) {
@@ -174,36 +189,47 @@ struct Rho {
             const uint2 id = RO ? __ldcs(p) : __ldg(p);
             return min(ld_tau<RO>(tau + id.x), ld_tau<RO>(tau + id.y));
         } else {
-            const uint32_t* p = row + 3 * (int64_t)j;
-            const uint32_t a = ld_id<RO>(p), b = ld_id<RO>(p + 1), c = ld_id<RO>(p + 2);
+            const uint32_t* p = row + j;
+            const uint32_t a = ld_id<RO>(p), b = ld_id<RO>(p + d), c = ld_id<RO>(p + 2 * (int64_t)d);
             return min(min(ld_tau<RO>(tau + a), ld_tau<RO>(tau + b)), ld_tau<RO>(tau + c));
         }
     }
 };
 
-// (2,3) rows with tau(R) > 65535 (so d_s > 65535, CTA rows): exact values,
-// CSR position -> edge id -> tau
-template <bool RO>
-struct RhoExact2 {
+// rows of slots with tau(R) > 65535 (so d_s > 65535, CTA rows): exact values,
+// slot -> r-clique -> tau
+template <int Q, bool RO>
+struct RhoExact {
     const uint32_t* __restrict__ row;
+    int d;
     const uint32_t* __restrict__ eid;
     const int32_t* tau;
     __device__ __forceinline__ int32_t operator()(int j) const {
-        const uint2 id = __ldg(reinterpret_cast<const uint2*>(row) + j);
-        return min(ld_tau<RO>(tau + __ldg(eid + id.x)), ld_tau<RO>(tau + __ldg(eid + id.y)));
+        if constexpr (Q == 2) {
+            const uint2 id = __ldg(reinterpret_cast<const uint2*>(row) + j);
+            return min(ld_tau<RO>(tau + __ldg(eid + id.x)), ld_tau<RO>(tau + __ldg(eid + id.y)));
+        } else {
+            const uint32_t* p = row + j;
+            return min(min(ld_tau<RO>(tau + __ldg(eid + __ldg(p))), ld_tau<RO>(tau + __ldg(eid + __ldg(p + d)))),
+                       ld_tau<RO>(tau + __ldg(eid + __ldg(p + 2 * (int64_t)d))));
+        }
     }
 };
 
 constexpr int32_t kTau16Max = 65535;
 
-// the gather of a row whose tau is at most 65535: the 16-bit copy for (1,2)
-// and (2,3).  (3,4) gathers int32 tau directly: its rows are not ordered, and
-// the 16-bit copy measured 3% slower there (Chung-Lu 100K (3,4) with planted
-// cliques) against 6% faster for a scale-24 k-core.
+// the row of a work item
+template <int Q>
+__device__ __forceinline__ const uint32_t* row_of(const SweepParams& P, int64_t jb) {
+    return P.inc + kWords<Q> * jb;
+}
+
+// the gather of a row whose tau is at most 65535: the 16-bit copy, or the
+// int32 values where entries are r-clique ids in no order (kIds)
 template <int Q, bool RO>
-__device__ __forceinline__ auto make_rho(const SweepParams& P, int64_t jb) {
-    if constexpr (Q == 3) return Rho<3, RO, int32_t>{P.inc + 3 * jb, P.tin};
-    else return Rho<Q, RO, uint16_t>{P.inc + Q * jb, P.gin};
+__device__ __forceinline__ auto make_rho(const SweepParams& P, int64_t jb, uint32_t d) {
+    if constexpr (Q == kIds) return Rho<3, RO, int32_t>{row_of<Q>(P, jb), (int)d, P.tin};
+    else return Rho<Q, RO, uint16_t>{row_of<Q>(P, jb), (int)d, P.gin};
 }
 
 // What a row's order says about the entries that are still to come.  Rows of a
@@ -513,7 +539,7 @@ __device__ __forceinline__ int32_t cta_hindex(const F& rho, const B& bound, int 
     }
 }
 
-// the new tau of R; (2,3) also writes it to both CSR entries of the edge.
+// the new tau of R, also written to all of its slots.
 // SND writes the buffer of two passes ago: where that holds h already (old),
 // all its copies do, and nothing is written.
 template <int Q>
@@ -525,13 +551,16 @@ __device__ __forceinline__ void store_tau(const SweepParams& P, uint32_t R, int3
         const uint2 ep = __ldg(P.epos + R);
         P.gout[ep.x] = v;
         P.gout[ep.y] = v;
+    } else if (Q == 3) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) P.gout[__ldg(P.tpos + 3 * (int64_t)R + k)] = v;
     } else if (Q == 1) {
         P.gout[R] = v;
     }
 }
 
-// (2,3): notify the edge at CSR position pos, whose tau read from the
-// 16-bit copy is tv, if h <= tau (the exact int32 value when h > 65535).
+// notify the r-clique at slot pos, whose tau read from the 16-bit copy is tv,
+// if h <= tau (the exact int32 value when h > 65535).
 // The caller has just seen its frontier bit clear, with a relaxed L2 read:
 // a bit set meanwhile only costs a redundant atomic, and a set bit is never
 // cleared within a pass.
@@ -551,116 +580,108 @@ __device__ __forceinline__ void notify_pos(const SweepParams& P, uint32_t pos, i
     notify_clear(P, pos, h, ld_tau<false>(P.gin + pos));
 }
 
-// is R in the current frontier?  (2,3): either bit of its two CSR positions
+__device__ __forceinline__ unsigned front_bit(const uint32_t* f, uint32_t i) {
+    return (__ldg(f + (i >> 5)) >> (i & 31)) & 1u;
+}
+
+// is R in the current frontier?  With slots: any bit of its slots
 template <int Q>
 __device__ __forceinline__ bool in_frontier(const SweepParams& P, uint32_t R) {
     if constexpr (Q == 2) {
         const uint2 ep = __ldg(P.epos + R);
-        return ((__ldg(P.cur + (ep.x >> 5)) >> (ep.x & 31)) & 1u) | ((__ldg(P.cur + (ep.y >> 5)) >> (ep.y & 31)) & 1u);
+        return front_bit(P.cur, ep.x) | front_bit(P.cur, ep.y);
+    } else if constexpr (Q == 3) {
+        const uint32_t* p = P.tpos + 3 * (int64_t)R;
+        const uint32_t a = __ldg(p), b = __ldg(p + 1), c = __ldg(p + 2);
+        return front_bit(P.cur, a) | front_bit(P.cur, b) | front_bit(P.cur, c);
     } else {
-        return (__ldg(P.cur + (R >> 5)) >> (R & 31)) & 1u;
+        return front_bit(P.cur, R);
+    }
+}
+
+// the ids of entry j of a row of d entries
+template <int Q>
+__device__ __forceinline__ void entry_ids(const uint32_t* __restrict__ row, uint32_t d, int64_t j,
+                                          uint32_t (&id)[kWords<Q>]) {
+    if constexpr (Q == 2) {
+        const uint2 x = __ldg(reinterpret_cast<const uint2*>(row) + j);
+        id[0] = x.x;
+        id[1] = x.y;
+    } else {
+#pragma unroll
+        for (int k = 0; k < kWords<Q>; ++k) id[k] = __ldg(row + j + k * (int64_t)d);
+    }
+}
+
+// one neighbour whose next-frontier word has been read as wd: set its bit if
+// it is clear and h <= tau.  A neighbour whose bit is already set needs
+// nothing, so the word (2 MB for 16M r-cliques, cache-resident) is read before
+// its tau, and an atomic is only issued for a bit that is still clear.
+// (Warp-wide merging of bits that share a word was measured slower: the match
+// runs for every neighbour, while most neighbours need no write.)
+template <int Q>
+__device__ __forceinline__ void notify_one(const SweepParams& P, uint32_t id, uint32_t wd, int32_t h) {
+    const uint32_t bit = 1u << (id & 31);
+    if (wd & bit) return;  // already active (or past the row's end)
+    if constexpr (kSlots<Q>) {
+        notify_clear(P, id, h, ld_tau<false>(P.gin + id));
+    } else {
+        if (P.members && !(__ldg(P.members + (id >> 5)) & bit)) return;  // PartialAnd
+        if (h <= ld_tau<false>(P.tin + id)) atomicOr(P.next + (id >> 5), bit);
     }
 }
 
 // notify every neighbour whose tau could still depend on R (Alg. 3, orange
-// lines): set its next-frontier bit if h <= tau(R').  A neighbour whose bit
-// is already set needs nothing, so the bitmap word (2 MB for 16M r-cliques,
-// cache-resident) is read before the neighbour's tau, and an atomic is only
-// issued for a bit that is still clear.  (Warp-wide merging of bits that
-// share a word was measured slower: the match runs for every neighbour,
-// while most neighbours need no write.)
+// lines): set its next-frontier bit if h <= tau(R').  With slots there is one
+// bit per slot, so the test reads the 16-bit copy and the bit sits next to it
+// (no r-clique id on this path).  U entries per lane and their bit words are
+// loaded before any is tested, so their latencies overlap.
 template <int Q>
-__device__ __forceinline__ void notify_row(const SweepParams& P, int64_t jb, int64_t je, int32_t h,
-                                           int first, int step) {
-    if constexpr (Q == 2) {
-        // (2,3): the entries are CSR positions; the frontier has one bit per
-        // position, so the test reads the 16-bit copy and the bit sits next
-        // to it (no edge id on this path).  kNotifyUnroll entries per lane
-        // are loaded before any is tested, so their latencies overlap.
-        const uint2* pairs = reinterpret_cast<const uint2*>(P.inc);
-        for (int64_t j0 = jb + first; j0 < je; j0 += (int64_t)kNotifyUnroll * step) {
-            uint2 id[kNotifyUnroll];
-            uint32_t wx[kNotifyUnroll], wy[kNotifyUnroll];
+__device__ __forceinline__ void notify_row(const SweepParams& P, const uint32_t* __restrict__ row, uint32_t d,
+                                           int32_t h, int first, int step) {
+    constexpr int W = kWords<Q>;
+    constexpr int U = W == 3 ? 2 : kNotifyUnroll;
+    // a relabelled (1,2) row: from this id on every tau is below h
+    const uint32_t limit = Q == 1 && P.oct_max ? id_limit(P.oct_max, h) : 0xffffffffu;
+    for (int64_t j0 = first; j0 < d; j0 += (int64_t)U * step) {
+        uint32_t id[U][W], wd[U][W];
 #pragma unroll
-            for (int u = 0; u < kNotifyUnroll; ++u) {
-                const int64_t j = j0 + (int64_t)u * step;
-                id[u] = j < je ? __ldg(pairs + j) : make_uint2(0u, 0u);
-            }
-            // the frontier words first: a neighbour whose bit is already set
-            // needs neither its tau nor an atomic
+        for (int u = 0; u < U; ++u) {
+            const int64_t j = j0 + (int64_t)u * step;
+            if (j < d) {
+                entry_ids<Q>(row, d, j, id[u]);
+            } else {
 #pragma unroll
-            for (int u = 0; u < kNotifyUnroll; ++u) {
-                const bool ok = j0 + (int64_t)u * step < je;
-                wx[u] = ok ? ld_front(P.next + (id[u].x >> 5)) : 0xffffffffu;
-                wy[u] = ok ? ld_front(P.next + (id[u].y >> 5)) : 0xffffffffu;
-            }
-#pragma unroll
-            for (int u = 0; u < kNotifyUnroll; ++u) {
-                if (!((wx[u] >> (id[u].x & 31)) & 1u)) notify_clear(P, id[u].x, h, ld_tau<false>(P.gin + id[u].x));
-                if (!((wy[u] >> (id[u].y & 31)) & 1u)) notify_clear(P, id[u].y, h, ld_tau<false>(P.gin + id[u].y));
+                for (int k = 0; k < W; ++k) id[u][k] = 0u;
             }
         }
-    } else {
-        // (1,2), (3,4): ids of r-cliques; the same overlap, kNotifyUnroll
-        // entries (Q ids each) and their bit words loaded before any test
-        constexpr int U = Q == 1 ? kNotifyUnroll : 2;
-        // a relabelled (1,2) row: from this id on every tau is below h
-        const uint32_t limit = Q == 1 && P.oct_max ? id_limit(P.oct_max, h) : 0xffffffffu;
-        for (int64_t j0 = jb + first; j0 < je; j0 += (int64_t)U * step) {
-            uint32_t id[U][Q], wd[U][Q];
+        if (Q == 1 && id[0][0] >= limit) break;  // so are this lane's later entries
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int64_t j = j0 + (int64_t)u * step;
+        for (int u = 0; u < U; ++u) {
+            const bool ok = j0 + (int64_t)u * step < d && (Q != 1 || id[u][0] < limit);
 #pragma unroll
-                for (int k = 0; k < Q; ++k) id[u][k] = j < je ? __ldg(P.inc + Q * j + k) : 0u;
-            }
-            if (Q == 1 && id[0][0] >= limit) break;  // so are this lane's later entries
+            for (int k = 0; k < W; ++k) wd[u][k] = ok ? ld_front(P.next + (id[u][k] >> 5)) : 0xffffffffu;
+        }
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const bool ok = j0 + (int64_t)u * step < je && (Q != 1 || id[u][0] < limit);
+        for (int u = 0; u < U; ++u) {
 #pragma unroll
-                for (int k = 0; k < Q; ++k) wd[u][k] = ok ? ld_front(P.next + (id[u][k] >> 5)) : 0xffffffffu;
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-#pragma unroll
-                for (int k = 0; k < Q; ++k) {
-                    const uint32_t Rp = id[u][k];
-                    const uint32_t bit = 1u << (Rp & 31);
-                    if (wd[u][k] & bit) continue;  // already active (or past the row's end)
-                    if (P.members && !(__ldg(P.members + (Rp >> 5)) & bit)) continue;  // PartialAnd
-                    if (h <= ld_tau<false>(P.tin + Rp)) atomicOr(P.next + (Rp >> 5), bit);
-                }
-            }
+            for (int k = 0; k < W; ++k) notify_one<Q>(P, id[u][k], wd[u][k], h);
         }
     }
 }
 
-// notification for one incidence entry j of a row whose tau dropped to h:
-// the same test as notify_row, for a single entry (the merged walk of group
-// rows below gives each lane entries of different rows)
+// notification for one entry j of a row whose tau dropped to h: the same
+// test as notify_row, for a single entry (the merged walk of group rows below
+// gives each lane entries of different rows)
 template <int Q>
-__device__ __forceinline__ void notify_entry(const SweepParams& P, int64_t j, int32_t h) {
-    if constexpr (Q == 2) {
-        const uint2 id = __ldg(reinterpret_cast<const uint2*>(P.inc) + j);
-        const uint32_t wx = ld_front(P.next + (id.x >> 5)), wy = ld_front(P.next + (id.y >> 5));
-        if (!((wx >> (id.x & 31)) & 1u)) notify_clear(P, id.x, h, ld_tau<false>(P.gin + id.x));
-        if (!((wy >> (id.y & 31)) & 1u)) notify_clear(P, id.y, h, ld_tau<false>(P.gin + id.y));
-    } else {
-        uint32_t id[Q], wd[Q];
+__device__ __forceinline__ void notify_entry(const SweepParams& P, int64_t jb, uint32_t d, int j, int32_t h) {
+    constexpr int W = kWords<Q>;
+    uint32_t id[W], wd[W];
+    entry_ids<Q>(row_of<Q>(P, jb), d, j, id);
 #pragma unroll
-        for (int k = 0; k < Q; ++k) id[k] = __ldg(P.inc + Q * j + k);
+    for (int k = 0; k < W; ++k) wd[k] = ld_front(P.next + (id[k] >> 5));
 #pragma unroll
-        for (int k = 0; k < Q; ++k) wd[k] = ld_front(P.next + (id[k] >> 5));
-#pragma unroll
-        for (int k = 0; k < Q; ++k) {
-            const uint32_t Rp = id[k];
-            const uint32_t bit = 1u << (Rp & 31);
-            if (wd[k] & bit) continue;
-            if (P.members && !(__ldg(P.members + (Rp >> 5)) & bit)) continue;  // PartialAnd
-            if (h <= ld_tau<false>(P.tin + Rp)) atomicOr(P.next + (Rp >> 5), bit);
-        }
-    }
+    for (int k = 0; k < W; ++k) notify_one<Q>(P, id[k], wd[k], h);
 }
 
 // batches (GB): has R's graph converged (no change in its previous pass)?
@@ -727,7 +748,7 @@ __device__ __forceinline__ void run_groups(const SweepParams& P, int64_t first, 
     const int d = run ? (int)it.d : 0;
     if (!run) t = 0;
     const int dmax = (int)__reduce_max_sync(0xffffffffu, (unsigned)d);
-    const int32_t h = group_hindex<G, C>(make_rho<Q, !AND>(P, it.jb), d, dmax, t);
+    const int32_t h = group_hindex<G, C>(make_rho<Q, !AND>(P, it.jb, it.d), d, dmax, t);
     if (run && (threadIdx.x & (G - 1)) == 0) {
         n.row(it.d, h != t0);
         if (h != t0) graph_changed<GB>(P, it.R);
@@ -746,18 +767,18 @@ __device__ __forceinline__ void run_warp_row(const SweepParams& P, const nd_item
     const bool direct = P.direct || (!AND && old != t0);
     int32_t h;
     if (Q == 1 && P.oct_max)
-        h = warp_hindex<true, HW>(make_rho<Q, !AND>(P, it.jb),
+        h = warp_hindex<true, HW>(make_rho<Q, !AND>(P, it.jb, it.d),
                                   IdBound{P.inc + it.jb, P.oct_max, direct ? 0u : id_limit(P.oct_max, t)}, (int)it.d, t,
                                   direct, bins);
     else
-        h = warp_hindex<true, HW>(make_rho<Q, !AND>(P, it.jb), NoBound{}, (int)it.d, t, direct, bins);
+        h = warp_hindex<true, HW>(make_rho<Q, !AND>(P, it.jb, it.d), NoBound{}, (int)it.d, t, direct, bins);
     const int lane = threadIdx.x & 31;
     if (lane == 0) {
         n.row(it.d, h != t0);
         if (h != t0) graph_changed<GB>(P, R);
         store_tau<Q>(P, R, h, old);
     }
-    if (AND && NOTIFY && h != t0) notify_row<Q>(P, it.jb, it.jb + it.d, h, lane, 32);
+    if (AND && NOTIFY && h != t0) notify_row<Q>(P, row_of<Q>(P, it.jb), it.d, h, lane, 32);
     __syncwarp();  // the bins are free again
 }
 
@@ -775,22 +796,24 @@ __device__ __forceinline__ void run_cta(const SweepParams& P, int64_t i, unsigne
     const int d = (int)it.d;
     const bool direct = P.direct || (!AND && old != t0);
     int32_t h;
-    if (Q == 2 && t > kTau16Max) {  // only then can a saturated value matter
-        h = cta_hindex<WORDS>(RhoExact2<!AND>{P.inc + 2 * it.jb, P.eid, P.tin}, NoBound{}, d, t, direct, bins, bounds);
+    if (kSlots<Q> && t > kTau16Max) {  // only then can a saturated value matter
+        h = cta_hindex<WORDS>(RhoExact<Q, !AND>{row_of<Q>(P, it.jb), d, P.eid, P.tin}, NoBound{}, d, t, direct, bins,
+                              bounds);
     } else if (Q == 1 && t > kTau16Max) {
-        h = cta_hindex<WORDS>(Rho<Q, !AND, int32_t>{P.inc + it.jb, P.tin}, NoBound{}, d, t, direct, bins, bounds);
+        h = cta_hindex<WORDS>(Rho<1, !AND, int32_t>{row_of<Q>(P, it.jb), d, P.tin}, NoBound{}, d, t, direct, bins,
+                              bounds);
     } else if (Q == 1 && P.oct_max) {
         const IdBound bound{P.inc + it.jb, P.oct_max, id_limit(P.oct_max, t)};
-        h = cta_hindex<WORDS>(make_rho<Q, !AND>(P, it.jb), bound, d, t, direct, bins, bounds);
+        h = cta_hindex<WORDS>(make_rho<Q, !AND>(P, it.jb, it.d), bound, d, t, direct, bins, bounds);
     } else {
-        h = cta_hindex<WORDS>(make_rho<Q, !AND>(P, it.jb), NoBound{}, d, t, direct, bins, bounds);
+        h = cta_hindex<WORDS>(make_rho<Q, !AND>(P, it.jb, it.d), NoBound{}, d, t, direct, bins, bounds);
     }
     if (threadIdx.x == 0) {
         n.row(it.d, h != t0);
         if (h != t0) graph_changed<GB>(P, R);
         store_tau<Q>(P, R, h, old);
     }
-    if (AND && NOTIFY && h != t0) notify_row<Q>(P, it.jb, it.jb + d, h, threadIdx.x, kThreads);
+    if (AND && NOTIFY && h != t0) notify_row<Q>(P, row_of<Q>(P, it.jb), it.d, h, threadIdx.x, kThreads);
     __syncthreads();
 }
 
@@ -821,6 +844,20 @@ __device__ __forceinline__ void active_masks(const SweepParams& P, int64_t a, in
 #pragma unroll
         for (int w = 0; w < W; ++w)
             mask[w] = __ballot_sync(0xffffffffu, ok[w] && (((bx[w] >> (ep[w].x & 31)) | (by[w] >> (ep[w].y & 31))) & 1u));
+    } else if constexpr (Q == 3) {
+        uint32_t tp[W][3], bits[W];
+#pragma unroll
+        for (int w = 0; w < W; ++w)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) tp[w][k] = ok[w] ? __ldg(P.tpos + 3 * (int64_t)R[w] + k) : 0u;
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+            bits[w] = 0;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) bits[w] |= front_bit(P.cur, tp[w][k]);
+        }
+#pragma unroll
+        for (int w = 0; w < W; ++w) mask[w] = __ballot_sync(0xffffffffu, ok[w] && bits[w]);
     } else {
         uint32_t bw[W];
 #pragma unroll
@@ -870,7 +907,7 @@ __device__ __forceinline__ void run_groups_active(const SweepParams& P, int64_t 
         const int d = run ? (int)it.d : 0;
         if (!run) t = 0;
         const int dmax = (int)__reduce_max_sync(0xffffffffu, (unsigned)d);
-        const int32_t h = group_hindex<G, C>(make_rho<Q, false>(P, jb), d, dmax, t);
+        const int32_t h = group_hindex<G, C>(make_rho<Q, false>(P, jb, it.d), d, dmax, t);
         if (run && (lane & (G - 1)) == 0) {
             n.row(it.d, h != t0);
             store_tau<Q>(P, it.R, h, old);
@@ -882,18 +919,18 @@ __device__ __forceinline__ void run_groups_active(const SweepParams& P, int64_t 
         for (int q = 0; q < NG; ++q) tot += __shfl_sync(0xffffffffu, dn, q * G);
         for (int e0 = 0; e0 < tot; e0 += 32) {
             const int e = e0 + lane;
-            int64_t j = 0;
-            int32_t hh = 0;
-            int run = 0;
+            int64_t jr = 0;  // the row of entry e, its length and its own number there
+            int32_t hh = 0, dr = 0;
+            int j = 0, run = 0;
 #pragma unroll
             for (int q = 0; q < NG; ++q) {
                 const int v = __shfl_sync(0xffffffffu, dn, q * G);
                 const int64_t jq = __shfl_sync(0xffffffffu, jb, q * G);
                 const int32_t hq = __shfl_sync(0xffffffffu, h, q * G);
-                if (e >= run && e < run + v) { j = jq + (e - run); hh = hq; }
+                if (e >= run && e < run + v) { jr = jq; dr = v; j = e - run; hh = hq; }
                 run += v;
             }
-            if (e < tot) notify_entry<Q>(P, j, hh);
+            if (e < tot) notify_entry<Q>(P, jr, (uint32_t)dr, j, hh);
         }
     }
 }
@@ -1082,7 +1119,19 @@ __global__ void k_tau_to_adj(int64_t N, const uint2* __restrict__ epos, const in
     }
 }
 
-// tau -> its 16-bit gather copies indexed by r-clique id ((1,2), (3,4))
+// the same for the three list slots of every triangle
+__global__ void k_tau_to_lists(int64_t N, const uint32_t* __restrict__ tpos, const int32_t* __restrict__ tau,
+                               uint16_t* __restrict__ a, uint16_t* __restrict__ b) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < 3 * N;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t p = tpos[i];
+        const uint16_t v = (uint16_t)min(max(tau[i / 3], 0), kTau16Max);
+        a[p] = v;
+        if (b) b[p] = v;
+    }
+}
+
+// tau -> its 16-bit gather copies indexed by r-clique id ((1,2))
 __global__ void k_tau_to_16(int64_t N, const int32_t* __restrict__ tau, uint16_t* __restrict__ a,
                             uint16_t* __restrict__ b) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N;
@@ -1102,6 +1151,19 @@ __global__ void k_member_pos(int64_t N, const uint32_t* __restrict__ members, co
         const uint2 ep = epos[i];
         atomicOr(f + (ep.x >> 5), 1u << (ep.x & 31));
         atomicOr(f + (ep.y >> 5), 1u << (ep.y & 31));
+    }
+}
+
+// and with the (3,4) layout: the three list slots of every member
+__global__ void k_member_lists(int64_t N, const uint32_t* __restrict__ members, const uint32_t* __restrict__ tpos,
+                               uint32_t* __restrict__ f) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        if (!((members[i >> 5] >> (i & 31)) & 1u)) continue;
+        for (int k = 0; k < 3; ++k) {
+            const uint32_t p = tpos[3 * i + k];
+            atomicOr(f + (p >> 5), 1u << (p & 31));
+        }
     }
 }
 
@@ -1158,10 +1220,8 @@ __global__ void k_add_const(const int32_t* __restrict__ in, int64_t n, int32_t c
 //    shorter list is walked by degree class, high first: the w of high degree
 //    close most triangles and hold the largest tau, and past a class no tau
 //    exceeds its degrees (DegreeBound).
-//  - Otherwise, where the lists are of like length (kMergeRatio), blocks of 128
-//    entries of the longer one pass through shared memory, each loaded once
-//    per sweep, and a lane searches its w there;
-//  - otherwise every lane searches the rest of the longer list.
+//  - Otherwise blocks of the longer list pass through shared memory, or, where
+//    it is much longer, every lane searches it (nd_list_cursor).
 // A search of the whole list per entry (the only way before) takes some 250 L1
 // wavefronts per 32 entries of a list of 4,000, because its lanes part after
 // the first steps.  The blocks alone were little faster: about 150 instructions
@@ -1169,35 +1229,17 @@ __global__ void k_add_const(const int32_t* __restrict__ in, int64_t n, int32_t c
 // (33.4M incidences, 101 passes): 109 ms with searches, 95 with blocks, 45 with
 // tables, 34 with the lists by degree class (late passes 0.31 ms; 0.43 in CSR
 // order).
-constexpr int kMergeRatio = 16;
-constexpr int kOtfBlock = 128;
-
 template <bool RO, bool EXACT>
 struct OtfRow {
     const int32_t* __restrict__ scol;   // N(s), sn entries: in CSR order from slot sb, or
     const uint32_t* __restrict__ slot;  // with a table, by degree class, and their slots
-    const int32_t* __restrict__ lcol;  // N(l), ln entries from CSR slot lb
-    int64_t sb, lb;
-    int sn, ln;
+    int64_t sb, lb;  // first slots of N(s) and of the longer list N(l)
+    int sn;
     const uint2* __restrict__ table;  // of the longer list's vertex, or null
-    int32_t* buf;  // kOtfBlock words of the warp
     const uint16_t* tau16;
     const uint32_t* __restrict__ eid;
     const int32_t* tau32;
-    mutable int at;   // merging: the block in buf starts here; searching: no earlier entry can match
-    mutable int last;  // merging: the largest vertex in buf
-
-    __device__ __forceinline__ void load_block() const {
-        const int lane = threadIdx.x & 31;
-        __syncwarp();
-#pragma unroll
-        for (int u = 0; u < kOtfBlock / 32; ++u) {
-            const int k = at + 32 * u + lane;
-            buf[32 * u + lane] = k < ln ? __ldg(lcol + k) : INT32_MAX;
-        }
-        __syncwarp();
-        last = buf[kOtfBlock - 1];
-    }
+    mutable nd_list_cursor longer;
 
     // the entry of w in the longer list, -1 if it is none
     static __device__ __forceinline__ int at_table(uint2 x, int32_t w) {
@@ -1232,39 +1274,11 @@ struct OtfRow {
             }
             return;
         }
-        const bool merge = ln <= kMergeRatio * (int64_t)sn;
-        if (i == 0) {
-            at = 0;
-            if (merge) load_block();
-        }
+        if (i == 0) longer.restart(sn);
         for (; i < end; i += 32) {
             const int j = i + lane;
-            const int32_t w = j < end ? __ldg(scol + j) : INT32_MAX;
-            int k = -1;
-            if (merge) {
-                const int32_t top = __reduce_max_sync(0xffffffffu, j < end ? w : 0);
-                bool open = j < end;
-                for (;;) {
-                    if (open && w <= last) {
-                        int lo = 0;  // entries of the block below w
-#pragma unroll
-                        for (int h = kOtfBlock / 2; h > 0; h >>= 1) lo += buf[lo + h - 1] < w ? h : 0;
-                        if (buf[lo] == w) k = at + lo;
-                        open = false;
-                    }
-                    if (top <= last || at + kOtfBlock >= ln) break;
-                    at += kOtfBlock;
-                    load_block();
-                }
-            } else {
-                int p = ln;
-                if (j < end) {
-                    p = at + nd_lower_bound_n(lcol + at, ln - at, w);
-                    if (p < ln && __ldg(lcol + p) == w) k = p;
-                }
-                at = __shfl_sync(0xffffffffu, p, min(end - i, 32) - 1);
-            }
-            f(j, k);
+            const int32_t w = j < end ? __ldg(scol + j) : 0;
+            f(j, longer.find(w, j < end, __reduce_max_sync(0xffffffffu, w)));
         }
     }
     __device__ __forceinline__ int32_t rho(int j, int k) const {
@@ -1278,7 +1292,6 @@ struct OtfRow {
 // a list by degree class: past an entry of degree d, no edge to a later entry
 // has a tau above the largest degree of d's class, less one
 struct DegreeBound {
-    static constexpr bool kOn = true;
     const int32_t* __restrict__ scol;  // null: the list is in another order
     const int64_t* __restrict__ rp;
     int32_t t;
@@ -1307,7 +1320,7 @@ template <bool AND, bool NOTIFY>
 __global__ void __launch_bounds__(kThreads, kPassBlocks) k_pass_otf(SweepParams P) {
     if (P.prev != nullptr && *(volatile const unsigned long long*)P.prev == 0ull) return;  // converged
     __shared__ __align__(16) unsigned hist[kThreads / 32][kHistWords];
-    __shared__ int32_t blocks[kThreads / 32][kOtfBlock];
+    __shared__ int32_t blocks[kThreads / 32][nd_list_cursor::kBlock];
     Tally<true> n;
     const int lane = threadIdx.x & 31;
     unsigned* const bins = hist[threadIdx.x >> 5];
@@ -1367,11 +1380,11 @@ __global__ void __launch_bounds__(kThreads, kPassBlocks) k_pass_otf(SweepParams 
             const uint2* const table = hub >= 0 ? P.hub_bits + hub * P.hub_words : nullptr;
             const int32_t* const scol = (table && P.by_degree ? P.by_degree : P.col) + sb;
             const uint32_t* const slot = table && P.by_degree ? P.slot_of + sb : nullptr;
-            const OtfRow<!AND, false> row{scol, slot, P.col + lb, sb, lb, sn, ln, table, buf, P.gin, P.eid, P.tin, 0, 0};
+            const nd_list_cursor longer{P.col + lb, ln, buf, false, 0, 0};
+            const OtfRow<!AND, false> row{scol, slot, sb, lb, sn, table, P.gin, P.eid, P.tin, longer};
             int32_t h;
             if (t > kTau16Max) {
-                const OtfRow<!AND, true> exact{scol, slot, P.col + lb, sb, lb, sn, ln, table, buf,
-                                               P.gin, P.eid, P.tin, 0, 0};
+                const OtfRow<!AND, true> exact{scol, slot, sb, lb, sn, table, P.gin, P.eid, P.tin, longer};
                 h = warp_hindex<false, kHistWords>(exact, NoBound{}, sn, t, direct, bins);
             } else {
                 h = warp_hindex<false, kHistWords>(row, DegreeBound{slot && P.bounded ? scol : nullptr, P.rp, t}, sn, t,
@@ -1395,7 +1408,7 @@ __global__ void __launch_bounds__(kThreads, kPassBlocks) k_pass_otf(SweepParams 
                     if (bound.past(i)) break;  // no later edge has a tau of h or more
                 }
             }
-            __syncwarp();  // the bins and the block are free again
+            __syncwarp();  // the bins and the block of the list are free again
         }
     }
     flush_tally(P, n);
@@ -1471,7 +1484,9 @@ pass_fn pick(const nd_incidence* h, int mode, bool late) {
     // mode: ND_SND, ND_AND (notify), ND_AND_NN
     if (h->otf) return mode == ND_SND ? k_pass_otf<false, false> : (mode == ND_AND ? k_pass_otf<true, true> : k_pass_otf<true, false>);
     const bool batch = h->gid && mode != ND_AND;  // converged graphs are skipped
-    return h->q == 1 ? pick_q<1>(mode, batch, late) : (h->q == 2 ? pick_q<2>(mode, batch, late) : pick_q<3>(mode, batch, late));
+    if (h->q == 1) return pick_q<1>(mode, batch, late);
+    if (h->q == 2) return pick_q<2>(mode, batch, late);
+    return h->t_pos ? pick_q<3>(mode, batch, late) : pick_q<kIds>(mode, batch, late);
 }
 
 // bucket ranges of a pass
@@ -1517,15 +1532,16 @@ nd_status ensure_state(nd_incidence* h, bool and_mode, cudaStream_t st) {
     const int64_t N = h->num_r > 0 ? h->num_r : 1;
     if (!h->tau[0]) ND_TRY(nd_alloc((void**)&h->tau[0], sizeof(int32_t) * N, st, h));
     if (!and_mode && !h->tau[1]) ND_TRY(nd_alloc((void**)&h->tau[1], sizeof(int32_t) * N, st, h));
-    if (h->q != 3) {
-        // 16-bit gather copies: one per CSR slot for (2,3), per vertex for (1,2)
-        const int64_t E = h->adj ? (h->nnz > 0 ? h->nnz : 1) : N;
+    const int64_t slots = nd_slots(h);
+    if (h->q != 3 || slots > 0) {
+        // 16-bit gather copies: one per slot, or per vertex for (1,2)
+        const int64_t E = slots > 0 ? slots : N;
         if (!h->tg[0]) ND_TRY(nd_alloc((void**)&h->tg[0], sizeof(uint16_t) * E, st, h));
         if (!and_mode && !h->tg[1]) ND_TRY(nd_alloc((void**)&h->tg[1], sizeof(uint16_t) * E, st, h));
     }
-    // (2,3): one frontier bit per CSR position (notification sets the bit of
-    // the slot it has just read); otherwise one per r-clique
-    const int64_t words = ((h->adj ? h->nnz : N) + 31) / 32;
+    // one frontier bit per slot (notification sets the bit of the slot it has
+    // just read), or per r-clique
+    const int64_t words = ((slots > 0 ? slots : N) + 31) / 32;
     if (and_mode && !h->front[0]) {
         ND_TRY(nd_alloc((void**)&h->front[0], sizeof(uint32_t) * words, st, h));
         ND_TRY(nd_alloc((void**)&h->front[1], sizeof(uint32_t) * words, st, h));
@@ -1796,9 +1812,12 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
             k_init_tau<<<blocks, kThreads, 0, st>>>(N, h->inc_ptr, h->tau[0], and_mode ? nullptr : h->tau[1]);
             ND_CUDA(cudaGetLastError());
         }
-        if (h->q != 3) {
+        if (h->q != 3 || h->t_pos) {
             nd_prof_scope ps("init_tau", st);
-            if (h->adj)
+            if (h->t_pos)
+                k_tau_to_lists<<<nd_blocks_for(3 * N, kThreads, h->sm_count * 8), kThreads, 0, st>>>(
+                    N, h->t_pos, h->tau[0], h->tg[0], and_mode ? nullptr : h->tg[1]);
+            else if (h->adj)
                 k_tau_to_adj<<<blocks, kThreads, 0, st>>>(N, h->e_pos, h->tau[0], h->tg[0],
                                                           and_mode ? nullptr : h->tg[1]);
             else
@@ -1811,11 +1830,16 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
         *converged = (N == 0);
         return ND_OK;
     }
-    const int64_t fbits = h->adj ? h->nnz : N;  // frontier bits (see ensure_state)
+    const int64_t fbits = nd_slots(h) > 0 ? nd_slots(h) : N;  // frontier bits (see ensure_state)
     const int64_t words = (fbits + 31) / 32;
     if (mode == ND_AND && members) {
         // PartialAnd: the members start active (end of Section 4.3)
-        if (h->adj) {
+        if (h->t_pos) {
+            ND_CUDA(cudaMemsetAsync(h->front[0], 0, sizeof(uint32_t) * words, st));
+            nd_prof_scope ps("fill_front", st);
+            k_member_lists<<<blocks, kThreads, 0, st>>>(N, members, h->t_pos, h->front[0]);
+            ND_CUDA(cudaGetLastError());
+        } else if (h->adj) {
             ND_CUDA(cudaMemsetAsync(h->front[0], 0, sizeof(uint32_t) * words, st));
             nd_prof_scope ps("fill_front", st);
             k_member_pos<<<blocks, kThreads, 0, st>>>(N, members, h->e_pos, h->front[0]);
@@ -1831,7 +1855,8 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
     SweepParams P;
     P.inc = h->inc;
     P.epos = h->e_pos;
-    P.eid = h->eid;
+    P.tpos = h->t_pos;
+    P.eid = h->t_pos ? h->t_id : h->eid;
     P.rp = h->rp;
     P.col = h->col;
     P.eu = h->e_u;

@@ -75,6 +75,15 @@ struct nd_incidence {
     int64_t* tri_ptr = nullptr;    // [m+1] triangles (u<v<w) grouped by edge (u,v)
     int32_t* tri_w = nullptr;      // [T] third vertex w, ascending inside a group
     uint32_t* tri_e = nullptr;     // [T] owning edge (u,v)
+    // (3,4) list layout: the triangles of every edge, by third vertex, form
+    // one array of 3T slots, where a triangle has three (one per edge).  An
+    // incidence entry of triangle {u,v,w} for the 4-clique {u,v,w,z} is the
+    // slots of z in the lists of its three edges, so a row ordered by z
+    // gathers at ascending slots of three lists; tau is gathered from a 16-bit
+    // copy indexed by slot.  Null where the slots do not fit (32-bit slots, the
+    // handle's memory limit): entries are then triangle ids.
+    uint32_t* t_pos = nullptr;     // [3T] the slots of every triangle
+    uint32_t* t_id = nullptr;      // [3T] the triangle at every slot
     // incidence (r-clique -> other r-cliques of each s-clique)
     int64_t* inc_ptr = nullptr;    // [num_r+1]
     uint32_t* inc = nullptr;       // [num_inc*q]
@@ -204,6 +213,11 @@ struct nd_tmp {
         return ND_OK;
     }
     operator T*() const { return p; }
+    T* take() {  // the caller's from now on
+        T* q = p;
+        p = nullptr;
+        return q;
+    }
 };
 
 // device memory helpers (stream-ordered)
@@ -221,13 +235,22 @@ nd_status nd_sort_u64(unsigned long long* keys, unsigned long long* alt, int64_t
                       unsigned long long** result, cudaStream_t st);
 int nd_id_bits(int64_t n);
 
+// the limit of nd_set_handle_memory_limit (0: none)
+int64_t nd_handle_limit();
+
+// slots of the handle's slot-indexed arrays (16-bit gather copies and frontier
+// bits): CSR slots for (2,3), list slots for (3,4); 0 where they are indexed by
+// r-clique
+static inline int64_t nd_slots(const nd_incidence* h) {
+    return h->adj ? h->nnz : (h->t_pos ? 3 * h->num_tri : 0);
+}
+
 // build steps (nd_build.cu)
 // the handle's CSR copy, validated and split; truss_relabel: a (2,3) build
 // that will renumber the graph (nd_relabel_truss_graph) next
 nd_status nd_build_graph(nd_incidence* h, const nd_csr* g, cudaStream_t st, bool truss_relabel);
 nd_status nd_build_edges(nd_incidence* h, cudaStream_t st);
 nd_status nd_build_tri_incidence(nd_incidence* h, cudaStream_t st);
-nd_status nd_build_triangles(nd_incidence* h, cudaStream_t st);
 nd_status nd_build_k4_incidence(nd_incidence* h, cudaStream_t st);
 nd_status nd_build_buckets(nd_incidence* h, cudaStream_t st);
 nd_status nd_relabel_by_degree(nd_incidence* h, cudaStream_t st);
@@ -283,6 +306,72 @@ static __device__ __forceinline__ int nd_lower_bound_n(const int32_t* __restrict
     }
     return lo;
 }
+
+// Positions in a sorted list l[0, n) of the elements of another one, taken 32
+// at a time and in order by one warp.  Lists of like length (kMergeRatio):
+// blocks of kBlock entries pass through shared memory, each loaded once, and a
+// lane searches its element there; a list much longer than the other is
+// searched by every lane, from where the elements before ended.
+struct nd_list_cursor {
+    static constexpr int kBlock = 128, kMergeRatio = 16;
+    const int32_t* __restrict__ l;
+    int n;
+    int32_t* buf;  // kBlock words of the warp
+    bool merge;
+    int at;    // merging: the block in buf starts here; searching: no earlier entry can match
+    int last;  // merging: the largest element in buf
+
+    // others: elements that will be looked up
+    __device__ __forceinline__ void start(const int32_t* list, int count, int64_t others, int32_t* buffer) {
+        l = list;
+        n = count;
+        buf = buffer;
+        restart(others);
+    }
+    __device__ __forceinline__ void restart(int64_t others) {
+        merge = n <= kMergeRatio * others;
+        at = 0;
+        if (merge) load();
+    }
+    __device__ __forceinline__ void load() {
+        const int lane = threadIdx.x & 31;
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < kBlock / 32; ++u) {
+            const int k = at + 32 * u + lane;
+            buf[32 * u + lane] = k < n ? __ldg(l + k) : INT32_MAX;
+        }
+        __syncwarp();
+        last = buf[kBlock - 1];
+    }
+    // where w is (open lanes only; -1: nowhere).  top: the warp's largest w,
+    // closed lanes included, which later calls do not go below
+    __device__ __forceinline__ int find(int32_t w, bool open, int32_t top) {
+        int k = -1;
+        if (merge) {
+            for (;;) {
+                if (open && w <= last) {
+                    int lo = 0;  // entries of the block below w
+#pragma unroll
+                    for (int h = kBlock / 2; h > 0; h >>= 1) lo += buf[lo + h - 1] < w ? h : 0;
+                    if (buf[lo] == w) k = at + lo;
+                    open = false;
+                }
+                if (top <= last || at + kBlock >= n || !__any_sync(0xffffffffu, open)) break;
+                at += kBlock;
+                load();
+            }
+        } else {
+            int p = at;
+            if (open) {
+                p = at + nd_lower_bound_n(l + at, n - at, w);
+                if (p < n && __ldg(l + p) == w) k = p;
+            }
+            at = (int)__reduce_max_sync(0xffffffffu, (unsigned)p);
+        }
+        return k;
+    }
+};
 
 // launch geometry
 static inline int nd_blocks_for(int64_t work_items, int per_block, int cap) {

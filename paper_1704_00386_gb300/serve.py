@@ -60,6 +60,7 @@ def footprint_bytes(row_ptr: np.ndarray, col: np.ndarray, r: int) -> int:
             num_r = tri_bound // 3 + 1
             inc = tri_bound * int(deg.max() if n else 0) // 3
             q = 3
+            base += 48 * num_r  # triangle lists and their slots; then slots, ids and 16-bit copies
         base += 12 * (nnz // 2)
     return int(base + 8 * (num_r + 1) + copies * 4 * q * inc + 16 * num_r + 8 * num_r + num_r // 4 + (1 << 20))
 

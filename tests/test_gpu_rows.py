@@ -95,3 +95,29 @@ def test_no_storage_rows_with_hub_tables(nd):
     members = torch.arange(0, inc.num_r, 3, dtype=torch.int32, device="cuda")
     np.testing.assert_array_equal(inc.and_partial(members)[0].cpu().numpy(),
                                   stored.and_partial(members)[0].cpu().numpy())
+
+
+def test_nuclei_by_triangle_ids(nd):
+    """A (3,4) handle whose memory limit leaves no room for the list slots
+    keeps triangle ids in its rows: the same results, fewer bytes."""
+    rp, col = G.hub_graph(2000, 5, seed=71)
+    drp, dcol = torch.from_numpy(rp).cuda(), torch.from_numpy(col).cuda()
+
+    def results(inc):
+        kap, passes = inc.snd()
+        t2, _ = inc.iterate_k("snd", 2)
+        members = torch.arange(0, inc.num_r, 5, dtype=torch.int32, device="cuda")
+        out = [kap, t2, inc.and_()[0], inc.and_(notify=False)[0], inc.and_partial(members)[0], inc.s_degree()]
+        return [x.cpu().numpy() for x in out], passes, inc.incidence_bytes()
+
+    want, passes, held = results(nd.build_incidence(drp, dcol, 3, 4))
+    g = oracle.Graph(rp, col, 3, 4)
+    np.testing.assert_array_equal(want[0], g.peel())
+    try:
+        nd.set_handle_memory_limit(held - 20 * len(want[0]))
+        got, passes_ids, held_ids = results(nd.build_incidence(drp, dcol, 3, 4))
+    finally:
+        nd.set_handle_memory_limit(0)
+    assert held_ids < held - 20 * len(want[0]) and passes_ids == passes
+    for a, b in zip(got, want):
+        np.testing.assert_array_equal(a, b)

@@ -50,7 +50,7 @@ constexpr int kThreads = 256;
 #ifndef ND_WARP_CHUNK
 #define ND_WARP_CHUNK 16  // consecutive warp tasks per counter grab
 #endif
-constexpr int kWarpChunk = ND_WARP_CHUNK;  // at most: pass_chunk
+constexpr int kWarpChunk = ND_WARP_CHUNK;  // at most: warp_chunk
 #ifndef ND_NOTIFY_UNROLL
 #define ND_NOTIFY_UNROLL 4  // notification entries in flight per lane ((2,3))
 #endif
@@ -125,7 +125,7 @@ struct SweepParams {
     bool bounded;                           // tau <= d_s throughout: a run from d_s
     const nd_item* __restrict__ items;
     int64_t lo[ND_NB], hi[ND_NB];  // bucket ranges in items
-    int chunk;                     // warp tasks per counter grab (pass_chunk)
+    int chunk;                     // warp tasks per counter grab (warp_chunk)
     bool direct;                   // AND: rows are expected to fail the count (see warp_hindex)
     const uint32_t* cur;  // AND + notification: frontier read in this pass
     uint32_t* next;       // and the frontier written for the next pass
@@ -139,8 +139,11 @@ struct SweepParams {
     const uint32_t* __restrict__ gid;
     const uint8_t* gact_in;
     uint8_t* gact_out;
-    unsigned long long* ctr;         // this pass: [0] changed, [1] evaluated, [2] next CTA row,
-                                     // [3] incidences of the evaluated rows, [4] next warp chunk
+    // AND with notification: the active work items, and where each bucket's
+    // begin there (their numbers are in ctr)
+    const uint32_t* __restrict__ list;
+    int64_t list_lo[ND_NB];
+    unsigned long long* ctr;         // this pass's counters (ND_CTR_*)
     const unsigned long long* prev;  // previous pass (null on the first)
 };
 
@@ -267,26 +270,26 @@ __device__ __forceinline__ void stream_row(const F& rho, int i, int end, G&& f) 
 #pragma unroll
         for (int u = 0; u < 4; ++u) r[u] = rho(i + u * STEP + lane);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) f(i + u * STEP + lane, r[u]);
+        for (int u = 0; u < 4; ++u) f((int)((unsigned)i + u * STEP + lane), r[u]);
     }
     if (end - i > 2 * STEP) {
         int32_t r[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const int j = i + u * STEP + lane;
-            r[u] = j < end ? rho(j) : -1;
+            const unsigned j = (unsigned)i + u * STEP + lane;  // may leave 31 bits
+            r[u] = j < (unsigned)end ? rho((int)j) : -1;
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) f(i + u * STEP + lane, r[u]);
+        for (int u = 0; u < 4; ++u) f((int)((unsigned)i + u * STEP + lane), r[u]);
     } else if (end > i) {
         int32_t r[2];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-            const int j = i + u * STEP + lane;
-            r[u] = j < end ? rho(j) : -1;
+            const unsigned j = (unsigned)i + u * STEP + lane;  // may leave 31 bits
+            r[u] = j < (unsigned)end ? rho((int)j) : -1;
         }
 #pragma unroll
-        for (int u = 0; u < 2; ++u) f(i + u * STEP + lane, r[u]);
+        for (int u = 0; u < 2; ++u) f((int)((unsigned)i + u * STEP + lane), r[u]);
     }
 }
 
@@ -412,7 +415,8 @@ __device__ __forceinline__ int32_t warp_hindex(const F& rho, const B& bound, int
     if (!direct) {
         int cnt = 0, have = 0;
         for (int i = 0; i < d;) {
-            const int end = min(d, i + max((t - have + 31) & ~31, 64));
+            const int need = max((min(t - have, 1 << 30) + 31) & ~31, 64);
+            const int end = d - i > need ? i + need : d;
             stream_row<32>(rho, i, end, [&](int, int32_t r) { cnt += (r >= t); });
             i = end;
             have = (int)__reduce_add_sync(0xffffffffu, (unsigned)cnt);
@@ -482,7 +486,7 @@ __device__ __forceinline__ int32_t cta_hindex(const F& rho, const B& bound, int 
     if (!direct) {
         int cnt = 0, have = 0;
         for (int i = 0; i < d;) {
-            const int need = max((t - have + 4 * kThreads - 1) & ~(4 * kThreads - 1), kCtaSegment);
+            const int need = max((min(t - have, 1 << 30) + 4 * kThreads - 1) & ~(4 * kThreads - 1), kCtaSegment);
             const int end = d - i > need ? i + need : d;
             stream_row<kThreads>(rho, i, end, [&](int, int32_t r) { cnt += (r >= t); });
             i = end;
@@ -584,24 +588,15 @@ __device__ __forceinline__ unsigned front_bit(const uint32_t* f, uint32_t i) {
     return (__ldg(f + (i >> 5)) >> (i & 31)) & 1u;
 }
 
-// is R in the current frontier?  With slots: any bit of its slots
-template <int Q>
+// (2,3): is R in the current frontier?  Either bit of its two slots
 __device__ __forceinline__ bool in_frontier(const SweepParams& P, uint32_t R) {
-    if constexpr (Q == 2) {
-        const uint2 ep = __ldg(P.epos + R);
-        return front_bit(P.cur, ep.x) | front_bit(P.cur, ep.y);
-    } else if constexpr (Q == 3) {
-        const uint32_t* p = P.tpos + 3 * (int64_t)R;
-        const uint32_t a = __ldg(p), b = __ldg(p + 1), c = __ldg(p + 2);
-        return front_bit(P.cur, a) | front_bit(P.cur, b) | front_bit(P.cur, c);
-    } else {
-        return front_bit(P.cur, R);
-    }
+    const uint2 ep = __ldg(P.epos + R);
+    return front_bit(P.cur, ep.x) | front_bit(P.cur, ep.y);
 }
 
 // the ids of entry j of a row of d entries
 template <int Q>
-__device__ __forceinline__ void entry_ids(const uint32_t* __restrict__ row, uint32_t d, int64_t j,
+__device__ __forceinline__ void entry_ids(const uint32_t* __restrict__ row, int d, int j,
                                           uint32_t (&id)[kWords<Q>]) {
     if constexpr (Q == 2) {
         const uint2 x = __ldg(reinterpret_cast<const uint2*>(row) + j);
@@ -609,79 +604,101 @@ __device__ __forceinline__ void entry_ids(const uint32_t* __restrict__ row, uint
         id[1] = x.y;
     } else {
 #pragma unroll
-        for (int k = 0; k < kWords<Q>; ++k) id[k] = __ldg(row + j + k * (int64_t)d);
+        for (int k = 0; k < kWords<Q>; ++k) id[k] = __ldg(row + j + (int64_t)k * d);
     }
 }
 
-// one neighbour whose next-frontier word has been read as wd: set its bit if
-// it is clear and h <= tau.  A neighbour whose bit is already set needs
-// nothing, so the word (2 MB for 16M r-cliques, cache-resident) is read before
-// its tau, and an atomic is only issued for a bit that is still clear.
-// (Warp-wide merging of bits that share a word was measured slower: the match
-// runs for every neighbour, while most neighbours need no write.)
+// one neighbour whose next-frontier bit was clear: set it if h <= tau
 template <int Q>
-__device__ __forceinline__ void notify_one(const SweepParams& P, uint32_t id, uint32_t wd, int32_t h) {
-    const uint32_t bit = 1u << (id & 31);
-    if (wd & bit) return;  // already active (or past the row's end)
+__device__ __forceinline__ void notify_one(const SweepParams& P, uint32_t id, int32_t h) {
     if constexpr (kSlots<Q>) {
         notify_clear(P, id, h, ld_tau<false>(P.gin + id));
     } else {
+        const uint32_t bit = 1u << (id & 31);
         if (P.members && !(__ldg(P.members + (id >> 5)) & bit)) return;  // PartialAnd
         if (h <= ld_tau<false>(P.tin + id)) atomicOr(P.next + (id >> 5), bit);
     }
 }
 
+// U entries of one lane (ok: those that exist): which of their neighbours'
+// next-frontier bits are clear, then those neighbours.  A neighbour whose bit
+// is already set needs nothing, so the words (2 MB for 16M r-cliques,
+// cache-resident) are read before any tau, all of them before any is tested,
+// and one branch skips an entry block whose bits are all set, which most are.
+// (Warp-wide merging of bits that share a word was measured slower: the match
+// runs for every neighbour, while most neighbours need no write.)
+template <int Q, int U>
+__device__ __forceinline__ void notify_block(const SweepParams& P, const uint32_t (&id)[U][kWords<Q>],
+                                             const bool (&ok)[U], int32_t h) {
+    constexpr int W = kWords<Q>;
+    uint32_t wd[U][W];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int k = 0; k < W; ++k) wd[u][k] = ok[u] ? ld_front(P.next + (id[u][k] >> 5)) : 0xffffffffu;
+    unsigned clear = 0;
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int k = 0; k < W; ++k) clear |= ((~wd[u][k] >> (id[u][k] & 31)) & 1u) << (u * W + k);
+    if (!clear) return;
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int k = 0; k < W; ++k)
+            if ((clear >> (u * W + k)) & 1u) notify_one<Q>(P, id[u][k], h);
+}
+
 // notify every neighbour whose tau could still depend on R (Alg. 3, orange
 // lines): set its next-frontier bit if h <= tau(R').  With slots there is one
 // bit per slot, so the test reads the 16-bit copy and the bit sits next to it
-// (no r-clique id on this path).  U entries per lane and their bit words are
-// loaded before any is tested, so their latencies overlap.
+// (no r-clique id on this path).
 template <int Q>
-__device__ __forceinline__ void notify_row(const SweepParams& P, const uint32_t* __restrict__ row, uint32_t d,
-                                           int32_t h, int first, int step) {
+__device__ __forceinline__ void notify_row(const SweepParams& P, const uint32_t* __restrict__ row, int d, int32_t h,
+                                           int first, int step) {
     constexpr int W = kWords<Q>;
     constexpr int U = W == 3 ? 2 : kNotifyUnroll;
     // a relabelled (1,2) row: from this id on every tau is below h
     const uint32_t limit = Q == 1 && P.oct_max ? id_limit(P.oct_max, h) : 0xffffffffu;
-    for (int64_t j0 = first; j0 < d; j0 += (int64_t)U * step) {
-        uint32_t id[U][W], wd[U][W];
+    for (unsigned j0 = 0; j0 < (unsigned)d; j0 += U * step) {  // past d it may leave 31 bits
+        uint32_t id[U][W];
+        bool ok[U];
+        if ((unsigned)d - j0 >= (unsigned)(U * step)) {  // a whole block: no test per entry
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int64_t j = j0 + (int64_t)u * step;
-            if (j < d) {
-                entry_ids<Q>(row, d, j, id[u]);
-            } else {
+            for (int u = 0; u < U; ++u) {
+                entry_ids<Q>(row, d, (int)(j0 + u * step + first), id[u]);
+                ok[u] = true;
+            }
+        } else {
 #pragma unroll
-                for (int k = 0; k < W; ++k) id[u][k] = 0u;
+            for (int u = 0; u < U; ++u) {
+                const unsigned j = j0 + u * step + first;
+                ok[u] = j < (unsigned)d;
+                if (ok[u]) {
+                    entry_ids<Q>(row, d, (int)j, id[u]);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < W; ++k) id[u][k] = 0u;
+                }
             }
         }
-        if (Q == 1 && id[0][0] >= limit) break;  // so are this lane's later entries
+        if (Q == 1) {
+            if (id[0][0] >= limit) break;  // so are this lane's later entries
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const bool ok = j0 + (int64_t)u * step < d && (Q != 1 || id[u][0] < limit);
-#pragma unroll
-            for (int k = 0; k < W; ++k) wd[u][k] = ok ? ld_front(P.next + (id[u][k] >> 5)) : 0xffffffffu;
+            for (int u = 0; u < U; ++u) ok[u] = ok[u] && id[u][0] < limit;
         }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-#pragma unroll
-            for (int k = 0; k < W; ++k) notify_one<Q>(P, id[u][k], wd[u][k], h);
-        }
+        notify_block<Q, U>(P, id, ok, h);
     }
 }
 
-// notification for one entry j of a row whose tau dropped to h: the same
-// test as notify_row, for a single entry (the merged walk of group rows below
-// gives each lane entries of different rows)
+// notification for one entry j of a row whose tau dropped to h (the merged
+// walk of group rows below gives each lane entries of different rows)
 template <int Q>
-__device__ __forceinline__ void notify_entry(const SweepParams& P, int64_t jb, uint32_t d, int j, int32_t h) {
-    constexpr int W = kWords<Q>;
-    uint32_t id[W], wd[W];
-    entry_ids<Q>(row_of<Q>(P, jb), d, j, id);
-#pragma unroll
-    for (int k = 0; k < W; ++k) wd[k] = ld_front(P.next + (id[k] >> 5));
-#pragma unroll
-    for (int k = 0; k < W; ++k) notify_one<Q>(P, id[k], wd[k], h);
+__device__ __forceinline__ void notify_entry(const SweepParams& P, int64_t jb, int d, int j, int32_t h) {
+    uint32_t id[1][kWords<Q>];
+    const bool ok[1] = {true};
+    entry_ids<Q>(row_of<Q>(P, jb), d, j, id[0]);
+    notify_block<Q, 1>(P, id, ok, h);
 }
 
 // batches (GB): has R's graph converged (no change in its previous pass)?
@@ -708,9 +725,10 @@ __device__ __forceinline__ nd_item load_item(const nd_item* __restrict__ items, 
     return it;
 }
 
-// counters of one thread over a pass.  FULL (AND with notification, batches):
-// evaluated rows and their incidences too; the other passes evaluate every
-// row, so the host knows both.
+// counters of one thread over a pass.  FULL (batches, no-storage passes):
+// evaluated rows and their incidences too; k_active_list counts them for AND
+// with notification, and the other passes evaluate every row, so the host
+// knows both.
 template <bool FULL>
 struct Tally {
     unsigned changed = 0, evals = 0;
@@ -735,13 +753,23 @@ __device__ __forceinline__ void load_tau(const SweepParams& P, const nd_item& it
     t = min(t0, (int32_t)min(it.d, (uint32_t)INT32_MAX));
 }
 
+// work item i of a pass: AND with notification takes them from its list
+template <bool NOTIFY>
+__device__ __forceinline__ nd_item pass_item(const SweepParams& P, int64_t i) {
+    return load_item(P.items, NOTIFY ? (int64_t)__ldg(P.list + i) : i);
+}
+
 // work items [first, last): one r-clique per group of G lanes of the calling
-// warp, at most 32/G of them
-template <int Q, int G, int C, bool AND, bool GB, bool FULL>
+// warp, at most 32/G of them.  NOTIFY: the entries of all rows that changed
+// are then walked by the 32 lanes together, instead of each row by its own G
+// lanes while the other groups wait.
+template <int Q, int G, int C, bool AND, bool NOTIFY, bool GB, bool FULL>
 __device__ __forceinline__ void run_groups(const SweepParams& P, int64_t first, int64_t last, Tally<FULL>& n) {
-    const int64_t i = first + (int64_t)((threadIdx.x & 31) / G);
+    constexpr int NG = 32 / G;
+    const int lane = threadIdx.x & 31;
+    const int64_t i = first + lane / G;
     const bool ok = i < last;
-    const nd_item it = load_item(P.items, ok ? i : first);
+    const nd_item it = pass_item<NOTIFY>(P, ok ? i : first);
     const bool run = ok && !graph_done<GB>(P, it.R);
     int32_t t0, t, old;
     load_tau<AND>(P, it, t0, t, old);
@@ -749,10 +777,35 @@ __device__ __forceinline__ void run_groups(const SweepParams& P, int64_t first, 
     if (!run) t = 0;
     const int dmax = (int)__reduce_max_sync(0xffffffffu, (unsigned)d);
     const int32_t h = group_hindex<G, C>(make_rho<Q, !AND>(P, it.jb, it.d), d, dmax, t);
-    if (run && (threadIdx.x & (G - 1)) == 0) {
+    if (run && (lane & (G - 1)) == 0) {
         n.row(it.d, h != t0);
         if (h != t0) graph_changed<GB>(P, it.R);
         store_tau<Q>(P, it.R, h, old);
+    }
+    if constexpr (NOTIFY) {
+        // entry e of the changed rows' concatenation belongs to the last row q
+        // that begins at or before e (the beginnings are kept in registers)
+        const int dn = h != t0 ? d : 0;
+        int begin[NG], tot = 0;
+#pragma unroll
+        for (int q = 0; q < NG; ++q) {
+            begin[q] = tot;
+            tot += __shfl_sync(0xffffffffu, dn, q * G);
+        }
+        for (int e0 = 0; e0 < tot; e0 += 32) {
+            const int e = e0 + lane;
+            int q = 0, b = 0;
+#pragma unroll
+            for (int r = 1; r < NG; ++r)
+                if (e >= begin[r] && begin[r] < tot) {  // an empty row's beginning is the next one's
+                    q = r;
+                    b = begin[r];
+                }
+            const int64_t jr = __shfl_sync(0xffffffffu, it.jb, q * G);
+            const int32_t hh = __shfl_sync(0xffffffffu, h, q * G);
+            const int dr = __shfl_sync(0xffffffffu, dn, q * G);
+            if (e < tot) notify_entry<Q>(P, jr, dr, e - b, hh);
+        }
     }
 }
 
@@ -778,7 +831,7 @@ __device__ __forceinline__ void run_warp_row(const SweepParams& P, const nd_item
         if (h != t0) graph_changed<GB>(P, R);
         store_tau<Q>(P, R, h, old);
     }
-    if (AND && NOTIFY && h != t0) notify_row<Q>(P, row_of<Q>(P, it.jb), it.d, h, lane, 32);
+    if (AND && NOTIFY && h != t0) notify_row<Q>(P, row_of<Q>(P, it.jb), (int)it.d, h, lane, 32);
     __syncwarp();  // the bins are free again
 }
 
@@ -786,9 +839,8 @@ __device__ __forceinline__ void run_warp_row(const SweepParams& P, const nd_item
 template <int Q, bool AND, bool NOTIFY, bool GB, int WORDS, bool FULL>
 __device__ __forceinline__ void run_cta(const SweepParams& P, int64_t i, unsigned* bins, int* bounds,
                                         Tally<FULL>& n) {
-    const nd_item it = load_item(P.items, i);
+    const nd_item it = pass_item<NOTIFY>(P, i);
     const uint32_t R = it.R;
-    if (AND && NOTIFY && !in_frontier<Q>(P, R)) return;
     if (graph_done<GB>(P, R)) return;  // the same R for the whole block
     int32_t t0, t, old;
     load_tau<AND>(P, it, t0, t, old);
@@ -813,125 +865,111 @@ __device__ __forceinline__ void run_cta(const SweepParams& P, int64_t i, unsigne
         if (h != t0) graph_changed<GB>(P, R);
         store_tau<Q>(P, R, h, old);
     }
-    if (AND && NOTIFY && h != t0) notify_row<Q>(P, row_of<Q>(P, it.jb), it.d, h, threadIdx.x, kThreads);
+    if (AND && NOTIFY && h != t0) notify_row<Q>(P, row_of<Q>(P, it.jb), d, h, threadIdx.x, kThreads);
     __syncthreads();
 }
 
-// AND with notification: the frontier bits of the rows [a, b) of a warp
-// chunk (at most 32 * W rows), tested by all lanes at once (one row per lane
-// per word, every load issued before any test) and returned as W ballots.
-template <int Q, int W>
-__device__ __forceinline__ void active_masks(const SweepParams& P, int64_t a, int64_t b, unsigned (&mask)[W]) {
-    const int lane = threadIdx.x & 31;
-    uint32_t R[W];
-    bool ok[W];
-#pragma unroll
-    for (int w = 0; w < W; ++w) {
-        const int64_t i = a + (int64_t)w * 32 + lane;
-        ok[w] = i < b;
-        R[w] = ok[w] ? __ldg(reinterpret_cast<const uint32_t*>(P.items + i) + 2) : 0u;  // nd_item::R
-    }
-    if constexpr (Q == 2) {
-        uint2 ep[W];
-#pragma unroll
-        for (int w = 0; w < W; ++w) ep[w] = ok[w] ? __ldg(P.epos + R[w]) : make_uint2(0u, 0u);
-        uint32_t bx[W], by[W];
-#pragma unroll
-        for (int w = 0; w < W; ++w) {
-            bx[w] = __ldg(P.cur + (ep[w].x >> 5));
-            by[w] = __ldg(P.cur + (ep[w].y >> 5));
-        }
-#pragma unroll
-        for (int w = 0; w < W; ++w)
-            mask[w] = __ballot_sync(0xffffffffu, ok[w] && (((bx[w] >> (ep[w].x & 31)) | (by[w] >> (ep[w].y & 31))) & 1u));
-    } else if constexpr (Q == 3) {
-        uint32_t tp[W][3], bits[W];
-#pragma unroll
-        for (int w = 0; w < W; ++w)
-#pragma unroll
-            for (int k = 0; k < 3; ++k) tp[w][k] = ok[w] ? __ldg(P.tpos + 3 * (int64_t)R[w] + k) : 0u;
-#pragma unroll
-        for (int w = 0; w < W; ++w) {
-            bits[w] = 0;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) bits[w] |= front_bit(P.cur, tp[w][k]);
-        }
-#pragma unroll
-        for (int w = 0; w < W; ++w) mask[w] = __ballot_sync(0xffffffffu, ok[w] && bits[w]);
-    } else {
-        uint32_t bw[W];
-#pragma unroll
-        for (int w = 0; w < W; ++w) bw[w] = __ldg(P.cur + (R[w] >> 5));
-#pragma unroll
-        for (int w = 0; w < W; ++w) mask[w] = __ballot_sync(0xffffffffu, ok[w] && ((bw[w] >> (R[w] & 31)) & 1u));
-    }
-}
+// AND with notification, before each pass: the work items whose r-clique is in
+// the frontier, compacted bucket by bucket, in order inside a tile; the pass
+// then takes dense tasks from the list, and splits few rows over all warps.
+// (With the frontier tested by each warp for its own chunk of work items, a
+// chunk of long rows that happened to be active together kept one warp busy:
+// 0.2 ms for a pass of 9,000 of 3.8M edges.)  It also clears the next frontier
+// and counts the pass's evaluations.  Streams 16 B per work item and its slots;
+// one atomic per tile.
+constexpr int kListTile = 2048;
 
-// position of the k-th (0-based) set bit of m, for k < popc(m): halves by popcount
-__device__ __forceinline__ int nth_set_bit(unsigned m, int k) {
-    int pos = 0;
-#pragma unroll
-    for (int w = 16; w >= 1; w >>= 1) {
-        const unsigned low = m & ((1u << w) - 1u);
-        const int c = __popc(low);
-        if (k >= c) {
-            k -= c;
-            m >>= w;
-            pos += w;
-        } else {
-            m = low;
-        }
-    }
-    return pos;
-}
+struct ListParams {
+    const uint2* __restrict__ epos;
+    const uint32_t* __restrict__ tpos;
+    const nd_item* __restrict__ items;
+    const uint32_t* cur;
+    uint32_t* next;
+    int64_t words;               // of the next frontier to clear
+    int64_t lo[ND_NB + 1];       // bucket ranges in items
+    int64_t tile_lo[ND_NB + 1];  // tiles of kListTile items, none across buckets
+    int64_t first, last;         // the tiles of this list
+    uint32_t* list;
+    unsigned long long* ctr;
+    const unsigned long long* prev;
+};
 
-// AND with notification, group rows: the active rows among the 32 rows
-// a + {bits of mask}, packed densely onto the 32/G groups of the warp (no
-// group idles on an inactive row).  After each round the entries of every
-// row that changed are walked by all 32 lanes together (the merged
-// notification), instead of by each row's own G lanes while the groups whose
-// rows did not change wait.
-template <int Q, int G, int C>
-__device__ __forceinline__ void run_groups_active(const SweepParams& P, int64_t a, unsigned mask, Tally<true>& n) {
-    constexpr int NG = 32 / G;
-    const int lane = threadIdx.x & 31;
-    const int grp = lane / G;
-    const int cnt = __popc(mask);
-    for (int base = 0; base < cnt; base += NG) {
-        const int k = base + grp;  // this group's k-th active row
-        const bool run = k < cnt;
-        const nd_item it = load_item(P.items, a + nth_set_bit(mask, run ? k : 0));
-        int32_t t0, t, old;
-        load_tau<true>(P, it, t0, t, old);
-        const int64_t jb = it.jb;
-        const int d = run ? (int)it.d : 0;
-        if (!run) t = 0;
-        const int dmax = (int)__reduce_max_sync(0xffffffffu, (unsigned)d);
-        const int32_t h = group_hindex<G, C>(make_rho<Q, false>(P, jb, it.d), d, dmax, t);
-        if (run && (lane & (G - 1)) == 0) {
-            n.row(it.d, h != t0);
-            store_tau<Q>(P, it.R, h, old);
+template <int Q>
+__global__ void __launch_bounds__(kThreads) k_active_list(ListParams L) {
+    if (L.prev != nullptr && *(volatile const unsigned long long*)L.prev == 0ull) return;  // converged
+    constexpr int K = kListTile / kThreads;
+    __shared__ unsigned wsum[kThreads / 32];
+    __shared__ unsigned long long s_base, s_in[kThreads / 32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < L.words; i += (int64_t)gridDim.x * kThreads)
+        L.next[i] = 0u;
+    unsigned long long evals = 0, incs = 0;
+    for (int64_t t = L.first + blockIdx.x; t < L.last; t += gridDim.x) {
+        int b = 0;
+        while (t >= L.tile_lo[b + 1]) ++b;
+        const int64_t i0 = L.lo[b] + (t - L.tile_lo[b]) * kListTile + (int64_t)w * (kListTile / (kThreads / 32)) + lane;
+        uint32_t R[K], d[K];
+        bool act[K];
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const int64_t i = i0 + 32 * k;
+            const uint2 x = i < L.lo[b + 1] ? __ldg(reinterpret_cast<const uint2*>(L.items + i) + 1) : make_uint2(0u, 0u);
+            R[k] = x.x;
+            d[k] = x.y;  // 0: past the bucket
         }
-        const int32_t dn = h != t0 ? d : 0;
-        // merged notification over the changed rows of this round
-        int tot = 0;
+        if constexpr (Q == 2) {
+            uint2 ep[K];
 #pragma unroll
-        for (int q = 0; q < NG; ++q) tot += __shfl_sync(0xffffffffu, dn, q * G);
-        for (int e0 = 0; e0 < tot; e0 += 32) {
-            const int e = e0 + lane;
-            int64_t jr = 0;  // the row of entry e, its length and its own number there
-            int32_t hh = 0, dr = 0;
-            int j = 0, run = 0;
+            for (int k = 0; k < K; ++k) ep[k] = __ldg(L.epos + R[k]);
 #pragma unroll
-            for (int q = 0; q < NG; ++q) {
-                const int v = __shfl_sync(0xffffffffu, dn, q * G);
-                const int64_t jq = __shfl_sync(0xffffffffu, jb, q * G);
-                const int32_t hq = __shfl_sync(0xffffffffu, h, q * G);
-                if (e >= run && e < run + v) { jr = jq; dr = v; j = e - run; hh = hq; }
-                run += v;
+            for (int k = 0; k < K; ++k) act[k] = d[k] && (front_bit(L.cur, ep[k].x) | front_bit(L.cur, ep[k].y));
+        } else if constexpr (Q == 3) {
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                const uint32_t* p = L.tpos + 3 * (int64_t)R[k];
+                const uint32_t a0 = __ldg(p), a1 = __ldg(p + 1), a2 = __ldg(p + 2);
+                act[k] = d[k] && (front_bit(L.cur, a0) | front_bit(L.cur, a1) | front_bit(L.cur, a2));
             }
-            if (e < tot) notify_entry<Q>(P, jr, (uint32_t)dr, j, hh);
+        } else {
+#pragma unroll
+            for (int k = 0; k < K; ++k) act[k] = d[k] && front_bit(L.cur, R[k]);
         }
+        unsigned c = 0;
+        uint32_t at[K];
+        unsigned long long in = 0;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const unsigned m = __ballot_sync(0xffffffffu, act[k]);
+            at[k] = c + __popc(m & ((1u << lane) - 1u));
+            c += __popc(m);
+            if (act[k]) in += d[k];
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) in += __shfl_xor_sync(0xffffffffu, in, o);
+        if (lane == 0) { wsum[w] = c; s_in[w] = in; }
+        __syncthreads();
+        unsigned before = 0, total = 0;
+#pragma unroll
+        for (int v = 0; v < kThreads / 32; ++v) {
+            if (v < w) before += wsum[v];
+            total += wsum[v];
+        }
+        if (threadIdx.x == 0) {
+            s_base = total ? atomicAdd(L.ctr + ND_CTR_LIST + b, (unsigned long long)total) : 0ull;
+            evals += total;
+            for (int v = 0; v < kThreads / 32; ++v) incs += s_in[v];
+        }
+        __syncthreads();
+        // the bucket's part of the list begins at its first tile here
+        uint32_t* const out = L.list + (max(L.tile_lo[b], L.first) - L.first) * kListTile + s_base + before;
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+            if (act[k]) out[at[k]] = (uint32_t)(i0 + 32 * k);
+        __syncthreads();
+    }
+    if (threadIdx.x == 0 && evals) {
+        atomicAdd(L.ctr + ND_CTR_EVALS, evals);
+        atomicAdd(L.ctr + ND_CTR_INCS, incs);
     }
 }
 
@@ -955,10 +993,22 @@ __device__ __forceinline__ void flush_tally(const SweepParams& P, const Tally<FU
     if (threadIdx.x == 0) {
         unsigned long long a = 0, e = 0, c = 0;
         for (int w = 0; w < kThreads / 32; ++w) { a += s_ch[w]; e += s_ev[w]; c += s_in[w]; }
-        if (a) atomicAdd(P.ctr, a);
-        if (e) atomicAdd(P.ctr + 1, e);
-        if (c) atomicAdd(P.ctr + 3, c);
+        if (a) atomicAdd(P.ctr + ND_CTR_CHANGED, a);
+        if (e) atomicAdd(P.ctr + ND_CTR_EVALS, e);
+        if (c) atomicAdd(P.ctr + ND_CTR_INCS, c);
     }
+}
+
+// warp tasks per counter grab: kWarpChunk where there are many, fewer where
+// that would leave the resident warps with less than kChunksPerWarp grabs
+// each.  A graph of 2,000 vertices has 250 tasks: in chunks of 16 they kept 16
+// warps busy, one after the other (26 us per pass).  R-MAT of 100,003 vertices:
+// the first 16 SND passes 3.2 ms with 8 grabs, 3.9 with 4, 3.2 with 16 (whose
+// late passes are 12% slower).
+constexpr int kChunksPerWarp = 8;
+__host__ __device__ __forceinline__ int warp_chunk(int64_t tasks, int grid) {
+    const int64_t c = tasks / ((int64_t)(grid > 0 ? grid : 1) * (kThreads / 32) * kChunksPerWarp);
+    return (int)(c < 1 ? 1 : (c > kWarpChunk ? kWarpChunk : c));
 }
 
 constexpr int kPassBlocks = 6;  // resident blocks per SM the register budget of every pass kernel targets
@@ -971,7 +1021,7 @@ constexpr int kPassBlocks = 6;  // resident blocks per SM the register budget of
 template <int Q, bool AND, bool NOTIFY, bool GB, bool LATE>
 __global__ void __launch_bounds__(kThreads, kPassBlocks) k_pass(SweepParams P) {
     if (P.prev != nullptr && *(volatile const unsigned long long*)P.prev == 0ull) return;  // converged
-    constexpr bool FULL = NOTIFY || GB;
+    constexpr bool FULL = GB;
     constexpr int HW = LATE ? kLateHistWords : kHistWords;
     constexpr int kWords = (kThreads / 32) * HW;  // a CTA row uses every warp's histogram
     __shared__ __align__(16) unsigned hist[kThreads / 32][HW];
@@ -979,18 +1029,21 @@ __global__ void __launch_bounds__(kThreads, kPassBlocks) k_pass(SweepParams P) {
     __shared__ unsigned long long s_chunk;
     unsigned* const bins = hist[threadIdx.x >> 5];
     Tally<FULL> n;
+    // the rows of each bucket: [lo, lo + rows) of the work items, or of the list
+    auto lo = [&](int b) { return NOTIFY ? P.list_lo[b] : P.lo[b]; };
+    auto rows = [&](int b) { return NOTIFY ? (int64_t)__ldcg(P.ctr + ND_CTR_LIST + b) : P.hi[b] - P.lo[b]; };
     // phase 1: rows longer than the CTA threshold, one per block at a time,
     // taken from a per-pass counter (longest rows first)
-    const int64_t n3 = P.hi[3] - P.lo[3];
+    const int64_t n3 = rows(3);
     auto cta_phase = [&]() {
         if (n3 <= 0) return;
         for (;;) {
-            if (threadIdx.x == 0) s_chunk = atomicAdd(P.ctr + 2, 1ull);
+            if (threadIdx.x == 0) s_chunk = atomicAdd(P.ctr + ND_CTR_CTA, 1ull);
             __syncthreads();
             const int64_t c = (int64_t)s_chunk;
             __syncthreads();
             if (c >= n3) break;
-            run_cta<Q, AND, NOTIFY, GB, kWords>(P, P.lo[3] + c, &hist[0][0], bounds, n);
+            run_cta<Q, AND, NOTIFY, GB, kWords>(P, lo(3) + c, &hist[0][0], bounds, n);
         }
     };
     // AND updates in place, so a row evaluated later in a pass already sees
@@ -1007,82 +1060,42 @@ __global__ void __launch_bounds__(kThreads, kPassBlocks) k_pass(SweepParams P) {
     if (kCtaFirst) cta_phase();
     // phase 2: warp tasks (one warp row, four 8-lane rows or eight 4-lane
     // rows), longest first (SND) or shortest first (AND).  Each warp takes
-    // chunks of P.chunk consecutive tasks from a per-pass counter (one atomic
-    // per chunk, no barrier): consecutive r-cliques share a vertex and gather
-    // from the same part of tau, and dynamic chunks keep the warps balanced
-    // even when only a scattered subset of r-cliques is active (AND).
-    const int64_t n2 = P.hi[2] - P.lo[2];
-    const int64_t t1 = (P.hi[1] - P.lo[1] + 3) / 4;
-    const int64_t t0 = (P.hi[0] - P.lo[0] + 7) / 8;
+    // chunks of consecutive tasks from a per-pass counter (one atomic per
+    // chunk, no barrier): consecutive r-cliques share a vertex and gather from
+    // the same part of tau.
+    const int64_t n2 = rows(2), n1 = rows(1), n0 = rows(0);
+    const int64_t t1 = (n1 + 3) / 4, t0 = (n0 + 7) / 8;
     const int64_t tasks = n2 + t1 + t0;
     const int lane32 = threadIdx.x & 31;
-    const int chunk = P.chunk;
+    const int chunk = NOTIFY ? warp_chunk(tasks, gridDim.x) : P.chunk;
     const int64_t nchunks = (tasks + chunk - 1) / chunk;
     for (;;) {
         unsigned long long c = 0;
-        if (lane32 == 0) c = atomicAdd(P.ctr + 4, 1ull);
+        if (lane32 == 0) c = atomicAdd(P.ctr + ND_CTR_CHUNK, 1ull);
         c = __shfl_sync(0xffffffffu, c, 0);
         if ((int64_t)c >= nchunks) break;
         const int64_t cc = kShortFirst ? nchunks - 1 - (int64_t)c : (int64_t)c;
         int64_t t = cc * chunk;
         const int64_t te = min(t + (int64_t)chunk, tasks);
-        if constexpr (AND && NOTIFY) {
-            // the chunk's rows per bucket, their frontier bits tested up front;
-            // only active rows are evaluated
-            static_assert(kWarpChunk <= 32, "one mask word of warp rows per chunk");
-            const int64_t w_hi = min(te, n2);
-            if (t < w_hi) {
-                unsigned m2[1];
-                active_masks<Q, 1>(P, P.lo[2] + t, P.lo[2] + w_hi, m2);
-                unsigned mm = m2[0];
-                while (mm) {
-                    const int b = __ffs(mm) - 1;
-                    mm &= mm - 1;
-                    const nd_item it = load_item(P.items, P.lo[2] + t + b);
-                    run_warp_row<Q, AND, NOTIFY, false, HW>(P, it, bins, n);
-                }
+        const int64_t e2 = min(te, n2);
+        if (t < e2) {
+            // warp rows: the next row's work item is loaded before this one runs
+            nd_item it = pass_item<NOTIFY>(P, lo(2) + t);
+            while (t < e2) {
+                nd_item nx;
+                if (t + 1 < e2) nx = pass_item<NOTIFY>(P, lo(2) + t + 1);
+                run_warp_row<Q, AND, NOTIFY, GB, HW>(P, it, bins, n);
+                it = nx;
+                ++t;
             }
-            const int64_t t1_lo = max(t, n2), t1_hi = min(te, n2 + t1);
-            if (t1_lo < t1_hi) {
-                constexpr int W1 = (kWarpChunk * 4 + 31) / 32;
-                const int64_t a = P.lo[1] + 4 * (t1_lo - n2), b = min(P.lo[1] + 4 * (t1_hi - n2), P.hi[1]);
-                unsigned mk[W1];
-                active_masks<Q, W1>(P, a, b, mk);
-#pragma unroll
-                for (int w = 0; w < W1; ++w)
-                    if (mk[w]) run_groups_active<Q, 8, 8>(P, a + 32 * w, mk[w], n);
-            }
-            const int64_t t0_lo = max(t, n2 + t1);
-            if (t0_lo < te) {
-                constexpr int W0 = (kWarpChunk * 8 + 31) / 32;
-                const int64_t a = P.lo[0] + 8 * (t0_lo - n2 - t1), b = min(P.lo[0] + 8 * (te - n2 - t1), P.hi[0]);
-                unsigned mk[W0];
-                active_masks<Q, W0>(P, a, b, mk);
-#pragma unroll
-                for (int w = 0; w < W0; ++w)
-                    if (mk[w]) run_groups_active<Q, 4, 2>(P, a + 32 * w, mk[w], n);
-            }
-        } else {
-            const int64_t e2 = min(te, n2);
-            if (t < e2) {
-                // warp rows: the next row's work item is loaded before this one runs
-                nd_item it = load_item(P.items, P.lo[2] + t);
-                while (t < e2) {
-                    nd_item nx;
-                    if (t + 1 < e2) nx = load_item(P.items, P.lo[2] + t + 1);
-                    run_warp_row<Q, AND, NOTIFY, GB, HW>(P, it, bins, n);
-                    it = nx;
-                    ++t;
-                }
-            }
-            for (; t < te; ++t) {
-                if (t < n2 + t1) {
-                    const int64_t first = P.lo[1] + 4 * (t - n2);
-                    run_groups<Q, 8, 8, AND, GB>(P, first, min(first + 4, P.hi[1]), n);
-                } else {
-                    const int64_t first = P.lo[0] + 8 * (t - n2 - t1);
-                    run_groups<Q, 4, 2, AND, GB>(P, first, min(first + 8, P.hi[0]), n);
-                }
+        }
+        for (; t < te; ++t) {
+            if (t < n2 + t1) {
+                const int64_t first = 4 * (t - n2);
+                run_groups<Q, 8, 8, AND, NOTIFY, GB>(P, lo(1) + first, lo(1) + min(first + 4, n1), n);
+            } else {
+                const int64_t first = 8 * (t - n2 - t1);
+                run_groups<Q, 4, 2, AND, NOTIFY, GB>(P, lo(0) + first, lo(0) + min(first + 8, n0), n);
             }
         }
     }
@@ -1329,7 +1342,7 @@ __global__ void __launch_bounds__(kThreads, kPassBlocks) k_pass_otf(SweepParams 
     const int64_t n3 = P.hi[3] - P.lo[3], n2 = P.hi[2] - P.lo[2], g2 = (n2 + kOtfChunk2 - 1) / kOtfChunk2;
     for (;;) {
         unsigned long long c = 0;
-        if (lane == 0) c = atomicAdd(P.ctr + 4, 1ull);
+        if (lane == 0) c = atomicAdd(P.ctr + ND_CTR_CHUNK, 1ull);
         c = __shfl_sync(0xffffffffu, c, 0);
         // the grab's rows [r0, r0 + take): one at a time of the CTA bucket,
         // kOtfChunk2 of the warp bucket, then kOtfChunk
@@ -1354,7 +1367,7 @@ __global__ void __launch_bounds__(kThreads, kPassBlocks) k_pass_otf(SweepParams 
             const nd_item it = load_item(P.items, first + rows - 1 - r0 - lane);
             R = it.R;
             d = it.d;
-            if (AND && NOTIFY) run = in_frontier<2>(P, R);
+            if (AND && NOTIFY) run = in_frontier(P, R);
         }
         if (run) {
             my_t0 = ld_tau<!AND>(P.tin + R);
@@ -1516,18 +1529,6 @@ int pass_grid(const nd_incidence* h, const void* fn, int64_t units) {
     return (int)(g < 1 ? 1 : g);
 }
 
-// warp tasks per counter grab: kWarpChunk where there are many, fewer where
-// that would leave the resident warps with less than kChunksPerWarp grabs
-// each.  A graph of 2,000 vertices has 250 tasks: in chunks of 16 they kept 16
-// warps busy, one after the other (26 us per pass).  R-MAT of 100,003 vertices:
-// the first 16 SND passes 3.2 ms with 8 grabs, 3.9 with 4, 3.2 with 16 (whose
-// late passes are 12% slower).
-constexpr int kChunksPerWarp = 8;
-int pass_chunk(int64_t tasks, int grid) {
-    const int64_t c = tasks / ((int64_t)(grid > 0 ? grid : 1) * (kThreads / 32) * kChunksPerWarp);
-    return (int)(c < 1 ? 1 : (c > kWarpChunk ? kWarpChunk : c));
-}
-
 nd_status ensure_state(nd_incidence* h, bool and_mode, cudaStream_t st) {
     const int64_t N = h->num_r > 0 ? h->num_r : 1;
     if (!h->tau[0]) ND_TRY(nd_alloc((void**)&h->tau[0], sizeof(int32_t) * N, st, h));
@@ -1550,6 +1551,74 @@ nd_status ensure_state(nd_incidence* h, bool and_mode, cudaStream_t st) {
     return ND_OK;
 }
 
+
+// AND with notification: the list of a pass (k_active_list).  A handle keeps
+// room for all of its work items; where it may not (the memory limit), a run
+// takes a sixteenth of that as scratch and makes each pass in parts.
+struct ListPlan {
+    int64_t tile_lo[ND_NB + 1] = {0, 0, 0, 0, 0};
+    int64_t tiles = 0, room = 0;  // all tiles; those a list holds
+    uint32_t* list = nullptr;
+    int64_t words = 0;  // of the next frontier
+};
+
+nd_status plan_list(nd_incidence* h, int64_t words, nd_tmp<uint32_t>& scratch, ListPlan* L, cudaStream_t st) {
+    for (int b = 0; b < ND_NB; ++b)
+        L->tile_lo[b + 1] = L->tile_lo[b] + (h->bucket_lo[b + 1] - h->bucket_lo[b] + kListTile - 1) / kListTile;
+    L->tiles = L->tile_lo[ND_NB];
+    L->words = words;
+    if (L->tiles == 0) return ND_OK;
+    if (h->list && h->list_tiles < L->tiles) {  // other buckets than before
+        nd_release(h->list, st);
+        h->bytes -= h->list_tiles * kListTile * (int64_t)sizeof(uint32_t);
+        h->list = nullptr;
+    }
+    if (!h->list && nd_alloc((void**)&h->list, sizeof(uint32_t) * kListTile * L->tiles, st, h) == ND_OK)
+        h->list_tiles = L->tiles;
+    L->list = h->list;
+    L->room = L->tiles;
+    if (!h->list) {
+        nd_set_error("");
+        L->room = (L->tiles + 15) / 16;
+        ND_TRY(scratch.alloc(L->room * kListTile));
+        L->list = scratch;
+    }
+    return ND_OK;
+}
+
+typedef void (*list_fn)(ListParams);
+list_fn pick_list(const nd_incidence* h) {
+    return h->q == 2 ? k_active_list<2> : (h->t_pos ? k_active_list<3> : k_active_list<1>);
+}
+
+// the parameters of the list of the tiles [first, last) for the pass P, whose
+// list ranges it sets; returns the blocks to launch
+int list_params(const nd_incidence* h, const ListPlan& L, int64_t first, int64_t last, SweepParams& P, ListParams* out) {
+    out->epos = P.epos;
+    out->tpos = P.tpos;
+    out->items = P.items;
+    out->cur = P.cur;
+    out->next = P.next;
+    out->words = first == 0 ? L.words : 0;
+    for (int b = 0; b <= ND_NB; ++b) {
+        out->lo[b] = h->bucket_lo[b];
+        out->tile_lo[b] = L.tile_lo[b];
+    }
+    out->first = first;
+    out->last = last;
+    out->list = L.list;
+    out->ctr = P.ctr;
+    out->prev = P.prev;
+    P.list = L.list;
+    for (int b = 0; b < ND_NB; ++b) {
+        const int64_t lo = L.tile_lo[b] > first ? L.tile_lo[b] : first;
+        P.list_lo[b] = (lo - first) * kListTile;  // unused where the bucket has no tile here
+    }
+    const int cap = (h->sm_count > 0 ? h->sm_count : 152) * 8;
+    const int for_words = nd_blocks_for(out->words, kThreads * 16, cap);
+    const int for_tiles = (int)(last - first < cap ? last - first : cap);
+    return for_tiles > for_words ? for_tiles : for_words;
+}
 
 // the smallest shared-memory carve-out (percent of the SM's maximum) that
 // holds the resident blocks of a pass kernel (all are built for kPassBlocks)
@@ -1610,7 +1679,7 @@ SweepParams pass_params(const nd_incidence* h, int mode, const SweepParams& P0, 
 // capture) so that it also serves the legacy default stream.  On any
 // failure the handle falls back to ordinary launches for this kind.
 void make_batch_graph(nd_incidence* h, int mode, int kind, const SweepParams& P0, int grid0, pass_fn fn0,
-                      int grid1, pass_fn fn1, int64_t words) {
+                      int grid1, pass_fn fn1, const ListPlan& L) {
     const int base = (kind == 2) ? ND_BATCH : 0;
     cudaGraph_t g = nullptr;
     cudaGraphExec_t ex = nullptr;
@@ -1631,14 +1700,16 @@ void make_batch_graph(nd_incidence* h, int mode, int kind, const SweepParams& P0
         const int prev_slot = k > 0 ? base + k - 1 : (kind == 0 ? -1 : (base ^ ND_BATCH) + ND_BATCH - 1);
         SweepParams P = pass_params(h, mode, P0, base + k, prev_slot, k & 1, mode != ND_SND && kind == 0 && k < kAndDirect);
         if (mode == ND_AND) {
-            cudaMemsetParams ms = {};
-            ms.dst = P.next;
-            ms.value = 0;
-            ms.elementSize = 4;
-            ms.width = (size_t)words;
-            ms.height = 1;
+            ListParams lp;
+            const int blocks = list_params(h, L, 0, L.tiles, P, &lp);
+            cudaKernelNodeParams kp = {};
+            void* args[] = {&lp};
+            kp.func = (void*)pick_list(h);
+            kp.gridDim = dim3(blocks);
+            kp.blockDim = dim3(kThreads);
+            kp.kernelParams = args;
             cudaGraphNode_t n = nullptr;
-            ok = cudaGraphAddMemsetNode(&n, g, &last, 1, &ms) == cudaSuccess;
+            ok = cudaGraphAddKernelNode(&n, g, &last, 1, &kp) == cudaSuccess;
             last = n;
         }
         if (ok && P.gid) {  // batches: the graphs changing in this pass, from none
@@ -1855,6 +1926,8 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
     SweepParams P;
     P.inc = h->inc;
     P.epos = h->e_pos;
+    P.list = nullptr;
+    for (int b = 0; b < ND_NB; ++b) P.list_lo[b] = 0;
     P.tpos = h->t_pos;
     P.eid = h->t_pos ? h->t_id : h->eid;
     P.rp = h->rp;
@@ -1896,7 +1969,10 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
     const int64_t units = pass_units(h, P);
     const int grid0 = units > 0 ? pass_grid(h, (const void*)fn0, units) : 0;
     const int grid1 = units > 0 ? pass_grid(h, (const void*)fn1, units) : 0;
-    P.chunk = pass_chunk(units - (P.hi[3] - P.lo[3]), grid0 < grid1 ? grid0 : grid1);
+    P.chunk = warp_chunk(units - (P.hi[3] - P.lo[3]), grid0 < grid1 ? grid0 : grid1);
+    ListPlan L;
+    nd_tmp<uint32_t> list_scratch(st);
+    if (mode == ND_AND && !h->otf) ND_TRY(plan_list(h, words, list_scratch, &L, st));
     // passes that evaluate every row do not count rows and incidences (Tally)
     const bool counted = h->otf || mode == ND_AND || P.gid;
     const int64_t all_rows = P.hi[ND_NB - 1] - P.lo[0], all_incs = h->num_inc;
@@ -1932,9 +2008,9 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
         // handles run each mode once
         const bool seen = h->batch_seen[mode][kind];
         if (nb == kBatch) h->batch_seen[mode][kind] = true;
-        if (nb == kBatch && seen && grid0 > 0 && !members && !tau_in_dev && !h->otf && (start & 1) == 0 && !h->pass_graph_failed[mode][kind]) {
+        if (nb == kBatch && seen && grid0 > 0 && !members && !tau_in_dev && !h->otf && L.room == L.tiles && (start & 1) == 0 && !h->pass_graph_failed[mode][kind]) {
             if (!h->pass_graph[mode][kind])
-                make_batch_graph(h, mode, kind, P, grid0, fn0, grid1, fn1, words);
+                make_batch_graph(h, mode, kind, P, grid0, fn0, grid1, fn1, L);
             if (h->pass_graph[mode][kind]) {
                 // the graph's first pass reads the last slot of the other half
                 const int want = (base ^ ND_BATCH) + ND_BATCH - 1;
@@ -1952,14 +2028,26 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
             for (int k = 0; k < nb; ++k, ++pass) {
                 SweepParams Pk = pass_params(h, mode, P, base + k, k > 0 ? base + k - 1 : last_slot, pass & 1,
                                              mode != ND_SND && pass < kAndDirect);
-                if (mode == ND_AND)
-                    ND_CUDA(cudaMemsetAsync(Pk.next, 0, sizeof(uint32_t) * words, st));
                 if (Pk.gid) ND_CUDA(cudaMemsetAsync(Pk.gact_out, 0, (size_t)h->ngraphs, st));
-                if (grid0 > 0) {
-                    const bool late = pass >= kLateFrom;
-                    nd_prof_scope ps(pname, st);
+                if (mode == ND_AND && h->otf)
+                    ND_CUDA(cudaMemsetAsync(Pk.next, 0, sizeof(uint32_t) * words, st));
+                if (grid0 == 0) continue;
+                const bool late = pass >= kLateFrom, listed = mode == ND_AND && !h->otf;
+                // the parts of a pass: one, unless the list has no room for all
+                for (int64_t t = 0; t == 0 || (listed && t < L.tiles); t += L.room) {
+                    nd_prof_scope ps(pname, st, listed ? 2 : 1);
+                    if (listed) {
+                        if (t > 0)
+                            ND_CUDA(cudaMemsetAsync(Pk.ctr + ND_CTR_CTA, 0,
+                                                    sizeof(unsigned long long) * (ND_SLOT - ND_CTR_CTA), st));
+                        ListParams lp;
+                        const int blocks = list_params(h, L, t, t + L.room < L.tiles ? t + L.room : L.tiles, Pk, &lp);
+                        pick_list(h)<<<blocks, kThreads, 0, st>>>(lp);
+                        ND_CUDA(cudaGetLastError());
+                    }
                     (late ? fn1 : fn0)<<<late ? grid1 : grid0, kThreads, 0, st>>>(Pk);
                     ND_CUDA(cudaGetLastError());
+                    if (!listed) break;
                 }
             }
             ND_CUDA(cudaMemcpyAsync(h->h_counters + ND_SLOT * base, h->counters + ND_SLOT * base,
@@ -1969,8 +2057,9 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
         ND_TRY(nd_wait(st));
         for (int k = 0; k < nb; ++k) {
             const int32_t p = start + k;
-            unsigned long long ch = h->h_counters[ND_SLOT * (base + k)];
-            unsigned long long ev = counted ? h->h_counters[ND_SLOT * (base + k) + 1] : (unsigned long long)all_rows;
+            unsigned long long ch = h->h_counters[ND_SLOT * (base + k) + ND_CTR_CHANGED];
+            unsigned long long ev =
+                counted ? h->h_counters[ND_SLOT * (base + k) + ND_CTR_EVALS] : (unsigned long long)all_rows;
             // r-cliques with d_s = 0 are never launched: tau = H(empty) = 0 = d_s.
             // They count as evaluated in every SND / AND-nn pass and in the first
             // AND pass, as in the paper's sequential loops (in a batch, whose
@@ -1978,14 +2067,14 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
             if ((mode != ND_AND && !h->gid) || p == 0) ev += (unsigned long long)h->num_zero;
             h->last_changed.push_back((int64_t)ch);
             h->last_evals.push_back((int64_t)ev);
-            h->last_incs.push_back(counted ? (int64_t)h->h_counters[ND_SLOT * (base + k) + 3] : all_incs);
+            h->last_incs.push_back(counted ? (int64_t)h->h_counters[ND_SLOT * (base + k) + ND_CTR_INCS] : all_incs);
             *evals += (int64_t)ev;
             if (!and_mode) last_written = (p & 1) ^ 1;
             if (ch == 0) { done = true; break; }
             (*updating)++;
             // active-ratio rule (Section 5.2, Fig. 9): the fraction of r-cliques
             // evaluated in this pass predicts how close tau is to kappa
-            const double active = (double)h->h_counters[ND_SLOT * (base + k) + 1] / (double)N;
+            const double active = (double)h->h_counters[ND_SLOT * (base + k) + ND_CTR_EVALS] / (double)N;
             if (stop_active > 0.0 && active < stop_active) {
                 opts->stopped = true;
                 done = true;

@@ -137,6 +137,8 @@ struct nd_incidence {
     // iteration state
     int32_t* tau[2] = {nullptr, nullptr};
     uint32_t* front[2] = {nullptr, nullptr};
+    uint32_t* list = nullptr;                // AND: the active work items of a pass
+    int64_t list_tiles = 0;                  // tiles of work items it holds
     unsigned long long* counters = nullptr;  // ring of per-pass counters
     unsigned long long* h_counters = nullptr;  // pinned host mirror, at the head of the handle's pinned block
     int64_t* h_read = nullptr;                 // ND_READ pinned words after it, for counts read back in the build
@@ -179,7 +181,9 @@ struct nd_claim {
 
 // passes are enqueued in batches of ND_BATCH; the per-pass counters (ND_SLOT
 // u64 each) live in two halves of ND_BATCH slots used by alternate batches
-enum { ND_BATCH = 16, ND_RING = 2 * ND_BATCH, ND_SLOT = 6 };
+enum { ND_BATCH = 16, ND_RING = 2 * ND_BATCH, ND_SLOT = 9 };
+// a slot: results first, then what the kernels of the pass count with
+enum { ND_CTR_CHANGED = 0, ND_CTR_EVALS = 1, ND_CTR_INCS = 2, ND_CTR_CTA = 3, ND_CTR_CHUNK = 4, ND_CTR_LIST = 5 };
 enum { ND_READ = 64 };
 
 // a pinned block for a handle's counters and read-backs, from a bounded pool

@@ -62,7 +62,7 @@ def footprint_bytes(row_ptr: np.ndarray, col: np.ndarray, r: int) -> int:
             q = 3
             base += 48 * num_r  # triangle lists and their slots; then slots, ids and 16-bit copies
         base += 12 * (nnz // 2)
-    return int(base + 8 * (num_r + 1) + copies * 4 * q * inc + 16 * num_r + 8 * num_r + num_r // 4 + (1 << 20))
+    return int(base + 8 * (num_r + 1) + copies * 4 * q * inc + 28 * num_r + num_r // 4 + (1 << 20))
 
 
 @dataclass(eq=False)

@@ -121,3 +121,29 @@ def test_nuclei_by_triangle_ids(nd):
     assert held_ids < held - 20 * len(want[0]) and passes_ids == passes
     for a, b in zip(got, want):
         np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("r", [1, 2, 3])
+def test_active_list_in_parts(nd, r):
+    """AND with notification whose handle has no room for the list of active
+    rows makes every pass in parts, from a sixteenth of it."""
+    n, s, d = G.rmat(13 if r < 3 else 11, 12, seed=83)
+    rp, col = G.to_csr(n, s, d)
+    drp, dcol = torch.from_numpy(rp).cuda(), torch.from_numpy(col).cuda()
+    inc = nd.build_incidence(drp, dcol, r, r + 1)
+    want = inc.and_()[0].cpu().numpy()
+    np.testing.assert_array_equal(want, oracle.Graph(rp, col, r, r + 1).peel())
+    held = inc.incidence_bytes()
+    members = torch.arange(0, inc.num_r, 7, dtype=torch.int32, device="cuda")
+    part = inc.and_partial(members)[0].cpu().numpy()
+    try:
+        nd.set_handle_memory_limit(held - 4)
+        tight = nd.build_incidence(drp, dcol, r, r + 1)
+        for _ in range(3):  # the second run of a mode would take a graph
+            tau, _, evals = tight.and_()
+            np.testing.assert_array_equal(tau.cpu().numpy(), want)
+            assert evals >= len(want)
+        np.testing.assert_array_equal(tight.and_partial(members)[0].cpu().numpy(), part)
+        assert tight.incidence_bytes() < held
+    finally:
+        nd.set_handle_memory_limit(0)

@@ -1011,6 +1011,13 @@ __host__ __device__ __forceinline__ int warp_chunk(int64_t tasks, int grid) {
     return (int)(c < 1 ? 1 : (c > kWarpChunk ? kWarpChunk : c));
 }
 
+// AND ends its passes on the longest warp rows: the last kTailTasks tasks of
+// every resident warp come in chunks of kTailChunk, so that no warp is left
+// with a chunk of them.  AND without notification, the first eight passes, in
+// whole chunks / with the tail: 2.76 / 2.13 ms for R-MAT of 100,003 vertices,
+// 27.4 / 25.8 ms for scale 20 (k-truss).
+constexpr int kTailTasks = 8, kTailChunk = 2;
+
 constexpr int kPassBlocks = 6;  // resident blocks per SM the register budget of every pass kernel targets
 
 // GB: a batch handle's SND / AND-nn pass, which skips the rows of graphs
@@ -1048,15 +1055,13 @@ __global__ void __launch_bounds__(kThreads, kPassBlocks) k_pass(SweepParams P) {
     };
     // AND updates in place, so a row evaluated later in a pass already sees
     // what earlier rows lowered: AND takes the shortest rows first and the
-    // CTA rows last (measured 3% faster than longest first on R-MAT scale 20
-    // k-truss).  SND, whose pass reads only the previous pass, takes the
-    // longest rows first, for balance.  A k-core's CTA rows are the hub
-    // vertices, up to hundreds of thousands of entries each, and one block
-    // streams a row: taken last, they kept a few blocks busy long after the
-    // rest of the pass had finished (18% of the AND time of an R-MAT scale
-    // 26 k-core in ncu), so (1,2) AND takes them first.
-    constexpr bool kShortFirst = AND;
-    constexpr bool kCtaFirst = !AND || Q == 1;
+    // CTA rows last (the first eight passes with notification on the R-MAT
+    // scale-20 k-truss: 33.2 against 34.4 ms longest first).  SND, whose pass
+    // reads only the previous pass, takes the longest rows first, for balance,
+    // and so does (1,2), whose longest rows are hub vertices of up to hundreds
+    // of thousands of entries (R-MAT scale-24 k-core: 15.1 against 15.6 ms).
+    constexpr bool kShortFirst = AND && Q != 1;
+    constexpr bool kCtaFirst = !kShortFirst;
     if (kCtaFirst) cta_phase();
     // phase 2: warp tasks (one warp row, four 8-lane rows or eight 4-lane
     // rows), longest first (SND) or shortest first (AND).  Each warp takes
@@ -1068,15 +1073,24 @@ __global__ void __launch_bounds__(kThreads, kPassBlocks) k_pass(SweepParams P) {
     const int64_t tasks = n2 + t1 + t0;
     const int lane32 = threadIdx.x & 31;
     const int chunk = NOTIFY ? warp_chunk(tasks, gridDim.x) : P.chunk;
-    const int64_t nchunks = (tasks + chunk - 1) / chunk;
+    // the last tasks in small chunks
+    const int64_t tail = kShortFirst ? min(tasks, (int64_t)gridDim.x * (kThreads / 32) * kTailTasks) : 0;
+    const int tc = min(kTailChunk, chunk);
+    const int64_t big = (tasks - tail + chunk - 1) / chunk;
+    const int64_t nchunks = big + (tail + tc - 1) / tc;
     for (;;) {
         unsigned long long c = 0;
         if (lane32 == 0) c = atomicAdd(P.ctr + ND_CTR_CHUNK, 1ull);
         c = __shfl_sync(0xffffffffu, c, 0);
         if ((int64_t)c >= nchunks) break;
-        const int64_t cc = kShortFirst ? nchunks - 1 - (int64_t)c : (int64_t)c;
-        int64_t t = cc * chunk;
-        const int64_t te = min(t + (int64_t)chunk, tasks);
+        // [t, te) in the order of the pass
+        int64_t t = (int64_t)c < big ? (int64_t)c * chunk : tasks - tail + ((int64_t)c - big) * tc;
+        int64_t te = (int64_t)c < big ? min(t + (int64_t)chunk, tasks - tail) : min(t + (int64_t)tc, tasks);
+        if (kShortFirst) {
+            const int64_t x = tasks - te;
+            te = tasks - t;
+            t = x;
+        }
         const int64_t e2 = min(te, n2);
         if (t < e2) {
             // warp rows: the next row's work item is loaded before this one runs

@@ -139,8 +139,8 @@ struct SweepParams {
     const uint32_t* __restrict__ gid;
     const uint8_t* gact_in;
     uint8_t* gact_out;
-    // AND with notification: the active work items, and where each bucket's
-    // begin there (their numbers are in ctr)
+    // AND with notification and batches: the active work items, and where each
+    // bucket's begin there (their numbers are in ctr)
     const uint32_t* __restrict__ list;
     int64_t list_lo[ND_NB];
     unsigned long long* ctr;         // this pass's counters (ND_CTR_*)
@@ -701,15 +701,6 @@ __device__ __forceinline__ void notify_entry(const SweepParams& P, int64_t jb, i
     notify_block<Q, 1>(P, id, ok, h);
 }
 
-// batches (GB): has R's graph converged (no change in its previous pass)?
-// Its rows then keep their tau, as the graph's own run would have stopped.
-// The single-graph kernels (GB = false) carry no test at all.
-template <bool GB>
-__device__ __forceinline__ bool graph_done(const SweepParams& P, uint32_t R) {
-    if constexpr (GB) return !P.gact_in[__ldg(P.gid + R)];
-    return false;
-}
-
 // batches: R changed, so its graph is still changing
 template <bool GB>
 __device__ __forceinline__ void graph_changed(const SweepParams& P, uint32_t R) {
@@ -725,10 +716,9 @@ __device__ __forceinline__ nd_item load_item(const nd_item* __restrict__ items, 
     return it;
 }
 
-// counters of one thread over a pass.  FULL (batches, no-storage passes):
-// evaluated rows and their incidences too; k_active_list counts them for AND
-// with notification, and the other passes evaluate every row, so the host
-// knows both.
+// counters of one thread over a pass.  FULL (no-storage passes): evaluated
+// rows and their incidences too; k_active_list counts them for the passes that
+// take its list, and the others evaluate every row, so the host knows both.
 template <bool FULL>
 struct Tally {
     unsigned changed = 0, evals = 0;
@@ -753,24 +743,20 @@ __device__ __forceinline__ void load_tau(const SweepParams& P, const nd_item& it
     t = min(t0, (int32_t)min(it.d, (uint32_t)INT32_MAX));
 }
 
-// work item i of a pass: AND with notification takes them from its list
-template <bool NOTIFY>
+// work item i of a pass, or of its list
+template <bool LISTED>
 __device__ __forceinline__ nd_item pass_item(const SweepParams& P, int64_t i) {
-    return load_item(P.items, NOTIFY ? (int64_t)__ldg(P.list + i) : i);
+    return load_item(P.items, LISTED ? (int64_t)__ldg(P.list + i) : i);
 }
 
-// work items [first, last): one r-clique per group of G lanes of the calling
-// warp, at most 32/G of them.  NOTIFY: the entries of all rows that changed
-// are then walked by the 32 lanes together, instead of each row by its own G
-// lanes while the other groups wait.
-template <int Q, int G, int C, bool AND, bool NOTIFY, bool GB, bool FULL>
-__device__ __forceinline__ void run_groups(const SweepParams& P, int64_t first, int64_t last, Tally<FULL>& n) {
+// one r-clique per group of G lanes of the calling warp (run: the group has
+// one).  NOTIFY: the entries of all rows that changed are then walked by the
+// 32 lanes together, instead of each row by its own G lanes while the other
+// groups wait.
+template <int Q, int G, int C, bool AND, bool NOTIFY, bool GB>
+__device__ __forceinline__ void run_groups(const SweepParams& P, const nd_item& it, bool run, Tally<false>& n) {
     constexpr int NG = 32 / G;
     const int lane = threadIdx.x & 31;
-    const int64_t i = first + lane / G;
-    const bool ok = i < last;
-    const nd_item it = pass_item<NOTIFY>(P, ok ? i : first);
-    const bool run = ok && !graph_done<GB>(P, it.R);
     int32_t t0, t, old;
     load_tau<AND>(P, it, t0, t, old);
     const int d = run ? (int)it.d : 0;
@@ -810,11 +796,10 @@ __device__ __forceinline__ void run_groups(const SweepParams& P, int64_t first, 
 }
 
 // one r-clique per warp (rows of the warp bucket), streamed
-template <int Q, bool AND, bool NOTIFY, bool GB, int HW, bool FULL>
+template <int Q, bool AND, bool NOTIFY, bool GB, int HW>
 __device__ __forceinline__ void run_warp_row(const SweepParams& P, const nd_item& it, unsigned* bins,
-                                             Tally<FULL>& n) {
+                                             Tally<false>& n) {
     const uint32_t R = it.R;
-    if (graph_done<GB>(P, R)) return;
     int32_t t0, t, old;
     load_tau<AND>(P, it, t0, t, old);
     const bool direct = P.direct || (!AND && old != t0);
@@ -836,12 +821,11 @@ __device__ __forceinline__ void run_warp_row(const SweepParams& P, const nd_item
 }
 
 // one r-clique per CTA (rows past the warp threshold)
-template <int Q, bool AND, bool NOTIFY, bool GB, int WORDS, bool FULL>
+template <int Q, bool AND, bool NOTIFY, bool GB, int WORDS>
 __device__ __forceinline__ void run_cta(const SweepParams& P, int64_t i, unsigned* bins, int* bounds,
-                                        Tally<FULL>& n) {
-    const nd_item it = pass_item<NOTIFY>(P, i);
+                                        Tally<false>& n) {
+    const nd_item it = pass_item<NOTIFY || GB>(P, i);
     const uint32_t R = it.R;
-    if (graph_done<GB>(P, R)) return;  // the same R for the whole block
     int32_t t0, t, old;
     load_tau<AND>(P, it, t0, t, old);
     __syncthreads();  // AND: every thread has read tau(R) before it is written
@@ -869,8 +853,9 @@ __device__ __forceinline__ void run_cta(const SweepParams& P, int64_t i, unsigne
     __syncthreads();
 }
 
-// AND with notification, before each pass: the work items whose r-clique is in
-// the frontier, compacted bucket by bucket, in order inside a tile; the pass
+// Before each pass of AND with notification: the work items whose r-clique is
+// in the frontier (of a batch's SND and AND-nn passes: whose graph changed in
+// the pass before), compacted bucket by bucket, in order inside a tile; the pass
 // then takes dense tasks from the list, and splits few rows over all warps.
 // (With the frontier tested by each warp for its own chunk of work items, a
 // chunk of long rows that happened to be active together kept one warp busy:
@@ -882,6 +867,8 @@ constexpr int kListTile = 2048;
 struct ListParams {
     const uint2* __restrict__ epos;
     const uint32_t* __restrict__ tpos;
+    const uint32_t* __restrict__ gid;  // batches: the graph of every r-clique, and the graphs still changing
+    const uint8_t* gact_in;
     const nd_item* __restrict__ items;
     const uint32_t* cur;
     uint32_t* next;
@@ -894,6 +881,7 @@ struct ListParams {
     const unsigned long long* prev;
 };
 
+constexpr int kByGraph = 0;  // k_active_list: by graph instead of by frontier bit (Q)
 template <int Q>
 __global__ void __launch_bounds__(kThreads) k_active_list(ListParams L) {
     if (L.prev != nullptr && *(volatile const unsigned long long*)L.prev == 0ull) return;  // converged
@@ -917,7 +905,13 @@ __global__ void __launch_bounds__(kThreads) k_active_list(ListParams L) {
             R[k] = x.x;
             d[k] = x.y;  // 0: past the bucket
         }
-        if constexpr (Q == 2) {
+        if constexpr (Q == kByGraph) {
+            uint32_t g[K];
+#pragma unroll
+            for (int k = 0; k < K; ++k) g[k] = __ldg(L.gid + R[k]);
+#pragma unroll
+            for (int k = 0; k < K; ++k) act[k] = d[k] && L.gact_in[g[k]];
+        } else if constexpr (Q == 2) {
             uint2 ep[K];
 #pragma unroll
             for (int k = 0; k < K; ++k) ep[k] = __ldg(L.epos + R[k]);
@@ -1018,27 +1012,33 @@ __host__ __device__ __forceinline__ int warp_chunk(int64_t tasks, int grid) {
 // 27.4 / 25.8 ms for scale 20 (k-truss).
 constexpr int kTailTasks = 8, kTailChunk = 2;
 
+// lanes of a group, and entries per lane of its longest row
+template <int G, int C>
+struct GroupOf {
+    static constexpr int lanes = G, entries = C;
+};
+
 constexpr int kPassBlocks = 6;  // resident blocks per SM the register budget of every pass kernel targets
 
-// GB: a batch handle's SND / AND-nn pass, which skips the rows of graphs
-// that have converged
+// GB: a batch handle's SND / AND-nn pass, which leaves out the rows of graphs
+// that have converged, and marks those that change
 // LATE: the passes after the first of a run, where few rows search: a
 // quarter of the histogram, and the shared memory it frees serves as L1 for
 // the gathers
 template <int Q, bool AND, bool NOTIFY, bool GB, bool LATE>
 __global__ void __launch_bounds__(kThreads, kPassBlocks) k_pass(SweepParams P) {
     if (P.prev != nullptr && *(volatile const unsigned long long*)P.prev == 0ull) return;  // converged
-    constexpr bool FULL = GB;
+    constexpr bool LISTED = NOTIFY || GB;
     constexpr int HW = LATE ? kLateHistWords : kHistWords;
     constexpr int kWords = (kThreads / 32) * HW;  // a CTA row uses every warp's histogram
     __shared__ __align__(16) unsigned hist[kThreads / 32][HW];
     __shared__ int bounds[kThreads / 32];
     __shared__ unsigned long long s_chunk;
     unsigned* const bins = hist[threadIdx.x >> 5];
-    Tally<FULL> n;
+    Tally<false> n;
     // the rows of each bucket: [lo, lo + rows) of the work items, or of the list
-    auto lo = [&](int b) { return NOTIFY ? P.list_lo[b] : P.lo[b]; };
-    auto rows = [&](int b) { return NOTIFY ? (int64_t)__ldcg(P.ctr + ND_CTR_LIST + b) : P.hi[b] - P.lo[b]; };
+    auto lo = [&](int b) { return LISTED ? P.list_lo[b] : P.lo[b]; };
+    auto rows = [&](int b) { return LISTED ? (int64_t)__ldcg(P.ctr + ND_CTR_LIST + b) : P.hi[b] - P.lo[b]; };
     // phase 1: rows longer than the CTA threshold, one per block at a time,
     // taken from a per-pass counter (longest rows first)
     const int64_t n3 = rows(3);
@@ -1072,7 +1072,7 @@ __global__ void __launch_bounds__(kThreads, kPassBlocks) k_pass(SweepParams P) {
     const int64_t t1 = (n1 + 3) / 4, t0 = (n0 + 7) / 8;
     const int64_t tasks = n2 + t1 + t0;
     const int lane32 = threadIdx.x & 31;
-    const int chunk = NOTIFY ? warp_chunk(tasks, gridDim.x) : P.chunk;
+    const int chunk = LISTED ? warp_chunk(tasks, gridDim.x) : P.chunk;
     // the last tasks in small chunks
     const int64_t tail = kShortFirst ? min(tasks, (int64_t)gridDim.x * (kThreads / 32) * kTailTasks) : 0;
     const int tc = min(kTailChunk, chunk);
@@ -1094,24 +1094,37 @@ __global__ void __launch_bounds__(kThreads, kPassBlocks) k_pass(SweepParams P) {
         const int64_t e2 = min(te, n2);
         if (t < e2) {
             // warp rows: the next row's work item is loaded before this one runs
-            nd_item it = pass_item<NOTIFY>(P, lo(2) + t);
+            nd_item it = pass_item<LISTED>(P, lo(2) + t);
             while (t < e2) {
                 nd_item nx;
-                if (t + 1 < e2) nx = pass_item<NOTIFY>(P, lo(2) + t + 1);
+                if (t + 1 < e2) nx = pass_item<LISTED>(P, lo(2) + t + 1);
                 run_warp_row<Q, AND, NOTIFY, GB, HW>(P, it, bins, n);
                 it = nx;
                 ++t;
             }
         }
-        for (; t < te; ++t) {
-            if (t < n2 + t1) {
-                const int64_t first = 4 * (t - n2);
-                run_groups<Q, 8, 8, AND, NOTIFY, GB>(P, lo(1) + first, lo(1) + min(first + 4, n1), n);
-            } else {
-                const int64_t first = 8 * (t - n2 - t1);
-                run_groups<Q, 4, 2, AND, NOTIFY, GB>(P, lo(0) + first, lo(0) + min(first + 8, n0), n);
+        // group rows, the same: the next task's items are loaded before this
+        // one runs (the first group's item stands in where a group has none).
+        // SND 2 to 4% faster; with notification, whose registers are short, 2
+        // to 5% slower, so not there.
+        auto group_tasks = [&](int64_t from, int64_t to, int64_t begin, int64_t count, auto group) {
+            constexpr int G = decltype(group)::lanes, NG = 32 / G;
+            if (from >= to) return;
+            auto item = [&](int64_t task) {
+                const int64_t i = NG * task + lane32 / G;
+                return pass_item<LISTED>(P, begin + (i < count ? i : NG * task));
+            };
+            nd_item it = item(from);
+            for (int64_t k = from; k < to; ++k) {
+                nd_item nx;
+                if (!NOTIFY && k + 1 < to) nx = item(k + 1);
+                run_groups<Q, G, decltype(group)::entries, AND, NOTIFY, GB>(P, it, NG * k + lane32 / G < count, n);
+                if (NOTIFY && k + 1 < to) nx = item(k + 1);
+                it = nx;
             }
-        }
+        };
+        group_tasks(max(t, n2) - n2, min(te, n2 + t1) - n2, lo(1), n1, GroupOf<8, 8>{});
+        group_tasks(max(t, n2 + t1) - n2 - t1, te - n2 - t1, lo(0), n0, GroupOf<4, 2>{});
     }
     if (!kCtaFirst) cta_phase();
     flush_tally(P, n);
@@ -1566,7 +1579,7 @@ nd_status ensure_state(nd_incidence* h, bool and_mode, cudaStream_t st) {
 }
 
 
-// AND with notification: the list of a pass (k_active_list).  A handle keeps
+// The list of a pass (k_active_list).  A handle keeps
 // room for all of its work items; where it may not (the memory limit), a run
 // takes a sixteenth of that as scratch and makes each pass in parts.
 struct ListPlan {
@@ -1601,7 +1614,8 @@ nd_status plan_list(nd_incidence* h, int64_t words, nd_tmp<uint32_t>& scratch, L
 }
 
 typedef void (*list_fn)(ListParams);
-list_fn pick_list(const nd_incidence* h) {
+list_fn pick_list(const nd_incidence* h, bool by_graph) {
+    if (by_graph) return k_active_list<kByGraph>;
     return h->q == 2 ? k_active_list<2> : (h->t_pos ? k_active_list<3> : k_active_list<1>);
 }
 
@@ -1610,10 +1624,12 @@ list_fn pick_list(const nd_incidence* h) {
 int list_params(const nd_incidence* h, const ListPlan& L, int64_t first, int64_t last, SweepParams& P, ListParams* out) {
     out->epos = P.epos;
     out->tpos = P.tpos;
+    out->gid = P.gid;
+    out->gact_in = P.gact_in;
     out->items = P.items;
     out->cur = P.cur;
     out->next = P.next;
-    out->words = first == 0 ? L.words : 0;
+    out->words = first == 0 && !P.gid ? L.words : 0;
     for (int b = 0; b <= ND_NB; ++b) {
         out->lo[b] = h->bucket_lo[b];
         out->tile_lo[b] = L.tile_lo[b];
@@ -1713,19 +1729,6 @@ void make_batch_graph(nd_incidence* h, int mode, int kind, const SweepParams& P0
         // of the other half (the caller puts the previous pass's counters there)
         const int prev_slot = k > 0 ? base + k - 1 : (kind == 0 ? -1 : (base ^ ND_BATCH) + ND_BATCH - 1);
         SweepParams P = pass_params(h, mode, P0, base + k, prev_slot, k & 1, mode != ND_SND && kind == 0 && k < kAndDirect);
-        if (mode == ND_AND) {
-            ListParams lp;
-            const int blocks = list_params(h, L, 0, L.tiles, P, &lp);
-            cudaKernelNodeParams kp = {};
-            void* args[] = {&lp};
-            kp.func = (void*)pick_list(h);
-            kp.gridDim = dim3(blocks);
-            kp.blockDim = dim3(kThreads);
-            kp.kernelParams = args;
-            cudaGraphNode_t n = nullptr;
-            ok = cudaGraphAddKernelNode(&n, g, &last, 1, &kp) == cudaSuccess;
-            last = n;
-        }
         if (ok && P.gid) {  // batches: the graphs changing in this pass, from none
             cudaMemsetParams ms = {};
             ms.dst = P.gact_out;
@@ -1735,6 +1738,19 @@ void make_batch_graph(nd_incidence* h, int mode, int kind, const SweepParams& P0
             ms.height = 1;
             cudaGraphNode_t n = nullptr;
             ok = cudaGraphAddMemsetNode(&n, g, &last, 1, &ms) == cudaSuccess;
+            last = n;
+        }
+        if (ok && (mode == ND_AND || P.gid)) {
+            ListParams lp;
+            const int blocks = list_params(h, L, 0, L.tiles, P, &lp);
+            cudaKernelNodeParams kp = {};
+            void* args[] = {&lp};
+            kp.func = (void*)pick_list(h, P.gid != nullptr);
+            kp.gridDim = dim3(blocks);
+            kp.blockDim = dim3(kThreads);
+            kp.kernelParams = args;
+            cudaGraphNode_t n = nullptr;
+            ok = cudaGraphAddKernelNode(&n, g, &last, 1, &kp) == cudaSuccess;
             last = n;
         }
         if (!ok) break;
@@ -1986,7 +2002,7 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
     P.chunk = warp_chunk(units - (P.hi[3] - P.lo[3]), grid0 < grid1 ? grid0 : grid1);
     ListPlan L;
     nd_tmp<uint32_t> list_scratch(st);
-    if (mode == ND_AND && !h->otf) ND_TRY(plan_list(h, words, list_scratch, &L, st));
+    if ((mode == ND_AND && !h->otf) || P.gid) ND_TRY(plan_list(h, words, list_scratch, &L, st));
     // passes that evaluate every row do not count rows and incidences (Tally)
     const bool counted = h->otf || mode == ND_AND || P.gid;
     const int64_t all_rows = P.hi[ND_NB - 1] - P.lo[0], all_incs = h->num_inc;
@@ -2046,7 +2062,7 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
                 if (mode == ND_AND && h->otf)
                     ND_CUDA(cudaMemsetAsync(Pk.next, 0, sizeof(uint32_t) * words, st));
                 if (grid0 == 0) continue;
-                const bool late = pass >= kLateFrom, listed = mode == ND_AND && !h->otf;
+                const bool late = pass >= kLateFrom, listed = (mode == ND_AND && !h->otf) || Pk.gid;
                 // the parts of a pass: one, unless the list has no room for all
                 for (int64_t t = 0; t == 0 || (listed && t < L.tiles); t += L.room) {
                     nd_prof_scope ps(pname, st, listed ? 2 : 1);
@@ -2056,7 +2072,7 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
                                                     sizeof(unsigned long long) * (ND_SLOT - ND_CTR_CTA), st));
                         ListParams lp;
                         const int blocks = list_params(h, L, t, t + L.room < L.tiles ? t + L.room : L.tiles, Pk, &lp);
-                        pick_list(h)<<<blocks, kThreads, 0, st>>>(lp);
+                        pick_list(h, Pk.gid != nullptr)<<<blocks, kThreads, 0, st>>>(lp);
                         ND_CUDA(cudaGetLastError());
                     }
                     (late ? fn1 : fn0)<<<late ? grid1 : grid0, kThreads, 0, st>>>(Pk);

@@ -137,7 +137,7 @@ struct nd_incidence {
     // iteration state
     int32_t* tau[2] = {nullptr, nullptr};
     uint32_t* front[2] = {nullptr, nullptr};
-    uint32_t* list = nullptr;                // AND: the active work items of a pass
+    uint32_t* list = nullptr;                // the active work items of a pass (AND; batches)
     int64_t list_tiles = 0;                  // tiles of work items it holds
     unsigned long long* counters = nullptr;  // ring of per-pass counters
     unsigned long long* h_counters = nullptr;  // pinned host mirror, at the head of the handle's pinned block

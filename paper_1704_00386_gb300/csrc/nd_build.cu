@@ -45,7 +45,76 @@ __device__ __forceinline__ int64_t warp_count_global() {
     return ((int64_t)gridDim.x * blockDim.x) >> 5;
 }
 
-// ---- validation and degree split (one warp per vertex) -------------------
+// ---- 32 rows per warp ------------------------------------------------------
+// Most rows of these graphs hold fewer entries than a warp has lanes.  The
+// kernels below therefore give a warp up to 32 consecutive rows: lane l loads what
+// leads to row l, and the entries of all are then walked as one sequence,
+// 32 at a time, every lane finding its entry's row by five steps over the
+// rows' prefix sums in shared memory.  Rows of more than kPoolRow entries go to
+// a second walk, one at a time and spread over all warps: consecutive rows are
+// of like length (degree classes, the edges of one hub), and 32 long ones would
+// keep one warp busy long after the others.  (A warp per row spent a chain of loads
+// on every row, empty ones included: 30 of the 97 ms of a batch of 256 small
+// graphs went to such kernels.)
+constexpr int kPoolRow = 128;
+// Rows per warp: 32 where that still gives every resident warp some, fewer
+// otherwise (a 2,800-vertex graph validated in 37 instead of 18 us with 32).
+int rows_per_warp(int64_t rows) {
+    const int64_t r = rows / (152 * 64);
+    return (int)(r < 1 ? 1 : (r > 32 ? 32 : r));
+}
+int pool_blocks(int64_t rows, int per, int cap) { return nd_blocks_for((rows + per - 1) / per * 32, kThreads, cap); }
+
+// the rows of [0, n) for which pick(row) holds, spread over the warps: f(row)
+template <typename P, typename F>
+__device__ __forceinline__ void spread_rows(int64_t n, P&& pick, F&& f) {
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = warp_count_global();
+    for (int64_t first = warp_id_global(); first < n; first += 32 * warps) {
+        const int64_t mine = first + lane * warps;
+        for (unsigned todo = __ballot_sync(kFull, mine < n && pick(mine)); todo; todo &= todo - 1)
+            f(first + (__ffs(todo) - 1) * warps);
+    }
+}
+
+struct row_pool {
+    uint32_t* pre;  // the warp's 32 words: entries before each row
+    int total;
+    // len: entries of this lane's row (their sum fits 31 bits)
+    __device__ __forceinline__ row_pool(uint32_t* words, int len) : pre(words) {
+        const int lane = threadIdx.x & 31;
+        int incl = len;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o) incl += t;
+        }
+        __syncwarp();
+        pre[lane] = (uint32_t)(incl - len);
+        total = __shfl_sync(kFull, incl, 31);
+        __syncwarp();
+    }
+    // the row of entry e < total: the last one that begins at or before it
+    __device__ __forceinline__ int row(int e) const {
+        int r = 0;
+#pragma unroll
+        for (int h = 16; h > 0; h >>= 1) r += (int)pre[r + h] <= e ? h : 0;
+        return r;
+    }
+    // the lanes that hold entries of this lane's row (rows ascend with the lanes)
+    static __device__ __forceinline__ unsigned same_row(int r) {
+        const int lane = threadIdx.x & 31;
+        const int before = __shfl_up_sync(kFull, r, 1);
+        const unsigned starts = __ballot_sync(kFull, lane == 0 || before != r);
+        const unsigned upto = 0xffffffffu >> (31 - lane);
+        const unsigned later = starts & ~upto;
+        const int first = 31 - __clz(starts & upto);
+        const unsigned from_first = 0xffffffffu << first;
+        return later ? from_first & ((1u << (__ffs(later) - 1)) - 1u) : from_first;
+    }
+};
+
+// ---- validation and degree split ------------------------------------------
 // A row must lie inside [0, nnz], be strictly increasing and hold ids in
 // [0, n) other than its own, and every entry v of row u needs u in row v.
 // Writes nlow[u] = #neighbours < u and upcnt[u] = #neighbours > u.  Reads
@@ -69,29 +138,61 @@ __device__ __forceinline__ int64_t warp_count_global() {
 // search.
 
 // FP (k-core builds, which need no reverse entries): symmetry by
-// fingerprint instead of searches.  Every entry (u, v) adds
-// f(u, v) - f(v, u) to two 64-bit sums, each with its own mixing function f
-// (the splitmix64 finalizer, after Steele, Lea and Flood, on different
-// inputs).  A symmetric graph sums to zero exactly.  Otherwise the sums are
-// those of f over the entries without a reverse minus f over the missing
-// reverses, and both are zero only by a coincidence of two 64-bit hashes.
-// It streams col once and gathers nothing.
+// fingerprint instead of searches.  Every entry (u, v) adds +f(u, v), if
+// u < v, or -f(v, u) to two 64-bit sums, each with its own mixing function f
+// (the splitmix64 finalizer, after Steele, Lea and Flood, and the finalizer of
+// its result).  A symmetric graph sums to zero exactly.  Otherwise the sums
+// are those of +-f over the entries without a reverse, and both are zero only
+// by a coincidence of two 64-bit hashes.  It streams col once and gathers
+// nothing; the hashing bounds it, so an entry takes two finalizers (f(u, v) -
+// f(v, u) with unrelated inputs took six).
 __device__ __forceinline__ unsigned long long fp_mix(unsigned long long z) {
     z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
     z = (z ^ (z >> 27)) * 0x94d049bb133111ebull;
     return z ^ (z >> 31);
 }
 __device__ __forceinline__ void fp_add(unsigned long long (&fp)[2], int64_t u, int32_t v) {
-    const unsigned long long k = ((unsigned long long)u << 32) | (uint32_t)v;
-    const unsigned long long r = ((unsigned long long)(uint32_t)v << 32) | (unsigned long long)u;
-    fp[0] += fp_mix(k ^ 0x9e3779b97f4a7c15ull) - fp_mix(r ^ 0x9e3779b97f4a7c15ull);
-    fp[1] += fp_mix(fp_mix(k) + 0x632be59bd9b4e019ull) - fp_mix(fp_mix(r) + 0x632be59bd9b4e019ull);
+    const bool up = u < v;
+    const unsigned long long lo = up ? (unsigned long long)u : (unsigned long long)v;
+    const unsigned long long hi = up ? (unsigned long long)v : (unsigned long long)u;
+    const unsigned long long a = fp_mix(((lo << 32) | hi) ^ 0x9e3779b97f4a7c15ull);
+    const unsigned long long b = fp_mix(a + 0x632be59bd9b4e019ull);
+    fp[0] += up ? a : 0ull - a;
+    fp[1] += up ? b : 0ull - b;
 }
 
 // the checks of entries [pb, pe) of row u (which spans [b, e)), one entry
 // per lane: the count of entries below the diagonal, of searching entries,
 // and whether any check failed (FP: fp collects this lane's fingerprint
 // terms, summed over the warp by the caller)
+template <bool BY_LENGTH, bool FP>
+__device__ __forceinline__ bool validate_entry(int64_t n, int64_t nnz, const int64_t* __restrict__ rp,
+                                               const int32_t* __restrict__ col, int64_t u, int64_t b, int64_t e,
+                                               int64_t p, uint32_t* __restrict__ mirror, bool& low, int& found,
+                                               unsigned long long (&fp)[2]) {
+    const int32_t v = col[p];
+    if (v < 0 || v >= n || v == u) return false;
+    low = v < u;
+    const bool ok = p <= b || col[p - 1] < v;
+    if constexpr (FP) {
+        fp_add(fp, u, v);
+        return ok;
+    }
+    if (!BY_LENGTH && v < u) return ok;
+    const int64_t vb = rp[v], ve = rp[v + 1];
+    // a row longer than n - 1 cannot be simple (and would not fit the 32-bit search)
+    if (vb < 0 || ve < vb || ve > nnz || ve - vb >= n) return false;
+    if (BY_LENGTH && (e - b < ve - vb || (e - b == ve - vb && u < v))) return ok;
+    const int64_t pos = vb + nd_lower_bound_n(col + vb, (int)(ve - vb), (int32_t)u);
+    if (pos >= ve || col[pos] != (int32_t)u) return false;
+    ++found;
+    if (mirror) {
+        mirror[p] = (uint32_t)pos;
+        mirror[pos] = (uint32_t)p;
+    }
+    return ok;
+}
+
 template <bool BY_LENGTH, bool FP = false>
 __device__ __forceinline__ void validate_entries(int64_t n, int64_t nnz, const int64_t* __restrict__ rp,
                                                  const int32_t* __restrict__ col, int64_t u, int64_t b, int64_t e,
@@ -99,26 +200,9 @@ __device__ __forceinline__ void validate_entries(int64_t n, int64_t nnz, const i
                                                  int& found, bool& rowbad, unsigned long long (&fp)[2]) {
     const int lane = threadIdx.x & 31;
     for (int64_t p = pb + lane; p < pe; p += 32) {
-        int32_t v = col[p];
-        if (v < 0 || v >= n || v == u) { rowbad = true; continue; }
-        if (p > b && col[p - 1] >= v) rowbad = true;
-        low += (v < u);
-        if constexpr (FP) {
-            fp_add(fp, u, v);
-            continue;
-        }
-        if (!BY_LENGTH && v < u) continue;
-        int64_t vb = rp[v], ve = rp[v + 1];
-        // a row longer than n - 1 cannot be simple (and would not fit the 32-bit search)
-        if (vb < 0 || ve < vb || ve > nnz || ve - vb >= n) { rowbad = true; continue; }
-        if (BY_LENGTH && (e - b < ve - vb || (e - b == ve - vb && u < v))) continue;
-        const int64_t pos = vb + nd_lower_bound_n(col + vb, (int)(ve - vb), (int32_t)u);
-        if (pos >= ve || col[pos] != (int32_t)u) { rowbad = true; continue; }
-        ++found;
-        if (mirror) {
-            mirror[p] = (uint32_t)pos;
-            mirror[pos] = (uint32_t)p;
-        }
+        bool below = false;
+        if (!validate_entry<BY_LENGTH, FP>(n, nnz, rp, col, u, b, e, p, mirror, below, found, fp)) rowbad = true;
+        low += below;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -186,39 +270,79 @@ __device__ __forceinline__ void fp_flush(unsigned long long (&fp)[2], unsigned l
 }
 
 template <bool BY_LENGTH, bool FP = false>
-__global__ void k_validate_split(int64_t n, int64_t nnz, const int64_t* __restrict__ rp,
+__global__ void k_validate_split(int per, int64_t n, int64_t nnz, const int64_t* __restrict__ rp,
                                  const int32_t* __restrict__ col, int32_t* __restrict__ nlow,
                                  int64_t* __restrict__ upcnt, int* __restrict__ err,
                                  unsigned long long* __restrict__ searched, uint32_t* __restrict__ mirror,
                                  unsigned long long* __restrict__ fp_out) {
-    const int lane = threadIdx.x & 31;
+    __shared__ uint32_t pre[kThreads / 32][32];
+    __shared__ int64_t begin[kThreads / 32][32];
+    __shared__ int lows[kThreads / 32][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     unsigned long long fp[2] = {0ull, 0ull};
-    for (int64_t u = warp_id_global(); u < n; u += warp_count_global()) {
-        int64_t b = rp[u], e = rp[u + 1];
-        bool bad = (b < 0) || (e < b) || (e > nnz) || (u == 0 && b != 0) || (u == n - 1 && e != nnz);
-        if (bad) {
-            if (lane == 0) { atomicOr(err, 1); nlow[u] = 0; upcnt[u] = 0; }
-            continue;
-        }
-        if (is_long_row(b, e)) {  // counted by k_validate_long
-            if (lane == 0) {
-                nlow[u] = 0;
-                upcnt[u] = 0;
+    int found = 0;
+    bool bad_entry = false;
+    const int64_t groups = (n + per - 1) / per;
+    for (int64_t g = warp_id_global(); g < groups; g += warp_count_global()) {
+        const int64_t u0 = per * g, mine = lane < per ? u0 + lane : n;
+        int64_t b = 0;
+        int len = 0;
+        if (mine < n) {
+            b = rp[mine];
+            const int64_t e = rp[mine + 1];
+            if (b < 0 || e < b || e > nnz || (mine == 0 && b != 0) || (mine == n - 1 && e != nnz)) {
+                atomicOr(err, 1);
+            } else if (is_long_row(b, e)) {  // counted by k_validate_long
                 // a graph of at most kLongRow vertices: too long to be simple
                 if (n <= kLongRow) atomicOr(err, 2);
+            } else if (e - b <= kPoolRow) {
+                len = (int)(e - b);
             }
-            continue;
         }
-        int low = 0, found = 0;
-        bool rowbad = false;
-        validate_entries<BY_LENGTH, FP>(n, nnz, rp, col, u, b, e, b, e, mirror, low, found, rowbad, fp);
-        if (lane == 0) {
-            nlow[u] = low;
-            upcnt[u] = (e - b) - low;
-            if (found) atomicAdd(searched, (unsigned long long)found);
-            if (rowbad) atomicOr(err, 2);
+        begin[w][lane] = b;
+        lows[w][lane] = 0;
+        const row_pool pool(pre[w], len);
+        for (int e0 = 0; e0 < pool.total; e0 += 32) {
+            const int x = e0 + lane;
+            const int r = pool.row(min(x, pool.total - 1));
+            bool low = false;
+            if (x < pool.total) {
+                const int64_t rb = begin[w][r], p = rb + (x - (int)pool.pre[r]);
+                const int64_t re = rb + ((r < 31 ? (int)pool.pre[r + 1] : pool.total) - (int)pool.pre[r]);
+                if (!validate_entry<BY_LENGTH, FP>(n, nnz, rp, col, u0 + r, rb, re, p, mirror, low, found, fp))
+                    bad_entry = true;
+            }
+            const unsigned same = row_pool::same_row(r), m = __ballot_sync(kFull, low) & same;
+            if (lane == __ffs(same) - 1) lows[w][r] += __popc(m);
+            __syncwarp();
+        }
+        if (mine < n && len > 0) {  // the others are zeroed beforehand, and may have been counted since
+            nlow[mine] = lows[w][lane];
+            upcnt[mine] = len - lows[w][lane];
         }
     }
+    spread_rows(
+        n,
+        [&](int64_t u) {
+            const int64_t b = rp[u], e = rp[u + 1];
+            return b >= 0 && e <= nnz && e - b > kPoolRow && !is_long_row(b, e);
+        },
+        [&](int64_t u) {
+            const int64_t b = rp[u], e = rp[u + 1];
+            int low = 0, in_row = 0;
+            bool bad = false;
+            validate_entries<BY_LENGTH, FP>(n, nnz, rp, col, u, b, e, b, e, mirror, low, in_row, bad, fp);
+            if (lane == 0) {
+                found += in_row;
+                nlow[u] = low;
+                upcnt[u] = (e - b) - low;
+            }
+            bad_entry |= bad;
+        });
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) found += __shfl_xor_sync(kFull, found, o);
+    if (lane == 0 && found) atomicAdd(searched, (unsigned long long)found);
+    if (bad_entry) atomicOr(err, 2);
     if constexpr (FP) fp_flush(fp, fp_out);
 }
 
@@ -355,52 +479,84 @@ struct DegreeOrder {  // no-storage passes: the caller's ids with their slots, b
     }
 };
 
-// one warp per row of up to kSortRow entries; up to 32 are ranked across the
-// warp, longer rows go through 32 shared counters
+// rows of up to kSortRow entries: up to 8 are ranked across eight lanes, up to
+// 32 across the warp; longer rows go through 32 shared counters, one warp each
 template <typename K>
-__global__ void __launch_bounds__(kThreads) k_order_rows(int64_t n, const int64_t* __restrict__ rp, K k) {
+__global__ void __launch_bounds__(kThreads) k_order_rows(int per, int64_t n, const int64_t* __restrict__ rp, K k) {
     __shared__ uint32_t stage[kThreads / 32][kSortRow];
     __shared__ uint32_t cur[kThreads / 32][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int64_t u = warp_id_global(); u < n; u += warp_count_global()) {
-        const int64_t b = rp[u];
-        const int64_t len = rp[u + 1] - b;
-        if (len == 0 || len > kSortRow) continue;  // k_sort_count, k_sort_scatter
-        const int d = (int)len;
-        const int64_t out = k.begin(u, b);
-        if (d <= 32) {
-            const uint32_t key = lane < d ? k.key(b + lane) : 0xffffffffu;
+    const int64_t groups = (n + per - 1) / per;
+    for (int64_t g = warp_id_global(); g < groups; g += warp_count_global()) {
+        const int64_t u0 = per * g, mine = lane < per ? u0 + lane : n;
+        const int64_t b = mine < n ? rp[mine] : 0, d = mine < n ? rp[mine + 1] - b : 0;
+        const int64_t out = d > 0 && d <= 32 ? k.begin(mine, b) : 0;
+        if (d == 1) k.write(out, b, k.key(b));
+        for (unsigned todo = __ballot_sync(kFull, d >= 2 && d <= 8); todo;) {
+            int r = -1;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int f = todo ? __ffs(todo) - 1 : -1;
+                if (lane / 8 == q) r = f;
+                todo &= todo - 1;  // 0 stays 0
+            }
+            const int64_t rb = __shfl_sync(kFull, b, max(r, 0)), ro = __shfl_sync(kFull, out, max(r, 0));
+            const int64_t any_d = __shfl_sync(kFull, d, max(r, 0));
+            const int j = lane & 7, rd = r >= 0 ? (int)any_d : 0;
+            const uint32_t key = j < rd ? k.key(rb + j) : 0xffffffffu;
             int rank = 0;
-            for (int o = 0; o < d; ++o) {
+#pragma unroll
+            for (int o = 0; o < 8; ++o) {
+                const uint32_t x = __shfl_sync(kFull, key, o, 8);
+                rank += x < key || (x == key && o < j);
+            }
+            if (j < rd) k.write(ro + rank, rb + j, key);
+        }
+        for (unsigned todo = __ballot_sync(kFull, d > 8 && d <= 32); todo; todo &= todo - 1) {
+            const int r = __ffs(todo) - 1;
+            const int64_t rb = __shfl_sync(kFull, b, r), ro = __shfl_sync(kFull, out, r);
+            const int rd = (int)__shfl_sync(kFull, d, r);
+            const uint32_t key = lane < rd ? k.key(rb + lane) : 0xffffffffu;
+            int rank = 0;
+            for (int o = 0; o < rd; ++o) {
                 const uint32_t x = __shfl_sync(kFull, key, o);
                 rank += x < key || (x == key && o < lane);
             }
-            if (lane < d) k.write(out + rank, b + lane, key);
-            continue;
+            if (lane < rd) k.write(ro + rank, rb + lane, key);
         }
-        cur[w][lane] = 0;
-        __syncwarp();
-        for (int j = lane; j < d; j += 32) {
-            const uint32_t key = k.key(b + j);
-            stage[w][j] = key;
-            atomicAdd(&cur[w][K::bucket(key)], 1u);
-        }
-        __syncwarp();
-        const uint32_t c = cur[w][lane];
-        uint32_t incl = c;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(kFull, incl, o);
-            if (lane >= o) incl += t;
-        }
-        cur[w][lane] = incl - c;
-        __syncwarp();
-        for (int j = lane; j < d; j += 32) {
-            const uint32_t key = stage[w][j];
-            k.write(out + atomicAdd(&cur[w][K::bucket(key)], 1u), b + j, key);
-        }
-        __syncwarp();
     }
+    spread_rows(
+        n,
+        [&](int64_t u) {
+            const int64_t d = rp[u + 1] - rp[u];
+            return d > 32 && d <= kSortRow;  // longer: k_sort_count, k_sort_scatter
+        },
+        [&](int64_t u) {
+            const int64_t b = rp[u], out = k.begin(u, b);
+            const int d = (int)(rp[u + 1] - b);
+            cur[w][lane] = 0;
+            __syncwarp();
+            for (int j = lane; j < d; j += 32) {
+                const uint32_t key = k.key(b + j);
+                stage[w][j] = key;
+                atomicAdd(&cur[w][K::bucket(key)], 1u);
+            }
+            __syncwarp();
+            const uint32_t c = cur[w][lane];
+            uint32_t incl = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(kFull, incl, o);
+                if (lane >= o) incl += t;
+            }
+            cur[w][lane] = incl - c;
+            __syncwarp();
+            for (int j = lane; j < d; j += 32) {
+                const uint32_t key = stage[w][j];
+                k.write(out + atomicAdd(&cur[w][K::bucket(key)], 1u), b + j, key);
+            }
+            __syncwarp();
+        });
 }
 
 // the rows longer than kSortRow and the number of their kLongSeg segments
@@ -627,73 +783,107 @@ __device__ __forceinline__ bool precedes(int64_t du, int32_t u, int64_t dv, int3
     return du < dv || (du == dv && u < v);
 }
 
-// one warp per vertex: count / list the out-neighbours of u in id order
-// (with out_pos: also the CSR positions of the entry and of its reverse)
+// count / list the out-neighbours of every vertex in id order, 32 vertices per
+// warp (with out_pos: also the CSR positions of the entry and of its reverse)
 template <bool FILL>
-__global__ void k_orient(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ col,
-                         const uint32_t* __restrict__ eid, int64_t* __restrict__ out_ptr,
-                         int32_t* __restrict__ out_col, uint32_t* __restrict__ out_eid,
-                         int32_t* __restrict__ out_src, const uint32_t* __restrict__ mirror,
-                         uint32_t* __restrict__ out_pos, uint32_t* __restrict__ out_mir) {
-    const int lane = threadIdx.x & 31;
-    for (int64_t u = warp_id_global(); u < n; u += warp_count_global()) {
-        const int64_t b = rp[u], e = rp[u + 1], du = e - b;
-        const int64_t base = FILL ? out_ptr[u] : 0;
-        int64_t cnt = 0;
-        for (int64_t p0 = b; p0 < e; p0 += 32) {
-            const int64_t p = p0 + lane;
+__global__ void __launch_bounds__(kThreads) k_orient(int per, int64_t n, const int64_t* __restrict__ rp,
+                                                     const int32_t* __restrict__ col,
+                                                     const uint32_t* __restrict__ eid, int64_t* __restrict__ out_ptr,
+                                                     int32_t* __restrict__ out_col, uint32_t* __restrict__ out_eid,
+                                                     int32_t* __restrict__ out_src,
+                                                     const uint32_t* __restrict__ mirror,
+                                                     uint32_t* __restrict__ out_pos, uint32_t* __restrict__ out_mir) {
+    __shared__ uint32_t pre[kThreads / 32][32];
+    __shared__ int64_t begin[kThreads / 32][32], slots[kThreads / 32][32];  // slots: next output slot of each row
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    auto put = [&](int64_t slot, int32_t u, int32_t v, int64_t p) {
+        out_col[slot] = v;
+        out_eid[slot] = __ldg(eid + p);
+        out_src[slot] = u;
+        if (out_pos) {
+            out_pos[slot] = (uint32_t)p;
+            out_mir[slot] = __ldg(mirror + p);
+        }
+    };
+    const int64_t groups = (n + per - 1) / per;
+    for (int64_t g = warp_id_global(); g < groups; g += warp_count_global()) {
+        const int64_t u0 = per * g, mine = lane < per ? u0 + lane : n;
+        const int64_t b = mine < n ? rp[mine] : 0, len = mine < n ? rp[mine + 1] - b : 0;
+        __syncwarp();
+        begin[w][lane] = b;
+        slots[w][lane] = FILL && mine < n ? out_ptr[mine] : 0;
+        const row_pool pool(pre[w], len > kPoolRow ? 0 : (int)len);
+        auto entry = [&](bool ok, int r, int64_t p, int64_t du) {
             bool keep = false;
             int32_t v = 0;
-            if (p < e) {
+            if (ok) {
                 v = __ldg(col + p);
-                keep = precedes(du, (int32_t)u, __ldg(rp + v + 1) - __ldg(rp + v), v);
+                keep = precedes(du, (int32_t)(u0 + r), __ldg(rp + v + 1) - __ldg(rp + v), v);
             }
-            const unsigned bal = __ballot_sync(kFull, keep);
-            if (FILL && keep) {
-                const int64_t slot = base + cnt + __popc(bal & lanemask_lt());
-                out_col[slot] = v;
-                out_eid[slot] = __ldg(eid + p);
-                out_src[slot] = (int32_t)u;
-                if (out_pos) {
-                    out_pos[slot] = (uint32_t)p;
-                    out_mir[slot] = __ldg(mirror + p);
-                }
-            }
-            cnt += __popc(bal);
+            const unsigned same = row_pool::same_row(r), m = __ballot_sync(kFull, keep) & same;
+            const int64_t first = slots[w][r];
+            __syncwarp();
+            if (lane == __ffs(same) - 1) slots[w][r] = first + __popc(m);
+            if (FILL && keep) put(first + __popc(m & lanemask_lt()), (int32_t)(u0 + r), v, p);
+            __syncwarp();
+        };
+        for (int e0 = 0; e0 < pool.total; e0 += 32) {
+            const int x = e0 + lane;
+            const int r = pool.row(min(x, pool.total - 1));
+            const int at = (int)pool.pre[r];
+            entry(x < pool.total, r, begin[w][r] + (x - at), (r < 31 ? (int)pool.pre[r + 1] : pool.total) - at);
         }
-        if (!FILL && lane == 0) out_ptr[u] = cnt;
+        if (!FILL && mine < n && len <= kPoolRow) out_ptr[mine] = slots[w][lane];
     }
+    spread_rows(
+        n, [&](int64_t u) { return rp[u + 1] - rp[u] > kPoolRow; },
+        [&](int64_t u) {
+            const int64_t b = rp[u], e = rp[u + 1], du = e - b;
+            int64_t slot = FILL ? out_ptr[u] : 0;
+            for (int64_t p0 = b; p0 < e; p0 += 32) {
+                const int64_t p = p0 + lane;
+                bool keep = false;
+                int32_t v = 0;
+                if (p < e) {
+                    v = __ldg(col + p);
+                    keep = precedes(du, (int32_t)u, __ldg(rp + v + 1) - __ldg(rp + v), v);
+                }
+                const unsigned m = __ballot_sync(kFull, keep);
+                if (FILL && keep) put(slot + __popc(m & lanemask_lt()), (int32_t)u, v, p);
+                slot += __popc(m);
+            }
+            if (!FILL && lane == 0) out_ptr[u] = slot;
+        });
 }
 
-// one warp per oriented edge u -> v: the triangles {u, v, w}, w in out(u) /\ out(v).
-// ADJ: the entries are CSR positions, each pair ordered by its edge's
-// canonical endpoints (the entry of the smaller endpoint first).
 #ifndef ND_TRI_COUNT_MIN_BLOCKS
 #define ND_TRI_COUNT_MIN_BLOCKS 8  // the count pass (with its records) at full occupancy
 #endif
 #ifndef ND_TRI_MIN_BLOCKS
 #define ND_TRI_MIN_BLOCKS 6  // resident blocks per SM for the searching fill (used when the records do not fit)
 #endif
-// REC (count pass): also record every triangle found from edge k, as the
-// offsets of w in the shorter and in the longer out-list (16 bits each: an
-// out-list holds at most sqrt(2m) < 65536 entries, since each of its
-// vertices has at least the owner's degree and nnz < 2^32), at
-// rec[rec_ptr[k] + i]; rec_ptr[k] reserves min(|out(u)|, |out(v)|) slots,
-// the most edge k can find.  rec_cnt[k] = triangles found.
-template <bool FILL, bool ADJ, typename C = unsigned long long, bool REC = false>
-__global__ void __launch_bounds__(kThreads, FILL ? ND_TRI_MIN_BLOCKS : ND_TRI_COUNT_MIN_BLOCKS) k_tri_oriented(int64_t m, const int64_t* __restrict__ out_ptr,
-                               const int32_t* __restrict__ out_col, const uint32_t* __restrict__ out_eid,
-                               const int32_t* __restrict__ out_src, const uint32_t* __restrict__ out_pos,
-                               const uint32_t* __restrict__ out_mir, C* __restrict__ ctr,
-                               uint2* __restrict__ inc, const int64_t* __restrict__ rec_ptr = nullptr,
-                               uint32_t* __restrict__ rec = nullptr, uint32_t* __restrict__ rec_cnt = nullptr) {
+// The searching fill (small builds, and where the records do not fit): one
+// warp per oriented edge u -> v, the triangles {u, v, w}, w in out(u) /\
+// out(v); the lanes walk the shorter list and search the longer.  The entries
+// are CSR positions, each pair ordered by its edge's canonical endpoints (the
+// entry of the smaller endpoint first).
+// Records (the count pass's, for the fill from records): every triangle found
+// from edge k, as the offsets of w in the shorter and in the longer out-list
+// (16 bits each: an out-list holds at most sqrt(2m) < 65536 entries, since
+// each of its vertices has at least the owner's degree and nnz < 2^32), at
+// rec[rec_ptr[k] + i]; rec_ptr[k] reserves min(|out(u)|, |out(v)|) slots, the
+// most edge k can find.  rec_cnt[k] = triangles found.
+template <typename C>
+__global__ void __launch_bounds__(kThreads, ND_TRI_MIN_BLOCKS)
+    k_tri_fill_search(int64_t m, const int64_t* __restrict__ out_ptr, const int32_t* __restrict__ out_col,
+                      const uint32_t* __restrict__ out_eid, const int32_t* __restrict__ out_src,
+                      const uint32_t* __restrict__ out_pos, const uint32_t* __restrict__ out_mir, C* __restrict__ ctr,
+                      uint2* __restrict__ inc) {
     const int lane = threadIdx.x & 31;
     for (int64_t k = warp_id_global(); k < m; k += warp_count_global()) {
-        uint32_t nrec = 0;  // REC: triangles recorded so far for edge k
         const int32_t u = out_src[k], v = out_col[k];
         const uint32_t e_uv = out_eid[k];
-        uint32_t Puv = 0, Pvu = 0;
-        if (ADJ) { Puv = __ldg(out_pos + k); Pvu = __ldg(out_mir + k); }
+        const uint32_t Puv = __ldg(out_pos + k), Pvu = __ldg(out_mir + k);
         int64_t ab = out_ptr[u], ae = out_ptr[u + 1], bb = out_ptr[v], be = out_ptr[v + 1];
         bool a_is_u = true;
         if (ae - ab > be - bb) {
@@ -706,125 +896,178 @@ __global__ void __launch_bounds__(kThreads, FILL ? ND_TRI_MIN_BLOCKS : ND_TRI_CO
             bool found = false;
             int64_t pb = 0;
             int32_t x = 0;
-            // FILL: the values at p are loaded with x, ahead of the search
+            // the values at p are loaded with x, ahead of the search
             // (coalesced), so only the loads at pb wait for it
             uint32_t ea = 0, pa = 0, ma = 0;
             if (p < ae) {
                 x = __ldg(out_col + p);
-                if (FILL) {
-                    ea = __ldg(out_eid + p);
-                    if (ADJ) {
-                        pa = __ldg(out_pos + p);
-                        ma = __ldg(out_mir + p);
-                    }
-                }
+                ea = __ldg(out_eid + p);
+                pa = __ldg(out_pos + p);
+                ma = __ldg(out_mir + p);
                 pb = lo + nd_lower_bound_n(out_col + lo, (int)(be - lo), x);
                 found = (pb < be) && (__ldg(out_col + pb) == x);
             }
             const unsigned bal = __ballot_sync(kFull, found);
             const int nf = __popc(bal);
             if (nf) {
-                uint32_t e_uw = 0, e_vw = 0;
-                if (!FILL) {
-                    if (found) {
-                        const uint32_t ea0 = __ldg(out_eid + p), eb = __ldg(out_eid + pb);
-                        e_uw = a_is_u ? ea0 : eb;
-                        e_vw = a_is_u ? eb : ea0;
-                    }
-                    if (lane == 0) atomicAdd(ctr + e_uv, (C)nf);
-                    if (found) {
-                        atomicAdd(ctr + e_uw, (C)1);
-                        atomicAdd(ctr + e_vw, (C)1);
-                    }
-                    if (REC) {
-                        if (found)
-                            rec[rec_ptr[k] + nrec + __popc(bal & lanemask_lt())] =
-                                (uint32_t)(p - ab) | ((uint32_t)(pb - bb) << 16);
-                        nrec += (uint32_t)nf;
-                    }
-                } else {
-                    uint32_t pbp = 0, mb = 0;
-                    if (found) {
-                        const uint32_t eb = __ldg(out_eid + pb);
-                        if (ADJ) {
-                            pbp = __ldg(out_pos + pb);
-                            mb = __ldg(out_mir + pb);
-                        }
-                        e_uw = a_is_u ? ea : eb;
-                        e_vw = a_is_u ? eb : ea;
-                    }
-                    // the three slot reservations are independent: issue them together
-                    C s0 = 0, s_uw = 0, s_vw = 0;
-                    if (lane == 0) s0 = atomicAdd(ctr + e_uv, (C)nf);
-                    if (found) {
-                        s_uw = atomicAdd(ctr + e_uw, (C)1);
-                        s_vw = atomicAdd(ctr + e_vw, (C)1);
-                    }
-                    s0 = __shfl_sync(kFull, s0, 0);
-                    if (found) {
-                        uint2 r_uv, r_uw, r_vw;
-                        if (ADJ) {
-                            // third vertex w = x; positions P(.,.) of the six entries
-                            const uint32_t Puw = a_is_u ? pa : pbp, Pwu = a_is_u ? ma : mb;
-                            const uint32_t Pvw = a_is_u ? pbp : pa, Pwv = a_is_u ? mb : ma;
-                            r_uv = u < v ? make_uint2(Puw, Pvw) : make_uint2(Pvw, Puw);
-                            r_uw = u < x ? make_uint2(Puv, Pwv) : make_uint2(Pwv, Puv);
-                            r_vw = v < x ? make_uint2(Pvu, Pwu) : make_uint2(Pwu, Pvu);
-                        } else {
-                            r_uv = make_uint2(e_uw, e_vw);
-                            r_uw = make_uint2(e_uv, e_vw);
-                            r_vw = make_uint2(e_uv, e_uw);
-                        }
-                        inc[s0 + __popc(bal & lanemask_lt())] = r_uv;
-                        inc[s_uw] = r_uw;
-                        inc[s_vw] = r_vw;
-                    }
+                uint32_t eb = 0, pbp = 0, mb = 0;
+                if (found) {
+                    eb = __ldg(out_eid + pb);
+                    pbp = __ldg(out_pos + pb);
+                    mb = __ldg(out_mir + pb);
+                }
+                const uint32_t e_uw = a_is_u ? ea : eb, e_vw = a_is_u ? eb : ea;
+                // the three slot reservations are independent: issue them together
+                C s0 = 0, s_uw = 0, s_vw = 0;
+                if (lane == 0) s0 = atomicAdd(ctr + e_uv, (C)nf);
+                if (found) {
+                    s_uw = atomicAdd(ctr + e_uw, (C)1);
+                    s_vw = atomicAdd(ctr + e_vw, (C)1);
+                }
+                s0 = __shfl_sync(kFull, s0, 0);
+                if (found) {
+                    // third vertex w = x; positions P(.,.) of the six entries
+                    const uint32_t Puw = a_is_u ? pa : pbp, Pwu = a_is_u ? ma : mb;
+                    const uint32_t Pvw = a_is_u ? pbp : pa, Pwv = a_is_u ? mb : ma;
+                    inc[s0 + __popc(bal & lanemask_lt())] = u < v ? make_uint2(Puw, Pvw) : make_uint2(Pvw, Puw);
+                    inc[s_uw] = u < x ? make_uint2(Puv, Pwv) : make_uint2(Pwv, Puv);
+                    inc[s_vw] = v < x ? make_uint2(Pvu, Pwu) : make_uint2(Pwu, Pvu);
                 }
             }
             const int64_t last_pb = __shfl_sync(kFull, pb, 31);
             if (base + 32 <= ae) lo = last_pb;
         }
-        if (REC && lane == 0) rec_cnt[k] = nrec;
     }
 }
 
-// the fill from the count pass's records: one warp per oriented edge k, one
-// recorded triangle per lane, so no search is repeated.  The six positions
-// of a triangle are read at the recorded offsets of w in the two out-lists
-// (the shorter list's reads coalesce, as in the searching fill); slots and
-// entries are as in k_tri_oriented<true, true>.
+// The count: 32 consecutive oriented edges per warp.  The elements of an
+// edge's shorter out-list, in whole blocks of 32, are looked up in the longer
+// one by the warp; the rests of all 32 edges are then walked as one sequence.
+template <bool REC>
+__global__ void __launch_bounds__(kThreads, ND_TRI_COUNT_MIN_BLOCKS)
+    k_tri_count(int per, int64_t m, const int64_t* __restrict__ out_ptr, const int32_t* __restrict__ out_col,
+                const uint32_t* __restrict__ out_eid, const int32_t* __restrict__ out_src, unsigned* __restrict__ ctr,
+                const int64_t* __restrict__ rec_ptr, uint32_t* __restrict__ rec, uint32_t* __restrict__ rec_cnt) {
+    __shared__ uint32_t pre[kThreads / 32][32];
+    __shared__ uint32_t ab[kThreads / 32][32], bb[kThreads / 32][32], bn[kThreads / 32][32], an[kThreads / 32][32];
+    __shared__ uint32_t nf[kThreads / 32][32];  // triangles found from each edge so far
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t groups = (m + per - 1) / per;
+    for (int64_t g = warp_id_global(); g < groups; g += warp_count_global()) {
+        const int64_t k0 = per * g, mine = lane < per ? k0 + lane : m;
+        uint32_t a = 0, b = 0;
+        int na = 0, nb = 0;  // out-lists have fewer than 65,536 entries
+        if (mine < m) {
+            const int32_t u = out_src[mine], v = out_col[mine];
+            const int64_t ub = out_ptr[u], ue = out_ptr[u + 1], vb = out_ptr[v], ve = out_ptr[v + 1];
+            const bool us = ue - ub <= ve - vb;
+            a = (uint32_t)(us ? ub : vb);
+            b = (uint32_t)(us ? vb : ub);
+            na = (int)(us ? ue - ub : ve - vb);
+            nb = (int)(us ? ve - vb : ue - ub);
+        }
+        __syncwarp();
+        ab[w][lane] = a;
+        bb[w][lane] = b;
+        an[w][lane] = (uint32_t)na;
+        bn[w][lane] = (uint32_t)nb;
+        nf[w][lane] = 0;
+        const row_pool pool(pre[w], na & 31);
+        // element j of edge r's shorter list
+        auto element = [&](bool ok, int r, int j) {
+            bool found = false;
+            uint32_t p = 0, pb = 0;
+            if (ok) {
+                p = ab[w][r] + j;
+                const uint32_t lb = bb[w][r];
+                const int32_t x = __ldg(out_col + p);
+                const int at = nd_lower_bound_n(out_col + lb, (int)bn[w][r], x);
+                pb = lb + at;
+                found = at < (int)bn[w][r] && __ldg(out_col + pb) == x;
+            }
+            const unsigned all = __ballot_sync(kFull, found);
+            if (!all) return;
+            const unsigned same = row_pool::same_row(r), hit = all & same;
+            const uint32_t before = nf[w][r];
+            __syncwarp();
+            if (lane == __ffs(same) - 1 && hit) nf[w][r] = before + __popc(hit);
+            if (found) {
+                atomicAdd(ctr + __ldg(out_eid + p), 1u);
+                atomicAdd(ctr + __ldg(out_eid + pb), 1u);
+                if (REC)
+                    rec[rec_ptr[k0 + r] + before + __popc(hit & lanemask_lt())] =
+                        (uint32_t)j | ((pb - bb[w][r]) << 16);
+            }
+            __syncwarp();
+        };
+        for (unsigned todo = __ballot_sync(kFull, na >= 32); todo; todo &= todo - 1) {
+            const int r = __ffs(todo) - 1, whole = (int)an[w][r] & ~31;
+            for (int j = 0; j < whole; j += 32) element(true, r, j + lane);
+        }
+        for (int e0 = 0; e0 < pool.total; e0 += 32) {
+            const int x = e0 + lane;
+            const int r = pool.row(min(x, pool.total - 1));
+            element(x < pool.total, r, ((int)an[w][r] & ~31) + x - (int)pool.pre[r]);
+        }
+        if (mine < m) {
+            const uint32_t c = nf[w][lane];
+            if (c) atomicAdd(ctr + out_eid[mine], c);
+            if (REC) rec_cnt[mine] = c;
+        }
+    }
+}
+
+// the fill from the count pass's records, 32 consecutive oriented edges per
+// warp and one recorded triangle per lane, so no search is repeated.  The six
+// positions of a triangle are read at the recorded offsets of w in the two
+// out-lists; slots and entries are as in the searching fill.
 #ifndef ND_FILL_MIN_BLOCKS
-#define ND_FILL_MIN_BLOCKS 5  // the fill from records: 48 registers, no spills (24.1 against 25.0 ms at 6 blocks)
+#define ND_FILL_MIN_BLOCKS 5  // the fill from records: 48 registers (24.1 against 25.0 ms at 6 blocks)
 #endif
 template <typename C>
 __global__ void __launch_bounds__(kThreads, ND_FILL_MIN_BLOCKS)
-    k_tri_fill_rec(int64_t m, const int64_t* __restrict__ out_ptr, const int32_t* __restrict__ out_col,
+    k_tri_fill_rec(int per, int64_t m, const int64_t* __restrict__ out_ptr, const int32_t* __restrict__ out_col,
                    const uint32_t* __restrict__ out_eid, const int32_t* __restrict__ out_src,
                    const uint32_t* __restrict__ out_pos, const uint32_t* __restrict__ out_mir, C* __restrict__ ctr,
                    uint2* __restrict__ inc, const int64_t* __restrict__ rec_ptr, const uint32_t* __restrict__ rec,
                    const uint32_t* __restrict__ rec_cnt) {
-    const int lane = threadIdx.x & 31;
-    for (int64_t k = warp_id_global(); k < m; k += warp_count_global()) {
-        const uint32_t c = __ldg(rec_cnt + k);
-        if (c == 0) continue;
-        const int32_t u = out_src[k], v = out_col[k];
-        const uint32_t e_uv = out_eid[k];
-        const uint32_t Puv = __ldg(out_pos + k), Pvu = __ldg(out_mir + k);
-        int64_t ab = out_ptr[u], ae = out_ptr[u + 1], bb = out_ptr[v], be = out_ptr[v + 1];
-        bool a_is_u = true;
-        if (ae - ab > be - bb) {  // the same choice of the shorter list as the count pass
-            int64_t t = ab; ab = bb; bb = t; t = ae; ae = be; be = t;
-            a_is_u = false;
+    __shared__ uint32_t pre[kThreads / 32][32];
+    __shared__ uint32_t ab[kThreads / 32][32], bb[kThreads / 32][32];
+    __shared__ int32_t vu[kThreads / 32][32], vv[kThreads / 32][32];
+    __shared__ bool a_is[kThreads / 32][32];  // the shorter list is out(u)
+    __shared__ int64_t rp0[kThreads / 32][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t groups = (m + per - 1) / per;
+    for (int64_t g = warp_id_global(); g < groups; g += warp_count_global()) {
+        const int64_t k0 = per * g, mine = lane < per ? k0 + lane : m;
+        const int c = mine < m ? (int)__ldg(rec_cnt + mine) : 0;
+        if (!__any_sync(kFull, c > 0)) continue;
+        __syncwarp();
+        if (c > 0) {
+            const int32_t u = out_src[mine], v = out_col[mine];
+            const int64_t ub = out_ptr[u], ue = out_ptr[u + 1], vb = out_ptr[v], ve = out_ptr[v + 1];
+            const bool us = ue - ub <= ve - vb;  // the same choice of the shorter list as the count pass
+            ab[w][lane] = (uint32_t)(us ? ub : vb);
+            bb[w][lane] = (uint32_t)(us ? vb : ub);
+            vu[w][lane] = u;
+            vv[w][lane] = v;
+            a_is[w][lane] = us;
+            rp0[w][lane] = rec_ptr[mine];
         }
-        const int64_t r0 = rec_ptr[k];
-        for (uint32_t base = 0; base < c; base += 32) {
-            const uint32_t i = base + lane;
-            const bool found = i < c;
-            uint32_t ea = 0, pa = 0, ma = 0, eb = 0, pbp = 0, mb = 0;
+        const row_pool pool(pre[w], c);
+        for (int e0 = 0; e0 < pool.total; e0 += 32) {
+            const int i = e0 + lane;
+            const bool found = i < pool.total;
+            const int r = pool.row(min(i, pool.total - 1));
+            const int64_t k = k0 + r;
+            uint32_t ea = 0, pa = 0, ma = 0, eb = 0, pbp = 0, mb = 0, e_uv = 0, Puv = 0, Pvu = 0;
             int32_t x = 0;
             if (found) {
-                const uint32_t r = __ldg(rec + r0 + i);
-                const int64_t p = ab + (r & 0xffffu), pb = bb + (r >> 16);
+                const uint32_t q = __ldg(rec + rp0[w][r] + (i - (int)pool.pre[r]));
+                const uint32_t p = ab[w][r] + (q & 0xffffu), pb = bb[w][r] + (q >> 16);
+                e_uv = __ldg(out_eid + k);
+                Puv = __ldg(out_pos + k);
+                Pvu = __ldg(out_mir + k);
                 x = __ldg(out_col + p);
                 ea = __ldg(out_eid + p);
                 pa = __ldg(out_pos + p);
@@ -833,20 +1076,23 @@ __global__ void __launch_bounds__(kThreads, ND_FILL_MIN_BLOCKS)
                 pbp = __ldg(out_pos + pb);
                 mb = __ldg(out_mir + pb);
             }
-            const unsigned bal = __ballot_sync(kFull, found);
-            const int nf = __popc(bal);
+            const unsigned same = row_pool::same_row(r) & __ballot_sync(kFull, found);
+            const bool a_is_u = a_is[w][r];
+            const int32_t u = vu[w][r], v = vv[w][r];
             const uint32_t e_uw = a_is_u ? ea : eb, e_vw = a_is_u ? eb : ea;
+            // the three slot reservations are independent: issue them together
             C s0 = 0, s_uw = 0, s_vw = 0;
-            if (lane == 0) s0 = atomicAdd(ctr + e_uv, (C)nf);
+            const int leader = __ffs(same) - 1;
+            if (found && lane == leader) s0 = atomicAdd(ctr + e_uv, (C)__popc(same));
             if (found) {
                 s_uw = atomicAdd(ctr + e_uw, (C)1);
                 s_vw = atomicAdd(ctr + e_vw, (C)1);
             }
-            s0 = __shfl_sync(kFull, s0, 0);
+            s0 = __shfl_sync(kFull, s0, found ? leader : lane);
             if (found) {
                 const uint32_t Puw = a_is_u ? pa : pbp, Pwu = a_is_u ? ma : mb;
                 const uint32_t Pvw = a_is_u ? pbp : pa, Pwv = a_is_u ? mb : ma;
-                inc[s0 + __popc(bal & lanemask_lt())] = u < v ? make_uint2(Puw, Pvw) : make_uint2(Pvw, Puw);
+                inc[s0 + __popc(same & lanemask_lt())] = u < v ? make_uint2(Puw, Pvw) : make_uint2(Pvw, Puw);
                 inc[s_uw] = u < x ? make_uint2(Puv, Pwv) : make_uint2(Pwv, Puv);
                 inc[s_vw] = v < x ? make_uint2(Pvu, Pwu) : make_uint2(Pwu, Pvu);
             }
@@ -881,8 +1127,9 @@ __global__ void k_narrow_u32(int64_t m, const int64_t* __restrict__ in, unsigned
 // adjacency lists, N(s): one bit per position of N(s) marks the row's
 // entries, and rank = (bits set in earlier words) + (bits below it in its
 // word).  O(d + deg(s)/32) per row, no comparison sort.  Rows up to 32
-// entries are ranked by comparing keys across the warp instead.  One warp
-// per row; the bit and prefix words sit in shared memory (kRankWords per
+// entries are ranked by comparing keys across eight lanes or the warp instead.
+// A warp takes 32 rows at a time, the longer ones one by one; the bit and prefix
+// words sit in shared memory (kRankWords per
 // warp); a row whose shorter list needs more words is left to the overflow
 // pass, which uses global scratch.
 constexpr int kRankWarps = 8;
@@ -895,18 +1142,6 @@ __device__ __forceinline__ void rank_row(const uint2* __restrict__ src, uint2* _
                                          int64_t d, int comp, uint32_t base, int64_t nw,
                                          uint32_t* __restrict__ bm, uint32_t* __restrict__ pre) {
     const int lane = threadIdx.x & 31;
-    if (d <= 32) {
-        uint2 e = make_uint2(0u, 0u);
-        uint32_t key = 0xffffffffu;
-        if (lane < d) {
-            e = src[jb + lane];
-            key = comp ? e.y : e.x;
-        }
-        int rank = 0;
-        for (int o = 0; o < d; ++o) rank += (__shfl_sync(kFull, key, o) < key);
-        if (lane < d) dst[jb + rank] = e;
-        return;
-    }
     for (int64_t w = lane; w < nw; w += 32) bm[w] = 0u;
     __syncwarp();
     for (int64_t j = jb + lane; j < jb + d; j += 32) {
@@ -944,7 +1179,7 @@ __device__ __forceinline__ void rank_row(const uint2* __restrict__ src, uint2* _
 // global scratch of 2 * scratch_words words per warp.
 template <bool BIG>
 __global__ void __launch_bounds__(32 * kRankWarps)
-k_row_rank(int64_t N, const int64_t* __restrict__ inc_ptr, const int32_t* __restrict__ e_u,
+k_row_rank(int per, int64_t N, const int64_t* __restrict__ inc_ptr, const int32_t* __restrict__ e_u,
            const int32_t* __restrict__ e_v, const int64_t* __restrict__ rp, const uint2* __restrict__ src,
            uint2* __restrict__ dst, uint32_t* __restrict__ over, unsigned long long* __restrict__ over_ctr,
            uint32_t* __restrict__ scratch, int64_t scratch_words) {
@@ -959,28 +1194,72 @@ k_row_rank(int64_t N, const int64_t* __restrict__ inc_ptr, const int32_t* __rest
         bm = rank_smem + (size_t)2 * kRankWords * wib;
         pre = bm + kRankWords;
     }
-    const int64_t rows = BIG ? (int64_t)over_ctr[0] : N;
-    for (int64_t i = warp_id_global(); i < rows; i += warp_count_global()) {
-        const int64_t R = BIG ? (int64_t)over[i] : i;
-        const int64_t jb = inc_ptr[R], d = inc_ptr[R + 1] - jb;
-        if (d <= 1) {
-            if (d == 1 && lane == 0) dst[jb] = src[jb];
-            continue;
-        }
+    auto long_row = [&](int64_t R, int64_t jb, int64_t d) {
         const int32_t x = e_u[R], y = e_v[R];
         const int64_t dx = rp[x + 1] - rp[x], dy = rp[y + 1] - rp[y];
         const int comp = dx <= dy ? 0 : 1;
         const uint32_t base = (uint32_t)rp[comp ? y : x];
         const int64_t nw = ((comp ? dy : dx) + 31) / 32;
-        if (!BIG && d > 32 && nw > kRankWords) {
+        if (!BIG && nw > kRankWords) {
             if (lane == 0) {
                 over[atomicAdd(over_ctr, 1ull)] = (uint32_t)R;
                 atomicMax(over_ctr + 1, (unsigned long long)nw);
             }
-            continue;
+            return;
         }
         rank_row(src, dst, jb, d, comp, base, nw, bm, pre);
+    };
+    if (BIG) {
+        const int64_t rows = (int64_t)over_ctr[0];
+        for (int64_t i = warp_id_global(); i < rows; i += warp_count_global()) {
+            const int64_t R = (int64_t)over[i], jb = inc_ptr[R];
+            long_row(R, jb, inc_ptr[R + 1] - jb);
+        }
+        return;
     }
+    const int64_t groups = (N + per - 1) / per;
+    for (int64_t g = warp_id_global(); g < groups; g += warp_count_global()) {
+        const int64_t mine = lane < per ? per * g + lane : N;
+        int64_t jb = 0, d = 0;
+        if (mine < N) {
+            jb = inc_ptr[mine];
+            d = inc_ptr[mine + 1] - jb;
+        }
+        if (d == 1) dst[jb] = src[jb];
+        // up to eight entries: four rows at a time, eight lanes each
+        for (unsigned todo = __ballot_sync(kFull, d >= 2 && d <= 8); todo;) {
+            int r = -1;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int f = todo ? __ffs(todo) - 1 : -1;
+                if (lane / 8 == q) r = f;
+                todo &= todo - 1;  // 0 stays 0
+            }
+            const int64_t rj = __shfl_sync(kFull, jb, max(r, 0)), any_d = __shfl_sync(kFull, d, max(r, 0));
+            const int rd = r >= 0 ? (int)any_d : 0;
+            const bool ok = (lane & 7) < rd;
+            const uint2 e = ok ? src[rj + (lane & 7)] : make_uint2(0xffffffffu, 0u);
+            int rank = 0;
+#pragma unroll
+            for (int o = 0; o < 8; ++o) rank += __shfl_sync(kFull, e.x, o, 8) < e.x;
+            if (ok) dst[rj + rank] = e;
+        }
+        for (unsigned todo = __ballot_sync(kFull, d > 8 && d <= kPoolRow); todo; todo &= todo - 1) {
+            const int r = __ffs(todo) - 1;
+            const int64_t rj = __shfl_sync(kFull, jb, r), rd = __shfl_sync(kFull, d, r);
+            if (rd > 32) {
+                long_row(per * g + r, rj, rd);
+                continue;
+            }
+            const uint2 e = lane < rd ? src[rj + lane] : make_uint2(0xffffffffu, 0u);
+            int rank = 0;
+            for (int o = 0; o < (int)rd; ++o) rank += __shfl_sync(kFull, e.x, o) < e.x;
+            if (lane < rd) dst[rj + rank] = e;
+        }
+    }
+    spread_rows(
+        N, [&](int64_t R) { return inc_ptr[R + 1] - inc_ptr[R] > kPoolRow; },
+        [&](int64_t R) { long_row(R, inc_ptr[R], inc_ptr[R + 1] - inc_ptr[R]); });
 }
 
 // ---- (3,4): the triangles of every edge, and the 4-cliques of every triangle --
@@ -1398,12 +1677,13 @@ static nd_status validate_split(nd_incidence* h, cudaStream_t st, bool by_length
     ND_CUDA(cudaMemsetAsync(dsearched, 0, 4 * sizeof(unsigned long long), st));
     int* const derr = (int*)(dsearched.p + 3);
     ND_CUDA(cudaMemsetAsync(h->up_start, 0, sizeof(int64_t) * (g->n + 1), st));
+    ND_CUDA(cudaMemsetAsync(h->nlow, 0, sizeof(int32_t) * (g->n > 0 ? g->n : 1), st));
     ND_TRY(find_long_rows(h, st));
     if (g->n > 0) {
         nd_prof_scope ps("validate_split", st);
-        int blocks = nd_blocks_for(g->n * 32, kThreads, grid_cap(h) * 4);
+        const int per = rows_per_warp(g->n), blocks = pool_blocks(g->n, per, grid_cap(h) * 4);
         auto split = fp ? k_validate_split<true, true> : (by_length ? k_validate_split<true> : k_validate_split<false>);
-        split<<<blocks, kThreads, 0, st>>>(g->n, g->nnz, h->rp, h->col, h->nlow, h->up_start, derr, dsearched,
+        split<<<blocks, kThreads, 0, st>>>(per, g->n, g->nnz, h->rp, h->col, h->nlow, h->up_start, derr, dsearched,
                                            h->mirror, dsearched.p + 1);
         ND_CUDA(cudaGetLastError());
         if (h->long_segs > 0) {
@@ -1610,7 +1890,8 @@ struct nd_row_segments {
 // every row of h->rp in the order of k's buckets
 template <typename K>
 static nd_status order_rows(nd_incidence* h, const K& k, const nd_row_segments& sg, cudaStream_t st) {
-    k_order_rows<K><<<nd_blocks_for(h->n * 32, kThreads, grid_cap(h) * 4), kThreads, 0, st>>>(h->n, h->rp, k);
+    const int per = rows_per_warp(h->n);
+    k_order_rows<K><<<pool_blocks(h->n, per, grid_cap(h) * 4), kThreads, 0, st>>>(per, h->n, h->rp, k);
     ND_CUDA(cudaGetLastError());
     if (sg.segs == 0) return ND_OK;
     const int blocks = nd_blocks_for(sg.segs * 32, kThreads, grid_cap(h) * 4);
@@ -1732,17 +2013,17 @@ static nd_status orient_graph(nd_incidence* h, nd_oriented* o, cudaStream_t st) 
         ND_TRY(o->out_mir.alloc(m));
     }
     ND_CUDA(cudaMemsetAsync(o->out_ptr.p + n, 0, sizeof(int64_t), st));
-    const int vblocks = nd_blocks_for(n * 32, kThreads, grid_cap(h) * 4);
+    const int per = rows_per_warp(n), vblocks = pool_blocks(n, per, grid_cap(h) * 4);
     if (n > 0) {
         nd_prof_scope ps("orient", st);
-        k_orient<false><<<vblocks, kThreads, 0, st>>>(n, h->rp, h->col, h->eid, o->out_ptr, nullptr, nullptr, nullptr,
+        k_orient<false><<<vblocks, kThreads, 0, st>>>(per, n, h->rp, h->col, h->eid, o->out_ptr, nullptr, nullptr, nullptr,
                                                       nullptr, nullptr, nullptr);
         ND_CUDA(cudaGetLastError());
     }
     ND_TRY(nd_scan_i64(o->out_ptr, n, st));
     if (n > 0) {
         nd_prof_scope ps("orient", st);
-        k_orient<true><<<vblocks, kThreads, 0, st>>>(n, h->rp, h->col, h->eid, o->out_ptr, o->out_col, o->out_eid,
+        k_orient<true><<<vblocks, kThreads, 0, st>>>(per, n, h->rp, h->col, h->eid, o->out_ptr, o->out_col, o->out_eid,
                                                      o->out_src, h->mirror, positions ? o->out_pos.p : nullptr,
                                                      o->out_mir);
         ND_CUDA(cudaGetLastError());
@@ -1772,8 +2053,9 @@ static nd_status sort_tri_rows(nd_incidence* h, cudaStream_t st) {
     ND_CUDA(cudaFuncSetAttribute(k_row_rank<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     {
         nd_prof_scope ps("row_rank", st);
-        const int blocks = nd_blocks_for(N * 32, 32 * kRankWarps, grid_cap(h) * 8);
-        k_row_rank<false><<<blocks, 32 * kRankWarps, smem, st>>>(N, h->inc_ptr, h->e_u, h->e_v, h->rp,
+        const int per = rows_per_warp(N);
+        const int blocks = nd_blocks_for((N + per - 1) / per * 32, 32 * kRankWarps, grid_cap(h) * 8);
+        k_row_rank<false><<<blocks, 32 * kRankWarps, smem, st>>>(per, N, h->inc_ptr, h->e_u, h->e_v, h->rp,
                                                                   (const uint2*)h->inc, dst, over, over_ctr,
                                                                   nullptr, 0);
         ND_CUDA(cudaGetLastError());
@@ -1792,7 +2074,7 @@ static nd_status sort_tri_rows(nd_incidence* h, cudaStream_t st) {
         ND_TRY(scratch.alloc((int64_t)2 * (int64_t)hc[1] * warps));
         nd_prof_scope ps("row_rank", st);
         k_row_rank<true><<<warps / kRankWarps, 32 * kRankWarps, 0, st>>>(
-            N, h->inc_ptr, h->e_u, h->e_v, h->rp, (const uint2*)h->inc, dst, over, over_ctr, scratch,
+            1, N, h->inc_ptr, h->e_u, h->e_v, h->rp, (const uint2*)h->inc, dst, over, over_ctr, scratch,
             (int64_t)hc[1]);
         ND_CUDA(cudaGetLastError());
     }
@@ -1814,7 +2096,8 @@ nd_status nd_build_tri_incidence(nd_incidence* h, cudaStream_t st) {
     if (m == 0) { h->num_inc = 0; ND_TRY(nd_alloc((void**)&h->inc, 16, st, h)); return ND_OK; }
     nd_oriented o(st);
     ND_TRY(orient_graph(h, &o, st));
-    const int eblocks = nd_blocks_for(m * 32, kThreads, grid_cap(h) * 4);
+    const int eblocks = nd_blocks_for(m * 32, kThreads, grid_cap(h) * 4);  // a warp per oriented edge
+    const int per = rows_per_warp(m), pblocks = pool_blocks(m, per, grid_cap(h) * 4);
     // the stored adjacency layout keeps the count pass's triangles as records
     // (4 B each, min(|out(u)|, |out(v)|) slots reserved per oriented edge), so
     // that the fill does not search again; without the memory for them the
@@ -1839,14 +2122,10 @@ nd_status nd_build_tri_incidence(nd_incidence* h, cudaStream_t st) {
         ND_TRY(cnt32.alloc(m));
         ND_CUDA(cudaMemsetAsync(cnt32, 0, sizeof(unsigned) * m, st));
         nd_prof_scope ps("tri_count", st, 2);
-        if (use_rec)
-            k_tri_oriented<false, false, unsigned, true><<<eblocks, kThreads, 0, st>>>(
-                m, o.out_ptr, o.out_col, o.out_eid, o.out_src, nullptr, nullptr, cnt32.p, nullptr, rec_ptr, rec,
-                rec_cnt);
-        else
-            k_tri_oriented<false, false, unsigned><<<eblocks, kThreads, 0, st>>>(m, o.out_ptr, o.out_col, o.out_eid,
-                                                                                 o.out_src, nullptr, nullptr, cnt32.p,
-                                                                                 nullptr);
+        auto count = use_rec ? k_tri_count<true> : k_tri_count<false>;
+        count<<<pblocks, kThreads, 0, st>>>(
+            per, m, o.out_ptr, o.out_col, o.out_eid, o.out_src, cnt32.p, use_rec ? rec_ptr.p : nullptr,
+            use_rec ? rec.p : nullptr, use_rec ? rec_cnt.p : nullptr);
         ND_CUDA(cudaGetLastError());
         k_widen_u32<<<nd_blocks_for(m, kThreads, grid_cap(h) * 4), kThreads, 0, st>>>(m, cnt32, h->inc_ptr);
         ND_CUDA(cudaGetLastError());
@@ -1875,23 +2154,21 @@ nd_status nd_build_tri_incidence(nd_incidence* h, cudaStream_t st) {
         }
         nd_prof_scope ps("tri_fill", st);
         if (use_rec && narrow)
-            k_tri_fill_rec<unsigned><<<eblocks, kThreads, 0, st>>>(m, o.out_ptr, o.out_col, o.out_eid, o.out_src,
+            k_tri_fill_rec<unsigned><<<pblocks, kThreads, 0, st>>>(per, m, o.out_ptr, o.out_col, o.out_eid, o.out_src,
                                                                    o.out_pos, o.out_mir, cursor32.p, (uint2*)h->inc,
                                                                    rec_ptr, rec, rec_cnt);
         else if (use_rec)
-            k_tri_fill_rec<unsigned long long><<<eblocks, kThreads, 0, st>>>(
-                m, o.out_ptr, o.out_col, o.out_eid, o.out_src, o.out_pos, o.out_mir, cursor.p, (uint2*)h->inc, rec_ptr,
+            k_tri_fill_rec<unsigned long long><<<pblocks, kThreads, 0, st>>>(
+                per, m, o.out_ptr, o.out_col, o.out_eid, o.out_src, o.out_pos, o.out_mir, cursor.p, (uint2*)h->inc, rec_ptr,
                 rec, rec_cnt);
         else if (narrow)
-            k_tri_oriented<true, true, unsigned><<<eblocks, kThreads, 0, st>>>(
-                m, o.out_ptr, o.out_col, o.out_eid, o.out_src, o.out_pos, o.out_mir, cursor32.p, (uint2*)h->inc);
-        else if (h->adj)
-            k_tri_oriented<true, true><<<eblocks, kThreads, 0, st>>>(m, o.out_ptr, o.out_col, o.out_eid, o.out_src,
-                                                                     o.out_pos, o.out_mir, cursor.p, (uint2*)h->inc);
-        else
-            k_tri_oriented<true, false><<<eblocks, kThreads, 0, st>>>(m, o.out_ptr, o.out_col, o.out_eid,
-                                                                      o.out_src, nullptr, nullptr, cursor.p,
+            k_tri_fill_search<unsigned><<<eblocks, kThreads, 0, st>>>(m, o.out_ptr, o.out_col, o.out_eid, o.out_src,
+                                                                      o.out_pos, o.out_mir, cursor32.p,
                                                                       (uint2*)h->inc);
+        else
+            k_tri_fill_search<unsigned long long><<<eblocks, kThreads, 0, st>>>(m, o.out_ptr, o.out_col, o.out_eid,
+                                                                                o.out_src, o.out_pos, o.out_mir,
+                                                                                cursor.p, (uint2*)h->inc);
         ND_CUDA(cudaGetLastError());
     }
     // the records are no longer needed: free them before the row ranking

@@ -242,7 +242,7 @@ void nd_free(nd_incidence* h) {
     cudaStream_t st = h->last_stream;
     cudaStreamSynchronize(st);
     void* ptrs[] = {h->nlow, h->up_start, h->eid, h->e_u, h->e_v, h->tri_ptr, h->tri_w, h->tri_e,
-                    h->items, h->tau[0], h->tau[1], h->front[0], h->front[1], h->list, h->counters,
+                    h->items, h->tau[0], h->tau[1], h->front[0], h->front[1], h->front[2], h->front[3], h->list, h->counters,
                     h->mirror, h->e_pos, h->tg[0], h->tg[1], h->long_rows, h->long_seg, h->to_new, h->to_old,
                     h->vto_old, h->oct_max, h->t_pos, h->t_id, h->c_rp, h->c_up, h->c_col, h->c_nlow, h->gid, h->gact[0], h->gact[1]};
     for (void* p : ptrs) nd_release(p, st);

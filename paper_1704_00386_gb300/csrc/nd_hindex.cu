@@ -129,6 +129,8 @@ struct SweepParams {
     bool direct;                   // AND: rows are expected to fail the count (see warp_hindex)
     const uint32_t* cur;  // AND + notification: frontier read in this pass
     uint32_t* next;       // and the frontier written for the next pass
+    uint32_t* spare;      // INLINE: the one of the pass after that, to be cleared
+    int64_t spare_words;
     // relabelled (1,2) runs from d_s: the largest degree, so the largest tau, of
     // the ids from 2^o on; rows are ordered by floor(log2 id).  Null: no bound
     const int32_t* __restrict__ oct_max;
@@ -588,10 +590,19 @@ __device__ __forceinline__ unsigned front_bit(const uint32_t* f, uint32_t i) {
     return (__ldg(f + (i >> 5)) >> (i & 31)) & 1u;
 }
 
-// (2,3): is R in the current frontier?  Either bit of its two slots
+// is R in the current frontier?  With slots: any bit of its slots
+template <int Q>
 __device__ __forceinline__ bool in_frontier(const SweepParams& P, uint32_t R) {
-    const uint2 ep = __ldg(P.epos + R);
-    return front_bit(P.cur, ep.x) | front_bit(P.cur, ep.y);
+    if constexpr (Q == 2) {
+        const uint2 ep = __ldg(P.epos + R);
+        return front_bit(P.cur, ep.x) | front_bit(P.cur, ep.y);
+    } else if constexpr (Q == 3) {
+        const uint32_t* p = P.tpos + 3 * (int64_t)R;
+        const uint32_t a = __ldg(p), b = __ldg(p + 1), c = __ldg(p + 2);
+        return front_bit(P.cur, a) | front_bit(P.cur, b) | front_bit(P.cur, c);
+    } else {
+        return front_bit(P.cur, R);
+    }
 }
 
 // the ids of entry j of a row of d entries
@@ -753,8 +764,9 @@ __device__ __forceinline__ nd_item pass_item(const SweepParams& P, int64_t i) {
 // one).  NOTIFY: the entries of all rows that changed are then walked by the
 // 32 lanes together, instead of each row by its own G lanes while the other
 // groups wait.
-template <int Q, int G, int C, bool AND, bool NOTIFY, bool GB>
-__device__ __forceinline__ void run_groups(const SweepParams& P, const nd_item& it, bool run, Tally<false>& n) {
+template <int Q, int G, int C, bool AND, bool NOTIFY, bool GB, bool INLINE>
+__device__ __forceinline__ void run_groups(const SweepParams& P, const nd_item& it, bool run, Tally<INLINE>& n) {
+    if (INLINE) run = run && in_frontier<Q>(P, it.R);
     constexpr int NG = 32 / G;
     const int lane = threadIdx.x & 31;
     int32_t t0, t, old;
@@ -796,10 +808,11 @@ __device__ __forceinline__ void run_groups(const SweepParams& P, const nd_item& 
 }
 
 // one r-clique per warp (rows of the warp bucket), streamed
-template <int Q, bool AND, bool NOTIFY, bool GB, int HW>
+template <int Q, bool AND, bool NOTIFY, bool GB, int HW, bool INLINE>
 __device__ __forceinline__ void run_warp_row(const SweepParams& P, const nd_item& it, unsigned* bins,
-                                             Tally<false>& n) {
+                                             Tally<INLINE>& n) {
     const uint32_t R = it.R;
+    if (INLINE && !in_frontier<Q>(P, R)) return;
     int32_t t0, t, old;
     load_tau<AND>(P, it, t0, t, old);
     const bool direct = P.direct || (!AND && old != t0);
@@ -821,11 +834,12 @@ __device__ __forceinline__ void run_warp_row(const SweepParams& P, const nd_item
 }
 
 // one r-clique per CTA (rows past the warp threshold)
-template <int Q, bool AND, bool NOTIFY, bool GB, int WORDS>
+template <int Q, bool AND, bool NOTIFY, bool GB, int WORDS, bool INLINE>
 __device__ __forceinline__ void run_cta(const SweepParams& P, int64_t i, unsigned* bins, int* bounds,
-                                        Tally<false>& n) {
-    const nd_item it = pass_item<NOTIFY || GB>(P, i);
+                                        Tally<INLINE>& n) {
+    const nd_item it = pass_item<(NOTIFY && !INLINE) || GB>(P, i);
     const uint32_t R = it.R;
+    if (INLINE && !in_frontier<Q>(P, R)) return;  // the same R for the whole block
     int32_t t0, t, old;
     load_tau<AND>(P, it, t0, t, old);
     __syncthreads();  // AND: every thread has read tau(R) before it is written
@@ -1025,17 +1039,25 @@ constexpr int kPassBlocks = 6;  // resident blocks per SM the register budget of
 // LATE: the passes after the first of a run, where few rows search: a
 // quarter of the histogram, and the shared memory it frees serves as L1 for
 // the gathers
-template <int Q, bool AND, bool NOTIFY, bool GB, bool LATE>
+// INLINE: AND with notification on a handle of at most kInlineItems work items
+// takes no list: a launch costs more than the rows' own frontier tests.  The
+// pass clears the frontier of the pass after next, of four (a clear by memset
+// or with the list costs a launch of its own).  A 2,000-vertex k-core: 16
+// passes in 0.13 instead of 0.23 ms.
+template <int Q, bool AND, bool NOTIFY, bool GB, bool LATE, bool INLINE = false>
 __global__ void __launch_bounds__(kThreads, kPassBlocks) k_pass(SweepParams P) {
     if (P.prev != nullptr && *(volatile const unsigned long long*)P.prev == 0ull) return;  // converged
-    constexpr bool LISTED = NOTIFY || GB;
+    constexpr bool LISTED = (NOTIFY && !INLINE) || GB;
     constexpr int HW = LATE ? kLateHistWords : kHistWords;
     constexpr int kWords = (kThreads / 32) * HW;  // a CTA row uses every warp's histogram
     __shared__ __align__(16) unsigned hist[kThreads / 32][HW];
     __shared__ int bounds[kThreads / 32];
     __shared__ unsigned long long s_chunk;
     unsigned* const bins = hist[threadIdx.x >> 5];
-    Tally<false> n;
+    Tally<INLINE> n;
+    if (INLINE)
+        for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < P.spare_words; i += (int64_t)gridDim.x * kThreads)
+            P.spare[i] = 0u;
     // the rows of each bucket: [lo, lo + rows) of the work items, or of the list
     auto lo = [&](int b) { return LISTED ? P.list_lo[b] : P.lo[b]; };
     auto rows = [&](int b) { return LISTED ? (int64_t)__ldcg(P.ctr + ND_CTR_LIST + b) : P.hi[b] - P.lo[b]; };
@@ -1050,7 +1072,7 @@ __global__ void __launch_bounds__(kThreads, kPassBlocks) k_pass(SweepParams P) {
             const int64_t c = (int64_t)s_chunk;
             __syncthreads();
             if (c >= n3) break;
-            run_cta<Q, AND, NOTIFY, GB, kWords>(P, lo(3) + c, &hist[0][0], bounds, n);
+            run_cta<Q, AND, NOTIFY, GB, kWords, INLINE>(P, lo(3) + c, &hist[0][0], bounds, n);
         }
     };
     // AND updates in place, so a row evaluated later in a pass already sees
@@ -1098,7 +1120,7 @@ __global__ void __launch_bounds__(kThreads, kPassBlocks) k_pass(SweepParams P) {
             while (t < e2) {
                 nd_item nx;
                 if (t + 1 < e2) nx = pass_item<LISTED>(P, lo(2) + t + 1);
-                run_warp_row<Q, AND, NOTIFY, GB, HW>(P, it, bins, n);
+                run_warp_row<Q, AND, NOTIFY, GB, HW, INLINE>(P, it, bins, n);
                 it = nx;
                 ++t;
             }
@@ -1118,7 +1140,7 @@ __global__ void __launch_bounds__(kThreads, kPassBlocks) k_pass(SweepParams P) {
             for (int64_t k = from; k < to; ++k) {
                 nd_item nx;
                 if (!NOTIFY && k + 1 < to) nx = item(k + 1);
-                run_groups<Q, G, decltype(group)::entries, AND, NOTIFY, GB>(P, it, NG * k + lane32 / G < count, n);
+                run_groups<Q, G, decltype(group)::entries, AND, NOTIFY, GB, INLINE>(P, it, NG * k + lane32 / G < count, n);
                 if (NOTIFY && k + 1 < to) nx = item(k + 1);
                 it = nx;
             }
@@ -1394,7 +1416,7 @@ __global__ void __launch_bounds__(kThreads, kPassBlocks) k_pass_otf(SweepParams 
             const nd_item it = load_item(P.items, first + rows - 1 - r0 - lane);
             R = it.R;
             d = it.d;
-            if (AND && NOTIFY) run = in_frontier(P, R);
+            if (AND && NOTIFY) run = in_frontier<2>(P, R);
         }
         if (run) {
             my_t0 = ld_tau<!AND>(P.tin + R);
@@ -1511,7 +1533,8 @@ typedef void (*pass_fn)(SweepParams);
 // the pass kernel of a run; late: for the passes from kLateFrom on
 constexpr int kLateFrom = ND_BATCH;
 template <int Q>
-pass_fn pick_q(int mode, bool batch, bool late) {
+pass_fn pick_q(int mode, bool batch, bool late, bool in_line) {
+    if (in_line) return k_pass<Q, true, true, false, false, true>;
     if (mode == ND_AND) return late ? k_pass<Q, true, true, false, true> : k_pass<Q, true, true, false, false>;
     if (mode == ND_SND) {
         if (batch) return late ? k_pass<Q, false, false, true, true> : k_pass<Q, false, false, true, false>;
@@ -1520,13 +1543,13 @@ pass_fn pick_q(int mode, bool batch, bool late) {
     if (batch) return late ? k_pass<Q, true, false, true, true> : k_pass<Q, true, false, true, false>;
     return late ? k_pass<Q, true, false, false, true> : k_pass<Q, true, false, false, false>;
 }
-pass_fn pick(const nd_incidence* h, int mode, bool late) {
+pass_fn pick(const nd_incidence* h, int mode, bool late, bool in_line) {
     // mode: ND_SND, ND_AND (notify), ND_AND_NN
     if (h->otf) return mode == ND_SND ? k_pass_otf<false, false> : (mode == ND_AND ? k_pass_otf<true, true> : k_pass_otf<true, false>);
     const bool batch = h->gid && mode != ND_AND;  // converged graphs are skipped
-    if (h->q == 1) return pick_q<1>(mode, batch, late);
-    if (h->q == 2) return pick_q<2>(mode, batch, late);
-    return h->t_pos ? pick_q<3>(mode, batch, late) : pick_q<kIds>(mode, batch, late);
+    if (h->q == 1) return pick_q<1>(mode, batch, late, in_line);
+    if (h->q == 2) return pick_q<2>(mode, batch, late, in_line);
+    return h->t_pos ? pick_q<3>(mode, batch, late, in_line) : pick_q<kIds>(mode, batch, late, in_line);
 }
 
 // bucket ranges of a pass
@@ -1671,12 +1694,26 @@ nd_status request_carveout(const void* fn) {
 // scale-20 k-truss, 71.9 / 68.0 / 66.1 / 62.9 / 62.7 on the scale-24 k-core
 constexpr int kAndDirect = 6;
 
+// AND with notification without a list (INLINE): small handles, with room for
+// two more frontiers
+constexpr int64_t kInlineItems = 1 << 15, kInlineBits = 1 << 22;
+bool take_inline(nd_incidence* h, int64_t words, cudaStream_t st) {
+    if (h->bucket_lo[ND_NB] > kInlineItems || 32 * words > kInlineBits) return false;
+    for (int b = 2; b < 4; ++b)
+        if (!h->front[b] && nd_alloc((void**)&h->front[b], sizeof(uint32_t) * words, st, h) != ND_OK) {
+            nd_set_error("");
+            return false;
+        }
+    return true;
+}
+
 // parameters of one pass: its counter slot, the slot of the pass before it
-// (-1: none), and the parity of its index in the run (SND reads tau[parity]
+// (-1: none), its index in the run (by whose parity SND reads tau[parity]
 // and writes the other buffer; AND reads the frontier front[parity])
 // and whether an AND pass takes its rows for changing ones (its first passes)
 SweepParams pass_params(const nd_incidence* h, int mode, const SweepParams& P0, int slot, int prev_slot,
-                        int parity, bool direct) {
+                        int index, bool direct) {
+    const int parity = index & 1;
     SweepParams P = P0;
     P.direct = direct;
     P.ctr = h->counters + ND_SLOT * slot;
@@ -1690,8 +1727,9 @@ SweepParams pass_params(const nd_incidence* h, int mode, const SweepParams& P0, 
         P.tout = h->tau[0];
         P.gin = h->tg[0];
         P.gout = h->tg[0];
-        P.cur = h->front[parity];
-        P.next = h->front[parity ^ 1];
+        P.cur = h->front[P0.spare_words > 0 ? index & 3 : parity];
+        P.next = h->front[P0.spare_words > 0 ? (index + 1) & 3 : parity ^ 1];
+        P.spare = h->front[(index + 2) & 3];
     } else {
         P.tin = h->tau[parity];
         P.tout = h->tau[parity ^ 1];
@@ -1728,7 +1766,7 @@ void make_batch_graph(nd_incidence* h, int mode, int kind, const SweepParams& P0
         // a batch starts at an even pass; its first pass reads the last slot
         // of the other half (the caller puts the previous pass's counters there)
         const int prev_slot = k > 0 ? base + k - 1 : (kind == 0 ? -1 : (base ^ ND_BATCH) + ND_BATCH - 1);
-        SweepParams P = pass_params(h, mode, P0, base + k, prev_slot, k & 1, mode != ND_SND && kind == 0 && k < kAndDirect);
+        SweepParams P = pass_params(h, mode, P0, base + k, prev_slot, k, mode != ND_SND && kind == 0 && k < kAndDirect);
         if (ok && P.gid) {  // batches: the graphs changing in this pass, from none
             cudaMemsetParams ms = {};
             ms.dst = P.gact_out;
@@ -1740,7 +1778,7 @@ void make_batch_graph(nd_incidence* h, int mode, int kind, const SweepParams& P0
             ok = cudaGraphAddMemsetNode(&n, g, &last, 1, &ms) == cudaSuccess;
             last = n;
         }
-        if (ok && (mode == ND_AND || P.gid)) {
+        if (ok && ((mode == ND_AND && !P.spare_words) || P.gid)) {
             ListParams lp;
             const int blocks = list_params(h, L, 0, L.tiles, P, &lp);
             cudaKernelNodeParams kp = {};
@@ -1956,6 +1994,11 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
     SweepParams P;
     P.inc = h->inc;
     P.epos = h->e_pos;
+    // small handles test the frontier row by row
+    const bool in_line = mode == ND_AND && !h->otf && take_inline(h, words, st);
+    P.spare = nullptr;
+    P.spare_words = in_line ? words : 0;
+    if (in_line) ND_CUDA(cudaMemsetAsync(h->front[1], 0, sizeof(uint32_t) * words, st));
     P.list = nullptr;
     for (int b = 0; b < ND_NB; ++b) P.list_lo[b] = 0;
     P.tpos = h->t_pos;
@@ -1987,7 +2030,7 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
     P.by_degree = nullptr;
     P.slot_of = nullptr;
     if (h->otf) ND_TRY(make_hub_tables(h, &hubs, P, st));
-    pass_fn fn0 = pick(h, mode, false), fn1 = pick(h, mode, true);
+    pass_fn fn0 = pick(h, mode, false, in_line), fn1 = pick(h, mode, true, in_line);
     // ask for a shared-memory carve-out that just holds each kernel's
     // resident blocks (plus the 1 KB each block reserves), leaving the rest
     // of the SM's memory as L1 for the gathers.  Left to itself the driver
@@ -2002,7 +2045,7 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
     P.chunk = warp_chunk(units - (P.hi[3] - P.lo[3]), grid0 < grid1 ? grid0 : grid1);
     ListPlan L;
     nd_tmp<uint32_t> list_scratch(st);
-    if ((mode == ND_AND && !h->otf) || P.gid) ND_TRY(plan_list(h, words, list_scratch, &L, st));
+    if ((mode == ND_AND && !h->otf && !in_line) || P.gid) ND_TRY(plan_list(h, words, list_scratch, &L, st));
     // passes that evaluate every row do not count rows and incidences (Tally)
     const bool counted = h->otf || mode == ND_AND || P.gid;
     const int64_t all_rows = P.hi[ND_NB - 1] - P.lo[0], all_incs = h->num_inc;
@@ -2056,13 +2099,13 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
         if (!launched) {
             ND_CUDA(cudaMemsetAsync(h->counters + ND_SLOT * base, 0, sizeof(unsigned long long) * ND_SLOT * nb, st));
             for (int k = 0; k < nb; ++k, ++pass) {
-                SweepParams Pk = pass_params(h, mode, P, base + k, k > 0 ? base + k - 1 : last_slot, pass & 1,
+                SweepParams Pk = pass_params(h, mode, P, base + k, k > 0 ? base + k - 1 : last_slot, pass,
                                              mode != ND_SND && pass < kAndDirect);
                 if (Pk.gid) ND_CUDA(cudaMemsetAsync(Pk.gact_out, 0, (size_t)h->ngraphs, st));
                 if (mode == ND_AND && h->otf)
                     ND_CUDA(cudaMemsetAsync(Pk.next, 0, sizeof(uint32_t) * words, st));
                 if (grid0 == 0) continue;
-                const bool late = pass >= kLateFrom, listed = (mode == ND_AND && !h->otf) || Pk.gid;
+                const bool late = pass >= kLateFrom, listed = (mode == ND_AND && !h->otf && !in_line) || Pk.gid;
                 // the parts of a pass: one, unless the list has no room for all
                 for (int64_t t = 0; t == 0 || (listed && t < L.tiles); t += L.room) {
                     nd_prof_scope ps(pname, st, listed ? 2 : 1);

@@ -136,7 +136,7 @@ struct nd_incidence {
     int32_t thr[3] = {8, 64, 2048};  // bucket thresholds t0, t1, t2
     // iteration state
     int32_t* tau[2] = {nullptr, nullptr};
-    uint32_t* front[2] = {nullptr, nullptr};
+    uint32_t* front[4] = {nullptr, nullptr, nullptr, nullptr};  // the last two: small handles
     uint32_t* list = nullptr;                // the active work items of a pass (AND; batches)
     int64_t list_tiles = 0;                  // tiles of work items it holds
     unsigned long long* counters = nullptr;  // ring of per-pass counters

@@ -784,7 +784,7 @@ __device__ __forceinline__ bool precedes(int64_t du, int32_t u, int64_t dv, int3
 }
 
 // count / list the out-neighbours of every vertex in id order, 32 vertices per
-// warp (with out_pos: also the CSR positions of the entry and of its reverse)
+// warp (with out_pm: also the CSR positions of the entry and of its reverse)
 template <bool FILL>
 __global__ void __launch_bounds__(kThreads) k_orient(int per, int64_t n, const int64_t* __restrict__ rp,
                                                      const int32_t* __restrict__ col,
@@ -792,7 +792,7 @@ __global__ void __launch_bounds__(kThreads) k_orient(int per, int64_t n, const i
                                                      int32_t* __restrict__ out_col, uint32_t* __restrict__ out_eid,
                                                      int32_t* __restrict__ out_src,
                                                      const uint32_t* __restrict__ mirror,
-                                                     uint32_t* __restrict__ out_pos, uint32_t* __restrict__ out_mir) {
+                                                     uint2* __restrict__ out_pm) {
     __shared__ uint32_t pre[kThreads / 32][32];
     __shared__ int64_t begin[kThreads / 32][32], slots[kThreads / 32][32];  // slots: next output slot of each row
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -800,10 +800,7 @@ __global__ void __launch_bounds__(kThreads) k_orient(int per, int64_t n, const i
         out_col[slot] = v;
         out_eid[slot] = __ldg(eid + p);
         out_src[slot] = u;
-        if (out_pos) {
-            out_pos[slot] = (uint32_t)p;
-            out_mir[slot] = __ldg(mirror + p);
-        }
+        if (out_pm) out_pm[slot] = make_uint2((uint32_t)p, __ldg(mirror + p));
     };
     const int64_t groups = (n + per - 1) / per;
     for (int64_t g = warp_id_global(); g < groups; g += warp_count_global()) {
@@ -877,13 +874,12 @@ template <typename C>
 __global__ void __launch_bounds__(kThreads, ND_TRI_MIN_BLOCKS)
     k_tri_fill_search(int64_t m, const int64_t* __restrict__ out_ptr, const int32_t* __restrict__ out_col,
                       const uint32_t* __restrict__ out_eid, const int32_t* __restrict__ out_src,
-                      const uint32_t* __restrict__ out_pos, const uint32_t* __restrict__ out_mir, C* __restrict__ ctr,
-                      uint2* __restrict__ inc) {
+                      const uint2* __restrict__ out_pm, C* __restrict__ ctr, uint2* __restrict__ inc) {
     const int lane = threadIdx.x & 31;
     for (int64_t k = warp_id_global(); k < m; k += warp_count_global()) {
         const int32_t u = out_src[k], v = out_col[k];
         const uint32_t e_uv = out_eid[k];
-        const uint32_t Puv = __ldg(out_pos + k), Pvu = __ldg(out_mir + k);
+        const uint2 uv = __ldg(out_pm + k);  // P(u,v), P(v,u)
         int64_t ab = out_ptr[u], ae = out_ptr[u + 1], bb = out_ptr[v], be = out_ptr[v + 1];
         bool a_is_u = true;
         if (ae - ab > be - bb) {
@@ -898,23 +894,23 @@ __global__ void __launch_bounds__(kThreads, ND_TRI_MIN_BLOCKS)
             int32_t x = 0;
             // the values at p are loaded with x, ahead of the search
             // (coalesced), so only the loads at pb wait for it
-            uint32_t ea = 0, pa = 0, ma = 0;
+            uint32_t ea = 0;
+            uint2 pa = make_uint2(0, 0);
             if (p < ae) {
                 x = __ldg(out_col + p);
                 ea = __ldg(out_eid + p);
-                pa = __ldg(out_pos + p);
-                ma = __ldg(out_mir + p);
+                pa = __ldg(out_pm + p);
                 pb = lo + nd_lower_bound_n(out_col + lo, (int)(be - lo), x);
                 found = (pb < be) && (__ldg(out_col + pb) == x);
             }
             const unsigned bal = __ballot_sync(kFull, found);
             const int nf = __popc(bal);
             if (nf) {
-                uint32_t eb = 0, pbp = 0, mb = 0;
+                uint32_t eb = 0;
+                uint2 pq = make_uint2(0, 0);
                 if (found) {
                     eb = __ldg(out_eid + pb);
-                    pbp = __ldg(out_pos + pb);
-                    mb = __ldg(out_mir + pb);
+                    pq = __ldg(out_pm + pb);
                 }
                 const uint32_t e_uw = a_is_u ? ea : eb, e_vw = a_is_u ? eb : ea;
                 // the three slot reservations are independent: issue them together
@@ -927,11 +923,10 @@ __global__ void __launch_bounds__(kThreads, ND_TRI_MIN_BLOCKS)
                 s0 = __shfl_sync(kFull, s0, 0);
                 if (found) {
                     // third vertex w = x; positions P(.,.) of the six entries
-                    const uint32_t Puw = a_is_u ? pa : pbp, Pwu = a_is_u ? ma : mb;
-                    const uint32_t Pvw = a_is_u ? pbp : pa, Pwv = a_is_u ? mb : ma;
-                    inc[s0 + __popc(bal & lanemask_lt())] = u < v ? make_uint2(Puw, Pvw) : make_uint2(Pvw, Puw);
-                    inc[s_uw] = u < x ? make_uint2(Puv, Pwv) : make_uint2(Pwv, Puv);
-                    inc[s_vw] = v < x ? make_uint2(Pvu, Pwu) : make_uint2(Pwu, Pvu);
+                    const uint2 uw = a_is_u ? pa : pq, vw = a_is_u ? pq : pa;  // P(u,w), P(w,u); P(v,w), P(w,v)
+                    inc[s0 + __popc(bal & lanemask_lt())] = u < v ? make_uint2(uw.x, vw.x) : make_uint2(vw.x, uw.x);
+                    inc[s_uw] = u < x ? make_uint2(uv.x, vw.y) : make_uint2(vw.y, uv.x);
+                    inc[s_vw] = v < x ? make_uint2(uv.y, uw.y) : make_uint2(uw.y, uv.y);
                 }
             }
             const int64_t last_pb = __shfl_sync(kFull, pb, 31);
@@ -1017,19 +1012,28 @@ __global__ void __launch_bounds__(kThreads, ND_TRI_COUNT_MIN_BLOCKS)
     }
 }
 
-// the fill from the count pass's records, 32 consecutive oriented edges per
-// warp and one recorded triangle per lane, so no search is repeated.  The six
-// positions of a triangle are read at the recorded offsets of w in the two
-// out-lists; slots and entries are as in the searching fill.
+// The fill from the count pass's records: 32 consecutive oriented edges per
+// warp, two recorded triangles per lane at a time, so no search is repeated.
+// The six positions of a triangle are read at the recorded offsets of w in the
+// two out-lists; slots and entries are as in the searching fill.
+// Bound by the chain record -> list entries -> slots -> writes and by the L2
+// traffic of the slot atomics and scattered 8-byte writes.  Registers for two
+// tasks in flight are worth more than warps: one task at 5 blocks per SM takes
+// 22.8 ms on an R-MAT of 1,048,576 vertices (390M triangles), two at 3 blocks 20.6, at 4 blocks
+// 21.4, four at 2 blocks 19.7 (but 0.846 ms against 0.804 on the 100K-vertex
+// R-MAT, where few warps leave the last groups on few SMs; one task 0.833).
+#ifndef ND_FILL_TASKS
+#define ND_FILL_TASKS 2
+#endif
 #ifndef ND_FILL_MIN_BLOCKS
-#define ND_FILL_MIN_BLOCKS 5  // the fill from records: 48 registers (24.1 against 25.0 ms at 6 blocks)
+#define ND_FILL_MIN_BLOCKS 3
 #endif
 template <typename C>
 __global__ void __launch_bounds__(kThreads, ND_FILL_MIN_BLOCKS)
     k_tri_fill_rec(int per, int64_t m, const int64_t* __restrict__ out_ptr, const int32_t* __restrict__ out_col,
                    const uint32_t* __restrict__ out_eid, const int32_t* __restrict__ out_src,
-                   const uint32_t* __restrict__ out_pos, const uint32_t* __restrict__ out_mir, C* __restrict__ ctr,
-                   uint2* __restrict__ inc, const int64_t* __restrict__ rec_ptr, const uint32_t* __restrict__ rec,
+                   const uint2* __restrict__ out_pm, C* __restrict__ ctr, uint2* __restrict__ inc,
+                   const int64_t* __restrict__ rec_ptr, const uint32_t* __restrict__ rec,
                    const uint32_t* __restrict__ rec_cnt) {
     __shared__ uint32_t pre[kThreads / 32][32];
     __shared__ uint32_t ab[kThreads / 32][32], bb[kThreads / 32][32];
@@ -1055,46 +1059,61 @@ __global__ void __launch_bounds__(kThreads, ND_FILL_MIN_BLOCKS)
             rp0[w][lane] = rec_ptr[mine];
         }
         const row_pool pool(pre[w], c);
-        for (int e0 = 0; e0 < pool.total; e0 += 32) {
-            const int i = e0 + lane;
-            const bool found = i < pool.total;
-            const int r = pool.row(min(i, pool.total - 1));
-            const int64_t k = k0 + r;
-            uint32_t ea = 0, pa = 0, ma = 0, eb = 0, pbp = 0, mb = 0, e_uv = 0, Puv = 0, Pvu = 0;
-            int32_t x = 0;
-            if (found) {
-                const uint32_t q = __ldg(rec + rp0[w][r] + (i - (int)pool.pre[r]));
-                const uint32_t p = ab[w][r] + (q & 0xffffu), pb = bb[w][r] + (q >> 16);
-                e_uv = __ldg(out_eid + k);
-                Puv = __ldg(out_pos + k);
-                Pvu = __ldg(out_mir + k);
-                x = __ldg(out_col + p);
-                ea = __ldg(out_eid + p);
-                pa = __ldg(out_pos + p);
-                ma = __ldg(out_mir + p);
-                eb = __ldg(out_eid + pb);
-                pbp = __ldg(out_pos + pb);
-                mb = __ldg(out_mir + pb);
+        constexpr int U = ND_FILL_TASKS;
+        for (int e0 = 0; e0 < pool.total; e0 += 32 * U) {
+            int r[U];
+            uint32_t p[U], pb[U];
+            bool found[U];
+#pragma unroll
+            for (int t = 0; t < U; ++t) {
+                const int i = e0 + 32 * t + lane;
+                found[t] = i < pool.total;
+                r[t] = pool.row(min(i, pool.total - 1));
+                p[t] = found[t] ? __ldg(rec + rp0[w][r[t]] + (i - (int)pool.pre[r[t]])) : 0;
             }
-            const unsigned same = row_pool::same_row(r) & __ballot_sync(kFull, found);
-            const bool a_is_u = a_is[w][r];
-            const int32_t u = vu[w][r], v = vv[w][r];
-            const uint32_t e_uw = a_is_u ? ea : eb, e_vw = a_is_u ? eb : ea;
-            // the three slot reservations are independent: issue them together
-            C s0 = 0, s_uw = 0, s_vw = 0;
-            const int leader = __ffs(same) - 1;
-            if (found && lane == leader) s0 = atomicAdd(ctr + e_uv, (C)__popc(same));
-            if (found) {
-                s_uw = atomicAdd(ctr + e_uw, (C)1);
-                s_vw = atomicAdd(ctr + e_vw, (C)1);
+            uint32_t ea[U], eb[U], e_uv[U];
+            uint2 pa[U], pq[U], uv[U];
+            int32_t x[U];
+#pragma unroll
+            for (int t = 0; t < U; ++t) {
+                if (found[t]) {
+                    pb[t] = bb[w][r[t]] + (p[t] >> 16);
+                    p[t] = ab[w][r[t]] + (p[t] & 0xffffu);
+                    e_uv[t] = __ldg(out_eid + k0 + r[t]);
+                    ea[t] = __ldg(out_eid + p[t]);
+                    eb[t] = __ldg(out_eid + pb[t]);
+                    uv[t] = __ldg(out_pm + k0 + r[t]);
+                    x[t] = __ldg(out_col + p[t]);
+                    pa[t] = __ldg(out_pm + p[t]);
+                    pq[t] = __ldg(out_pm + pb[t]);
+                }
             }
-            s0 = __shfl_sync(kFull, s0, found ? leader : lane);
-            if (found) {
-                const uint32_t Puw = a_is_u ? pa : pbp, Pwu = a_is_u ? ma : mb;
-                const uint32_t Pvw = a_is_u ? pbp : pa, Pwv = a_is_u ? mb : ma;
-                inc[s0 + __popc(same & lanemask_lt())] = u < v ? make_uint2(Puw, Pvw) : make_uint2(Pvw, Puw);
-                inc[s_uw] = u < x ? make_uint2(Puv, Pwv) : make_uint2(Pwv, Puv);
-                inc[s_vw] = v < x ? make_uint2(Pvu, Pwu) : make_uint2(Pwu, Pvu);
+            unsigned same[U];
+            C s0[U], s_uw[U], s_vw[U];
+            // the slot reservations are independent: issue them together
+#pragma unroll
+            for (int t = 0; t < U; ++t) {
+                same[t] = row_pool::same_row(r[t]) & __ballot_sync(kFull, found[t]);
+                const bool a_is_u = a_is[w][r[t]];
+                s0[t] = 0;
+                if (found[t]) {
+                    if (lane == __ffs(same[t]) - 1) s0[t] = atomicAdd(ctr + e_uv[t], (C)__popc(same[t]));
+                    s_uw[t] = atomicAdd(ctr + (a_is_u ? ea[t] : eb[t]), (C)1);
+                    s_vw[t] = atomicAdd(ctr + (a_is_u ? eb[t] : ea[t]), (C)1);
+                }
+            }
+#pragma unroll
+            for (int t = 0; t < U; ++t) {
+                const bool a_is_u = a_is[w][r[t]];
+                const C first = __shfl_sync(kFull, s0[t], found[t] ? __ffs(same[t]) - 1 : lane);
+                if (found[t]) {
+                    const int32_t u = vu[w][r[t]], v = vv[w][r[t]];
+                    const uint2 uw = a_is_u ? pa[t] : pq[t], vw = a_is_u ? pq[t] : pa[t];
+                    inc[first + __popc(same[t] & lanemask_lt())] =
+                        u < v ? make_uint2(uw.x, vw.x) : make_uint2(vw.x, uw.x);
+                    inc[s_uw[t]] = u < x[t] ? make_uint2(uv[t].x, vw.y) : make_uint2(vw.y, uv[t].x);
+                    inc[s_vw[t]] = v < x[t] ? make_uint2(uv[t].y, uw.y) : make_uint2(uw.y, uv[t].y);
+                }
             }
         }
     }
@@ -1996,9 +2015,10 @@ nd_status nd_build_edges(nd_incidence* h, cudaStream_t st) {
 struct nd_oriented {
     nd_tmp<int64_t> out_ptr;
     nd_tmp<int32_t> out_col, out_src;
-    nd_tmp<uint32_t> out_eid, out_pos, out_mir;
+    nd_tmp<uint32_t> out_eid;
+    nd_tmp<uint2> out_pm;  // CSR positions of the entry and of its reverse
     explicit nd_oriented(cudaStream_t st)
-        : out_ptr(st), out_col(st), out_src(st), out_eid(st), out_pos(st), out_mir(st) {}
+        : out_ptr(st), out_col(st), out_src(st), out_eid(st), out_pm(st) {}
 };
 
 static nd_status orient_graph(nd_incidence* h, nd_oriented* o, cudaStream_t st) {
@@ -2008,24 +2028,20 @@ static nd_status orient_graph(nd_incidence* h, nd_oriented* o, cudaStream_t st) 
     ND_TRY(o->out_src.alloc(m));
     ND_TRY(o->out_eid.alloc(m));
     const bool positions = h->adj && !h->otf;  // only the stored (2,3) fill uses them
-    if (positions) {
-        ND_TRY(o->out_pos.alloc(m));
-        ND_TRY(o->out_mir.alloc(m));
-    }
+    if (positions) ND_TRY(o->out_pm.alloc(m));
     ND_CUDA(cudaMemsetAsync(o->out_ptr.p + n, 0, sizeof(int64_t), st));
     const int per = rows_per_warp(n), vblocks = pool_blocks(n, per, grid_cap(h) * 4);
     if (n > 0) {
         nd_prof_scope ps("orient", st);
         k_orient<false><<<vblocks, kThreads, 0, st>>>(per, n, h->rp, h->col, h->eid, o->out_ptr, nullptr, nullptr, nullptr,
-                                                      nullptr, nullptr, nullptr);
+                                                      nullptr, nullptr);
         ND_CUDA(cudaGetLastError());
     }
     ND_TRY(nd_scan_i64(o->out_ptr, n, st));
     if (n > 0) {
         nd_prof_scope ps("orient", st);
         k_orient<true><<<vblocks, kThreads, 0, st>>>(per, n, h->rp, h->col, h->eid, o->out_ptr, o->out_col, o->out_eid,
-                                                     o->out_src, h->mirror, positions ? o->out_pos.p : nullptr,
-                                                     o->out_mir);
+                                                     o->out_src, h->mirror, positions ? o->out_pm.p : nullptr);
         ND_CUDA(cudaGetLastError());
     }
     return ND_OK;
@@ -2155,20 +2171,19 @@ nd_status nd_build_tri_incidence(nd_incidence* h, cudaStream_t st) {
         nd_prof_scope ps("tri_fill", st);
         if (use_rec && narrow)
             k_tri_fill_rec<unsigned><<<pblocks, kThreads, 0, st>>>(per, m, o.out_ptr, o.out_col, o.out_eid, o.out_src,
-                                                                   o.out_pos, o.out_mir, cursor32.p, (uint2*)h->inc,
-                                                                   rec_ptr, rec, rec_cnt);
+                                                                   o.out_pm, cursor32.p, (uint2*)h->inc, rec_ptr, rec,
+                                                                   rec_cnt);
         else if (use_rec)
             k_tri_fill_rec<unsigned long long><<<pblocks, kThreads, 0, st>>>(
-                per, m, o.out_ptr, o.out_col, o.out_eid, o.out_src, o.out_pos, o.out_mir, cursor.p, (uint2*)h->inc, rec_ptr,
+                per, m, o.out_ptr, o.out_col, o.out_eid, o.out_src, o.out_pm, cursor.p, (uint2*)h->inc, rec_ptr,
                 rec, rec_cnt);
         else if (narrow)
             k_tri_fill_search<unsigned><<<eblocks, kThreads, 0, st>>>(m, o.out_ptr, o.out_col, o.out_eid, o.out_src,
-                                                                      o.out_pos, o.out_mir, cursor32.p,
-                                                                      (uint2*)h->inc);
+                                                                      o.out_pm, cursor32.p, (uint2*)h->inc);
         else
             k_tri_fill_search<unsigned long long><<<eblocks, kThreads, 0, st>>>(m, o.out_ptr, o.out_col, o.out_eid,
-                                                                                o.out_src, o.out_pos, o.out_mir,
-                                                                                cursor.p, (uint2*)h->inc);
+                                                                                o.out_src, o.out_pm, cursor.p,
+                                                                                (uint2*)h->inc);
         ND_CUDA(cudaGetLastError());
     }
     // the records are no longer needed: free them before the row ranking

@@ -71,6 +71,23 @@ def test_rows_at_the_edges(nd, r, pad):
     np.testing.assert_array_equal(ta.cpu().numpy(), kap)
 
 
+# builds that keep the count pass's triangles as records: warps with thousands
+# of triangles (whole blocks of two per lane), and with none, one or a few
+@pytest.mark.parametrize("n,m", [(700, 70_000), (9000, 90_000), (40_000, 68_000)])
+def test_fill_from_records(nd, n, m):
+    rng = np.random.default_rng(n)
+    key = np.unique(rng.integers(0, n, 3 * m) * n + rng.integers(0, n, 3 * m))
+    u, v = key // n, key % n
+    rp, col = G.to_csr(n, u[u < v][:m], v[u < v][:m])
+    assert rp[-1] // 2 >= 1 << 16
+    g = oracle.Graph(rp, col, 2, 3)
+    inc = nd.build_incidence(torch.from_numpy(rp).cuda(), torch.from_numpy(col).cuda(), 2, 3)
+    np.testing.assert_array_equal(inc.s_degree().cpu().numpy(), g.s_degree())
+    for k in (1, 2, 3):
+        np.testing.assert_array_equal(inc.iterate_k("snd", k)[0].cpu().numpy(), g.snd(max_sweeps=k)[0])
+    np.testing.assert_array_equal(inc.snd()[0].cpu().numpy(), g.peel())
+
+
 def test_no_storage_rows_with_hub_tables(nd):
     """The no-storage passes of a graph large enough for hub tables: lists by
     degree class, their bound, and the lists below the tables' degree."""

@@ -1628,9 +1628,12 @@ nd_status plan_list(nd_incidence* h, int64_t words, nd_tmp<uint32_t>& scratch, L
     L->list = h->list;
     L->room = L->tiles;
     if (!h->list) {
+        // parts of a sixteenth, or of what the device still has room for
+        nd_status e;
+        for (L->room = (L->tiles + 15) / 16; (e = scratch.alloc(L->room * kListTile)) != ND_OK && L->room > 1;)
+            L->room = (L->room + 3) / 4;
+        ND_TRY(e);
         nd_set_error("");
-        L->room = (L->tiles + 15) / 16;
-        ND_TRY(scratch.alloc(L->room * kListTile));
         L->list = scratch;
     }
     return ND_OK;

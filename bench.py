@@ -48,12 +48,12 @@ METRIC = "r-clique h-index updates/sec to convergence; HBM GB/s vs peak; batched
 UNIT = "updates/s"
 PEEL_SAMPLE_SCALE = 14    # the single-threaded peeling oracle, timed on a bounded sample
 CPU_SND_SECONDS = 10.0    # time budget of the multi-threaded SND passes of the CPU baseline
-# ncu DRAM bytes per incidence of the SND pass (k-truss, q = 2), measured on the
-# current kernels on R-MAT scale 18: pass 12, with the rho cache (dram__bytes_read.sum +
-# dram__bytes_write.sum = 2.197118 GB + 32.99328 MB per pass over 247,767,033
-# incidences, 9.00 B), and pass 21 of the late-pass kernel without it (2.195024 GB +
-# 26.116608 MB, 8.96 B); None once a kernel changes until it is measured again.
-NCU_SND_TRAFFIC_PER_INCIDENCE = (2.197118e9 + 32.99328e6) / 247767033
+# ncu DRAM bytes per incidence of a SND pass (k-truss, q = 2): dram__bytes_read.sum +
+# dram__bytes_write.sum over the 41 working passes of one run on R-MAT scale 18, 72.154 GB, by
+# 247,767,033 incidences per pass: 7.10 B on average, 9.4 B in pass 1 (whole rows), 6.0 B in
+# late passes, which stop once a row's h-index is settled.  None once a kernel changes
+# until it is measured again.
+NCU_SND_TRAFFIC_PER_INCIDENCE = 72.154e9 / 41 / 247767033
 
 
 def parse():
@@ -378,7 +378,9 @@ def run_ours(args, rank, world, local_rank):
     # the gather layout, 4 B first touch of the second copy), for (1,2) 4 B
     # more (the 2 B write of its 16-bit copy and the first touch of it).  The q gathered
     # tau values per incidence are L2 hits while tau fits in L2, so they are
-    # not DRAM bytes.
+    # not DRAM bytes.  The incidences are those of whole rows: a pass stops
+    # reading a row once its h-index is settled, so this model is an upper
+    # bound, and where the DRAM bytes were measured those are used instead.
     info = infos[-1]
     peak, peak_kind = load_peaks()
     top = max(prof.items(), key=lambda kv: kv[1][1])
@@ -398,15 +400,17 @@ def run_ours(args, rank, world, local_rank):
         units = "8 B per incidence written (fill) or CSR bytes read"
     avg_ms = ms / max(eff, 1)
     achieved = per_launch / (avg_ms / 1000.0) / 1e9
-    # DRAM traffic per SND pass: the ncu bytes per incidence of the R-MAT scale 18 k-truss pass,
-    # scaled by the incidences of this workload (a full SND pass streams every row); None for any
-    # other kernel or once the kernel has changed.
+    # DRAM traffic per SND pass: the ncu bytes per incidence of the R-MAT scale 18 k-truss passes,
+    # scaled by the incidences of this workload; None for any other kernel or once the kernel has
+    # changed.
     traffic = None
     if name == "snd_pass" and q == 2 and NCU_SND_TRAFFIC_PER_INCIDENCE is not None:
         traffic = NCU_SND_TRAFFIC_PER_INCIDENCE * M
-    # Three byte models of the same pass, each over its measured average time:
-    #   frac       compulsory DRAM bytes: 4q B per incidence streamed + the per-row
-    #              bytes above (the gathered tau values are L2 hits);
+        per_launch, achieved = traffic, traffic / (avg_ms / 1000.0) / 1e9
+        units = "ncu DRAM bytes per SND pass (rows are read only until their h-index is settled)"
+    # Byte models of the same pass, each over its measured average time:
+    #   frac       the DRAM bytes ncu measured, where known; else the compulsory bytes
+    #              of whole rows above;
     #   frac_survey every operand counted once, gathers included:
     #              16 B per r-clique + 8q B per incidence (4 B id + 4 B gathered tau);
     #   frac_dram  the DRAM bytes ncu measured (traffic), when known.
@@ -424,7 +428,7 @@ def run_ours(args, rank, world, local_rank):
                 "frac_survey": survey_gbs / peak if survey_gbs else None,
                 "achieved_survey": survey_gbs,
                 "bytes_per_launch_survey": survey_bytes,
-                "units_survey": "16 B x r-cliques evaluated + 8q B x incidences streamed (4 B id + 4 B gathered tau)",
+                "units_survey": "16 B x r-cliques evaluated + 8q B x incidences of whole rows (4 B id + 4 B gathered tau)",
                 "frac_dram": dram_gbs / peak if dram_gbs else None,
                 "achieved_dram": dram_gbs,
                 "units_dram": "ncu dram__bytes_read.sum + dram__bytes_write.sum per pass (traffic) / average pass time",

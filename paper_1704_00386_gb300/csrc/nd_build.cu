@@ -49,8 +49,7 @@ __device__ __forceinline__ int64_t warp_count_global() {
 // Most rows of these graphs hold fewer entries than a warp has lanes.  The
 // kernels below therefore give a warp up to 32 consecutive rows: lane l loads what
 // leads to row l, and the entries of all are then walked as one sequence,
-// 32 at a time, every lane finding its entry's row by five steps over the
-// rows' prefix sums in shared memory.  Rows of more than kPoolRow entries go to
+// 32 at a time (row_pool).  Rows of more than kPoolRow entries go to
 // a second walk, one at a time and spread over all warps: consecutive rows are
 // of like length (degree classes, the edges of one hub), and 32 long ones would
 // keep one warp busy long after the others.  (A warp per row spent a chain of loads
@@ -78,10 +77,19 @@ __device__ __forceinline__ void spread_rows(int64_t n, P&& pick, F&& f) {
 }
 
 struct row_pool {
-    uint32_t* pre;  // the warp's 32 words: entries before each row
+    struct place {
+        int row, at;    // the entry's row, and the entries before it
+        unsigned same;  // the lanes with entries of that row
+    };
+    // the warp's words: entries before each row, then of each row that is not
+    // empty, in order, the same * 32 + its index (a row has fewer than 2^22)
+    uint32_t* pre;
     int total;
-    // len: entries of this lane's row (their sum fits 31 bits)
-    __device__ __forceinline__ row_pool(uint32_t* words, int len) : pre(words) {
+    int start;   // the first entry of this lane's row, -1 if it is empty
+    int before;  // rows, not empty, that begin before the next block
+    static constexpr int kWords = 64;
+    // len: entries of this lane's row
+    __device__ __forceinline__ row_pool(uint32_t* words, int len) : pre(words), before(0) {
         const int lane = threadIdx.x & 31;
         int incl = len;
 #pragma unroll
@@ -89,29 +97,32 @@ struct row_pool {
             const int t = __shfl_up_sync(kFull, incl, o);
             if (lane >= o) incl += t;
         }
+        const unsigned filled = __ballot_sync(kFull, len > 0);
         __syncwarp();
         pre[lane] = (uint32_t)(incl - len);
+        if (len > 0) pre[32 + __popc(filled & lanemask_lt())] = (uint32_t)(incl - len) << 5 | lane;
+        start = len > 0 ? incl - len : -1;
         total = __shfl_sync(kFull, incl, 31);
         __syncwarp();
     }
-    // the row of entry e < total: the last one that begins at or before it
-    __device__ __forceinline__ int row(int e) const {
-        int r = 0;
-#pragma unroll
-        for (int h = 16; h > 0; h >>= 1) r += (int)pre[r + h] <= e ? h : 0;
-        return r;
-    }
-    // the lanes that hold entries of this lane's row (rows ascend with the lanes)
-    static __device__ __forceinline__ unsigned same_row(int r) {
+    // where this lane's entry of the block of 32 from e0 lies; blocks are asked
+    // for in order, and lanes past the last entry get the last row.  One bit per
+    // row that begins in the block, so one shared load finds the row, where a
+    // search of the prefix sums takes five in a row (triangle count of the R-MAT
+    // k-truss of 1,048,576 vertices: 13.3 against 12.5 ms).
+    __device__ __forceinline__ place block(int e0) {
         const int lane = threadIdx.x & 31;
-        const int before = __shfl_up_sync(kFull, r, 1);
-        const unsigned starts = __ballot_sync(kFull, lane == 0 || before != r);
-        const unsigned upto = 0xffffffffu >> (31 - lane);
+        const unsigned d = (unsigned)(start - e0);
+        const unsigned begins = __reduce_or_sync(kFull, d < 32u ? 1u << d : 0u);
+        const unsigned upto = 0xffffffffu >> (31 - lane), starts = begins | 1u;
+        const uint32_t q = pre[31 + before + __popc(begins & upto)];
+        before += __popc(begins);
         const unsigned later = starts & ~upto;
-        const int first = 31 - __clz(starts & upto);
-        const unsigned from_first = 0xffffffffu << first;
-        return later ? from_first & ((1u << (__ffs(later) - 1)) - 1u) : from_first;
+        const unsigned from_first = 0xffffffffu << (31 - __clz(starts & upto));
+        return {(int)(q & 31u), (int)(q >> 5), later ? from_first & ((1u << (__ffs(later) - 1)) - 1u) : from_first};
     }
+    // the entries of row r
+    __device__ __forceinline__ int length(int r) const { return (r < 31 ? (int)pre[r + 1] : total) - (int)pre[r]; }
 };
 
 // ---- validation and degree split ------------------------------------------
@@ -275,7 +286,7 @@ __global__ void k_validate_split(int per, int64_t n, int64_t nnz, const int64_t*
                                  int64_t* __restrict__ upcnt, int* __restrict__ err,
                                  unsigned long long* __restrict__ searched, uint32_t* __restrict__ mirror,
                                  unsigned long long* __restrict__ fp_out) {
-    __shared__ uint32_t pre[kThreads / 32][32];
+    __shared__ uint32_t pre[kThreads / 32][row_pool::kWords];
     __shared__ int64_t begin[kThreads / 32][32];
     __shared__ int lows[kThreads / 32][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -301,18 +312,17 @@ __global__ void k_validate_split(int per, int64_t n, int64_t nnz, const int64_t*
         }
         begin[w][lane] = b;
         lows[w][lane] = 0;
-        const row_pool pool(pre[w], len);
+        row_pool pool(pre[w], len);
         for (int e0 = 0; e0 < pool.total; e0 += 32) {
             const int x = e0 + lane;
-            const int r = pool.row(min(x, pool.total - 1));
+            const auto [r, at, same] = pool.block(e0);
             bool low = false;
             if (x < pool.total) {
-                const int64_t rb = begin[w][r], p = rb + (x - (int)pool.pre[r]);
-                const int64_t re = rb + ((r < 31 ? (int)pool.pre[r + 1] : pool.total) - (int)pool.pre[r]);
+                const int64_t rb = begin[w][r], p = rb + (x - at), re = rb + pool.length(r);
                 if (!validate_entry<BY_LENGTH, FP>(n, nnz, rp, col, u0 + r, rb, re, p, mirror, low, found, fp))
                     bad_entry = true;
             }
-            const unsigned same = row_pool::same_row(r), m = __ballot_sync(kFull, low) & same;
+            const unsigned m = __ballot_sync(kFull, low) & same;
             if (lane == __ffs(same) - 1) lows[w][r] += __popc(m);
             __syncwarp();
         }
@@ -793,7 +803,7 @@ __global__ void __launch_bounds__(kThreads) k_orient(int per, int64_t n, const i
                                                      int32_t* __restrict__ out_src,
                                                      const uint32_t* __restrict__ mirror,
                                                      uint2* __restrict__ out_pm) {
-    __shared__ uint32_t pre[kThreads / 32][32];
+    __shared__ uint32_t pre[kThreads / 32][row_pool::kWords];
     __shared__ int64_t begin[kThreads / 32][32], slots[kThreads / 32][32];  // slots: next output slot of each row
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     auto put = [&](int64_t slot, int32_t u, int32_t v, int64_t p) {
@@ -809,15 +819,15 @@ __global__ void __launch_bounds__(kThreads) k_orient(int per, int64_t n, const i
         __syncwarp();
         begin[w][lane] = b;
         slots[w][lane] = FILL && mine < n ? out_ptr[mine] : 0;
-        const row_pool pool(pre[w], len > kPoolRow ? 0 : (int)len);
-        auto entry = [&](bool ok, int r, int64_t p, int64_t du) {
+        row_pool pool(pre[w], len > kPoolRow ? 0 : (int)len);
+        auto entry = [&](bool ok, int r, unsigned same, int64_t p, int64_t du) {
             bool keep = false;
             int32_t v = 0;
             if (ok) {
                 v = __ldg(col + p);
                 keep = precedes(du, (int32_t)(u0 + r), __ldg(rp + v + 1) - __ldg(rp + v), v);
             }
-            const unsigned same = row_pool::same_row(r), m = __ballot_sync(kFull, keep) & same;
+            const unsigned m = __ballot_sync(kFull, keep) & same;
             const int64_t first = slots[w][r];
             __syncwarp();
             if (lane == __ffs(same) - 1) slots[w][r] = first + __popc(m);
@@ -826,9 +836,8 @@ __global__ void __launch_bounds__(kThreads) k_orient(int per, int64_t n, const i
         };
         for (int e0 = 0; e0 < pool.total; e0 += 32) {
             const int x = e0 + lane;
-            const int r = pool.row(min(x, pool.total - 1));
-            const int at = (int)pool.pre[r];
-            entry(x < pool.total, r, begin[w][r] + (x - at), (r < 31 ? (int)pool.pre[r + 1] : pool.total) - at);
+            const auto [r, at, same] = pool.block(e0);
+            entry(x < pool.total, r, same, begin[w][r] + (x - at), pool.length(r));
         }
         if (!FILL && mine < n && len <= kPoolRow) out_ptr[mine] = slots[w][lane];
     }
@@ -943,7 +952,7 @@ __global__ void __launch_bounds__(kThreads, ND_TRI_COUNT_MIN_BLOCKS)
     k_tri_count(int per, int64_t m, const int64_t* __restrict__ out_ptr, const int32_t* __restrict__ out_col,
                 const uint32_t* __restrict__ out_eid, const int32_t* __restrict__ out_src, unsigned* __restrict__ ctr,
                 const int64_t* __restrict__ rec_ptr, uint32_t* __restrict__ rec, uint32_t* __restrict__ rec_cnt) {
-    __shared__ uint32_t pre[kThreads / 32][32];
+    __shared__ uint32_t pre[kThreads / 32][row_pool::kWords];
     __shared__ uint32_t ab[kThreads / 32][32], bb[kThreads / 32][32], bn[kThreads / 32][32], an[kThreads / 32][32];
     __shared__ uint32_t nf[kThreads / 32][32];  // triangles found from each edge so far
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -967,9 +976,9 @@ __global__ void __launch_bounds__(kThreads, ND_TRI_COUNT_MIN_BLOCKS)
         an[w][lane] = (uint32_t)na;
         bn[w][lane] = (uint32_t)nb;
         nf[w][lane] = 0;
-        const row_pool pool(pre[w], na & 31);
+        row_pool pool(pre[w], na & 31);
         // element j of edge r's shorter list
-        auto element = [&](bool ok, int r, int j) {
+        auto element = [&](bool ok, int r, unsigned same, int j) {
             bool found = false;
             uint32_t p = 0, pb = 0;
             if (ok) {
@@ -982,7 +991,7 @@ __global__ void __launch_bounds__(kThreads, ND_TRI_COUNT_MIN_BLOCKS)
             }
             const unsigned all = __ballot_sync(kFull, found);
             if (!all) return;
-            const unsigned same = row_pool::same_row(r), hit = all & same;
+            const unsigned hit = all & same;
             const uint32_t before = nf[w][r];
             __syncwarp();
             if (lane == __ffs(same) - 1 && hit) nf[w][r] = before + __popc(hit);
@@ -997,12 +1006,12 @@ __global__ void __launch_bounds__(kThreads, ND_TRI_COUNT_MIN_BLOCKS)
         };
         for (unsigned todo = __ballot_sync(kFull, na >= 32); todo; todo &= todo - 1) {
             const int r = __ffs(todo) - 1, whole = (int)an[w][r] & ~31;
-            for (int j = 0; j < whole; j += 32) element(true, r, j + lane);
+            for (int j = 0; j < whole; j += 32) element(true, r, kFull, j + lane);
         }
         for (int e0 = 0; e0 < pool.total; e0 += 32) {
             const int x = e0 + lane;
-            const int r = pool.row(min(x, pool.total - 1));
-            element(x < pool.total, r, ((int)an[w][r] & ~31) + x - (int)pool.pre[r]);
+            const auto [r, at, same] = pool.block(e0);
+            element(x < pool.total, r, same, ((int)an[w][r] & ~31) + x - at);
         }
         if (mine < m) {
             const uint32_t c = nf[w][lane];
@@ -1013,20 +1022,20 @@ __global__ void __launch_bounds__(kThreads, ND_TRI_COUNT_MIN_BLOCKS)
 }
 
 // The fill from the count pass's records: 32 consecutive oriented edges per
-// warp, two recorded triangles per lane at a time, so no search is repeated.
+// warp, four recorded triangles per lane at a time, so no search is repeated.
 // The six positions of a triangle are read at the recorded offsets of w in the
 // two out-lists; slots and entries are as in the searching fill.
 // Bound by the chain record -> list entries -> slots -> writes and by the L2
-// traffic of the slot atomics and scattered 8-byte writes.  Registers for two
-// tasks in flight are worth more than warps: one task at 5 blocks per SM takes
-// 22.8 ms on an R-MAT of 1,048,576 vertices (390M triangles), two at 3 blocks 20.6, at 4 blocks
-// 21.4, four at 2 blocks 19.7 (but 0.846 ms against 0.804 on the 100K-vertex
-// R-MAT, where few warps leave the last groups on few SMs; one task 0.833).
+// traffic of the slot atomics and scattered 8-byte writes.  Registers for tasks
+// in flight are worth more than warps: one task at 5 blocks per SM takes 22.8 ms
+// on an R-MAT of 1,048,576 vertices (390M triangles), two at 3 blocks 20.5, at
+// 4 blocks 21.5, four at 2 blocks 19.6; 100K vertices 0.833, 0.822, 0.821 and
+// 0.833 ms.
 #ifndef ND_FILL_TASKS
-#define ND_FILL_TASKS 2
+#define ND_FILL_TASKS 4
 #endif
 #ifndef ND_FILL_MIN_BLOCKS
-#define ND_FILL_MIN_BLOCKS 3
+#define ND_FILL_MIN_BLOCKS 2
 #endif
 template <typename C>
 __global__ void __launch_bounds__(kThreads, ND_FILL_MIN_BLOCKS)
@@ -1035,7 +1044,7 @@ __global__ void __launch_bounds__(kThreads, ND_FILL_MIN_BLOCKS)
                    const uint2* __restrict__ out_pm, C* __restrict__ ctr, uint2* __restrict__ inc,
                    const int64_t* __restrict__ rec_ptr, const uint32_t* __restrict__ rec,
                    const uint32_t* __restrict__ rec_cnt) {
-    __shared__ uint32_t pre[kThreads / 32][32];
+    __shared__ uint32_t pre[kThreads / 32][row_pool::kWords];
     __shared__ uint32_t ab[kThreads / 32][32], bb[kThreads / 32][32];
     __shared__ int32_t vu[kThreads / 32][32], vv[kThreads / 32][32];
     __shared__ bool a_is[kThreads / 32][32];  // the shorter list is out(u)
@@ -1058,18 +1067,21 @@ __global__ void __launch_bounds__(kThreads, ND_FILL_MIN_BLOCKS)
             a_is[w][lane] = us;
             rp0[w][lane] = rec_ptr[mine];
         }
-        const row_pool pool(pre[w], c);
+        row_pool pool(pre[w], c);
         constexpr int U = ND_FILL_TASKS;
         for (int e0 = 0; e0 < pool.total; e0 += 32 * U) {
             int r[U];
+            unsigned same[U];
             uint32_t p[U], pb[U];
             bool found[U];
 #pragma unroll
             for (int t = 0; t < U; ++t) {
                 const int i = e0 + 32 * t + lane;
                 found[t] = i < pool.total;
-                r[t] = pool.row(min(i, pool.total - 1));
-                p[t] = found[t] ? __ldg(rec + rp0[w][r[t]] + (i - (int)pool.pre[r[t]])) : 0;
+                const row_pool::place of = pool.block(e0 + 32 * t);
+                r[t] = of.row;
+                same[t] = of.same;
+                p[t] = found[t] ? __ldg(rec + rp0[w][of.row] + (i - of.at)) : 0;
             }
             uint32_t ea[U], eb[U], e_uv[U];
             uint2 pa[U], pq[U], uv[U];
@@ -1088,12 +1100,11 @@ __global__ void __launch_bounds__(kThreads, ND_FILL_MIN_BLOCKS)
                     pq[t] = __ldg(out_pm + pb[t]);
                 }
             }
-            unsigned same[U];
             C s0[U], s_uw[U], s_vw[U];
             // the slot reservations are independent: issue them together
 #pragma unroll
             for (int t = 0; t < U; ++t) {
-                same[t] = row_pool::same_row(r[t]) & __ballot_sync(kFull, found[t]);
+                same[t] &= __ballot_sync(kFull, found[t]);
                 const bool a_is_u = a_is[w][r[t]];
                 s0[t] = 0;
                 if (found[t]) {

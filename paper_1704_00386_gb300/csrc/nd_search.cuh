@@ -131,12 +131,12 @@ __device__ __forceinline__ int bin_shift(unsigned span, int bins) {
 // The bin of a histogram that holds H, by one full warp.  Bin b counts rho in
 // [lo + (b << shift), lo + ((b + 1) << shift)); `above` counts rho past the
 // last bin.  #{rho >= lo + (b << shift)} is above plus the suffix sum from b,
-// and H lies in the last bin whose sum reaches its lower edge (bin 0 always
-// qualifies: #{rho >= lo} >= lo).  Blocks of 128 bins from the top, four to a
-// lane; returns the bin, and in `above` the count past it.
+// and H lies in the last bin whose sum reaches its lower edge (bin 0 where none
+// does: #{rho >= lo} >= lo has been seen).  Blocks of 128 bins from the top, four
+// to a lane.
 // PK: 16-bit counters, bin b in half b / HW of word b % HW.
 template <bool PK, int HW>
-__device__ __forceinline__ int select_bin(const unsigned* bins, int lo, int shift, int nb, int& above) {
+__device__ __forceinline__ int select_bin(const unsigned* bins, int lo, int shift, int nb, int above) {
     const int lane = threadIdx.x & 31;
     for (int c = (nb - 1) >> 7;; --c) {
         const int b0 = 128 * c;
@@ -155,15 +155,14 @@ __device__ __forceinline__ int select_bin(const unsigned* bins, int lo, int shif
         const int after = above + incl - s0;  // rho past this lane's bins
         // lower edges; unsigned, because those of the padding past nb may leave 31 bits
         const unsigned e0 = (unsigned)lo + ((unsigned)(b0 + 4 * lane) << shift), w1 = 1u << shift;
-        int best = -1, past = 0;
-        if ((unsigned)(after + s0) >= e0) { best = 0; past = after + s1; }
-        if ((unsigned)(after + s1) >= e0 + w1) { best = 1; past = after + s2; }
-        if ((unsigned)(after + s2) >= e0 + 2 * w1) { best = 2; past = after + s3; }
-        if ((unsigned)(after + s3) >= e0 + 3 * w1) { best = 3; past = after; }
+        int best = -1;
+        if ((unsigned)(after + s0) >= e0) best = 0;
+        if ((unsigned)(after + s1) >= e0 + w1) best = 1;
+        if ((unsigned)(after + s2) >= e0 + 2 * w1) best = 2;
+        if ((unsigned)(after + s3) >= e0 + 3 * w1) best = 3;
         const unsigned hit = __ballot_sync(0xffffffffu, best >= 0);
         if (hit || c == 0) {
             const int src = hit ? 31 - __clz(hit) : 0;
-            above = __shfl_sync(0xffffffffu, past, src);
             return b0 + 4 * src + max(__shfl_sync(0xffffffffu, best, src), 0);
         }
         above += __shfl_sync(0xffffffffu, incl, 0);
@@ -183,13 +182,20 @@ __device__ __forceinline__ int select_bin(const unsigned* bins, int lo, int shif
 // rows of fewer than 65,536 entries; else HW bins of 32 bits), one per value
 // while t allows, so H is exact after one sweep there, and after two for
 // longer rows.
+// AND lowers tau between the sweeps of a row, so a sweep counts all that its
+// sums need: the entries past its bins (ge) too.  With the count of an earlier
+// sweep in its place, a neighbour X that fell to x in between would count twice,
+// and R would keep an h below x that x does not support: X notifies R only if
+// x <= tau(R).  With one sweep's counts, what no longer supports h has fallen
+// below h, and so notifies R.  The same holds for lo, the bound of an earlier
+// sweep.  (tests/test_row_search.py plays the interleaving.)
 // bound: a count also stops where the rest of the row cannot reach t.
 template <bool PK, int HW, typename F, typename B>
 __device__ __forceinline__ int32_t warp_hindex(const F& rho, const B& bound, int d, int32_t t, bool direct,
                                                unsigned* bins) {
     const int lane = threadIdx.x & 31;
     if (t <= 0) return 0;
-    int lo = 0, hi = t, above = 0;
+    int lo = 0, hi = t;
     if (!direct) {
         int cnt = 0, have = 0;
         for (int i = 0; i < d;) {
@@ -201,7 +207,7 @@ __device__ __forceinline__ int32_t warp_hindex(const F& rho, const B& bound, int
             if (have >= t) return t;
             if (bound.past(end)) break;
         }
-        lo = above = have;  // #{rho >= lo} >= lo holds; at hi it fails
+        lo = have;  // #{rho >= lo} >= lo holds; at hi it fails
         if (hi - lo <= 1) return lo;
     }
     for (;;) {
@@ -223,11 +229,8 @@ __device__ __forceinline__ int32_t warp_hindex(const F& rho, const B& bound, int
             }
         });
         __syncwarp();
-        if (direct) {
-            above = (int)__reduce_add_sync(0xffffffffu, (unsigned)ge);
-            if (above >= t) return t;
-            direct = false;
-        }
+        const int above = (int)__reduce_add_sync(0xffffffffu, (unsigned)ge);
+        if (above >= hi) return hi;  // a direct row's first sweep: hi is t
         const int b = select_bin<PK, HW>(bins, lo, shift, nb, above);
         lo += b << shift;
         hi = min(hi, lo + (1 << shift));
@@ -242,7 +245,8 @@ constexpr int kCtaSegment = 2048;
 // The same by the whole CTA (the longest rows): 32-bit counters, as many bins
 // as the block's histogram has words; warp 0 selects the bin.  A sweep also
 // stops where u, the most the rest of the row can reach, is settled: once
-// #{rho >= u} >= u, H is at least u, and the rest counts for no larger value.
+// #{rho >= u} >= u, H is at least u, and the rest, which is below hi, counts for
+// no larger value.
 // That is what keeps the hub rows of a k-core short: on R-MAT scale 20 the
 // rows past 2,048 entries hold 22% of all entries, and a search needs a third
 // of those, a converged count an eighth.
@@ -260,7 +264,7 @@ __device__ __forceinline__ int32_t cta_hindex(const F& rho, const B& bound, int 
         __syncthreads();
         return tot;
     };
-    int lo = 0, hi = t, above = 0;
+    int lo = 0, hi = t;
     if (!direct) {
         int cnt = 0, have = 0;
         for (int i = 0; i < d;) {
@@ -272,7 +276,7 @@ __device__ __forceinline__ int32_t cta_hindex(const F& rho, const B& bound, int 
             if (have >= t) return t;
             if (bound.past(end)) break;
         }
-        lo = above = have;
+        lo = have;
         if (hi - lo <= 1) return lo;
     }
     for (;;) {
@@ -296,25 +300,19 @@ __device__ __forceinline__ int32_t cta_hindex(const F& rho, const B& bound, int 
             u = m;
             __syncthreads();  // the bins so far are complete
             // #{rho >= u} from the bins at or past u
-            int c = direct ? ge : (threadIdx.x == 0 ? above : 0);
+            int c = ge;
             for (int b = (int)(((unsigned)(u - lo) + (1u << shift) - 1) >> shift) + threadIdx.x; b < nb; b += kThreads)
                 c += (int)bins[b];
             if (total(c) >= u) break;
         }
-        if (direct) {
-            above = total(ge);  // with its barriers, the bins are complete too
-            if (above >= t) return t;
-            direct = false;
-        } else {
-            __syncthreads();
-        }
+        const int above = total(ge);  // with its barriers, the bins are complete too
+        if (above >= hi) return hi;
         if (threadIdx.x < 32) {
             const int b = select_bin<false, WORDS>(bins, lo, shift, nb, above);
-            if (threadIdx.x == 0) { bounds[0] = b; bounds[1] = above; }
+            if (threadIdx.x == 0) bounds[0] = b;
         }
         __syncthreads();
         lo += bounds[0] << shift;
-        above = bounds[1];
         __syncthreads();
         hi = min(hi, lo + (1 << shift));
         if (hi - lo <= 1) return lo;

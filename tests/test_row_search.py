@@ -1,0 +1,225 @@
+"""The row search of the passes (csrc/nd_search.cuh) while AND lowers tau.
+
+AND updates tau in place, so a row that is read more than once can meet a
+neighbour X that falls between two readings.  X then tests whether its new value
+is at most tau(R) before it notifies R, and if R has stored its result by then,
+X compares with that.  So the result h of R must be one that the values support
+after X's fall, or one that X's fall to h or below lets X correct: anything else
+would stay, and AND would return a tau above kappa.
+
+The routines are compiled for the host here, every lane a coroutine that runs to
+the next warp or block barrier.  The interleaving is the worst one, spelled out
+per row: the first reading of every entry, the stores of the neighbours, the
+later readings, the store of R, the walks of the neighbours.  Integers: exact.
+"""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_1704_00386_gb300", "csrc")
+
+PROGRAM = r"""
+#include <stdint.h>
+#include <stdio.h>
+#include <string.h>
+#include <ucontext.h>
+
+#include <algorithm>
+#include <functional>
+#include <memory>
+#include <random>
+#include <vector>
+
+// ---- lanes as coroutines, and the intrinsics that the header uses ----
+#define __device__
+#define __forceinline__ inline
+struct alignas(16) uint4 { unsigned x, y, z, w; };
+struct lane_index { int x; };
+static int g_lane;
+#define threadIdx (lane_index{g_lane})
+constexpr int kLanes = 256;
+static ucontext_t g_main, g_ctx[kLanes];
+static bool g_done[kLanes];
+struct Barrier { int size, count; unsigned gen; };
+static Barrier g_warp[kLanes / 32], g_block;
+static unsigned long long g_slot[kLanes];
+static std::function<void()> g_body;
+
+static void arrive(Barrier& b) {
+    const unsigned gen = b.gen;
+    if (++b.count == b.size) { b.count = 0; ++b.gen; return; }
+    while (b.gen == gen) swapcontext(&g_ctx[g_lane], &g_main);
+}
+static void entry() { g_body(); g_done[g_lane] = true; swapcontext(&g_ctx[g_lane], &g_main); }
+static void run_lanes(int n, std::function<void()> body) {
+    static std::unique_ptr<char[]> stacks(new char[(size_t)kLanes * 65536]);
+    g_body = body;
+    for (auto& w : g_warp) w = {32, 0, 0};
+    g_block = {n, 0, 0};
+    for (int i = 0; i < n; ++i) {
+        getcontext(&g_ctx[i]);
+        g_ctx[i].uc_stack.ss_sp = stacks.get() + (size_t)i * 65536;
+        g_ctx[i].uc_stack.ss_size = 65536;
+        g_ctx[i].uc_link = nullptr;
+        g_done[i] = false;
+        makecontext(&g_ctx[i], entry, 0);
+    }
+    for (bool more = true; more;) {
+        more = false;
+        for (g_lane = 0; g_lane < n; ++g_lane)
+            if (!g_done[g_lane]) { more = true; swapcontext(&g_main, &g_ctx[g_lane]); }
+    }
+}
+static void __syncwarp() { arrive(g_warp[g_lane >> 5]); }
+static void __syncthreads() { arrive(g_block); }
+template <typename F> static auto exchange(unsigned long long v, F f) {
+    g_slot[g_lane] = v;
+    __syncwarp();
+    const auto r = f(g_slot + (g_lane & ~31));
+    __syncwarp();
+    return r;
+}
+static int __shfl_sync(unsigned, int v, int src, int width = 32) {
+    return exchange((unsigned)v, [&](unsigned long long* s) {
+        return (int)(unsigned)s[(g_lane & 31 & ~(width - 1)) + (src & (width - 1))]; });
+}
+static int __shfl_down_sync(unsigned, int v, int o) {
+    return exchange((unsigned)v, [&](unsigned long long* s) { return (int)(unsigned)s[std::min((g_lane & 31) + o, 31)]; });
+}
+static int __shfl_xor_sync(unsigned, int v, int o) {
+    return exchange((unsigned)v, [&](unsigned long long* s) { return (int)(unsigned)s[(g_lane & 31) ^ o]; });
+}
+static unsigned __reduce_add_sync(unsigned, unsigned v) {
+    return exchange(v, [&](unsigned long long* s) { unsigned t = 0; for (int i = 0; i < 32; ++i) t += (unsigned)s[i]; return t; });
+}
+static unsigned __ballot_sync(unsigned, bool p) {
+    return exchange(p, [&](unsigned long long* s) { unsigned t = 0; for (int i = 0; i < 32; ++i) t |= (unsigned)s[i] << i; return t; });
+}
+static bool __any_sync(unsigned m, bool p) { return __ballot_sync(m, p) != 0; }
+static int __clz(unsigned x) { return x ? __builtin_clz(x) : 32; }
+static int __ffs(unsigned x) { return __builtin_ffs((int)x); }
+static int __popc(unsigned x) { return __builtin_popcount(x); }
+template <typename T> static T __ldg(const T* p) { return *p; }
+static void atomicAdd(unsigned* p, unsigned v) { *p += v; }
+static uint4 make_uint4(unsigned x, unsigned y, unsigned z, unsigned w) { return {x, y, z, w}; }
+using std::max;
+using std::min;
+
+#include "nd_search.cuh"
+
+// ---- rows whose entries fall from one reading to the next ----
+struct Row {
+    std::vector<std::vector<int>> v;  // v[k][j]: entry j at its reading k
+    std::vector<uint32_t> id;
+    std::vector<int> oct;             // 32 bounds
+    int t;
+};
+struct Falling {
+    const Row* row;
+    int* reads;
+    int operator()(int j) const { return row->v[std::min(reads[j]++, (int)row->v.size() - 1)][j]; }
+};
+static int hindex(std::vector<int> a, int t) {
+    std::sort(a.rbegin(), a.rend());
+    int h = 0;
+    while (h < (int)a.size() && a[h] >= h + 1) ++h;
+    return std::min(h, t);
+}
+
+// kind 0: a warp, 16-bit bins; 1: a warp, 32-bit bins; 2: a block; 3: a block, rows bounded by octave
+static int search(const Row& row, int kind, bool direct) {
+    alignas(16) static unsigned bins[1024];
+    static int bounds[8];
+    const int d = (int)row.v[0].size();
+    std::vector<int> reads(d, 0);
+    const Falling rho{&row, reads.data()};
+    int h = -1;
+    run_lanes(kind < 2 ? 32 : kLanes, [&] {
+        int x;
+        if (kind == 0) x = warp_hindex<true, 128>(rho, NoBound{}, d, row.t, direct, bins);
+        else if (kind == 1) x = warp_hindex<false, 128>(rho, NoBound{}, d, row.t, direct, bins);
+        else if (kind == 2) x = cta_hindex<128>(rho, NoBound{}, d, row.t, direct, bins, bounds);
+        else {
+            const uint32_t limit = id_limit(row.oct.data(), row.t);
+            x = cta_hindex<128>(rho, IdBound{row.id.data(), row.oct.data(), limit}, d, row.t, direct, bins, bounds);
+        }
+        if (g_lane == 0) h = x;
+    });
+    return h;
+}
+
+int main() {
+    std::mt19937 rng(20);
+    auto below = [&](int n) { return (int)(rng() % (unsigned)n); };
+    int bad = 0, high = 0, rows = 0;
+    for (int trial = 0; trial < 4200 && bad < 20; ++trial) {
+        const int kind = trial % 4;
+        const bool block = kind >= 2, wide = trial % 3 == 0, direct = trial % 5 == 0;
+        if (block && trial % 40 >= 4 && trial % 40 < 36) continue;  // fewer of the larger rows
+        // wide: more values than bins, so several sweeps
+        const int top = wide ? 300 + below(500) : 3 + below(20);
+        const int d = kind == 3 ? 4100 + below(3000) : top + below(2 * top);
+        Row row;
+        row.t = 2 + below(top);
+        std::vector<int> a(d);
+        for (int j = 0; j < d; ++j) a[j] = below(4) ? below(row.t + 3) : row.t + below(3);
+        if (kind == 3) {
+            // ids in order of their octave, values below the octave's bound
+            row.oct.assign(32, 0);
+            for (int o = 0; o < 32; ++o) row.oct[o] = max(0, 2 * row.t - o * (row.t / 6 + 1));
+            for (int j = 0; j < d; ++j) {
+                const int o = min(13, 14 * j / d);
+                row.id.push_back((1u << o) + (unsigned)below(1 << o));
+                a[j] = min(below(3) ? below(row.t / 4 + 1) : a[j], row.oct[o]);
+            }
+        } else {
+            // a row that fails its count by a little, as rows do when neighbours fall
+            int have = 0, keep = max(1, row.t - 1 - below(3));
+            for (int j = 0; j < d; ++j)
+                if (a[j] >= row.t && ++have > keep) a[j] = below(row.t);
+        }
+        row.v.push_back(a);
+        const int fall = 1 + below(4);
+        for (int k = 1; k < 4; ++k) {
+            for (int f = 0; f < fall; ++f) {
+                const int j = below(d);
+                // mostly a neighbour above the row's tau, to just below it
+                if (a[j] > 0) a[j] = a[j] >= row.t && below(4) ? max(0, row.t - 1 - below(3)) : below(a[j]);
+            }
+            row.v.push_back(a);
+        }
+        ++rows;
+        const int h = search(row, kind, direct);
+        const int truth = hindex(a, row.t), first = hindex(row.v[0], row.t);
+        // the walks, after the store of h
+        bool notified = false;
+        for (int j = 0; j < d; ++j)
+            for (int k = 1; k < 4; ++k) notified |= row.v[k][j] < row.v[k - 1][j] && row.v[k][j] <= h;
+        high += h > truth;
+        if (h < truth || h > first || (h > truth && !notified)) {
+            ++bad;
+            printf("row %d, kind %d, direct %d: d %d, t %d, h %d, h-index %d at the first reading, %d after the stores%s\n",
+                   trial, kind, (int)direct, d, row.t, h, first, truth, notified ? "" : ", not notified");
+        }
+    }
+    printf("%d rows, %d briefly too high, %d wrong\n", rows, high, bad);
+    return bad ? 1 : 0;
+}
+"""
+
+
+def test_a_result_is_supported_or_its_row_is_notified(tmp_path):
+    cxx = os.environ.get("CXX") or shutil.which("g++") or shutil.which("c++")
+    if not cxx:
+        pytest.skip("no C++ compiler")
+    src = tmp_path / "rows.cpp"
+    src.write_text(PROGRAM)
+    exe = tmp_path / "rows"
+    res = subprocess.run([cxx, "-std=c++17", "-O2", "-I", CSRC, str(src), "-o", str(exe)], capture_output=True, text=True)
+    assert res.returncode == 0, res.stderr
+    res = subprocess.run([str(exe)], capture_output=True, text=True, timeout=300)
+    assert res.returncode == 0, res.stdout + res.stderr
+    assert "0 wrong" in res.stdout

@@ -1770,13 +1770,15 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
         if (stop_active > 0.0) nb = 1;  // the stopping rule looks at every pass
         const int kind = batch == 0 ? 0 : ((batch & 1) ? 2 : 1);
         bool launched = false;
-        // graphs hold the plain parameters; runs with members, a stopping rule,
-        // a tau of the caller's or tables of their own launch directly, and so does the first batch of its kind on a
+        // graphs hold the plain parameters and the handle's own memory; runs with
+        // members, a stopping rule, a tau of the caller's, or tables or a list of
+        // their own launch directly, and so does the first batch of its kind on a
         // handle: building a graph costs more than its launches, and many
         // handles run each mode once
         const bool seen = h->batch_seen[mode][kind];
         if (nb == kBatch) h->batch_seen[mode][kind] = true;
-        if (nb == kBatch && seen && grid0 > 0 && !members && !tau_in_dev && !h->otf && L.room == L.tiles && (start & 1) == 0 && !h->pass_graph_failed[mode][kind]) {
+        if (nb == kBatch && seen && grid0 > 0 && !members && !tau_in_dev && !h->otf && !list_scratch.p &&
+            (start & 1) == 0 && !h->pass_graph_failed[mode][kind]) {
             if (!h->pass_graph[mode][kind])
                 make_batch_graph(h, mode, kind, P, grid0, fn0, grid1, fn1, L);
             if (h->pass_graph[mode][kind]) {

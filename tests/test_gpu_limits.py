@@ -1,0 +1,56 @@
+"""Handles at their memory limit: the library does without what it only keeps to
+be faster, and what ran without those arrays still runs."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1704_00386_gb300 import graphs as G
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def nd():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1704_00386_gb300 import nd as _nd
+    _nd.load()
+    return _nd
+
+
+def _cycle(n):
+    v = np.arange(n)
+    return G.to_csr(n, v, np.roll(v, -1))
+
+
+@pytest.mark.parametrize("r,mode", [(1, "snd"), (1, "and_nn"), (2, "snd"), (2, "and_nn")])
+def test_list_of_one_tile_is_the_run_s_own(nd, r, mode):
+    """A batch whose rows all lie in one bucket and fit one tile: a run without
+    room for the list on the handle has all of it as scratch.  Later runs must
+    not use that scratch again."""
+    graphs = [_cycle(n) if r == 1 else G.complete_graph(n % 4 + 4) for n in range(9, 60)]
+    graphs = [tuple(torch.from_numpy(x).cuda() for x in g) for g in graphs]
+
+    def run(inc):
+        return (inc.snd()[0] if mode == "snd" else inc.and_(notify=False)[0]).cpu().numpy()
+
+    inc, _ = nd.build_incidence_batch(graphs, r, r + 1)
+    assert inc.num_r <= 2048
+    want = run(inc)
+    np.testing.assert_array_equal(want, inc.s_degree().cpu().numpy())  # cycles and cliques are their own nuclei
+    held = inc.incidence_bytes()
+    other = G.hub_graph(3000, 6, seed=205)
+    core = oracle.decompose(*other, 1, 2)
+    try:
+        nd.set_handle_memory_limit(held - 4)
+        tight, _ = nd.build_incidence_batch(graphs, r, r + 1)
+        for _ in range(4):
+            np.testing.assert_array_equal(run(tight), want)
+            nd.set_handle_memory_limit(0)
+            between = nd.build_incidence(*other, 1, 2)  # takes the memory that runs have given back
+            np.testing.assert_array_equal(between.snd()[0], core)
+            nd.set_handle_memory_limit(held - 4)
+        assert tight.incidence_bytes() <= held - 4
+    finally:
+        nd.set_handle_memory_limit(0)

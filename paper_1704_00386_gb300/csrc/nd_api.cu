@@ -90,7 +90,7 @@ static std::atomic<int64_t> g_handle_limit{0};
 
 int64_t nd_handle_limit() { return g_handle_limit.load(); }
 
-nd_status nd_alloc(void** p, size_t bytes, cudaStream_t st, nd_incidence* owner) {
+static nd_status alloc_once(void** p, size_t bytes, cudaStream_t st, nd_incidence* owner) {
     if (bytes == 0) bytes = 16;
     const int64_t limit = g_handle_limit.load();
     if (owner && limit > 0 && owner->bytes + (int64_t)bytes > limit) {
@@ -112,6 +112,41 @@ nd_status nd_alloc(void** p, size_t bytes, cudaStream_t st, nd_incidence* owner)
     }
     if (owner) owner->bytes += (int64_t)bytes;
     return ND_OK;
+}
+
+nd_status nd_alloc(void** p, size_t bytes, cudaStream_t st, nd_incidence* owner) {
+    nd_status rc = alloc_once(p, bytes, st, owner);
+    if (rc == ND_OK || !owner || owner->spare_bytes == 0) return rc;
+    nd_release_spare(owner, st);
+    rc = alloc_once(p, bytes, st, owner);
+    if (rc == ND_OK) nd_set_error("");
+    return rc;
+}
+
+nd_status nd_alloc_spare(void** p, size_t bytes, cudaStream_t st, nd_incidence* owner) {
+    const int64_t before = owner->bytes;
+    const nd_status rc = alloc_once(p, bytes, st, owner);
+    owner->spare_bytes += owner->bytes - before;
+    if (rc != ND_OK) nd_set_error("");
+    return rc;
+}
+
+// the pass graphs hold addresses of spare memory and the bucket ranges
+void nd_drop_graphs(nd_incidence* h) {
+    for (auto& row : h->pass_graph)
+        for (auto& ex : row)
+            if (ex) { cudaGraphExecDestroy(ex); ex = nullptr; }
+}
+
+void nd_release_spare(nd_incidence* h, cudaStream_t st) {
+    nd_drop_graphs(h);
+    nd_release(h->list, st);
+    nd_release(h->front[2], st);
+    nd_release(h->front[3], st);
+    h->list = h->front[2] = h->front[3] = nullptr;
+    h->list_tiles = 0;
+    h->bytes -= h->spare_bytes;
+    h->spare_bytes = 0;
 }
 
 void nd_release(void* p, cudaStream_t st) {
@@ -246,9 +281,7 @@ void nd_free(nd_incidence* h) {
                     h->mirror, h->e_pos, h->tg[0], h->tg[1], h->long_rows, h->long_seg, h->to_new, h->to_old,
                     h->vto_old, h->oct_max, h->t_pos, h->t_id, h->c_rp, h->c_up, h->c_col, h->c_nlow, h->gid, h->gact[0], h->gact[1]};
     for (void* p : ptrs) nd_release(p, st);
-    for (auto& row : h->pass_graph)
-        for (auto& ex : row)
-            if (ex) cudaGraphExecDestroy(ex);
+    nd_drop_graphs(h);
     if (!h->inc_aliases_graph) {
         nd_release(h->inc_ptr, st);
         nd_release(h->inc, st);

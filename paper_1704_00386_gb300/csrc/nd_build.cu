@@ -2286,10 +2286,7 @@ nd_status nd_build_k4_incidence(nd_incidence* h, cudaStream_t st) {
 
 nd_status nd_build_buckets(nd_incidence* h, cudaStream_t st) {
     const int64_t N = h->num_r;
-    // pass graphs hold the bucket ranges of the old buckets
-    for (auto& row : h->pass_graph)
-        for (auto& ex : row)
-            if (ex) { cudaGraphExecDestroy(ex); ex = nullptr; }
+    nd_drop_graphs(h);  // they hold the old buckets
     for (int b = 0; b <= ND_NB; ++b) h->bucket_lo[b] = 0;
     h->num_zero = N;
     if (!h->items) ND_TRY(nd_alloc((void**)&h->items, sizeof(nd_item) * (N > 0 ? N : 1), st, h));

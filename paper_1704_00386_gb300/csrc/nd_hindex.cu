@@ -1310,12 +1310,8 @@ nd_status plan_list(nd_incidence* h, int64_t words, nd_tmp<uint32_t>& scratch, L
     L->tiles = L->tile_lo[ND_NB];
     L->words = words;
     if (L->tiles == 0) return ND_OK;
-    if (h->list && h->list_tiles < L->tiles) {  // other buckets than before
-        nd_release(h->list, st);
-        h->bytes -= h->list_tiles * kListTile * (int64_t)sizeof(uint32_t);
-        h->list = nullptr;
-    }
-    if (!h->list && nd_alloc((void**)&h->list, sizeof(uint32_t) * kListTile * L->tiles, st, h) == ND_OK)
+    if (h->list && h->list_tiles < L->tiles) nd_release_spare(h, st);  // other buckets than before
+    if (!h->list && nd_alloc_spare((void**)&h->list, sizeof(uint32_t) * kListTile * L->tiles, st, h) == ND_OK)
         h->list_tiles = L->tiles;
     L->list = h->list;
     L->room = L->tiles;
@@ -1394,11 +1390,11 @@ constexpr int kAndDirect = 6;
 constexpr int64_t kInlineItems = 1 << 15, kInlineBits = 1 << 22;
 bool take_inline(nd_incidence* h, int64_t words, cudaStream_t st) {
     if (h->bucket_lo[ND_NB] > kInlineItems || 32 * words > kInlineBits) return false;
-    for (int b = 2; b < 4; ++b)
-        if (!h->front[b] && nd_alloc((void**)&h->front[b], sizeof(uint32_t) * words, st, h) != ND_OK) {
-            nd_set_error("");
-            return false;
-        }
+    for (int b = 2; b < 4; ++b) {
+        if (h->front[b]) continue;
+        if (nd_alloc_spare((void**)&h->front[b], sizeof(uint32_t) * words, st, h) != ND_OK) return false;
+        nd_drop_graphs(h);  // those of AND take a list
+    }
     return true;
 }
 

@@ -136,9 +136,12 @@ struct nd_incidence {
     int32_t thr[3] = {8, 64, 2048};  // bucket thresholds t0, t1, t2
     // iteration state
     int32_t* tau[2] = {nullptr, nullptr};
-    uint32_t* front[4] = {nullptr, nullptr, nullptr, nullptr};  // the last two: small handles
+    // spare memory: what a handle keeps to be faster, and gives up where
+    // something it cannot do without needs the room (nd_alloc)
     uint32_t* list = nullptr;                // the active work items of a pass (AND; batches)
     int64_t list_tiles = 0;                  // tiles of work items it holds
+    uint32_t* front[4] = {nullptr, nullptr, nullptr, nullptr};  // the last two, of small handles, are spare
+    int64_t spare_bytes = 0;                 // of all of it, also counted in bytes
     unsigned long long* counters = nullptr;  // ring of per-pass counters
     unsigned long long* h_counters = nullptr;  // pinned host mirror, at the head of the handle's pinned block
     int64_t* h_read = nullptr;                 // ND_READ pinned words after it, for counts read back in the build
@@ -224,9 +227,14 @@ struct nd_tmp {
     }
 };
 
-// device memory helpers (stream-ordered)
+// device memory helpers (stream-ordered).  nd_alloc: memory that the owner
+// cannot do without; where there is no room for it, the owner's spare memory is
+// given back first.  nd_alloc_spare: memory that it can do without.
 nd_status nd_alloc(void** p, size_t bytes, cudaStream_t st, nd_incidence* owner);
+nd_status nd_alloc_spare(void** p, size_t bytes, cudaStream_t st, nd_incidence* owner);
 void nd_release(void* p, cudaStream_t st);
+void nd_release_spare(nd_incidence* h, cudaStream_t st);
+void nd_drop_graphs(nd_incidence* h);
 
 // exclusive scan of data[0..count] in place (count+1 entries; data[count]
 // becomes the total).  Uses stream-ordered scratch.

@@ -54,3 +54,32 @@ def test_list_of_one_tile_is_the_run_s_own(nd, r, mode):
         assert tight.incidence_bytes() <= held - 4
     finally:
         nd.set_handle_memory_limit(0)
+
+
+@pytest.mark.parametrize("r,scale", [(1, 16), (1, 9), (2, 13), (2, 8), (3, 10), (3, 6)])
+def test_and_leaves_room_for_the_other_modes(nd, r, scale):
+    """The list of active rows, and the frontiers of a small handle, give way to
+    what another mode cannot do without, in whatever order the modes come."""
+    n, s, d = G.rmat(scale, 8, seed=17 + r)
+    g = [torch.from_numpy(x).cuda() for x in G.to_csr(n, s, d)]
+    inc = nd.build_incidence(*g, r, r + 1)
+    kap = inc.snd()[0]
+    one = inc.iterate_k("snd", 1)[0]
+    inc.and_(notify=False)
+    held = inc.incidence_bytes()  # with all that SND and AND need
+    try:
+        nd.set_handle_memory_limit(held)
+        for order in (("and", "snd", "and_nn", "and"), ("and_nn", "and", "snd"), ("snd", "and", "snd", "and")):
+            tight = nd.build_incidence(*g, r, r + 1)
+            for mode in order:
+                for _ in range(3):  # the later runs take graphs
+                    assert torch.equal(tight.iterate_k(mode, 1 << 20)[0], kap), (order, mode)
+            assert torch.equal(tight.iterate_k("snd", 1)[0], one)
+            assert tight.incidence_bytes() <= held
+            nd.set_handle_memory_limit(0)  # room for the spare arrays again
+            assert torch.equal(tight.and_()[0], kap)
+            nd.set_handle_memory_limit(held)
+            assert torch.equal(tight.and_()[0], kap) and torch.equal(tight.snd()[0], kap)
+            tight.free()
+    finally:
+        nd.set_handle_memory_limit(0)

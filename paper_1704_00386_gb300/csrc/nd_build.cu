@@ -1800,56 +1800,44 @@ nd_status nd_relabel_truss_graph(nd_incidence* h, cudaStream_t st) {
     const int64_t n = h->n, nnz = h->nnz;
     if (n < kRelabelMinVertices || h->r != 2) return ND_OK;
     nd_prof_scope ps("relabel", st);
-    int32_t* vto_new = nullptr;
-    ND_TRY(nd_alloc((void**)&vto_new, sizeof(int32_t) * n, st, h));
+    nd_tmp<int32_t> vto_new(st), ncol(st);
+    nd_tmp<int64_t> nrp(st);
+    ND_TRY(nd_alloc((void**)&vto_new.p, sizeof(int32_t) * n, st, h));
     ND_TRY(nd_alloc((void**)&h->vto_old, sizeof(int32_t) * n, st, h));
-    nd_status rc = class_ids(h, vto_new, h->vto_old, st);
-    int64_t* nrp = nullptr;
-    int32_t* ncol = nullptr;
-    if (rc == ND_OK) rc = nd_alloc((void**)&nrp, sizeof(int64_t) * (n + 1), st, h);
-    if (rc == ND_OK) rc = nd_alloc((void**)&ncol, sizeof(int32_t) * (nnz > 0 ? nnz : 1), st, h);
-    if (rc == ND_OK && nnz > 0) {
+    ND_TRY(class_ids(h, vto_new, h->vto_old, st));
+    ND_TRY(nd_alloc((void**)&nrp.p, sizeof(int64_t) * (n + 1), st, h));
+    ND_TRY(nd_alloc((void**)&ncol.p, sizeof(int32_t) * (nnz > 0 ? nnz : 1), st, h));
+    if (nnz > 0) {
         nd_tmp<unsigned long long> keys(st), alt(st);
-        rc = keys.alloc(nnz);
-        if (rc == ND_OK) rc = alt.alloc(nnz);
+        ND_TRY(keys.alloc(nnz));
+        ND_TRY(alt.alloc(nnz));
         const int bits = nd_id_bits(n);
-        if (rc == ND_OK) {
-            k_relabel_keys<<<nd_blocks_for(n * 32, kThreads, grid_cap(h) * 4), kThreads, 0, st>>>(
-                n, h->rp, h->col, vto_new, bits, keys);
-            if (h->long_segs > 0)
-                k_relabel_keys_long<<<nd_blocks_for(h->long_segs * 32, kThreads, grid_cap(h) * 4), kThreads, 0, st>>>(
-                    h->rp, h->col, vto_new, bits, keys, h->long_rows, h->long_seg, h->long_count, h->long_segs);
-            const cudaError_t e = cudaGetLastError();
-            if (e != cudaSuccess) rc = nd_cuda_fail(e, "k_relabel_keys", __FILE__, __LINE__);
+        k_relabel_keys<<<nd_blocks_for(n * 32, kThreads, grid_cap(h) * 4), kThreads, 0, st>>>(n, h->rp, h->col, vto_new,
+                                                                                             bits, keys);
+        ND_CUDA(cudaGetLastError());
+        if (h->long_segs > 0) {
+            k_relabel_keys_long<<<nd_blocks_for(h->long_segs * 32, kThreads, grid_cap(h) * 4), kThreads, 0, st>>>(
+                h->rp, h->col, vto_new, bits, keys, h->long_rows, h->long_seg, h->long_count, h->long_segs);
+            ND_CUDA(cudaGetLastError());
         }
         unsigned long long* sorted = nullptr;
-        if (rc == ND_OK) rc = nd_sort_u64(keys, alt, nnz, 2 * bits, &sorted, st);
-        if (rc == ND_OK) {
-            k_keys_to_col<<<nd_blocks_for(nnz, kThreads, grid_cap(h) * 4), kThreads, 0, st>>>(nnz, sorted, bits, ncol);
-            const cudaError_t e = cudaGetLastError();
-            if (e != cudaSuccess) rc = nd_cuda_fail(e, "k_keys_to_col", __FILE__, __LINE__);
-        }
-    }
-    if (rc == ND_OK) {
-        ND_CUDA(cudaMemsetAsync(nrp + n, 0, sizeof(int64_t), st));
-        k_new_degrees<<<nd_blocks_for(n, kThreads, grid_cap(h) * 4), kThreads, 0, st>>>(n, h->rp, vto_new, nrp);
+        ND_TRY(nd_sort_u64(keys, alt, nnz, 2 * bits, &sorted, st));
+        k_keys_to_col<<<nd_blocks_for(nnz, kThreads, grid_cap(h) * 4), kThreads, 0, st>>>(nnz, sorted, bits, ncol);
         ND_CUDA(cudaGetLastError());
-        rc = nd_scan_i64(nrp, n, st);
     }
-    nd_release(vto_new, st);
-    if (rc != ND_OK) {
-        nd_release(nrp, st);
-        nd_release(ncol, st);
-        return rc;
-    }
+    ND_CUDA(cudaMemsetAsync(nrp + n, 0, sizeof(int64_t), st));
+    k_new_degrees<<<nd_blocks_for(n, kThreads, grid_cap(h) * 4), kThreads, 0, st>>>(n, h->rp, vto_new, nrp);
+    ND_CUDA(cudaGetLastError());
+    ND_TRY(nd_scan_i64(nrp, n, st));
+    nd_release(vto_new.take(), st);
     // keep the caller's graph and split for the edge map; the new graph
     // takes their place and is split again
     h->c_rp = h->rp;
     h->c_col = h->col;
     h->c_nlow = h->nlow;
     h->c_up = h->up_start;
-    h->rp = nrp;
-    h->col = ncol;
+    h->rp = nrp.take();
+    h->col = ncol.take();
     h->nlow = nullptr;
     h->up_start = nullptr;
     nd_release(h->mirror, st);
@@ -1961,19 +1949,19 @@ nd_status nd_relabel_by_degree(nd_incidence* h, cudaStream_t st) {
         }
         ND_TRY(nd_alloc((void**)&h->oct_max, sizeof(int32_t) * 32, st, h));
         ND_CUDA(cudaMemcpyAsync(h->oct_max, oct_max, sizeof(int32_t) * 32, cudaMemcpyHostToDevice, st));
-        int64_t* nrp = nullptr;
-        int32_t* ncol = nullptr;
-        ND_TRY(nd_alloc((void**)&nrp, sizeof(int64_t) * (n + 1), st, h));
+        nd_tmp<int64_t> nrp(st);
+        nd_tmp<int32_t> ncol(st);
+        ND_TRY(nd_alloc((void**)&nrp.p, sizeof(int64_t) * (n + 1), st, h));
         ND_CUDA(cudaMemsetAsync(nrp + n, 0, sizeof(int64_t), st));
         k_new_degrees<<<nd_blocks_for(n, kThreads, grid_cap(h) * 4), kThreads, 0, st>>>(n, h->rp, h->to_new, nrp);
         ND_CUDA(cudaGetLastError());
         ND_TRY(nd_scan_i64(nrp, n, st));
-        ND_TRY(nd_alloc((void**)&ncol, sizeof(int32_t) * (nnz > 0 ? nnz : 1), st, h));
+        ND_TRY(nd_alloc((void**)&ncol.p, sizeof(int32_t) * (nnz > 0 ? nnz : 1), st, h));
         if (nnz > 0) ND_TRY(order_rows(h, NewIdOrder{h->col, h->to_new, nrp, ncol}, segments, st));
         nd_release(h->rp, st);
         nd_release(h->col, st);
-        h->rp = nrp;
-        h->col = ncol;
+        h->rp = nrp.take();
+        h->col = ncol.take();
     }
     release_long_rows(h, st);
     return ND_OK;
@@ -2063,18 +2051,17 @@ static nd_status orient_graph(nd_incidence* h, nd_oriented* o, cudaStream_t st) 
 // does not depend on it; the gathers are only less local)
 static nd_status sort_tri_rows(nd_incidence* h, cudaStream_t st) {
     const int64_t N = h->num_r, M = h->num_inc;
-    uint2* dst = nullptr;
-    if (cudaMallocAsync((void**)&dst, sizeof(uint2) * (size_t)M, st) != cudaSuccess) {
-        cudaGetLastError();
+    nd_tmp<uint2> dst(st);
+    if (dst.alloc(M) != ND_OK) {
+        nd_set_error("");
         return ND_OK;
     }
     nd_tmp<uint32_t> over(st);
     nd_tmp<unsigned long long> over_ctr(st);
     // no adjacency list of n <= 32 * kRankWords vertices needs more words
     const bool can_overflow = h->n > 32 * (int64_t)kRankWords;
-    nd_status rc = over.alloc(can_overflow ? N : 1);
-    if (rc == ND_OK) rc = over_ctr.alloc(2);
-    if (rc != ND_OK) { cudaFreeAsync(dst, st); return rc; }
+    ND_TRY(over.alloc(can_overflow ? N : 1));
+    ND_TRY(over_ctr.alloc(2));
     if (can_overflow) ND_CUDA(cudaMemsetAsync(over_ctr, 0, sizeof(unsigned long long) * 2, st));
     const size_t smem = sizeof(uint32_t) * 2 * kRankWords * kRankWarps;
     ND_CUDA(cudaFuncSetAttribute(k_row_rank<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -2106,7 +2093,7 @@ static nd_status sort_tri_rows(nd_incidence* h, cudaStream_t st) {
         ND_CUDA(cudaGetLastError());
     }
     nd_release(h->inc, st);
-    h->inc = reinterpret_cast<uint32_t*>(dst);
+    h->inc = reinterpret_cast<uint32_t*>(dst.take());
     h->rows_sorted = true;
     return ND_OK;
 }

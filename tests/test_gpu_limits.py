@@ -1,5 +1,7 @@
 """Handles at their memory limit: the library does without what it only keeps to
 be faster, and what ran without those arrays still runs."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -83,3 +85,40 @@ def test_and_leaves_room_for_the_other_modes(nd, r, scale):
             tight.free()
     finally:
         nd.set_handle_memory_limit(0)
+
+
+def _pool_bytes():
+    """Bytes in use in the memory pool that the library allocates from."""
+    cu = ctypes.CDLL("libcuda.so.1")
+    dev, pool, used = ctypes.c_int(), ctypes.c_void_p(), ctypes.c_uint64()
+    torch.cuda.synchronize()
+    assert cu.cuDeviceGet(ctypes.byref(dev), torch.cuda.current_device()) == 0
+    assert cu.cuDeviceGetMemPool(ctypes.byref(pool), dev) == 0
+    assert cu.cuMemPoolGetAttribute(pool, 7, ctypes.byref(used)) == 0  # CU_MEMPOOL_ATTR_USED_MEM_CURRENT
+    return used.value
+
+
+@pytest.mark.parametrize("r", [1, 2, 3])
+def test_a_refused_build_frees_what_it_took(nd, r):
+    """Builds under limits from nothing to what the handle holds, so that they
+    fail at one allocation after the other; 65,536 vertices are renumbered."""
+    n, s, d = G.rmat(16, 4, seed=29)
+    g = [torch.from_numpy(x).cuda() for x in G.to_csr(n, s, d)]
+    before = _pool_bytes()
+    inc = nd.build_incidence(*g, r, r + 1)
+    held = inc.incidence_bytes()
+    inc.free()
+    assert _pool_bytes() == before
+    refused = 0
+    try:
+        for k in range(1, 65):
+            nd.set_handle_memory_limit(held * k // 64)
+            try:
+                nd.build_incidence(*g, r, r + 1).free()
+            except nd.NDError as e:
+                assert e.status == nd.ND_E_NOMEM
+                refused += 1
+            assert _pool_bytes() == before, k
+    finally:
+        nd.set_handle_memory_limit(0)
+    assert 32 <= refused < 64

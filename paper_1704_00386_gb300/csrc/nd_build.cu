@@ -2197,10 +2197,9 @@ nd_status nd_build_tri_incidence(nd_incidence* h, cudaStream_t st) {
 }
 
 // may a (3,4) handle of T triangles and M incidences take the list layout?
-// Its slots have 32 bits, and what it holds beyond the id layout must not make
-// a handle miss the memory limit that would do without.
+// What it holds beyond the id layout must not make a handle miss the memory
+// limit that would do without.
 static bool list_layout_fits(const nd_incidence* h, int64_t T, int64_t M) {
-    if (3 * T >= (int64_t)UINT32_MAX) return false;
     const int64_t limit = nd_handle_limit();
     if (limit <= 0) return true;
     const int64_t extra = 24 * T + 12 * T + T;          // t_pos, t_id; two 16-bit copies; frontier bits
@@ -2238,7 +2237,8 @@ nd_status nd_build_k4_incidence(nd_incidence* h, cudaStream_t st) {
     ND_TRY(lw.alloc(3 * T));
     ND_TRY(lid.alloc(3 * T));
     ND_TRY(te.alloc(3 * T));
-    if (3 * T < (int64_t)UINT32_MAX) ND_TRY(t_pos.alloc(3 * T));
+    // without the slots, whatever the reason, the rows hold triangle ids
+    if (3 * T < (int64_t)UINT32_MAX && t_pos.alloc(3 * T) != ND_OK) nd_set_error("");
     {
         nd_prof_scope ps("edge_lists", st, 2);
         k_edge_lists<true><<<eblocks, kThreads, 0, st>>>(m, h->rp, h->col, h->eid, h->e_u, h->e_v, lptr, h->tri_ptr, lw,
@@ -2255,8 +2255,14 @@ nd_status nd_build_k4_incidence(nd_incidence* h, cudaStream_t st) {
     }
     ND_TRY(nd_scan_i64(h->inc_ptr, T, st));
     ND_TRY(read_i64(h, h->inc_ptr + T, &h->num_inc, st));
-    const bool slots = list_layout_fits(h, T, h->num_inc);
-    ND_TRY(nd_alloc((void**)&h->inc, sizeof(uint32_t) * 3 * (h->num_inc > 0 ? h->num_inc : 1), st, h));
+    const size_t inc_bytes = sizeof(uint32_t) * 3 * (h->num_inc > 0 ? h->num_inc : 1);
+    bool slots = t_pos.p && list_layout_fits(h, T, h->num_inc);
+    if (!slots || nd_alloc((void**)&h->inc, inc_bytes, st, h) != ND_OK) {
+        slots = false;
+        nd_release(t_pos.take(), st);  // room for the rows
+        ND_TRY(nd_alloc((void**)&h->inc, inc_bytes, st, h));
+        nd_set_error("");
+    }
     if (h->num_inc > 0) {
         nd_prof_scope ps("k4_fill", st);
         auto fill = slots ? k_k4_rows<true, false> : k_k4_rows<true, true>;

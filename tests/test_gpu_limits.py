@@ -122,3 +122,70 @@ def test_a_refused_build_frees_what_it_took(nd, r):
     finally:
         nd.set_handle_memory_limit(0)
     assert 32 <= refused < 64
+
+
+class _PoolProps(ctypes.Structure):
+    _fields_ = [("alloc_type", ctypes.c_int), ("handle_types", ctypes.c_int), ("location_type", ctypes.c_int),
+                ("location_id", ctypes.c_int), ("security", ctypes.c_void_p), ("max_size", ctypes.c_size_t),
+                ("usage", ctypes.c_ushort), ("reserved", ctypes.c_ubyte * 54)]
+
+
+class _small_pool:
+    """The library's allocations come from a pool of at most max_size bytes:
+    a device without memory, as the library sees it."""
+
+    def __init__(self, max_size):
+        self.cu, self.dev, self.pool = ctypes.CDLL("libcuda.so.1"), ctypes.c_int(), ctypes.c_void_p()
+        torch.cuda.synchronize()
+        assert self.cu.cuDeviceGet(ctypes.byref(self.dev), torch.cuda.current_device()) == 0
+        props = _PoolProps(alloc_type=1, location_type=1, location_id=self.dev.value, max_size=max_size)
+        assert self.cu.cuMemPoolCreate(ctypes.byref(self.pool), ctypes.byref(props)) == 0
+
+    def __enter__(self):
+        self.old = ctypes.c_void_p()
+        assert self.cu.cuDeviceGetMemPool(ctypes.byref(self.old), self.dev) == 0
+        assert self.cu.cuDeviceSetMemPool(self.dev, self.pool) == 0
+
+    def __exit__(self, *exc):
+        torch.cuda.synchronize()
+        assert self.cu.cuDeviceSetMemPool(self.dev, self.old) == 0
+        assert self.cu.cuMemPoolDestroy(self.pool) == 0
+
+
+def test_nuclei_without_memory_for_the_slots(nd):
+    """A (3,4) build on a device with room for triangle ids, but not for list
+    slots, keeps ids.  3.4M triangles of a complete tripartite graph, in no
+    4-clique, and ten cliques of 20."""
+    a, k = 150, 20
+    part = [np.arange(a) + i * a for i in range(3)]
+    pairs = [np.meshgrid(part[i], part[j]) for i, j in ((0, 1), (0, 2), (1, 2))]
+    up = np.triu_indices(k, 1)
+    src = np.concatenate([p[0].ravel() for p in pairs] + [3 * a + c * k + up[0] for c in range(10)])
+    dst = np.concatenate([p[1].ravel() for p in pairs] + [3 * a + c * k + up[1] for c in range(10)])
+    g = [torch.from_numpy(x).cuda() for x in G.to_csr(3 * a + 10 * k, src, dst)]
+    inc = nd.build_incidence(*g, 3, 4)
+    want = np.concatenate([np.zeros(a ** 3, np.int32), np.full(10 * k * (k - 1) * (k - 2) // 6, k - 3, np.int32)])
+    np.testing.assert_array_equal(inc.snd()[0].cpu().numpy(), want)
+    held = inc.incidence_bytes()
+    inc.free()
+    outcomes = []
+    for mb in range(384, 64, -8):
+        with _small_pool(mb << 20):
+            try:
+                inc = nd.build_incidence(*g, 3, 4)
+            except nd.NDError as e:
+                assert e.status == nd.ND_E_NOMEM
+                outcomes.append("refused")
+                assert _pool_bytes() == 0
+                continue
+            try:
+                for tau in (inc.and_()[0], inc.snd()[0]):
+                    np.testing.assert_array_equal(tau.cpu().numpy(), want)
+                # ids hold neither the slots (24 B a triangle) nor their 16-bit copies
+                outcomes.append("ids" if inc.incidence_bytes() < held - 24 * len(want) else "slots")
+            except nd.NDError as e:
+                assert e.status == nd.ND_E_NOMEM
+                outcomes.append("built only")
+            inc.free()
+    assert outcomes[0] == "slots" and outcomes[-1] == "refused"
+    assert "ids" in outcomes, outcomes

@@ -119,10 +119,15 @@ nd_status nd_build_incidence(const nd_csr* g, int r, int s, void* stream, nd_inc
  * through the neighbourhoods on every update (Section 4.1, "Time
  * complexity"; Section 5); this mode does the same for memory-bound inputs.
  * Only the counts d_s are kept (tau_0 and the work buckets); every SND / AND
- * pass then finds the triangles of edge (x,y) by searching each entry of the
- * shorter of N(x), N(y) in the longer.  Results are identical to the stored
- * mode; a pass costs about sum over edges of min(deg) binary searches
- * instead of a stream of 8 B per incidence.  For (1,2) the CSR already is the
+ * pass then finds the triangles of edge (x,y) by looking up each entry of the
+ * shorter of N(x), N(y) in the longer: in a table where that is a hub's, else
+ * by merging or by binary search.  Results are identical to the stored
+ * mode; a pass costs about sum over edges of min(deg) look-ups
+ * instead of a stream of 8 B per incidence.  The hub tables, and the lists
+ * ordered by degree class that go with them (at most 128 MB, and 8 B per CSR
+ * entry and 4 B per vertex), are built by the first run that they pay for and
+ * stay with the handle: nd_incidence_bytes counts them, and where the memory
+ * limit or the device has no room the handle does without.  For (1,2) the CSR already is the
  * incidence and the flag changes nothing; (3,4) gives ND_E_UNSUPPORTED_RS.
  * Unknown flags give ND_E_INVAL. */
 #define ND_BUILD_ON_THE_FLY 1u
@@ -254,7 +259,10 @@ nd_status nd_autotune(nd_incidence* inc, int32_t passes, void* stream, int32_t* 
 nd_status nd_last_passes(const nd_incidence* inc, int64_t* changed, int64_t* evaluated, int64_t* incidences,
                          int32_t cap, int32_t* passes);
 
-/* Device memory held by the handle, in bytes. */
+/* Device memory held by the handle, in bytes.  Iteration calls add to it: the
+ * state of their modes, and arrays that only make them faster (the list of active
+ * rows, hub tables), which the handle gives back where the limit below or the
+ * device has no room for what a call needs. */
 nd_status nd_incidence_bytes(const nd_incidence* inc, int64_t* bytes);
 
 /* Core numbers ((r,s) = (1,2)) by SND without allocating anything.

@@ -140,10 +140,11 @@ void nd_drop_graphs(nd_incidence* h) {
 
 void nd_release_spare(nd_incidence* h, cudaStream_t st) {
     nd_drop_graphs(h);
-    nd_release(h->list, st);
-    nd_release(h->front[2], st);
-    nd_release(h->front[3], st);
-    h->list = h->front[2] = h->front[3] = nullptr;
+    void* const ptrs[] = {h->list, h->front[2], h->front[3], h->hub_of, h->hub_bits, h->by_degree, h->slot_of};
+    for (void* p : ptrs) nd_release(p, st);
+    h->list = h->front[2] = h->front[3] = h->slot_of = nullptr;
+    h->hub_of = h->by_degree = nullptr;
+    h->hub_bits = nullptr;
     h->list_tiles = 0;
     h->bytes -= h->spare_bytes;
     h->spare_bytes = 0;
@@ -276,12 +277,12 @@ void nd_free(nd_incidence* h) {
     // one, then release on it (other streams keep running)
     cudaStream_t st = h->last_stream;
     cudaStreamSynchronize(st);
+    nd_release_spare(h, st);
     void* ptrs[] = {h->nlow, h->up_start, h->eid, h->e_u, h->e_v, h->tri_ptr, h->tri_w, h->tri_e,
-                    h->items, h->tau[0], h->tau[1], h->front[0], h->front[1], h->front[2], h->front[3], h->list, h->counters,
+                    h->items, h->tau[0], h->tau[1], h->front[0], h->front[1], h->counters,
                     h->mirror, h->e_pos, h->tg[0], h->tg[1], h->long_rows, h->long_seg, h->to_new, h->to_old,
                     h->vto_old, h->oct_max, h->t_pos, h->t_id, h->c_rp, h->c_up, h->c_col, h->c_nlow, h->gid, h->gact[0], h->gact[1]};
     for (void* p : ptrs) nd_release(p, st);
-    nd_drop_graphs(h);
     if (!h->inc_aliases_graph) {
         nd_release(h->inc_ptr, st);
         nd_release(h->inc, st);
@@ -652,6 +653,7 @@ nd_status nd_and_partial(nd_incidence* h, const uint32_t* members, int64_t count
     if (herr) { nd_set_error("a member id is not an r-clique id"); return ND_E_INVAL; }
     nd_run_opts opts;
     opts.members = mask;
+    opts.num_members = count;
     return run_and_deliver(h, ND_AND, max_iters, nullptr, 0, tau_out, on_device, iters_out, evals_out, true, st,
                            &opts);
 }

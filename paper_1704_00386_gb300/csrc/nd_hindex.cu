@@ -1196,8 +1196,8 @@ __global__ void k_number_hubs(int64_t n, const int64_t* __restrict__ rp, int64_t
 
 // the table of every hub, one block each: word w covers the vertices
 // [32 w, 32 w + 32), x = which of them are neighbours, y = neighbours below.
-// The list is sorted, so a word's entries are one run: its first entry (found
-// by a search, as the word's count below) writes the word alone.
+// The list is sorted, so a word's entries are one run: its thread searches the
+// run's first entry, whose index is y, and walks the run.
 __global__ void __launch_bounds__(kThreads) k_hub_tables(const int32_t* __restrict__ hubs,
                                                          const int64_t* __restrict__ rp,
                                                          const int32_t* __restrict__ col, int64_t words,
@@ -1552,61 +1552,64 @@ nd_status nd_classic_truss(const int32_t* in, int64_t n, int32_t* out, cudaStrea
 
 namespace {
 
-// the hub tables of a run without a stored incidence, in the run's own
-// workspace.  The largest degree class whose tables, with those of the
-// classes above, fit kHubBytes (an L2's worth: past that the probes would go
-// to DRAM) bounds the hubs.  Small graphs, and a device without the memory,
-// do without.
+// The hub tables of a handle without a stored incidence.  The largest degree
+// class whose tables, with those of the classes above, fit kHubBytes (an L2's
+// worth: past that the probes would go to DRAM) bounds the hubs.  They are
+// spare memory of the handle: a program that calls it again finds them built,
+// and where the device or the handle's limit has no room a run does without.
+// Building them takes 0.14 to 0.35 ms (426,000 to 7.6M entries), which the first
+// pass of a run over triangle-rich rows wins back (SND of one pass over an
+// R-MAT of 426,000 entries: 0.40 ms with them built, 0.83 with searches).  Not
+// worth it, and so not built: small graphs; rows of few triangles (uniform
+// random, 1.3M entries with 131,000 incidences: the whole SND 0.54 against 0.47
+// ms); PartialAnd of few members (ten of a Chung-Lu k-truss of 60,000 vertices:
+// 0.49 against 0.41 ms).
 constexpr int64_t kHubBytes = int64_t(128) << 20;
 constexpr int64_t kHubMinEntries = 1 << 18;  // below, the tables cost more than the passes
 constexpr int kHubMinClass = 5;              // lists of 32 entries are searched as fast
+constexpr int64_t kHubMemberShare = 8;       // PartialAnd: members at least one row in so many
 
-struct hub_tables {
-    nd_tmp<int32_t> of, list, by_degree;
-    nd_tmp<uint32_t> slot_of;
-    nd_tmp<uint2> bits;
-    explicit hub_tables(cudaStream_t st) : of(st), list(st), by_degree(st), slot_of(st), bits(st) {}
-};
+bool hub_tables_pay(const nd_incidence* h, const nd_run_opts* opts) {
+    if (h->num_hubs == 0 || h->nnz < kHubMinEntries || h->num_inc < h->nnz) return false;
+    return !opts || !opts->members || opts->num_members >= h->bucket_lo[ND_NB] / kHubMemberShare;
+}
 
-nd_status make_hub_tables(nd_incidence* h, hub_tables* t, SweepParams& P, cudaStream_t st) {
+nd_status make_hub_tables(nd_incidence* h, cudaStream_t st) {
     const int64_t words = (h->n + 31) / 32;
-    if (h->nnz < kHubMinEntries) return ND_OK;
-    nd_tmp<unsigned long long> cnt(st);
-    nd_tmp<int> count(st);
-    ND_TRY(cnt.alloc(32));
-    ND_TRY(count.alloc(1));
-    ND_CUDA(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long) * 32, st));
-    ND_CUDA(cudaMemsetAsync(count, 0, sizeof(int), st));
     const int blocks = nd_blocks_for(h->n, kThreads, h->sm_count * 8);
     nd_prof_scope ps("hub_tables", st, 3);
-    k_degree_classes<<<blocks, kThreads, 0, st>>>(h->n, h->rp, cnt);
-    ND_CUDA(cudaGetLastError());
-    ND_CUDA(cudaMemcpyAsync(h->h_read, cnt, sizeof(unsigned long long) * 32, cudaMemcpyDeviceToHost, st));
-    ND_TRY(nd_wait(st));
-    int64_t hubs = 0;
-    int k = 32;
-    while (k > kHubMinClass && (hubs + h->h_read[k - 1]) * words * (int64_t)sizeof(uint2) <= kHubBytes) hubs += h->h_read[--k];
+    if (h->num_hubs < 0) {
+        nd_tmp<unsigned long long> cnt(st);
+        ND_TRY(cnt.alloc(32));
+        ND_CUDA(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long) * 32, st));
+        k_degree_classes<<<blocks, kThreads, 0, st>>>(h->n, h->rp, cnt);
+        ND_CUDA(cudaGetLastError());
+        ND_CUDA(cudaMemcpyAsync(h->h_read, cnt, sizeof(unsigned long long) * 32, cudaMemcpyDeviceToHost, st));
+        ND_TRY(nd_wait(st));
+        int64_t hubs = 0;
+        int k = 32;
+        while (k > kHubMinClass && (hubs + h->h_read[k - 1]) * words * (int64_t)sizeof(uint2) <= kHubBytes)
+            hubs += h->h_read[--k];
+        h->num_hubs = hubs;
+        h->hub_degree = k < 31 ? 1 << k : INT32_MAX;
+    }
+    const int64_t hubs = h->num_hubs;
     if (hubs == 0) return ND_OK;
-    if (t->of.alloc(h->n) != ND_OK || t->list.alloc(hubs) != ND_OK || t->bits.alloc(hubs * words) != ND_OK ||
-        t->by_degree.alloc(h->nnz) != ND_OK || t->slot_of.alloc(h->nnz) != ND_OK) {
-        nd_set_error("");
-        return ND_OK;
-    }
-    k_number_hubs<<<blocks, kThreads, 0, st>>>(h->n, h->rp, (int64_t)1 << k, t->of, t->list, count);
+    nd_tmp<int32_t> list(st);
+    nd_tmp<int> count(st);
+    nd_status rc = nd_alloc_spare((void**)&h->hub_of, sizeof(int32_t) * h->n, st, h);
+    if (rc == ND_OK) rc = nd_alloc_spare((void**)&h->by_degree, sizeof(int32_t) * h->nnz, st, h);
+    if (rc == ND_OK) rc = nd_alloc_spare((void**)&h->slot_of, sizeof(uint32_t) * h->nnz, st, h);
+    if (rc == ND_OK) rc = nd_alloc_spare((void**)&h->hub_bits, sizeof(uint2) * hubs * words, st, h);
+    if (rc == ND_OK) rc = list.alloc(hubs);
+    if (rc == ND_OK) rc = count.alloc(1);
+    if (rc == ND_OK) rc = nd_rows_by_degree(h, h->by_degree, h->slot_of, st);
+    if (rc != ND_OK) return rc;
+    ND_CUDA(cudaMemsetAsync(count, 0, sizeof(int), st));
+    k_number_hubs<<<blocks, kThreads, 0, st>>>(h->n, h->rp, h->hub_degree, h->hub_of, list, count);
     ND_CUDA(cudaGetLastError());
-    k_hub_tables<<<(unsigned)hubs, kThreads, 0, st>>>(t->list, h->rp, h->col, words, t->bits);
+    k_hub_tables<<<(unsigned)hubs, kThreads, 0, st>>>(list, h->rp, h->col, words, h->hub_bits);
     ND_CUDA(cudaGetLastError());
-    const nd_status rc = nd_rows_by_degree(h, t->by_degree, t->slot_of, st);
-    if (rc == ND_E_NOMEM) {
-        nd_set_error("");
-        return ND_OK;
-    }
-    ND_TRY(rc);
-    P.by_degree = t->by_degree;
-    P.slot_of = t->slot_of;
-    P.hub_of = t->of;
-    P.hub_bits = t->bits;
-    P.hub_words = words;
     return ND_OK;
 }
 
@@ -1714,13 +1717,17 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
         P.gid = h->gid;
     }
     plan_buckets(h, P);
-    hub_tables hubs(st);
-    P.hub_of = nullptr;
-    P.hub_bits = nullptr;
-    P.hub_words = 0;
-    P.by_degree = nullptr;
-    P.slot_of = nullptr;
-    if (h->otf) ND_TRY(make_hub_tables(h, &hubs, P, st));
+    if (h->otf && !h->hub_bits && hub_tables_pay(h, opts)) {
+        const nd_status rc = make_hub_tables(h, st);
+        if (rc != ND_OK) nd_release_spare(h, st);
+        if (rc != ND_OK && rc != ND_E_NOMEM) return rc;
+        if (rc != ND_OK) nd_set_error("");
+    }
+    P.hub_of = h->hub_bits ? h->hub_of : nullptr;
+    P.hub_bits = h->hub_bits;
+    P.hub_words = (h->n + 31) / 32;
+    P.by_degree = h->by_degree;
+    P.slot_of = h->slot_of;
     pass_fn fn0 = pick(h, mode, false, in_line), fn1 = pick(h, mode, true, in_line);
     // ask for a shared-memory carve-out that just holds each kernel's
     // resident blocks (plus the 1 KB each block reserves), leaving the rest
@@ -1767,8 +1774,8 @@ nd_status nd_run(nd_incidence* h, int mode, int32_t max_passes, const int32_t* t
         const int kind = batch == 0 ? 0 : ((batch & 1) ? 2 : 1);
         bool launched = false;
         // graphs hold the plain parameters and the handle's own memory; runs with
-        // members, a stopping rule, a tau of the caller's, or tables or a list of
-        // their own launch directly, and so does the first batch of its kind on a
+        // members, a stopping rule, a tau of the caller's, a list of their own or
+        // no storage launch directly, and so does the first batch of its kind on a
         // handle: building a graph costs more than its launches, and many
         // handles run each mode once
         const bool seen = h->batch_seen[mode][kind];

@@ -141,7 +141,15 @@ struct nd_incidence {
     uint32_t* list = nullptr;                // the active work items of a pass (AND; batches)
     int64_t list_tiles = 0;                  // tiles of work items it holds
     uint32_t* front[4] = {nullptr, nullptr, nullptr, nullptr};  // the last two, of small handles, are spare
-    int64_t spare_bytes = 0;                 // of all of it, also counted in bytes
+    // no storage: the hub tables (make_hub_tables in nd_hindex.cu), built by the
+    // first run that they pay for; num_hubs: -1 until they have been counted
+    int64_t num_hubs = -1;
+    int32_t hub_degree = 0;        // the smallest degree of a hub
+    int32_t* hub_of = nullptr;     // [n] hub index of a vertex, -1 for the others
+    uint2* hub_bits = nullptr;     // [num_hubs * ((n + 31) / 32)]
+    int32_t* by_degree = nullptr;  // [nnz] the adjacency lists by degree class, and
+    uint32_t* slot_of = nullptr;   // [nnz] the CSR slot of every entry
+    int64_t spare_bytes = 0;       // of all of it, also counted in bytes
     unsigned long long* counters = nullptr;  // ring of per-pass counters
     unsigned long long* h_counters = nullptr;  // pinned host mirror, at the head of the handle's pinned block
     int64_t* h_read = nullptr;                 // ND_READ pinned words after it, for counts read back in the build
@@ -294,6 +302,7 @@ nd_status nd_init_tau(nd_incidence* h, int32_t* tau, cudaStream_t st);
 // options of a run beyond the paper's plain SND / AND
 struct nd_run_opts {
     const uint32_t* members = nullptr;  // PartialAnd: member bitmap (device), AND modes only
+    int64_t num_members = 0;            // as the caller counts them, repeats included
     double stop_active = 0.0;           // AND: stop after a pass that evaluated < this fraction of N_R
     bool stopped = false;               // out: the active-ratio rule ended the run
 };

@@ -87,6 +87,49 @@ def test_and_leaves_room_for_the_other_modes(nd, r, scale):
         nd.set_handle_memory_limit(0)
 
 
+def test_hub_tables_are_counted_and_give_way(nd):
+    """A handle without storage keeps the hub tables that its first long run
+    builds; they count in its bytes, are left out where its limit has no room,
+    and go where another mode needs theirs.  Short questions build none."""
+    n, s, d = G.rmat(14, 16, seed=61)
+    rp, col = G.to_csr(n, s, d)
+    g = [torch.from_numpy(x).cuda() for x in (rp, col)]
+    new = lambda: nd.build_incidence(*g, 2, 3, on_the_fly=True)  # noqa: E731
+    inc = new()
+    few = torch.arange(0, 10, dtype=torch.int32, device="cuda")
+    part = inc.and_partial(few)[0]
+    bare = inc.incidence_bytes()  # what AND needs
+    snd_more = 4 * inc.num_r + 2 * int(rp[-1])  # and SND: the second tau and its copy
+    kap, passes = inc.snd()
+    tables = inc.incidence_bytes() - bare - snd_more
+    assert 8 * rp[-1] < tables <= 8 * rp[-1] + 4 * n + (128 << 20)
+    assert torch.equal(inc.and_()[0], kap) and torch.equal(inc.and_partial(few)[0], part)
+    assert inc.incidence_bytes() == bare + snd_more + tables  # built once
+    try:
+        for room in (bare + snd_more, bare + tables, bare + tables + snd_more // 2, bare + tables + snd_more):
+            nd.set_handle_memory_limit(room)
+            tight = new()
+            for _ in range(2):
+                assert torch.equal(tight.and_()[0], kap)
+                assert torch.equal(tight.and_partial(few)[0], part)
+                tau, it = tight.snd()
+                assert torch.equal(tau, kap) and it == passes
+            assert tight.incidence_bytes() == (room if room == bare + tables + snd_more else bare + snd_more)
+            tight.free()
+    finally:
+        nd.set_handle_memory_limit(0)
+    # rows of few triangles: none either
+    rng = np.random.default_rng(5)
+    rp, col = G.to_csr(20000, rng.integers(0, 20000, 300_000), rng.integers(0, 20000, 300_000))
+    grown = []
+    for otf in (True, False):
+        inc = nd.build_incidence(rp, col, 2, 3, on_the_fly=otf)
+        bare = inc.incidence_bytes()
+        np.testing.assert_array_equal(inc.snd()[0], oracle.decompose(rp, col, 2, 3))
+        grown.append(inc.incidence_bytes() - bare)
+    assert grown[0] == grown[1]  # the state of SND alone
+
+
 def _pool_bytes():
     """Bytes in use in the memory pool that the library allocates from."""
     cu = ctypes.CDLL("libcuda.so.1")

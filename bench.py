@@ -49,11 +49,11 @@ UNIT = "updates/s"
 PEEL_SAMPLE_SCALE = 14    # the single-threaded peeling oracle, timed on a bounded sample
 CPU_SND_SECONDS = 10.0    # time budget of the multi-threaded SND passes of the CPU baseline
 # ncu DRAM bytes per incidence of a SND pass (k-truss, q = 2): dram__bytes_read.sum +
-# dram__bytes_write.sum over the 41 working passes of one run on R-MAT scale 18, 72.154 GB, by
-# 247,767,033 incidences per pass: 7.10 B on average, 9.4 B in pass 1 (whole rows), 6.0 B in
+# dram__bytes_write.sum over the 41 working passes of one run on R-MAT scale 18, 72.048 GB, by
+# 247,767,033 incidences per pass: 7.09 B on average, 9.2 B in pass 1 (whole rows), 6.0 B in
 # late passes, which stop once a row's h-index is settled.  None once a kernel changes
 # until it is measured again.
-NCU_SND_TRAFFIC_PER_INCIDENCE = 72.154e9 / 41 / 247767033
+NCU_SND_TRAFFIC_PER_INCIDENCE = 72.048e9 / 41 / 247767033
 
 
 def parse():
@@ -380,7 +380,7 @@ def run_ours(args, rank, world, local_rank):
     # tau values per incidence are L2 hits while tau fits in L2, so they are
     # not DRAM bytes.  The incidences are those of whole rows: a pass stops
     # reading a row once its h-index is settled, so this model is an upper
-    # bound, and where the DRAM bytes were measured those are used instead.
+    # bound (frac_whole_rows).
     info = infos[-1]
     peak, peak_kind = load_peaks()
     top = max(prof.items(), key=lambda kv: kv[1][1])
@@ -400,20 +400,23 @@ def run_ours(args, rank, world, local_rank):
         units = "8 B per incidence written (fill) or CSR bytes read"
     avg_ms = ms / max(eff, 1)
     achieved = per_launch / (avg_ms / 1000.0) / 1e9
-    # DRAM traffic per SND pass: the ncu bytes per incidence of the R-MAT scale 18 k-truss passes,
-    # scaled by the incidences of this workload; None for any other kernel or once the kernel has
+    whole_rows = per_launch if name in ("snd_pass", "and_pass") else None
+    # DRAM traffic per SND pass of an R-MAT k-truss: the ncu bytes per incidence of the R-MAT scale 18
+    # passes, scaled by the incidences of this workload.  How far rows are read depends on the graph
+    # and on the number of passes, so None for any other workload or kernel, or once the kernel has
     # changed.
     traffic = None
-    if name == "snd_pass" and q == 2 and NCU_SND_TRAFFIC_PER_INCIDENCE is not None:
+    if name == "snd_pass" and q == 2 and args.workload.startswith("rmat_s") and NCU_SND_TRAFFIC_PER_INCIDENCE:
         traffic = NCU_SND_TRAFFIC_PER_INCIDENCE * M
         per_launch, achieved = traffic, traffic / (avg_ms / 1000.0) / 1e9
-        units = "ncu DRAM bytes per SND pass (rows are read only until their h-index is settled)"
+        units = ("DRAM bytes per SND pass, extrapolated by incidences from the ncu bytes of R-MAT scale 18 "
+                 "(rows are read only until their h-index is settled)")
     # Byte models of the same pass, each over its measured average time:
-    #   frac       the DRAM bytes ncu measured, where known; else the compulsory bytes
-    #              of whole rows above;
+    #   frac       traffic where there is one, else the whole rows;
+    #   frac_whole_rows the compulsory bytes of whole rows above, an upper bound;
     #   frac_survey every operand counted once, gathers included:
     #              16 B per r-clique + 8q B per incidence (4 B id + 4 B gathered tau);
-    #   frac_dram  the DRAM bytes ncu measured (traffic), when known.
+    #   frac_dram  traffic, when known.
     survey_bytes = None
     if name in ("snd_pass", "and_pass"):
         key = "snd" if name == "snd_pass" else "and"
@@ -421,17 +424,22 @@ def run_ours(args, rank, world, local_rank):
         survey_bytes = sb / max(eff, 1)
     survey_gbs = survey_bytes / (avg_ms / 1000.0) / 1e9 if survey_bytes else None
     dram_gbs = traffic / (avg_ms / 1000.0) / 1e9 if traffic else None
+    whole_gbs = whole_rows / (avg_ms / 1000.0) / 1e9 if whole_rows else None
     roofline = {"bound": "hbm", "kernel": name, "achieved": achieved, "peak": peak,
                 "peak_kind": peak_kind, "unit": "GB/s", "frac": achieved / peak, "traffic": traffic,
                 "bytes_per_launch": per_launch, "launches_effective": eff, "avg_launch_ms": avg_ms,
                 "units": units,
+                "frac_whole_rows": whole_gbs / peak if whole_gbs else None,
+                "bytes_per_launch_whole_rows": whole_rows,
+                "units_whole_rows": "compulsory bytes of whole rows: an upper bound, rows are read only until settled",
                 "frac_survey": survey_gbs / peak if survey_gbs else None,
                 "achieved_survey": survey_gbs,
                 "bytes_per_launch_survey": survey_bytes,
                 "units_survey": "16 B x r-cliques evaluated + 8q B x incidences of whole rows (4 B id + 4 B gathered tau)",
                 "frac_dram": dram_gbs / peak if dram_gbs else None,
                 "achieved_dram": dram_gbs,
-                "units_dram": "ncu dram__bytes_read.sum + dram__bytes_write.sum per pass (traffic) / average pass time",
+                "units_dram": "traffic (ncu dram__bytes_read.sum + dram__bytes_write.sum of R-MAT scale 18 passes, "
+                              "extrapolated by incidences) / average pass time",
                 "note": "gather-bound: the L1 wavefronts of the q tau gathers per incidence set the pace, not DRAM"}
 
     # ----- end to end through the public API with host buffers

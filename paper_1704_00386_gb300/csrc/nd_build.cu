@@ -12,9 +12,12 @@
 //   (3,4)  triangle (u,v,w): the z in the triangle lists of its three edges
 //          -> the slots of {u,v,z}, {u,w,z}, {v,w,z} in those lists.
 // Every step is a count pass, an exclusive scan and a fill pass over the same
-// enumeration.  Intersections: one warp per list pair; the lanes walk the
-// shorter list in order and binary-search each element in the other list(s)
-// (read-only path).
+// enumeration; the (2,3) fill of larger graphs takes the count's triangles as
+// records.  Intersections: (2,3), 32 oriented edges per warp, the elements of
+// their shorter out-lists walked as one sequence and binary-searched in the
+// longer ones; (3,4), a list pair or triple per warp, the longer lists passing
+// through shared memory in blocks (nd_list_cursor) or, where much longer,
+// binary-searched.
 #include "nd_internal.cuh"
 
 #include <vector>
@@ -58,8 +61,8 @@ __device__ __forceinline__ int64_t warp_count_global() {
 constexpr int kPoolRow = 128;
 // Rows per warp: 32 where that still gives every resident warp some, fewer
 // otherwise (a 2,800-vertex graph validated in 37 instead of 18 us with 32).
-int rows_per_warp(int64_t rows) {
-    const int64_t r = rows / (152 * 64);
+int rows_per_warp(const nd_incidence* h, int64_t rows) {
+    const int64_t r = rows / ((h->sm_count > 0 ? h->sm_count : 152) * 64);
     return (int)(r < 1 ? 1 : (r > 32 ? 32 : r));
 }
 int pool_blocks(int64_t rows, int per, int cap) { return nd_blocks_for((rows + per - 1) / per * 32, kThreads, cap); }
@@ -1711,7 +1714,7 @@ static nd_status validate_split(nd_incidence* h, cudaStream_t st, bool by_length
     ND_TRY(find_long_rows(h, st));
     if (g->n > 0) {
         nd_prof_scope ps("validate_split", st);
-        const int per = rows_per_warp(g->n), blocks = pool_blocks(g->n, per, grid_cap(h) * 4);
+        const int per = rows_per_warp(h, g->n), blocks = pool_blocks(g->n, per, grid_cap(h) * 4);
         auto split = fp ? k_validate_split<true, true> : (by_length ? k_validate_split<true> : k_validate_split<false>);
         split<<<blocks, kThreads, 0, st>>>(per, g->n, g->nnz, h->rp, h->col, h->nlow, h->up_start, derr, dsearched,
                                            h->mirror, dsearched.p + 1);
@@ -1908,7 +1911,7 @@ struct nd_row_segments {
 // every row of h->rp in the order of k's buckets
 template <typename K>
 static nd_status order_rows(nd_incidence* h, const K& k, const nd_row_segments& sg, cudaStream_t st) {
-    const int per = rows_per_warp(h->n);
+    const int per = rows_per_warp(h, h->n);
     k_order_rows<K><<<pool_blocks(h->n, per, grid_cap(h) * 4), kThreads, 0, st>>>(per, h->n, h->rp, k);
     ND_CUDA(cudaGetLastError());
     if (sg.segs == 0) return ND_OK;
@@ -2029,7 +2032,7 @@ static nd_status orient_graph(nd_incidence* h, nd_oriented* o, cudaStream_t st) 
     const bool positions = h->adj && !h->otf;  // only the stored (2,3) fill uses them
     if (positions) ND_TRY(o->out_pm.alloc(m));
     ND_CUDA(cudaMemsetAsync(o->out_ptr.p + n, 0, sizeof(int64_t), st));
-    const int per = rows_per_warp(n), vblocks = pool_blocks(n, per, grid_cap(h) * 4);
+    const int per = rows_per_warp(h, n), vblocks = pool_blocks(n, per, grid_cap(h) * 4);
     if (n > 0) {
         nd_prof_scope ps("orient", st);
         k_orient<false><<<vblocks, kThreads, 0, st>>>(per, n, h->rp, h->col, h->eid, o->out_ptr, nullptr, nullptr, nullptr,
@@ -2067,7 +2070,7 @@ static nd_status sort_tri_rows(nd_incidence* h, cudaStream_t st) {
     ND_CUDA(cudaFuncSetAttribute(k_row_rank<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     {
         nd_prof_scope ps("row_rank", st);
-        const int per = rows_per_warp(N);
+        const int per = rows_per_warp(h, N);
         const int blocks = nd_blocks_for((N + per - 1) / per * 32, 32 * kRankWarps, grid_cap(h) * 8);
         k_row_rank<false><<<blocks, 32 * kRankWarps, smem, st>>>(per, N, h->inc_ptr, h->e_u, h->e_v, h->rp,
                                                                   (const uint2*)h->inc, dst, over, over_ctr,
@@ -2111,7 +2114,7 @@ nd_status nd_build_tri_incidence(nd_incidence* h, cudaStream_t st) {
     nd_oriented o(st);
     ND_TRY(orient_graph(h, &o, st));
     const int eblocks = nd_blocks_for(m * 32, kThreads, grid_cap(h) * 4);  // a warp per oriented edge
-    const int per = rows_per_warp(m), pblocks = pool_blocks(m, per, grid_cap(h) * 4);
+    const int per = rows_per_warp(h, m), pblocks = pool_blocks(m, per, grid_cap(h) * 4);
     // the stored adjacency layout keeps the count pass's triangles as records
     // (4 B each, min(|out(u)|, |out(v)|) slots reserved per oriented edge), so
     // that the fill does not search again; without the memory for them the

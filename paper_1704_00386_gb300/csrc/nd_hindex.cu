@@ -183,6 +183,7 @@ __device__ __forceinline__ uint32_t ld_id(const uint32_t* p) {
 // registers and issue slots)
 template <int Q, bool RO, typename T>
 struct Rho {
+    static constexpr bool kCarry = RO && Q != 2;  // see warp_hindex
     const uint32_t* __restrict__ row;
     int d;  // (3,4): the length of the row's runs
     const T* tau;
@@ -205,6 +206,7 @@ struct Rho {
 // slot -> r-clique -> tau
 template <int Q, bool RO>
 struct RhoExact {
+    static constexpr bool kCarry = RO && Q != 2;
     const uint32_t* __restrict__ row;
     int d;
     const uint32_t* __restrict__ eid;
@@ -985,6 +987,7 @@ __global__ void k_add_const(const int32_t* __restrict__ in, int64_t n, int32_t c
 // order).
 template <bool RO, bool EXACT>
 struct OtfRow {
+    static constexpr bool kCarry = false;
     const int32_t* __restrict__ scol;   // N(s), sn entries: in CSR order from slot sb, or
     const uint32_t* __restrict__ slot;  // with a table, by degree class, and their slots
     int64_t sb, lb;  // first slots of N(s) and of the longer list N(l)

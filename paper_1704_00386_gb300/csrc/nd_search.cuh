@@ -133,10 +133,10 @@ __device__ __forceinline__ int bin_shift(unsigned span, int bins) {
 // last bin.  #{rho >= lo + (b << shift)} is above plus the suffix sum from b,
 // and H lies in the last bin whose sum reaches its lower edge (bin 0 where none
 // does: #{rho >= lo} >= lo has been seen).  Blocks of 128 bins from the top, four
-// to a lane.
+// to a lane; returns the bin, with CARRY also the count past it, in `above`.
 // PK: 16-bit counters, bin b in half b / HW of word b % HW.
-template <bool PK, int HW>
-__device__ __forceinline__ int select_bin(const unsigned* bins, int lo, int shift, int nb, int above) {
+template <bool PK, int HW, bool CARRY>
+__device__ __forceinline__ int select_bin(const unsigned* bins, int lo, int shift, int nb, int& above) {
     const int lane = threadIdx.x & 31;
     for (int c = (nb - 1) >> 7;; --c) {
         const int b0 = 128 * c;
@@ -155,14 +155,15 @@ __device__ __forceinline__ int select_bin(const unsigned* bins, int lo, int shif
         const int after = above + incl - s0;  // rho past this lane's bins
         // lower edges; unsigned, because those of the padding past nb may leave 31 bits
         const unsigned e0 = (unsigned)lo + ((unsigned)(b0 + 4 * lane) << shift), w1 = 1u << shift;
-        int best = -1;
-        if ((unsigned)(after + s0) >= e0) best = 0;
-        if ((unsigned)(after + s1) >= e0 + w1) best = 1;
-        if ((unsigned)(after + s2) >= e0 + 2 * w1) best = 2;
-        if ((unsigned)(after + s3) >= e0 + 3 * w1) best = 3;
+        int best = -1, past = 0;
+        if ((unsigned)(after + s0) >= e0) { best = 0; past = after + s1; }
+        if ((unsigned)(after + s1) >= e0 + w1) { best = 1; past = after + s2; }
+        if ((unsigned)(after + s2) >= e0 + 2 * w1) { best = 2; past = after + s3; }
+        if ((unsigned)(after + s3) >= e0 + 3 * w1) { best = 3; past = after; }
         const unsigned hit = __ballot_sync(0xffffffffu, best >= 0);
         if (hit || c == 0) {
             const int src = hit ? 31 - __clz(hit) : 0;
+            if (CARRY) above = __shfl_sync(0xffffffffu, past, src);
             return b0 + 4 * src + max(__shfl_sync(0xffffffffu, best, src), 0);
         }
         above += __shfl_sync(0xffffffffu, incl, 0);
@@ -189,13 +190,18 @@ __device__ __forceinline__ int select_bin(const unsigned* bins, int lo, int shif
 // x <= tau(R).  With one sweep's counts, what no longer supports h has fallen
 // below h, and so notifies R.  The same holds for lo, the bound of an earlier
 // sweep.  (tests/test_row_search.py plays the interleaving.)
+// F::kCarry: the values are the same at every reading (SND), and the count is
+// carried from sweep to sweep.  That is for (1,2) and (3,4): SND of an R-MAT
+// k-core of 16.7M vertices 76.6 against 78.5 ms with a fresh count, Chung-Lu 100K
+// (3,4) 40.2 against 41.0; the k-truss counts afresh, R-MAT of 1,048,576 vertices
+// 108.9 against 118.4 ms (the kernels spill differently).
 // bound: a count also stops where the rest of the row cannot reach t.
 template <bool PK, int HW, typename F, typename B>
 __device__ __forceinline__ int32_t warp_hindex(const F& rho, const B& bound, int d, int32_t t, bool direct,
                                                unsigned* bins) {
     const int lane = threadIdx.x & 31;
     if (t <= 0) return 0;
-    int lo = 0, hi = t;
+    int lo = 0, hi = t, above = 0;
     if (!direct) {
         int cnt = 0, have = 0;
         for (int i = 0; i < d;) {
@@ -207,7 +213,7 @@ __device__ __forceinline__ int32_t warp_hindex(const F& rho, const B& bound, int
             if (have >= t) return t;
             if (bound.past(end)) break;
         }
-        lo = have;  // #{rho >= lo} >= lo holds; at hi it fails
+        lo = above = have;  // #{rho >= lo} >= lo holds; at hi it fails
         if (hi - lo <= 1) return lo;
     }
     for (;;) {
@@ -229,9 +235,15 @@ __device__ __forceinline__ int32_t warp_hindex(const F& rho, const B& bound, int
             }
         });
         __syncwarp();
-        const int above = (int)__reduce_add_sync(0xffffffffu, (unsigned)ge);
-        if (above >= hi) return hi;  // a direct row's first sweep: hi is t
-        const int b = select_bin<PK, HW>(bins, lo, shift, nb, above);
+        if (!F::kCarry) {
+            above = (int)__reduce_add_sync(0xffffffffu, (unsigned)ge);
+            if (above >= hi) return hi;  // a direct row's first sweep: hi is t
+        } else if (direct) {
+            above = (int)__reduce_add_sync(0xffffffffu, (unsigned)ge);
+            if (above >= t) return t;
+            direct = false;
+        }
+        const int b = select_bin<PK, HW, F::kCarry>(bins, lo, shift, nb, above);
         lo += b << shift;
         hi = min(hi, lo + (1 << shift));
         if (hi - lo <= 1) return lo;
@@ -264,7 +276,7 @@ __device__ __forceinline__ int32_t cta_hindex(const F& rho, const B& bound, int 
         __syncthreads();
         return tot;
     };
-    int lo = 0, hi = t;
+    int lo = 0, hi = t, above = 0;
     if (!direct) {
         int cnt = 0, have = 0;
         for (int i = 0; i < d;) {
@@ -276,7 +288,7 @@ __device__ __forceinline__ int32_t cta_hindex(const F& rho, const B& bound, int 
             if (have >= t) return t;
             if (bound.past(end)) break;
         }
-        lo = have;
+        lo = above = have;
         if (hi - lo <= 1) return lo;
     }
     for (;;) {
@@ -300,19 +312,31 @@ __device__ __forceinline__ int32_t cta_hindex(const F& rho, const B& bound, int 
             u = m;
             __syncthreads();  // the bins so far are complete
             // #{rho >= u} from the bins at or past u
-            int c = ge;
+            int c = !F::kCarry || direct ? ge : (threadIdx.x == 0 ? above : 0);
             for (int b = (int)(((unsigned)(u - lo) + (1u << shift) - 1) >> shift) + threadIdx.x; b < nb; b += kThreads)
                 c += (int)bins[b];
             if (total(c) >= u) break;
         }
-        const int above = total(ge);  // with its barriers, the bins are complete too
-        if (above >= hi) return hi;
+        if (!F::kCarry) {
+            above = total(ge);  // with its barriers, the bins are complete too
+            if (above >= hi) return hi;
+        } else if (direct) {
+            above = total(ge);
+            if (above >= t) return t;
+            direct = false;
+        } else {
+            __syncthreads();
+        }
         if (threadIdx.x < 32) {
-            const int b = select_bin<false, WORDS>(bins, lo, shift, nb, above);
-            if (threadIdx.x == 0) bounds[0] = b;
+            const int b = select_bin<false, WORDS, F::kCarry>(bins, lo, shift, nb, above);
+            if (threadIdx.x == 0) {
+                bounds[0] = b;
+                if (F::kCarry) bounds[1] = above;
+            }
         }
         __syncthreads();
         lo += bounds[0] << shift;
+        if (F::kCarry) above = bounds[1];
         __syncthreads();
         hi = min(hi, lo + (1 << shift));
         if (hi - lo <= 1) return lo;

@@ -117,7 +117,9 @@ struct Row {
     std::vector<int> oct;             // 32 bounds
     int t;
 };
+template <bool CARRY>
 struct Falling {
+    static constexpr bool kCarry = CARRY;
     const Row* row;
     int* reads;
     int operator()(int j) const { return row->v[std::min(reads[j]++, (int)row->v.size() - 1)][j]; }
@@ -130,12 +132,14 @@ static int hindex(std::vector<int> a, int t) {
 }
 
 // kind 0: a warp, 16-bit bins; 1: a warp, 32-bit bins; 2: a block; 3: a block, rows bounded by octave
+// CARRY: for rows that do not fall (SND)
+template <bool CARRY>
 static int search(const Row& row, int kind, bool direct) {
     alignas(16) static unsigned bins[1024];
     static int bounds[8];
     const int d = (int)row.v[0].size();
     std::vector<int> reads(d, 0);
-    const Falling rho{&row, reads.data()};
+    const Falling<CARRY> rho{&row, reads.data()};
     int h = -1;
     run_lanes(kind < 2 ? 32 : kLanes, [&] {
         int x;
@@ -192,7 +196,7 @@ int main() {
             row.v.push_back(a);
         }
         ++rows;
-        const int h = search(row, kind, direct);
+        const int h = search<false>(row, kind, direct);
         const int truth = hindex(a, row.t), first = hindex(row.v[0], row.t);
         // the walks, after the store of h
         bool notified = false;
@@ -203,6 +207,13 @@ int main() {
             ++bad;
             printf("row %d, kind %d, direct %d: d %d, t %d, h %d, h-index %d at the first reading, %d after the stores%s\n",
                    trial, kind, (int)direct, d, row.t, h, first, truth, notified ? "" : ", not notified");
+        }
+        row.v.resize(1);
+        const int still = search<false>(row, kind, direct), carried = search<true>(row, kind, direct);
+        if (still != first || carried != first) {
+            ++bad;
+            printf("row %d, kind %d, direct %d, values that stay: %d, %d carried, h-index %d\n", trial, kind, (int)direct,
+                   still, carried, first);
         }
     }
     printf("%d rows, %d briefly too high, %d wrong\n", rows, high, bad);

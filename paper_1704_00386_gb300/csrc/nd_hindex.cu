@@ -20,12 +20,13 @@
 // counts rho >= tau(R) and stops at tau(R) of them; a row that fails, or is
 // expected to, goes through a shared-memory histogram of rho over the values
 // that can be H, whose suffix sums give H.
+// (The routines that search a row are in nd_search.cuh.)
 // What bounds a pass: the L1 wavefronts of the gathers, and in the early
 // passes the instructions of the search.  R-MAT scale-20 k-truss (1.17G
-// incidences), SND to convergence in 57 passes: 113.1 ms, against 184.3 ms
+// incidences), SND to convergence in 57 passes: 109.0 ms, against 184.3 ms
 // with 64-bit row offsets, a runtime division per binned value, whole rows
 // read in every pass and 16-bit values cached in shared memory between a
-// count and its search; AND 53.0 against 72.9 ms, AND-nn 63.6 against 105.8.
+// count and its search; AND 48.0 against 72.9 ms, AND-nn 64.4 against 105.8.
 // The paper's linear-time hashmap h-index (Section 4.4) is replaced by this
 // tau-bounded count; both compute Def. 3 exactly.
 //
